@@ -121,7 +121,7 @@ def _prepare_step(case, seed):
     lens, o, status = _lens(case, seed), torch.empty(b, h, 128, device="cuda"), _status()
     step = mqa.AppendStep(x["q"], x["K"], x["V"], x["k_new"], x["v_new"], lens, o, mqa.alloc_workspace(b, h, m, "cuda"), status,
                           advance=False, chained=case["chained"])
-    return dict(op="step", step=step, out=dict(o=o, K=x["K"], V=x["V"], lens=lens, status=status))
+    return dict(op="step", step=step, x=x, out=dict(o=o, K=x["K"], V=x["V"], lens=lens, status=status))
 
 
 def _prepare_loop(case, seed):
@@ -214,6 +214,89 @@ def run(state):
         return dict(o=state["o"], K=x["K"], V=x["V"], status=state["status"])
     mqa.mqa_prefill_attention(state["Q"], state["K"], state["V"], state["O"], state["ws"], state["start"], state["status"])
     return dict(O=state["O"], status=state["status"])
+
+
+def _attend(q, K, V, rows):
+    """In 64 bits: softmax(q K^T) V over the first `rows` rows of one sequence's cache (q [..., 128]; K, V [m, 128])."""
+    K, V = K[:rows].double(), V[:rows].double()
+    return torch.softmax(q.double() @ K.T, -1) @ V
+
+
+def _with_row(cache, new, row):
+    """One sequence's cache with the new row in its place (a copy; the given one stays as it is)."""
+    cache = cache.clone()
+    cache[row] = new.to(cache.dtype)
+    return cache
+
+
+def _exact_step(case, state):
+    x, lens = state["x"], state["out"]["lens"].tolist()
+    o = torch.stack([_attend(x["q"][i], _with_row(x["K"][i], x["k_new"][i], n), _with_row(x["V"][i], x["v_new"][i], n), n + 1)
+                     for i, n in enumerate(lens)])
+    return dict(o=o, K=None, V=None, lens=None, status=None)
+
+
+def _exact_loop(case, state):
+    q, k_new, v_new, _ = state["keep"]
+    keys, values = k_new.transpose(0, 1).double(), v_new.transpose(0, 1).double()
+    o = torch.stack([torch.softmax(q[t].double() @ keys[:, : t + 1].transpose(1, 2), -1) @ values[:, : t + 1] for t in range(case["m"])])
+    return dict(o=o, K=None, V=None, lens=None, status=None)
+
+
+def _exact_mha(case, state):
+    x, lens = state["x"], state["lens"].tolist()
+    o = torch.empty(case["b"], case["h"], 128, dtype=torch.float64, device="cuda")
+    for i, n in enumerate(lens):
+        K, V = x["K"][i, :, : n + 1].double(), x["V"][i, :, : n + 1].double()
+        K[:, n], V[:, n] = x["k_new"][i].double(), x["v_new"][i].double()
+        o[i] = (torch.softmax(x["q"][i].double().unsqueeze(1) @ K.transpose(1, 2), -1) @ V).squeeze(1)
+    return dict(o=o, K=None, V=None, status=None)
+
+
+def _exact_prefill(case, state):
+    b, h, n = case["b"], case["h"], case["n"]
+    Q, K, V = state["Q"], state["K"], state["V"]
+    starts = [0] * b if state["start"] is None else state["start"].tolist()
+    O = torch.empty(b, h, n, 128, dtype=torch.float64, device="cuda")
+    for i, first in enumerate(starts):
+        keys, values = K[i, : first + n].double(), V[i, : first + n].double()
+        hidden = torch.ones(n, first + n, dtype=torch.bool, device="cuda").triu(first + 1)
+        for g in range(h):
+            O[i, g] = torch.softmax((Q[i, g].double() @ keys.T).masked_fill_(hidden, -math.inf), -1) @ values
+    return dict(O=O, status=None)
+
+
+def _exact_layer(case, state):
+    y = []
+    for x, P_q, P_k, P_v, P_o, K, V, lens in state["keep"][0]:
+        x = x.double()
+        q, k_new, v_new = torch.einsum("bd,hdk->bhk", x, P_q.double()), x @ P_k.double(), x @ P_v.double()
+        o = []
+        for i, n in enumerate(lens.tolist()):
+            rows, values = K[i, : n + 1].double(), V[i, : n + 1].double()
+            rows[n], values[n] = k_new[i], v_new[i]
+            o.append(_attend(q[i], rows, values, n + 1))
+        y.append(torch.einsum("bhv,hdv->bd", torch.stack(o), P_o.double()))
+    return dict(y=torch.stack(y), status=None, K=None, V=None)
+
+
+def _exact_local(case, state):
+    w, o = case["window"], []
+    for q, K, V, k_new, v_new, pos in state["keep"]:
+        K, V, at = K.double(), V.double(), pos.long()
+        each = torch.arange(case["b"], device="cuda")
+        K[each, at % w], V[each, at % w] = k_new.double(), v_new.double()
+        unused = torch.arange(w, device="cuda") >= (at + 1).clamp(max=w)[:, None]
+        s = (q.double() @ K.transpose(1, 2)).masked_fill_(unused[:, None, :], -math.inf)
+        o.append(torch.softmax(s, -1) @ V)
+    return dict(o=torch.stack(o), status=None, K=None, V=None)
+
+
+def exact(case, seed):
+    """What ``run`` computes for these inputs, in 64 bits and without intermediate roundings; the caches and counters it also
+    returns are copies of bytes and whole numbers."""
+    by_op = dict(step=_exact_step, loop=_exact_loop, mha=_exact_mha, prefill=_exact_prefill, layer=_exact_layer, local=_exact_local)
+    return by_op[case["op"]](case, prepare(case, seed))
 
 
 def _mean_rows(case):
