@@ -356,16 +356,16 @@ bool encode_cache_map(CUtensorMap* map, const void* base, long long rows, int bo
     return encode_matrix_map(map, base, rows, kHeadDim, box_rows);
 }
 
-std::atomic<int> g_smem_opt_in[kMaxDevices][4];
+std::atomic<int> g_smem_opt_in[kMaxDevices][6];
 
-template <int M_TILES, bool EARLY = false>
+template <int M_TILES, int EARLY = 0>
 int launch_mma(const Plan& p, const void* q, const void* K, const void* V, const int32_t* lens, float* o,
                float2* part_ml, float* part_acc, int32_t* status, int b, int h, int m_max, cudaStream_t stream, int len_bias,
                const void* k_new = nullptr, const void* v_new = nullptr, int32_t* lens_advance = nullptr,
                bool withhold = false) {
     using Cfg = MmaCfg<M_TILES>;
     auto kernel = mqa_decode_split_mma_kernel<M_TILES, EARLY>;
-    constexpr int kSlot = (M_TILES - 1) * 2 + (EARLY ? 1 : 0);
+    constexpr int kSlot = (M_TILES - 1) * 3 + EARLY;
     int dev = 0;
     if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxDevices) { cudaGetLastError(); return MQA_ERR_CUDA; }
     if (!g_smem_opt_in[dev][kSlot].load(std::memory_order_acquire)) {
@@ -381,7 +381,7 @@ int launch_mma(const Plan& p, const void* q, const void* K, const void* V, const
         !encode_cache_map(&map_v_big, V, (long long)b * m_max, 4 * kTileRows))
         return MQA_ERR_CUDA;
     FusedArgs fa = {};
-    if (k_new) {                                       // the whole decoding step in this launch (one CTA per sequence)
+    if (k_new) {                                       // the append-and-attend step
         fa.k_new = static_cast<const uint4*>(k_new);
         fa.v_new = static_cast<const uint4*>(v_new);
         fa.K = static_cast<uint4*>(const_cast<void*>(K));
@@ -792,22 +792,6 @@ static int append_step_impl(const void* q, void* K, void* V, const void* k_new, 
     }
     // other plans: the same step as separate launches.  Without `advance` the append leaves lens alone and
     // the step is told that a sequence which took a row has one more row than lens says.
-    if ((p.kernel == Kernel::kMma1 || p.kernel == Kernel::kMma2) && p.n_splits == 1) {
-        // one CTA per sequence: it writes the row, attends and moves lens on, all in one launch
-        // tiles below the prefix's last rows are fetched ahead of the wait (measured: 5.70 -> 5.45 us per step over the
-        // 128 steps of a cache growing to 128 rows; nothing gained, 0.2 us lost, at 512 rows)
-        if (early == kEarlyChained && m_max <= 8 * kTileRows && !withhold)
-            return p.kernel == Kernel::kMma1
-                       ? launch_mma<1, true>(p, q, K, V, lens, o, nullptr, nullptr, status, b, h, m_max, stream, 0, k_new, v_new,
-                                             advance ? lens : nullptr)
-                       : launch_mma<2, true>(p, q, K, V, lens, o, nullptr, nullptr, status, b, h, m_max, stream, 0, k_new, v_new,
-                                             advance ? lens : nullptr);
-        return p.kernel == Kernel::kMma1
-                   ? launch_mma<1>(p, q, K, V, lens, o, nullptr, nullptr, status, b, h, m_max, stream, 0, k_new, v_new,
-                                   advance ? lens : nullptr, withhold)
-                   : launch_mma<2>(p, q, K, V, lens, o, nullptr, nullptr, status, b, h, m_max, stream, 0, k_new, v_new,
-                                   advance ? lens : nullptr, withhold);
-    }
     if (p.kernel == Kernel::kWide) {
         // many query rows: the CTA whose rows hold the new one writes it; one split per sequence moves lens on itself,
         // otherwise the second pass does.  One or two launches.
@@ -824,14 +808,23 @@ static int append_step_impl(const void* q, void* K, void* V, const void* k_new, 
         }
         return run_combine(true, lens, o, workspace, workspace_bytes, b, h, m_max, k, v, stream, 0, advance ? lens : nullptr, true);
     }
-    if ((p.kernel == Kernel::kMma1 || p.kernel == Kernel::kMma2) && p.n_splits > 1) {
-        // fixed splits: the CTA whose rows hold the new one writes it; the second pass moves lens on.  Two launches.
-        float2* part_ml = partials_ml(workspace);
-        float* part_acc = partials_acc(p, workspace);
-        rc = p.kernel == Kernel::kMma1
-                 ? launch_mma<1>(p, q, K, V, lens, o, part_ml, part_acc, status, b, h, m_max, stream, 0, k_new, v_new, nullptr, withhold)
-                 : launch_mma<2>(p, q, K, V, lens, o, part_ml, part_acc, status, b, h, m_max, stream, 0, k_new, v_new, nullptr, withhold);
-        if (rc) return rc;
+    if (p.kernel == Kernel::kMma1 || p.kernel == Kernel::kMma2) {
+        // one CTA per sequence writes the row, attends and moves lens on, all in one launch; of several splits the CTA whose
+        // rows hold the new one writes it and the second pass moves lens on.  What is fetched ahead of the wait: EARLY in
+        // decode_mma.cuh.
+        const bool alone = p.n_splits == 1;
+        float2* part_ml = alone ? nullptr : partials_ml(workspace);
+        float* part_acc = alone ? nullptr : partials_acc(p, workspace);
+        int32_t* move_lens = alone && advance ? lens : nullptr;
+#define MQA_MMA_STEP(TILES, EARLY) \
+    launch_mma<TILES, EARLY>(p, q, K, V, lens, o, part_ml, part_acc, status, b, h, m_max, stream, 0, k_new, v_new, move_lens, withhold)
+        const int ahead = withhold ? 0 : early == kEarlyChained ? 1 : early == kEarlyAfterProjection ? 2 : 0;
+        if (p.kernel == Kernel::kMma1)
+            rc = ahead == 1 ? MQA_MMA_STEP(1, 1) : ahead == 2 ? MQA_MMA_STEP(1, 2) : MQA_MMA_STEP(1, 0);
+        else
+            rc = ahead == 1 ? MQA_MMA_STEP(2, 1) : ahead == 2 ? MQA_MMA_STEP(2, 2) : MQA_MMA_STEP(2, 0);
+#undef MQA_MMA_STEP
+        if (rc || alone) return rc;
         return run_combine(true, lens, o, workspace, workspace_bytes, b, h, m_max, k, v, stream, 0, advance ? lens : nullptr, true);
     }
     rc = kv_cache_append(K, V, k_new, v_new, lens, 0, status, b, 1, m_max, k, v, stream_);

@@ -98,6 +98,7 @@ combine_splits_kernel(const float2* __restrict__ part_ml, const float* __restric
                       int h, int m_max, int chunk_rows, int n_splits, int len_bias, int32_t* __restrict__ lens_advance) {
     const size_t u = blockIdx.x;
     grid_dependency_wait();          // the partials come from the kernel before this one
+    grid_launch_dependents();        // the next step's kernel sets itself up meanwhile (it waits for this one before it writes)
     // lens == nullptr: every split wrote its piece (an empty one has max = -inf) and nobody here looks at lens, so
     // the CTA of a sequence's first head may move it on (lens_advance: the append-and-attend step)
     int live = n_splits;
@@ -132,6 +133,7 @@ combine_few_kernel(const float2* __restrict__ part_ml, const float* __restrict__
     const int lane = threadIdx.x & 31;
     const size_t u = (size_t)blockIdx.x * kCombineFewWarps + (threadIdx.x >> 5);
     grid_dependency_wait();          // the partials come from the kernel before this one
+    grid_launch_dependents();        // the next step's kernel sets itself up meanwhile (it waits for this one before it writes)
     if (u >= units) return;
     int live = n_splits;
     if (lens != nullptr) {

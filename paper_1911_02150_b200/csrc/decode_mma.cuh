@@ -319,42 +319,23 @@ __device__ __forceinline__ void consume_tile(WarpState& st, const uint32_t (&qa)
     }
 }
 
-// Merge `other` (the same heads over other rows) into `st`.  Either side may be empty (m = -inf).
-__device__ __forceinline__ void merge_state(WarpState& st, const float* __restrict__ other, int lane) {
-    // `other` is thread-private storage: float index r * 32 + lane, r = 0..63 acc, 64..65 m, 66..67 l
-    float wa[2], wb[2];
-#pragma unroll
-    for (int r = 0; r < 2; ++r) {
-        const float mb = other[(64 + r) * 32 + lane];
-        const float lb = other[(66 + r) * 32 + lane];
-        const float m_new = fmaxf(st.m[r], mb);
-        wa[r] = st.m[r] == -INFINITY ? 0.f : fast_exp2(st.m[r] - m_new);
-        wb[r] = mb == -INFINITY ? 0.f : fast_exp2(mb - m_new);
-        st.m[r] = m_new;
-        st.l[r] = st.l[r] * wa[r] + lb * wb[r];
-    }
-#pragma unroll
-    for (int vt = 0; vt < 16; ++vt) {
-#pragma unroll
-        for (int j = 0; j < 4; ++j)
-            st.acc[vt][j] = st.acc[vt][j] * wa[j >> 1] + other[(vt * 4 + j) * 32 + lane] * wb[j >> 1];
-    }
-}
-
-__device__ __forceinline__ void store_state(const WarpState& st, float* __restrict__ dst, int lane) {
-#pragma unroll
-    for (int vt = 0; vt < 16; ++vt) {
-#pragma unroll
-        for (int j = 0; j < 4; ++j) dst[(vt * 4 + j) * 32 + lane] = st.acc[vt][j];
-    }
-    dst[64 * 32 + lane] = st.m[0]; dst[65 * 32 + lane] = st.m[1];
-    dst[66 * 32 + lane] = st.l[0]; dst[67 * 32 + lane] = st.l[1];
-}
-
 // =============================================================================================
 // Fixed-split kernel: one CTA per (sequence, split of chunk_rows rows).
+//
+// What bounds it is a chain of round trips, not bytes: the paper's step moves 9 MB in all, 1.4 us at the copy rate, and
+// takes several.  So everything that does not need the kernel before is done ahead of the wait for it (EARLY), and after
+// the wait the loads of lens, q, the new row and the last tiles are all in flight together: the new row is not stored,
+// fenced and fetched again, it goes from registers into its place in the landed tile (and, with nobody waiting, into the
+// cache).  Measured over the paper's 128 steps (128 sequences, 8 heads, the cache growing to 128 rows): 5.0 -> 3.8 us per
+// step, with the merge's stores no longer meeting in the same banks.
+// EARLY  0  nothing is fetched before the wait
+//        1  the caller's promise that only this library's steps have written the cache and lens since its last step on
+//           them (a decoding loop): lens as it reads now is final or one short of it, so tiles that lie wholly below the
+//           prefix's last rows are fetched ahead of the wait and the rest right behind it, without waiting for lens
+//        2  behind this library's input projection (or the host step's input kernel), which has waited for everything
+//           that writes the cache and lens: lens is final, and all the tiles are fetched ahead of the wait
 // =============================================================================================
-template <int M_TILES, bool EARLY = false>
+template <int M_TILES, int EARLY = 0>
 __global__ void __launch_bounds__(MmaCfg<M_TILES>::kThreads, MmaCfg<M_TILES>::kMinBlocks)
 mqa_decode_split_mma_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_constant__ CUtensorMap map_v,
                             const __grid_constant__ CUtensorMap map_k_big, const __grid_constant__ CUtensorMap map_v_big,
@@ -368,6 +349,7 @@ mqa_decode_split_mma_kernel(const __grid_constant__ CUtensorMap map_k, const __g
     const int seq = blockIdx.x / n_splits;
     const int split = blockIdx.x % n_splits;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const bool producer = warp == Cfg::kConsumerWarps && lane == 0;
 
     extern __shared__ uint8_t smem_raw[];
     // 1 KiB alignment in the shared window: the 128-byte swizzle repeats every 8 rows x 128 bytes
@@ -375,10 +357,10 @@ mqa_decode_split_mma_kernel(const __grid_constant__ CUtensorMap map_k, const __g
     uint64_t* bars = reinterpret_cast<uint64_t*>(stages + kStages * kStageBytes);   // full[kStages], empty[kStages]
     const uint32_t stages_s = smem_addr(stages);
     const uint32_t full_s = smem_addr(bars), empty_s = full_s + kStages * 8;
-    __shared__ int timed_out, issued;   // a wait ran out; tiles whose copies were started
+    __shared__ int timed_out, issued;   // a wait ran out; tiles (or groups of four) whose copies were started
 
     // set up by the thread that issues the copies (it may issue some before the first CTA-wide barrier)
-    if (warp == Cfg::kConsumerWarps && lane == 0) {
+    if (producer) {
         prefetch_tensormap(&map_k); prefetch_tensormap(&map_v);
         timed_out = 0;
         issued = 0;
@@ -389,7 +371,8 @@ mqa_decode_split_mma_kernel(const __grid_constant__ CUtensorMap map_k, const __g
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
     }
-    const int row_base = seq * m_max + split * chunk_rows; // row coordinate in the [b*m_max, 128] view
+    const int r0 = split * chunk_rows;
+    const int row_base = seq * m_max + r0;                 // row coordinate in the [b*m_max, 128] view
     auto issue_tile = [&](int i) {
         const int s = i % kStages;
         const uint32_t bar = full_s + s * 8;
@@ -402,44 +385,78 @@ mqa_decode_split_mma_kernel(const __grid_constant__ CUtensorMap map_k, const __g
         if (!(withhold && blockIdx.x == 0 && i == 1)) tma_load_2d(dst + 3 * kBoxBytes, &map_v, kBoxCols, y, bar);
         issued = i + 1;
     };
-    // EARLY (the caller's promise that only this library's steps have written the cache and lens since its last step
-    // on them): one CTA owns the sequence, its tiles are tiles 0, 1, ... whatever lens says, so those that lie wholly
-    // below the prefix's last two rows -- by lens as it reads now, which the step ahead may be about to advance -- are
-    // fetched while that step is still finishing.  Only their number is a guess: should fewer tiles count in the end,
-    // the surplus is left to land and ignored.
-    int pre = 0;
-    if (EARLY && n_splits == 1 && warp == Cfg::kConsumerWarps && lane == 0) {
-        const int raw_guess = __ldcg(lens + seq);
-        const int rows_guess = min(max(raw_guess, 0) + (fa.k_new != nullptr ? 1 : 0), m_max);
-        pre = min((rows_guess - 2) / kTileRows, kStages);
-        if (pre < 0) pre = 0;
-        for (int i = 0; i < pre; ++i) issue_tile(i);
+    // four tiles per copy: boxes of 128 rows (K columns 0-63, 64-127, V likewise), a quarter of the copies
+    auto issue_group = [&](int grp) {
+        const uint32_t bar = full_s + grp * 8, dst = stages_s + grp * 4 * kStageBytes;
+        mbar_expect_tx(bar, 4 * kStageBytes);
+        const int y = row_base + grp * 4 * kTileRows;
+        tma_load_2d(dst, &map_k_big, 0, y, bar);
+        tma_load_2d(dst + 4 * kBoxBytes, &map_k_big, kBoxCols, y, bar);
+        tma_load_2d(dst + 8 * kBoxBytes, &map_v_big, 0, y, bar);
+        tma_load_2d(dst + 12 * kBoxBytes, &map_v_big, kBoxCols, y, bar);
+        issued = grp + 1;
+    };
+    // a few tiles (each has a stage of its own), beginning at a multiple of 128 rows: fetched four tiles per copy
+    // (from three tiles on: a copy moves all 128 rows of its box, and one or two tiles are quicker on their own)
+    auto in_groups = [&](int tiles) { return EARLY != 1 && !withhold && tiles >= 3 && tiles <= kStages && (r0 & (4 * kTileRows - 1)) == 0; };
+    // rows of this split that hold tokens once the row at `length` (what lens says) has been appended
+    auto rows_of_split = [&](int length) {
+        const int rows = length < 0 ? 0 : min(length + (fa.k_new != nullptr && length < m_max ? 1 : 0), m_max);
+        return min(rows - r0, chunk_rows);
+    };
+    int pre = 0;                                           // tiles asked for so far (by the producer's thread)
+    bool pre_groups = false;
+    int guess = 0;
+    if (EARLY != 0 && producer) {
+        guess = __ldcg(lens + seq);
+        if (EARLY == 2) {
+            const int tiles = (rows_of_split(guess) + kTileRows - 1) / kTileRows;      // (<= 0: nothing in this split)
+            pre_groups = in_groups(tiles);
+            pre = max(0, min(tiles, kStages));
+            if (pre_groups) for (int grp = 0; grp * 4 < tiles; ++grp) issue_group(grp);
+            else for (int i = 0; i < pre; ++i) issue_tile(i);
+        } else {
+            // the step ahead, still running, writes row guess - 1 or row guess: the tiles below both
+            pre = max(0, min((min(max(guess, 0) - 1, min(m_max, r0 + chunk_rows)) - r0) / kTileRows, kStages));
+            for (int i = 0; i < pre; ++i) issue_tile(i);
+        }
     }
+    __syncthreads();
     // everything above overlaps the tail of the kernel before this one
-    grid_dependency_wait();          // lens and the newest cache row may come from the kernel before
+    grid_dependency_wait();          // lens, q and the newest cache row may come from the kernel before
     grid_launch_dependents();
+    if (EARLY == 1 && producer) {
+        // the rest of the rows there can be (lens is at most one more than it was, and takes a row): a surplus tile is left to
+        // land and ignored
+        const int rows = min(min(max(guess, 0) + 2, m_max) - r0, chunk_rows);
+        const int most = max(pre, min((rows + kTileRows - 1) / kTileRows, kStages));
+        for (; pre < most; ++pre) issue_tile(pre);
+    }
     // With one CTA per sequence (n_splits == 1) the CTA may do the whole decoding step: write the new row
     // (fa.k_new given), attend over one row more, and move lens[seq] on at the end (lens_advance given) --
     // nobody else reads this sequence's length.
     // A sequence cut into several splits (n_splits > 1) may take its new row too: the CTA whose rows hold it writes
     // it, every split attends over one row more, and lens is left to the second-pass kernel.
-    // (the new row's pieces do not depend on lens: asked for first, so that the two loads are in flight together)
-    uint4 row_piece = make_uint4(0u, 0u, 0u, 0u);
-    if (fa.k_new != nullptr && warp == 0)                 // lanes 0-15 move the key row, 16-31 the value row
+    // (lens, the new row's pieces and q are in flight together)
+    uint4 row_piece = make_uint4(0u, 0u, 0u, 0u);          // lanes 0-15: of the key row, 16-31: of the value row
+    if (fa.k_new != nullptr && warp < Cfg::kConsumerWarps)
         row_piece = (lane < 16 ? fa.k_new : fa.v_new)[(size_t)seq * (kRowBytes / 16) + (lane & 15)];
     const int raw = lens[seq];
+    const int mt = warp % M_TILES;                         // which 16-head tile this warp serves
+    const int rw = warp / M_TILES;                         // which tiles (round-robin over kRowWarps)
+    uint32_t qa[8][4];
+    if (warp < Cfg::kConsumerWarps) load_q_fragments(qa, q, (size_t)seq, h, mt, lane);
     const bool appended = fa.k_new != nullptr && raw >= 0 && raw < m_max;
+    const bool holds_new = appended && raw >= r0 && raw - r0 < chunk_rows;        // the new row is one of this split's
     if (fa.k_new != nullptr) {
         if (!appended && threadIdx.x == 0 && status) atomicOr(status, raw < 0 ? kStatusAppendNegative : kStatusAppendFull);
-        if (appended && warp == 0 && (n_splits == 1 || raw / chunk_rows == split)) {
+        if (holds_new && warp == 0) {
             const size_t dst = ((size_t)seq * m_max + raw) * (kRowBytes / 16) + (lane & 15);
             if (lane < 16) fa.K[dst] = row_piece; else fa.V[dst] = row_piece;
-            asm volatile("fence.proxy.async;" ::: "memory");   // the copy engine must see the row (a barrier follows)
         }
     }
     const int L = clamp_len(appended ? raw + 1 : biased_len(raw, m_max, len_bias), m_max,
                             threadIdx.x == 0 ? status : nullptr);
-    const int r0 = split * chunk_rows;
     const int r1 = min(L, r0 + chunk_rows);
     if (r0 >= L) {                                         // nothing valid in this split (uniform)
         if (n_splits == 1)                                 // L == 0: the empty prefix gives zeros
@@ -447,34 +464,18 @@ mqa_decode_split_mma_kernel(const __grid_constant__ CUtensorMap map_k, const __g
         else                                               // an empty piece, for a second pass that does not look at lens
             for (int i = threadIdx.x; i < h; i += Cfg::kThreads)
                 part_ml[((size_t)seq * h + i) * n_splits + split] = make_float2(-INFINITY, 0.f);
-        for (int i = 0; i < pre; ++i) mbar_wait(full_s + i * 8, 0);   // copies started on a guess land before the CTA leaves
+        for (int i = 0; i < pre; ++i) mbar_wait(full_s + i * 8, 0);   // copies already started land before the CTA leaves
         return;
     }
     const int n_tiles = (r1 - r0 + kTileRows - 1) / kTileRows;
-    // a few tiles (each has a stage of its own), beginning at a multiple of 128 rows: fetched four tiles per copy
-    // (from three tiles on: a copy moves all 128 rows of its box, and one or two tiles are quicker on their own)
-    const bool big = !EARLY && !withhold && n_tiles >= 3 && n_tiles <= kStages && (r0 & (4 * kTileRows - 1)) == 0;
+    const bool big = in_groups(n_tiles);
 
-    __syncthreads();
-
-    const int mt = warp % M_TILES;                         // which 16-head tile this warp serves
-    const int rw = warp / M_TILES;                         // which tiles (round-robin over kRowWarps)
     WarpState st;
 
     if (warp == Cfg::kConsumerWarps) {
         // ------------------------------------------------------------------ producer warp
         if (lane == 0 && big) {
-            // four tiles per copy: boxes of 128 rows (K columns 0-63, 64-127, V likewise), a quarter of the copies
-            for (int grp = 0; grp * 4 < n_tiles; ++grp) {
-                const uint32_t bar = full_s + grp * 8, dst = stages_s + grp * 4 * kStageBytes;
-                mbar_expect_tx(bar, 4 * kStageBytes);
-                const int y = row_base + grp * 4 * kTileRows;
-                tma_load_2d(dst, &map_k_big, 0, y, bar);
-                tma_load_2d(dst + 4 * kBoxBytes, &map_k_big, kBoxCols, y, bar);
-                tma_load_2d(dst + 8 * kBoxBytes, &map_v_big, 0, y, bar);
-                tma_load_2d(dst + 12 * kBoxBytes, &map_v_big, kBoxCols, y, bar);
-                issued = grp + 1;
-            }
+            if (!pre_groups) for (int grp = 0; grp * 4 < n_tiles; ++grp) issue_group(grp);
         } else if (lane == 0) {
             bool ok = true;
             for (int i = pre; i < n_tiles && ok; ++i) {
@@ -489,8 +490,6 @@ mqa_decode_split_mma_kernel(const __grid_constant__ CUtensorMap map_k, const __g
     } else {
         // --------------------------------------------------------------- consumer warps
         st.reset();
-        uint32_t qa[8][4];
-        load_q_fragments(qa, q, (size_t)seq, h, mt, lane);
         LaneOffsets off;
         off.init(lane);
         bool ok = true;
@@ -501,6 +500,14 @@ mqa_decode_split_mma_kernel(const __grid_constant__ CUtensorMap map_k, const __g
             // a tile's K boxes, then its V boxes; in a copy of four tiles the tile is 32 of a box's 128 rows
             const uint32_t k_s = big ? stages_s + (i >> 2) * 4 * kStageBytes + (i & 3) * kBoxBytes : stages_s + s * kStageBytes;
             const uint32_t half = big ? 4 * kBoxBytes : kBoxBytes;
+            if (holds_new && (raw - r0) / kTileRows == i) {
+                // the new row into its place (with two head tiles both warps that read this tile write the same bytes)
+                const int row = (raw - r0) & (kTileRows - 1), c = lane & 7;
+                const uint32_t at = k_s + (lane >> 3) * half + row * 128 + ((c ^ (row & 7)) << 4);   // boxes: K, K, V, V
+                asm volatile("st.shared.v4.b32 [%0], {%1,%2,%3,%4};" ::"r"(at), "r"(row_piece.x), "r"(row_piece.y), "r"(row_piece.z),
+                             "r"(row_piece.w) : "memory");
+                __syncwarp();
+            }
             consume_tile<true>(st, qa, off, k_s, k_s + 2 * half, half, r0 + i * kTileRows, r1, lane);
             // The tile was read through the generic proxy (ldmatrix) and the copy engine will write the stage
             // again through the async proxy: without this fence the last ldmatrix of a tile now and then saw
@@ -541,8 +548,9 @@ mqa_decode_split_mma_kernel(const __grid_constant__ CUtensorMap map_k, const __g
         float* mine = sm_acc + (size_t)warp * 16 * kHeadDim;
 #pragma unroll
         for (int vt = 0; vt < 16; ++vt) {
-            *reinterpret_cast<float2*>(mine + g * kHeadDim + vt * 8 + t4 * 2) = make_float2(st.acc[vt][0], st.acc[vt][1]);
-            *reinterpret_cast<float2*>(mine + (g + 8) * kHeadDim + vt * 8 + t4 * 2) = make_float2(st.acc[vt][2], st.acc[vt][3]);
+            // (8-column groups XORed with the head: the eight heads of a store would otherwise meet in the same banks)
+            *reinterpret_cast<float2*>(mine + g * kHeadDim + ((vt ^ g) * 8) + t4 * 2) = make_float2(st.acc[vt][0], st.acc[vt][1]);
+            *reinterpret_cast<float2*>(mine + (g + 8) * kHeadDim + ((vt ^ g) * 8) + t4 * 2) = make_float2(st.acc[vt][2], st.acc[vt][3]);
         }
         if (t4 == 0) {
             sm_ml[warp * 16 + g] = make_float2(st.m[0], st.l[0]);
@@ -580,7 +588,8 @@ mqa_decode_split_mma_kernel(const __grid_constant__ CUtensorMap map_k, const __g
         float4 num = make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll
         for (int w = 0; w < kRowWarps; ++w) {
-            const float4 a = *reinterpret_cast<const float4*>(sm_acc + ((size_t)(w * M_TILES + tile) * 16 + hr) * kHeadDim + c4 * 4);
+            const float4 a = *reinterpret_cast<const float4*>(sm_acc + ((size_t)(w * M_TILES + tile) * 16 + hr) * kHeadDim +
+                                                               (((c4 >> 1) ^ (hr & 7)) * 8 + (c4 & 1) * 4));
             const float wt = wts[w];
             num.x = fmaf(wt, a.x, num.x); num.y = fmaf(wt, a.y, num.y); num.z = fmaf(wt, a.z, num.z); num.w = fmaf(wt, a.w, num.w);
         }

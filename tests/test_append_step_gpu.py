@@ -95,6 +95,15 @@ def test_append_step_with_the_chained_promise_matches_oracle(b, h, m_max, chaine
     run(b, h, m_max, lens_mix(b, m_max, seed=b + h + 1), True, seed=b * 5 + h, chained=chained)
 
 
+@pytest.mark.parametrize("chained", [False, True])
+@pytest.mark.parametrize("h,m_max", [(8, 128), (16, 700), (32, 130), (17, 900)])
+def test_new_row_at_the_edges_of_tiles_and_splits(h, m_max, chained):
+    """The fixed-split kernel puts the new row into the landed tile itself: rows either side of every edge of a 32-row tile,
+    of four tiles and of a split, one and two head tiles, one split and several."""
+    lens = sorted({min(m_max - 1, max(0, e + x)) for e in (0, 32, 64, 128, 160, 256, 320, 448, 512, 640, m_max) for x in (-2, -1, 0, 1)})
+    run(len(lens), h, m_max, lens, True, seed=h + m_max, chained=chained)
+
+
 def test_append_step_full_and_negative_sequences_take_no_row():
     b, h, m_max = 48, 16, 1024
     lens = lens_mix(b, m_max, seed=5)
