@@ -605,7 +605,7 @@ std::atomic<int> g_proj_opt_in[kMaxDevices][8];
 
 template <int NB>
 int launch_projections_in(const void* x, const void* P_q, const void* P_k, const void* P_v, void* q, void* k_new, void* v_new,
-                          int32_t* status, int b, int h, int d, cudaStream_t stream) {
+                          int32_t* status, int b, int h, int d, int parts, cudaStream_t stream) {
     using Cfg = ProjCfg<NB>;
     auto kernel = project_in_kernel<NB>;
     constexpr int kSlot = NB == 16 ? 0 : (NB == 32 ? 1 : (NB == 64 ? 2 : 3));
@@ -623,18 +623,34 @@ int launch_projections_in(const void* x, const void* P_q, const void* P_k, const
         !encode_matrix_map(&map_pv, P_v, d, kHeadDim, 128) || !encode_matrix_map(&map_x, x, b, d, NB))
         return MQA_ERR_CUDA;
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)(h + 2), (unsigned)((b + 127) / 128));
+    cfg.gridDim = dim3((unsigned)(h + 2), (unsigned)parts, (unsigned)((b + 127) / 128));
     cfg.blockDim = dim3(kProjThreads);
     cfg.dynamicSmemBytes = Cfg::kSmemBytes;
     cfg.stream = stream;
-    cudaLaunchAttribute attr[1];
+    cudaLaunchAttribute attr[2];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[0].val.programmaticStreamSerializationAllowed = 1;
+    attr[1].id = cudaLaunchAttributeClusterDimension;
+    attr[1].val.clusterDim.x = 1;
+    attr[1].val.clusterDim.y = (unsigned)parts;
+    attr[1].val.clusterDim.z = 1;
     cfg.attrs = attr;
-    cfg.numAttrs = 1;
+    cfg.numAttrs = parts > 1 ? 2 : 1;
     cudaLaunchKernelEx(&cfg, kernel, map_pq, map_pk, map_pv, map_x, static_cast<__nv_bfloat16*>(q),
                        static_cast<__nv_bfloat16*>(k_new), static_cast<__nv_bfloat16*>(v_new), status, b, h, d);
     return launch_status();
+}
+
+// CTAs (of one cluster) that share an input slab's d rows: as many as keep the kernel on half of the SMs.  A slab's rows are
+// a serial chain for one CTA, so a few CTAs per slab are quicker (per layer step, 1 / 2 / 4 / 8 CTAs per slab: 10 slabs of
+// 1024 rows 18.8 / 17.3 / 17.1 / 17.1 us; 4 slabs of 768 rows 29.1 / 28.1 / 27.6 / 26.8; 18 slabs of 2048 rows 22.1 / 19.8 / 18.0 /
+// 21.6), but the attention kernel behind it sets itself up and fetches its first stages on the SMs that this one leaves
+// free (34 slabs of 1024 rows in front of the streaming kernel 39.3 / 39.0 / 41.5 / 46.1; 34 of 2048: 26.3 / 24.3 / 27.8 / 31.0).
+int projection_parts(int b, int h, int d) {
+    const int slabs = (h + 2) * ((b + 127) / 128);
+    int parts = 1;
+    while (2 * parts <= kProjMaxParts && 2 * parts <= d / 128 && 4 * parts * slabs <= sm_count()) parts *= 2;
+    return parts;
 }
 
 // The output projection: the head groups of a (d tile, batch tile) are the CTAs of one thread-block cluster (see
@@ -982,12 +998,13 @@ int mqa_layer_decode_step(const void* x, const void* P_q, const void* P_k, const
     void* v_new = base + w.v_new;
     float* o = reinterpret_cast<float*>(base + w.o);
     const int nb = b >= 128 ? 128 : (b > 64 ? 128 : (b > 32 ? 64 : (b > 16 ? 32 : 16)));
+    const int parts = projection_parts(b, h, d);
     int rc;
     switch (nb) {
-        case 16: rc = launch_projections_in<16>(x, P_q, P_k, P_v, q, k_new, v_new, status, b, h, d, stream); break;
-        case 32: rc = launch_projections_in<32>(x, P_q, P_k, P_v, q, k_new, v_new, status, b, h, d, stream); break;
-        case 64: rc = launch_projections_in<64>(x, P_q, P_k, P_v, q, k_new, v_new, status, b, h, d, stream); break;
-        default: rc = launch_projections_in<128>(x, P_q, P_k, P_v, q, k_new, v_new, status, b, h, d, stream); break;
+        case 16: rc = launch_projections_in<16>(x, P_q, P_k, P_v, q, k_new, v_new, status, b, h, d, parts, stream); break;
+        case 32: rc = launch_projections_in<32>(x, P_q, P_k, P_v, q, k_new, v_new, status, b, h, d, parts, stream); break;
+        case 64: rc = launch_projections_in<64>(x, P_q, P_k, P_v, q, k_new, v_new, status, b, h, d, parts, stream); break;
+        default: rc = launch_projections_in<128>(x, P_q, P_k, P_v, q, k_new, v_new, status, b, h, d, parts, stream); break;
     }
     if (rc) return rc;
     rc = append_step_impl(q, K, V, k_new, v_new, lens, advance ? MQA_STEP_ADVANCE : 0, o, base + w.step, w.total - w.step, status,

@@ -11,10 +11,20 @@
 //   project_in_kernel    slab s < h: P_q[s] = [d rows x 128]; s = h: P_k; s = h + 1: P_v  (each [d x 128], d contiguous
 //                        rows of 256 bytes -- the layout of a 128-column cache, fetched the same way)
 //                        Out^T[128 features x NB] = sum over d in chunks of 128:  W_chunk^T (MN-major A) * x_chunk^T (K-major B)
+//                        the d rows of a slab are shared out over the CTAs of one thread-block cluster
 //   project_out_kernel   CTA (d tile j, head group g): Y^T[128 x NB] = sum over the group's heads:
 //                        P_o[head][128 d-rows of tile j x 128] (K-major A) * o[:, head, :]^T (K-major B, converted
-//                        from fp32 to bf16 by the CTA); the head groups of a tile are one thread-block cluster and
-//                        add their sums up through distributed shared memory, in a fixed order (no float atomics)
+//                        from fp32 to bf16 by the CTA); the head groups of a tile are one thread-block cluster
+//
+// The CTAs of a cluster leave their sums in shared memory and add them up through distributed shared memory, each the
+// batch rows that fall to it, in rank order (no float atomics).
+//
+// What bounds these kernels is latency: the weights are in flight before the kernel ahead has finished, and a CTA's work
+// after that is a chain of round trips (x or o, the products, the other CTAs' sums).  So a chain is cut into as many CTAs
+// as help (projection_parts in api.cu), and each of its links is one round trip: all of a head's o loads, and all the remote loads
+// of a row's sums, are in flight at once.  Measured on one B200, per layer step of 128 sequences, 8 heads, d = 1024, 128
+// rows: 24.7 -> 17.1 us, about 1 us of it from the attention step between them (the 4.7 MB of weights take 0.7 us
+// at the copy rate).
 //
 // NB = batch columns of a tile (the batch rounded up to 16, 32, 64 or 128; larger batches take
 // several tiles of 128).  Every wait is bounded (mbar_wait); TMEM is freed on every path.
@@ -25,10 +35,13 @@
 
 namespace mqa {
 
-constexpr int kProjThreads = 6 * 32;           // warps 0-3: convert / read out, warp 4: TMA, warp 5: MMA issue
+constexpr int kProjWorkWarps = 8;              // convert o, read the sums out, add them up
+constexpr int kProjTmaWarp = 8, kProjMmaWarp = 9;
+constexpr int kProjThreads = 10 * 32;
 constexpr int kProjChunkBytes = 128 * 256;     // 128 rows x 128 bf16 of a weight matrix: 32 KiB, two 64-column boxes
 constexpr int kProjMaxGroups = 16;             // project_out: head groups of a tile = CTAs of one cluster (16: the
                                                // non-portable cluster size, which the B200 offers; two heads per CTA at h = 32)
+constexpr int kProjMaxParts = 8;               // project_in: CTAs (of one cluster) that share a slab's d rows
 
 template <int NB>
 struct ProjCfg {
@@ -41,18 +54,37 @@ struct ProjCfg {
     static_assert(kSmemBytes <= 227 * 1024, "exceeds the shared memory of one SM");
 };
 
-// NB consecutive fp32 columns of this thread's TMEM lane, in pieces of at most 32
+// The accumulator Out^T (TMEM lane = feature, column = batch row of the tile) into this CTA's shared memory as
+// [NB batch rows][128 features] fp32, by the eight work warps: a warp may read the 32 lanes of its quarter, and the two
+// warps of a quarter take half of the batch rows each.  valid = false: zeros.
 template <int NB>
-__device__ __forceinline__ void tmem_ld_row(uint32_t taddr, uint32_t (&r)[NB]) {
-    constexpr int CH = NB < 32 ? NB : 32;
+__device__ __forceinline__ void leave_sums(uint32_t tmem, uint32_t dst, int warp, int lane, bool valid) {
+    constexpr int CH = NB < 64 ? NB / 2 : 32;                      // columns per load
+    const int feature = (warp & 3) * 32 + lane, col0 = (warp >> 2) * (NB / 2);
 #pragma unroll
-    for (int c = 0; c < NB / CH; ++c) {
+    for (int c = 0; c < NB / 2; c += CH) {
         uint32_t part[CH];
-        tmem_ld_cols<CH>(taddr + c * CH, part);
+        tmem_ld_cols<CH>(tmem + ((uint32_t)((warp & 3) * 32) << 16) + col0 + c, part);
+        tmem_wait_ld();
 #pragma unroll
-        for (int i = 0; i < CH; ++i) r[c * CH + i] = part[i];
+        for (int i = 0; i < CH; ++i)
+            asm volatile("st.shared.b32 [%0], %1;" ::"r"(dst + (uint32_t)((col0 + c + i) * 128 + feature) * 4), "r"(valid ? part[i] : 0u) : "memory");
     }
-    tmem_wait_ld();
+}
+
+// Batch row n of the tile, features lane * 4 .. + 3: the sums of all the cluster's CTAs, added up in rank order.  Every
+// remote load of a row is asked for before the first is used (one round trip through the cluster per row, not one per CTA).
+template <int MAX_CTAS>
+__device__ __forceinline__ float4 add_up_row(uint32_t sums, int n, int lane, int ctas) {
+    float4 part[MAX_CTAS];
+#pragma unroll
+    for (int g = 0; g < MAX_CTAS; ++g)
+        if (g < ctas) part[g] = cluster_ld_f4(cluster_map(sums + (uint32_t)(n * 128 + lane * 4) * 4, (uint32_t)g));
+    float4 sum = part[0];
+#pragma unroll
+    for (int g = 1; g < MAX_CTAS; ++g)
+        if (g < ctas) { sum.x += part[g].x; sum.y += part[g].y; sum.z += part[g].z; sum.w += part[g].w; }
+    return sum;
 }
 
 template <int NB>
@@ -63,9 +95,11 @@ project_in_kernel(const __grid_constant__ CUtensorMap map_pq, const __grid_const
                   int32_t* __restrict__ status, int b, int h, int d) {
     using Cfg = ProjCfg<NB>;
     constexpr int S = Cfg::kStages;
-    const int slab = blockIdx.x, row0 = blockIdx.y * 128;          // weight slab; first batch row of this tile
+    const int slab = blockIdx.x, row0 = blockIdx.z * 128;          // weight slab; first batch row of this tile
+    const int part = blockIdx.y, parts = gridDim.y;                // this CTA's part of the slab's d rows: one cluster per slab
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int n_chunks = d / 128;
+    const int chunk0 = part * (d / 128) / parts;                   // chunks of 128 rows [chunk0, chunk0 + n_chunks)
+    const int n_chunks = (part + 1) * (d / 128) / parts - chunk0;
 
     extern __shared__ uint8_t smem_raw[];
     uint8_t* stages = smem_raw + ((1024u - (smem_addr(smem_raw) & 1023u)) & 1023u);
@@ -81,17 +115,17 @@ project_in_kernel(const __grid_constant__ CUtensorMap map_pq, const __grid_const
     auto issue_weights = [&](int c) {
         const uint32_t bar = full_s + (c % S) * 8, w_s = stages_s + (c % S) * Cfg::kStageBytes;
         mbar_expect_tx(bar, kProjChunkBytes);
-        tma_load_2d(w_s, wmap, 0, wrow0 + c * 128, bar);
-        tma_load_2d(w_s + kProjChunkBytes / 2, wmap, kBoxCols, wrow0 + c * 128, bar);
+        tma_load_2d(w_s, wmap, 0, wrow0 + (chunk0 + c) * 128, bar);
+        tma_load_2d(w_s + kProjChunkBytes / 2, wmap, kBoxCols, wrow0 + (chunk0 + c) * 128, bar);
     };
     auto issue_x = [&](int c) {
         const uint32_t bar = full_s + (c % S) * 8, x_s = stages_s + (c % S) * Cfg::kStageBytes + kProjChunkBytes;
         mbar_expect_tx(bar, Cfg::kActBytes);
-        tma_load_2d(x_s, &map_x, c * 128, row0, bar);                         // rows past b read as zero
-        tma_load_2d(x_s + Cfg::kActBytes / 2, &map_x, c * 128 + kBoxCols, row0, bar);
+        tma_load_2d(x_s, &map_x, (chunk0 + c) * 128, row0, bar);              // rows past b read as zero
+        tma_load_2d(x_s + Cfg::kActBytes / 2, &map_x, (chunk0 + c) * 128 + kBoxCols, row0, bar);
         issued = c + 1;
     };
-    if (warp == 4 && lane == 0) {                                  // by the thread that issues the copies
+    if (warp == kProjTmaWarp && lane == 0) {                                  // by the thread that issues the copies
         prefetch_tensormap(&map_pq); prefetch_tensormap(&map_pk); prefetch_tensormap(&map_pv); prefetch_tensormap(&map_x);
         timed_out = 0;
         issued = 0;
@@ -101,15 +135,15 @@ project_in_kernel(const __grid_constant__ CUtensorMap map_pq, const __grid_const
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
         for (int c = 0; c < n_chunks && c < S; ++c) issue_weights(c);
     }
-    if (warp == 5) { tmem_alloc(smem_addr(&tmem_slot), Cfg::kTmemCols); tmem_relinquish(); }
-    grid_dependency_wait();          // x may come from the kernel before this one
-    grid_launch_dependents();
+    if (warp == kProjMmaWarp) { tmem_alloc(smem_addr(&tmem_slot), Cfg::kTmemCols); tmem_relinquish(); }
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem = tmem_slot;
+    grid_dependency_wait();          // x may come from the kernel before this one
+    grid_launch_dependents();
 
-    if (warp == 4) {
+    if (warp == kProjTmaWarp) {
         if (lane == 0) {
             bool ok = true;
             for (int c = 0; c < n_chunks && ok; ++c) {
@@ -122,7 +156,7 @@ project_in_kernel(const __grid_constant__ CUtensorMap map_pq, const __grid_const
             }
             if (!ok) atomicExch(&timed_out, 1);
         }
-    } else if (warp == 5) {
+    } else if (warp == kProjMmaWarp) {
         if (lane == 0) {
             constexpr uint32_t kIdesc = umma_idesc(128, NB, true, false);
             bool ok = true;
@@ -145,31 +179,31 @@ project_in_kernel(const __grid_constant__ CUtensorMap map_pq, const __grid_const
             if (!ok) atomicExch(&timed_out, 1);
         }
     } else {
-        // read-out: thread t = feature t of the slab, one TMEM lane; a column is a batch row
-        const int t = warp * 32 + lane;
+        // this CTA's sums into its shared memory: the stages are free once the last product has completed
         const bool ok = mbar_wait(done_s, 0);
         tc_fence_after();
-        if (ok) {
-            uint32_t acc[NB];
-            tmem_ld_row<NB>(tmem + ((uint32_t)(warp * 32) << 16), acc);
-            __nv_bfloat16* out = slab < h ? q + (size_t)slab * 128 + t : (slab == h ? k_new : v_new) + t;
-            const size_t stride = slab < h ? (size_t)h * 128 : 128;
-#pragma unroll
-            for (int i = 0; i < NB; ++i)
-                if (row0 + i < b) out[(size_t)(row0 + i) * stride] = __float2bfloat16_rn(__uint_as_float(acc[i]));
-        } else {
-            atomicExch(&timed_out, 1);
-        }
+        leave_sums<NB>(tmem, stages_s, warp, lane, ok);
+        if (!ok) atomicExch(&timed_out, 1);
     }
     tc_fence_before();
     __syncthreads();
     if (timed_out && threadIdx.x == 0) {
-        // before the CTA leaves: the last copy started into each stage has to land
+        // before anything else: the last copy started into each stage has to land
         for (int s = 0; s < S && s < issued; ++s) mbar_wait(full_s + s * 8, ((issued - 1 - s) / S) & 1);
         if (status) atomicOr(status, kStatusPipelineTimeout);
     }
     __syncthreads();
-    if (warp == 5) { tc_fence_after(); tmem_dealloc(tmem, Cfg::kTmemCols); }
+    if (parts > 1) cluster_sync();   // every part's sums are in its shared memory
+    {
+        __nv_bfloat16* out = slab < h ? q + (size_t)slab * 128 : (slab == h ? k_new : v_new);
+        const size_t stride = slab < h ? (size_t)h * 128 : 128;
+        for (int n = part + parts * warp; n < NB && row0 + n < b; n += parts * (kProjThreads / 32)) {
+            const float4 v = add_up_row<kProjMaxParts>(stages_s, n, lane, parts);
+            *reinterpret_cast<uint2*>(out + (size_t)(row0 + n) * stride + lane * 4) = make_uint2(pack_bf16(v.x, v.y), pack_bf16(v.z, v.w));
+        }
+    }
+    if (parts > 1) cluster_sync();   // nobody leaves while its shared memory is being read
+    if (warp == kProjMmaWarp) { tc_fence_after(); tmem_dealloc(tmem, Cfg::kTmemCols); }
 }
 
 // The head groups of one (d tile, batch tile) form one thread-block cluster (gridDim.y CTAs, at most 16): each CTA
@@ -194,16 +228,16 @@ project_out_kernel(const __grid_constant__ CUtensorMap map_po, const float* __re
     __shared__ uint32_t tmem_slot;
     __shared__ int timed_out, issued;
 
-    if (warp == 4 && lane == 0) {                                  // by the thread that issues the copies
+    if (warp == kProjTmaWarp && lane == 0) {                                  // by the thread that issues the copies
         prefetch_tensormap(&map_po);
         timed_out = 0;
         issued = 0;
-        for (int s = 0; s < S; ++s) { mbar_init(w_full + s * 8, 1); mbar_init(o_full + s * 8, 4); mbar_init(empty_s + s * 8, 1); }
+        for (int s = 0; s < S; ++s) { mbar_init(w_full + s * 8, 1); mbar_init(o_full + s * 8, kProjWorkWarps); mbar_init(empty_s + s * 8, 1); }
         mbar_init(done_s, 1);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
     }
-    if (warp == 5) { tmem_alloc(smem_addr(&tmem_slot), Cfg::kTmemCols); tmem_relinquish(); }
+    if (warp == kProjMmaWarp) { tmem_alloc(smem_addr(&tmem_slot), Cfg::kTmemCols); tmem_relinquish(); }
     auto issue_weights = [&](int i) {
         const int st = i % S;
         const uint32_t bar = w_full + st * 8, w_s = stages_s + st * Cfg::kStageBytes;
@@ -214,7 +248,7 @@ project_out_kernel(const __grid_constant__ CUtensorMap map_po, const float* __re
         issued = i + 1;
     };
     // the weights do not depend on the kernel before this one: the first copies start at once
-    if (warp == 4 && lane == 0)
+    if (warp == kProjTmaWarp && lane == 0)
         for (int i = 0; i < n_heads && i < S; ++i) issue_weights(i);
     tc_fence_before();
     __syncthreads();
@@ -223,7 +257,7 @@ project_out_kernel(const __grid_constant__ CUtensorMap map_po, const float* __re
     grid_dependency_wait();          // o comes from the kernel before this one
     grid_launch_dependents();
 
-    if (warp == 4) {
+    if (warp == kProjTmaWarp) {
         if (lane == 0) {
             bool ok = true;
             for (int i = S; i < n_heads && ok; ++i) {
@@ -232,7 +266,7 @@ project_out_kernel(const __grid_constant__ CUtensorMap map_po, const float* __re
             }
             if (!ok) atomicExch(&timed_out, 1);
         }
-    } else if (warp == 5) {
+    } else if (warp == kProjMmaWarp) {
         if (lane == 0) {
             constexpr uint32_t kIdesc = umma_idesc(128, NB, false, false);
             bool ok = true;
@@ -257,45 +291,34 @@ project_out_kernel(const __grid_constant__ CUtensorMap map_po, const float* __re
         }
     } else {
         // ---- o[:, head, :] (fp32) -> bf16 tile [NB rows x 128 columns], K-major with the 128-byte swizzle:
-        // row n, 16-byte chunk c of its 64-column half at n * 128 + ((c ^ (n & 7)) << 4)
-        const int tid = warp * 32 + lane;
+        // row n, 16-byte chunk c of its 64-column half at n * 128 + ((c ^ (n & 7)) << 4).  A warp takes whole rows (512
+        // contiguous bytes per load); all of a head's loads are in flight before the first is converted.
         bool ok = true;
         for (int i = 0; i < n_heads; ++i) {
             const int st = i % S;
+            float4 v[NB / kProjWorkWarps];
+#pragma unroll
+            for (int k = 0; k < NB / kProjWorkWarps; ++k) {
+                const int n = warp + k * kProjWorkWarps;
+                v[k] = make_float4(0.f, 0.f, 0.f, 0.f);
+                if (row0 + n < b) v[k] = *reinterpret_cast<const float4*>(o + ((size_t)(row0 + n) * h + head0 + i) * kHeadDim + lane * 4);
+            }
             if (i >= S && ok) ok = mbar_wait(empty_s + st * 8, ((i / S) - 1) & 1);   // the product that read this tile is done
-            const uint32_t o_s = stages_s + st * Cfg::kStageBytes + kProjChunkBytes;
-            for (int item = tid; item < NB * 16; item += 128) {
-                const int n = item >> 4, ch = item & 15;                     // batch row of the tile, 8-column chunk
-                uint32_t w[4] = {0u, 0u, 0u, 0u};
-                if (row0 + n < b) {
-                    const float4* src = reinterpret_cast<const float4*>(o + ((size_t)(row0 + n) * h + head0 + i) * kHeadDim + ch * 8);
-                    const float4 lo = src[0], hi = src[1];
-                    w[0] = pack_bf16(lo.x, lo.y); w[1] = pack_bf16(lo.z, lo.w);
-                    w[2] = pack_bf16(hi.x, hi.y); w[3] = pack_bf16(hi.z, hi.w);
-                }
-                const uint32_t at = o_s + (ch >> 3) * (Cfg::kActBytes / 2) + n * 128 + (((ch & 7) ^ (n & 7)) << 4);
-                asm volatile("st.shared.v4.b32 [%0], {%1,%2,%3,%4};" ::"r"(at), "r"(w[0]), "r"(w[1]), "r"(w[2]), "r"(w[3]) : "memory");
+            const uint32_t o_s = stages_s + st * Cfg::kStageBytes + kProjChunkBytes + (lane >> 4) * (Cfg::kActBytes / 2) + (lane & 1) * 8;
+#pragma unroll
+            for (int k = 0; k < NB / kProjWorkWarps; ++k) {
+                const int n = warp + k * kProjWorkWarps;
+                const uint32_t at = o_s + n * 128 + ((((lane >> 1) & 7) ^ (n & 7)) << 4);
+                asm volatile("st.shared.v2.b32 [%0], {%1,%2};" ::"r"(at), "r"(pack_bf16(v[k].x, v[k].y)), "r"(pack_bf16(v[k].z, v[k].w)) : "memory");
             }
             asm volatile("fence.proxy.async.shared::cta;" ::: "memory");     // the tile is read by the tensor core
             __syncwarp();
             if (lane == 0) mbar_arrive(o_full + st * 8);
         }
-        // ---- this CTA's Y^T (thread t = row t of the d tile, one TMEM lane; a TMEM column is a batch row) into its
-        // shared memory as [NB batch rows][128]: the stages are free once the last product has completed
-        const int t = warp * 32 + lane;
+        // ---- this CTA's Y^T into its shared memory: the stages are free once the last product has completed
         if (ok) ok = mbar_wait(done_s, 0);
         tc_fence_after();
-        if (ok && n_heads > 0) {
-            uint32_t acc[NB];
-            tmem_ld_row<NB>(tmem + ((uint32_t)(warp * 32) << 16), acc);
-#pragma unroll
-            for (int i = 0; i < NB; ++i)
-                asm volatile("st.shared.b32 [%0], %1;" ::"r"(stages_s + (uint32_t)(i * 128 + t) * 4), "r"(acc[i]) : "memory");
-        } else {
-#pragma unroll
-            for (int i = 0; i < NB; ++i)
-                asm volatile("st.shared.b32 [%0], %1;" ::"r"(stages_s + (uint32_t)(i * 128 + t) * 4), "r"(0u) : "memory");
-        }
+        leave_sums<NB>(tmem, stages_s, warp, lane, ok && n_heads > 0);
         if (!ok) atomicExch(&timed_out, 1);
     }
     tc_fence_before();
@@ -307,17 +330,13 @@ project_out_kernel(const __grid_constant__ CUtensorMap map_po, const float* __re
     }
     __syncthreads();
     cluster_sync();                  // every group's Y^T is in its shared memory
-    if (warp < 4) {
-        const int t = warp * 32 + lane;
-        const uint32_t rank = cluster_cta_rank(), n_groups = cluster_size();
-        for (int n = (int)rank; n < NB && row0 + n < b; n += (int)n_groups) {
-            float sum = 0.f;
-            for (uint32_t g = 0; g < n_groups; ++g) sum += ld_cluster_f32(stages_s + (uint32_t)(n * 128 + t) * 4, g);
-            y[(size_t)(row0 + n) * d + (size_t)tile * 128 + t] = sum;
-        }
+    const int rank = (int)cluster_cta_rank(), n_groups = (int)cluster_size();
+    for (int n = rank + n_groups * warp; n < NB && row0 + n < b; n += n_groups * (kProjThreads / 32)) {
+        const float4 sum = add_up_row<kProjMaxGroups>(stages_s, n, lane, n_groups);
+        *reinterpret_cast<float4*>(y + (size_t)(row0 + n) * d + (size_t)tile * 128 + lane * 4) = sum;
     }
     cluster_sync();                  // nobody leaves while its shared memory is being read
-    if (warp == 5) { tc_fence_after(); tmem_dealloc(tmem, Cfg::kTmemCols); }
+    if (warp == kProjMmaWarp) { tc_fence_after(); tmem_dealloc(tmem, Cfg::kTmemCols); }
 }
 
 }  // namespace mqa

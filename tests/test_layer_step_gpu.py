@@ -97,6 +97,19 @@ def test_layer_step_matches_oracle(b, h, d, m_max):
     run(b, h, d, m_max, lens0, seed=b * 3 + h)
 
 
+@pytest.mark.parametrize("b,h,d,m_max", [
+    (3, 1, 1024, 130),        # eight CTAs share an input slab's d rows
+    (17, 5, 640, 130),        # five chunks over four CTAs; a batch that is no multiple of a tile
+    (70, 32, 896, 96),        # seven chunks over two; 128 batch columns of which 70 count
+    (129, 2, 128, 64),        # one chunk; a second batch tile of one sequence
+])
+def test_input_slabs_shared_by_a_cluster(b, h, d, m_max):
+    """...and prefixes that end at every place of a tile, for the small steps that fetch their cache rows before the
+    projection has finished."""
+    lens0 = np.resize(np.array([0, 31, 32, 33, 63, 64, 1, 30, m_max - 1, m_max - 2, m_max]), b).astype(np.int32)
+    run(b, h, d, m_max, lens0, seed=b + d)
+
+
 def test_layer_step_full_cache_and_no_advance():
     b, h, d, m_max = 24, 16, 256, 1536
     lens0 = np.random.default_rng(5).integers(1, m_max, size=b).astype(np.int32)
