@@ -181,6 +181,16 @@ __host__ __device__ constexpr uint32_t umma_idesc(int M, int N, bool a_mn_major,
            ((uint32_t)(N >> 3) << 17) | ((uint32_t)(M >> 4) << 24);
 }
 
+// One lane of the warp, chosen by the hardware: the warp stays together (its values uniform) and only this lane's
+// instructions take effect.
+__device__ __forceinline__ bool elect_one() {
+    uint32_t chosen;
+    asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\tselp.u32 %0, 1, 0, p;\n\t}" : "=r"(chosen));
+    return chosen != 0;
+}
+// mbar_wait by a whole warp: the same answer on every lane.
+__device__ __forceinline__ bool warp_wait(uint32_t bar, uint32_t parity) { return __all_sync(0xffffffffu, mbar_wait(bar, parity)); }
+
 // ---- control block of the single-launch step ---------------------------------------------------
 // When a control block is given, the CTA that is last to deliver a piece of a sequence merges the pieces
 // itself (no second-pass kernel), and one CTA advances lens at the end.  The block is the first
@@ -371,7 +381,7 @@ mqa_decode_stream_umma_kernel(const __grid_constant__ CUtensorMap map_k, const _
     constexpr int kSubs = kUmmaStageRows / kTileRows;       // 4 sub-tiles of 32 rows per stage
     const bool appending = FUSED && fa.k_new != nullptr;
     const int cta = blockIdx.x, G = gridDim.x;
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int warp = __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0), lane = threadIdx.x & 31;
 
     extern __shared__ uint8_t smem_raw[];
     uint8_t* ring = smem_raw + ((1024u - (smem_addr(smem_raw) & 1023u)) & 1023u);   // K slots, then V slots
@@ -652,7 +662,7 @@ mqa_decode_stream_umma_kernel(const __grid_constant__ CUtensorMap map_k, const _
     float* piece_acc = reinterpret_cast<float*>(ring);                        // [h][128] in the first K slot (free by then)
     float2* piece_ml = reinterpret_cast<float2*>(ring + kUmmaSlotBytes);      // [h] (reference maximum, sum) in the second
     bool piece_left = false;                                // (softmax warps) this CTA has left a piece there
-    const uint32_t tmem_base = tmem_base_slot;
+    const uint32_t tmem_base = __shfl_sync(0xffffffffu, tmem_base_slot, 0);
     const uint32_t tmem_o = tmem_base + 2 * HP;             // S^T buffers at columns 0 and HP, two O^T buffers after them
 
     if (warp == kUmmaProducerWarp) {
@@ -708,27 +718,30 @@ mqa_decode_stream_umma_kernel(const __grid_constant__ CUtensorMap map_k, const _
         }
     } else if (warp == kUmmaSWarp) {
         // =============================================================== issuer of S^T = K Q^T
-        if (lane == 0 && t_begin < t_end) {
+        if (t_begin < t_end) {             // (the whole warp, one lane elected to issue: see elect_one)
             constexpr uint32_t kIdescS = umma_idesc(128, HP, false, false);
-            bool ok = !(GUESS && early >= 2) || mbar_wait(go, 0);
-            TS(14);
+            bool ok = !(GUESS && early >= 2) || warp_wait(go, 0);
+            if (lane == 0) TS(14);
             int j = 0, seg = 0;
             ShareWalker<kUmmaBoundaryPenalty> walk{prefix, t_begin, t_end, s_first};
             Segment g;
             for (; next_segment(walk, g, seg); ++seg) {
                 const int qi = seg % NQ;
-                if (ok) ok = mbar_wait(q_full + qi * 8, (seg / NQ) & 1);
-                if (seg == 0) TS(15);
+                g.lo = __shfl_sync(0xffffffffu, g.lo, 0);
+                g.hi = __shfl_sync(0xffffffffu, g.hi, 0);
+                if (ok) ok = warp_wait(q_full + qi * 8, (seg / NQ) & 1);
+                if (seg == 0 && lane == 0) TS(15);
                 for (int u = g.lo; u < g.hi; u += ustep, ++j) {
                     const int slot = j % NK, sb = j & 1;
-                    if (ok) ok = mbar_wait(k_full + slot * 8, (j / NK) & 1);
-                    if (j == 0) TS(2);
-                    TS(3);
-                    ST(j, 0);
-                    if (ok && j >= 2) ok = mbar_wait(s_free + sb * 8, ((j >> 1) - 1) & 1);
-                    ST(j, 1);
+                    if (ok) ok = warp_wait(k_full + slot * 8, (j / NK) & 1);
+                    if (j == 0 && lane == 0) TS(2);
+                    if (lane == 0) TS(3);
+                    if (lane == 0) ST(j, 0);
+                    if (ok && j >= 2) ok = warp_wait(s_free + sb * 8, ((j >> 1) - 1) & 1);
+                    if (lane == 0) ST(j, 1);
                     tc_fence_after();
-                    if (ok) {
+                    if (elect_one()) {
+                      if (ok) {
                         const uint32_t k_s = k_ring + slot * kUmmaSlotBytes;
 #pragma unroll
                         for (int ks = 0; ks < 8; ++ks) {             // 8 k-steps of 16 columns; 4 per 64-column box
@@ -736,17 +749,19 @@ mqa_decode_stream_umma_kernel(const __grid_constant__ CUtensorMap map_k, const _
                             const uint64_t bd = umma_desc(q_s + qi * Cfg::kQBytes + (ks >> 2) * (Cfg::kQBytes / 2) + (ks & 3) * 32, 16, 1024);
                             umma_ss(tmem_base + sb * HP, a, bd, kIdescS, ks ? 1u : 0u);
                         }
+                      }
+                      tc_commit(s_ready + sb * 8);
+                      tc_commit(k_empty + slot * 8);                 // the K rows are not needed again
+                      if (u + ustep >= g.hi) tc_commit(q_empty + qi * 8);   // last use of this segment's Q
                     }
-                    tc_commit(s_ready + sb * 8);
-                    tc_commit(k_empty + slot * 8);                   // the K rows are not needed again
-                    if (u + ustep >= g.hi) tc_commit(q_empty + qi * 8);   // last use of this segment's Q
+                    __syncwarp();
                 }
             }
-            if (!ok) atomicExch(&timed_out, 1);
+            if (!ok && lane == 0) atomicExch(&timed_out, 1);
         }
     } else if (warp == kUmmaPvWarp) {
         // =============================================================== issuer of O^T += V^T P^T
-        if (lane == 0 && t_begin < t_end) {
+        if (t_begin < t_end) {             // (the whole warp, one lane elected to issue: see elect_one)
             constexpr uint32_t kIdescO = umma_idesc(128, HP, true, true);
             bool ok = true;
             int j = 0, seg = 0;
@@ -754,19 +769,22 @@ mqa_decode_stream_umma_kernel(const __grid_constant__ CUtensorMap map_k, const _
             Segment g;
             for (; next_segment(walk, g, seg); ++seg) {
                 const int L = rows_of[g.s] & (kAppendBit - 1);
-                const int parts = L >= kSingleRoundingMinRows ? 1 : 2;   // P hi only, or hi then lo (as the softmax warps wrote it)
+                g.lo = __shfl_sync(0xffffffffu, g.lo, 0);
+                g.hi = __shfl_sync(0xffffffffu, g.hi, 0);
+                const int parts = __shfl_sync(0xffffffffu, L >= kSingleRoundingMinRows ? 1 : 2, 0);   // P hi only, or hi then lo (as the softmax warps wrote it)
                 for (int u = g.lo; u < g.hi; u += ustep, ++j) {
                     const int pb = j & 1, slot = j % NV;
                     // the weights first: they exist only once q has arrived, and before that a slot's barrier may
                     // still be on its way back from copies started on a guess (see early above)
-                    if (ok) ok = mbar_wait(p_ready + pb * 8, (j >> 1) & 1);
-                    ST(j, 5);
-                    if (ok) ok = mbar_wait(v_full + slot * 8, (j / NV) & 1);
-                    ST(j, 6);
+                    if (ok) ok = warp_wait(p_ready + pb * 8, (j >> 1) & 1);
+                    if (lane == 0) ST(j, 5);
+                    if (ok) ok = warp_wait(v_full + slot * 8, (j / NV) & 1);
+                    if (lane == 0) ST(j, 6);
                     // segments alternate between the two O^T buffers; the segment before the last has read this one out
-                    if (ok && u == g.lo && seg >= 2) ok = mbar_wait(o_free + (seg & 1) * 8, ((seg >> 1) - 1) & 1);
+                    if (ok && u == g.lo && seg >= 2) ok = warp_wait(o_free + (seg & 1) * 8, ((seg >> 1) - 1) & 1);
                     tc_fence_after();
-                    if (ok) {
+                    if (elect_one()) {
+                      if (ok) {
                         const uint32_t v_s = v_ring + slot * kUmmaSlotBytes;
                         for (int part = 0; part < parts; ++part) {
                             const uint32_t pt = p_s + (parts == 2 ? part : pb) * Cfg::kPBytes;
@@ -777,12 +795,14 @@ mqa_decode_stream_umma_kernel(const __grid_constant__ CUtensorMap map_k, const _
                                 umma_ss(tmem_o + (seg & 1) * HP, a, bd, kIdescO, (u == g.lo && part == 0 && kk == 0) ? 0u : 1u);
                             }
                         }
+                      }
+                      tc_commit(v_empty + slot * 8);
+                      tc_commit(pv_done + pb * 8);                   // this P^T buffer is free, O^T is up to date
                     }
-                    tc_commit(v_empty + slot * 8);
-                    tc_commit(pv_done + pb * 8);                     // this P^T buffer is free, O^T is up to date
+                    __syncwarp();
                 }
             }
-            if (!ok) atomicExch(&timed_out, 1);
+            if (!ok && lane == 0) atomicExch(&timed_out, 1);
         }
     } else {
         // =============================================================== softmax warps

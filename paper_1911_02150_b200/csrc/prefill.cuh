@@ -8,15 +8,28 @@
 // last position in stages of 128:
 //     S_w   = Q_w K_j^T       tcgen05.mma, M = 128 query rows (TMEM lanes), N = 128 cache rows, fp32 in TMEM
 //     P_w   = exp2(S_w log2e - m)   one thread per query row: the row's maximum and sum need no other thread
-//     O_w  += P_w V_j         tcgen05.mma with A = P_w read from TMEM (bf16 pairs written over S_w), B = V_j (MN-major)
-// for w = 0, 1.  While the four softmax warps of one head work on S_w, the tensor core computes the other head's
-// products: the issue order is S_0 S_1 | PV_0 S_0' | PV_1 S_1' | ...  TMEM: S_0, S_1, O_0, O_1 of 128 columns each
-// (all 512).  The reference maximum of a row moves only when the row's largest logit leads it by more than
+//     O_w  += P_w V_j         tcgen05.mma with A = P_w read from TMEM (bf16 pairs), B = V_j (MN-major)
+// for w = 0, 1.  TMEM: ONE buffer of logits (128 columns) that the two heads use in turn, P_0 and P_1 (64 columns each, bf16
+// pairs) and O_0, O_1 (128 each): all 512.  A head's logits are in registers a hundred cycles after they are there, the
+// buffer then takes the other head's, and the weights wait in registers until the product before them has read the ones
+// in tensor memory: so a head's logits are ready before it has finished the weights of the stage before, its product runs
+// under its next softmax, and the two heads fall half a period apart by themselves.  (With P written over S, every stage of a
+// head was a chain logits - softmax - product - logits; two heads' chains side by side left the tensor cores and the
+// exponentials half idle.)  The reference maximum of a row moves only when the row's largest logit leads it by more than
 // kPfMaxLead (then O_w's row is rescaled in TMEM by the row's own thread); P is bounded by 2^kPfMaxLead.
-// Rows of a tile whose memory is shorter than 1024 rows feed P as bf16 hi + lo parts (two products), like the
-// decoding kernels, so that the rounding of few large weights stays inside the tolerance.
+// Rows of a tile whose memory is shorter than 1024 rows feed P as bf16 hi + lo parts (two products, one after the other
+// out of the same columns), like the decoding kernels, so that the rounding of few large weights stays inside the
+// tolerance.
 //
-// Roles: warps 0-3 softmax of head 0, warps 4-7 softmax of head 1, warp 8 TMA producer, warp 9 MMA issuer.
+// Roles: warps 0-3 softmax of head 0, warps 4-7 softmax of head 1, warp 8 TMA producer, warp 9 issues the logits'
+// products, warp 10 the weights' (two warps: with one, the gaps between waiting for a barrier and the first instruction
+// added up to as much as the products).  The issuing warps stay together and elect a lane (elect_one): from code that
+// only lane 0 runs, every tcgen05.mma took its descriptors from per-thread registers one by one, 82 cycles instead of 54.
+//
+// What bounds it: power.  A stage of both heads takes 2630 cycles (4400 before the logits had a buffer of their own and
+// the issuers were taken apart; the tensor cores need 2048, the exponentials 2048), and at that rate the card holds its
+// clock near 1.2 GHz.  32 x 32 heads x 4096 positions, in a loop: 5.15 ms -> 4.13 ms (1070 TFLOP/s); 5 x 9 heads x 333
+// positions: 50 -> 35 us.
 // Every wait is bounded; a wait that runs out flags PIPELINE_TIMEOUT and the CTA drains and leaves.
 #pragma once
 #include "decode_umma.cuh"
@@ -28,12 +41,15 @@ constexpr int kPfTileBytes = kPfRows * kRowBytes;              // 32 KiB: 128 ro
 constexpr int kPfHalfBytes = kPfTileBytes / 2;
 constexpr int kPfKSlots = 2, kPfVSlots = 2;
 constexpr int kPfThreads = 12 * 32;                            // (warps 10 and 11 only complete the third warpgroup)
-constexpr int kPfProducerWarp = 8, kPfMmaWarp = 9;
+constexpr int kPfProducerWarp = 8, kPfSWarp = 9, kPfPvWarp = 10;
 constexpr int kPfRegsSoftmax = 216, kPfRegsOther = 72;
 constexpr float kPfMaxLead = 8.f;                              // log2 units a logit may exceed its row's reference by
-// barriers: q_full, k_full/k_empty[2], v_full/v_empty[2], s_ready[2], p_ready[2], pv_done[2]
-constexpr int kPfBarriers = 1 + 2 * kPfKSlots + 2 * kPfVSlots + 6 + 1;       // (+ q_empty)
-constexpr int kPfSmemBytes = (2 + kPfKSlots + kPfVSlots) * kPfTileBytes + kPfBarriers * 8 + 16 + 1024 /* alignment slack */;
+// barriers: q_full, k_full/k_empty[2], v_full/v_empty[2], s_ready[2], p_ready[2], pv_done[2], s_free, q_empty
+constexpr int kPfBarriers = 1 + 2 * kPfKSlots + 2 * kPfVSlots + 6 + 2;
+constexpr int kPfOutBytes = 32 * 128;                          // a softmax warp's rows of O on their way out, 32 columns at a time
+constexpr int kPfSmemBytes = (2 + kPfKSlots + kPfVSlots) * kPfTileBytes + 8 * kPfOutBytes + kPfBarriers * 8 + 16 + 1024 /* alignment slack */;
+// tensor memory columns: the logits of one stage and head, the two heads' weights, the two accumulators
+constexpr uint32_t kPfTmemP = 128, kPfTmemO = 256;
 static_assert(kPfSmemBytes <= 227 * 1024, "exceeds the shared memory of one SM");
 
 // two fp32 values in one 64-bit register: packed multiply-add and add (one instruction for two elements)
@@ -97,24 +113,26 @@ __global__ void __launch_bounds__(kPfThreads, 1)
 mqa_prefill_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CUtensorMap map_k,
                    const __grid_constant__ CUtensorMap map_v, const int32_t* __restrict__ start, float* __restrict__ O,
                    int32_t* __restrict__ status, int b, int h, int n, int m_max, int n_items) {
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int warp = __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0), lane = threadIdx.x & 31;
 
     extern __shared__ uint8_t smem_raw[];
     uint8_t* base = smem_raw + ((1024u - (smem_addr(smem_raw) & 1023u)) & 1023u);     // the 128-byte swizzle repeats every 1 KiB
     const uint32_t q_s = smem_addr(base);
     const uint32_t k_ring = q_s + 2 * kPfTileBytes, v_ring = k_ring + kPfKSlots * kPfTileBytes;
-    const uint32_t bars = v_ring + kPfVSlots * kPfTileBytes;
+    const uint32_t out_s = v_ring + kPfVSlots * kPfTileBytes, bars = out_s + 8 * kPfOutBytes;
     const uint32_t q_empty = bars + 8 * (kPfBarriers - 1);       // the unit's Q tiles have been read for the last time
+    const uint32_t s_free = bars + 8 * (kPfBarriers - 2);        // the logits have been read into registers
     const uint32_t q_full = bars, k_full = bars + 8, k_empty = k_full + 8 * kPfKSlots, v_full = k_empty + 8 * kPfKSlots,
                    v_empty = v_full + 8 * kPfVSlots, s_ready = v_empty + 8 * kPfVSlots, p_ready = s_ready + 16,
                    pv_done = p_ready + 16;
-    uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(base + (2 + kPfKSlots + kPfVSlots) * kPfTileBytes + kPfBarriers * 8);
+    uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(base + (2 + kPfKSlots + kPfVSlots) * kPfTileBytes + 8 * kPfOutBytes + kPfBarriers * 8);
     __shared__ int timed_out;
 
     if (threadIdx.x == 0) {
         prefetch_tensormap(&map_q); prefetch_tensormap(&map_k); prefetch_tensormap(&map_v);
         mbar_init(q_full, 1);
         mbar_init(q_empty, 1);
+        mbar_init(s_free, 4);
         for (int i = 0; i < kPfKSlots; ++i) { mbar_init(k_full + 8 * i, 1); mbar_init(k_empty + 8 * i, 1); }
         for (int i = 0; i < kPfVSlots; ++i) { mbar_init(v_full + 8 * i, 1); mbar_init(v_empty + 8 * i, 1); }
         for (int w = 0; w < 2; ++w) { mbar_init(s_ready + 8 * w, 1); mbar_init(p_ready + 8 * w, 4); mbar_init(pv_done + 8 * w, 1); }
@@ -122,14 +140,14 @@ mqa_prefill_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
     }
-    if (warp == kPfMmaWarp) {
+    if (warp == kPfSWarp) {
         tmem_alloc(smem_addr(tmem_slot), 512);
         tmem_relinquish();
     }
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
-    const uint32_t tmem_base = *tmem_slot;
+    const uint32_t tmem_base = __shfl_sync(0xffffffffu, *tmem_slot, 0);
     grid_dependency_wait();              // Q, K, V and start may come from the kernel before
     grid_launch_dependents();
     // the units of this CTA: c, 2G - 1 - c, 2G + c, 4G - 1 - c, ... (G CTAs; the units come longest first, so taking them
@@ -192,78 +210,87 @@ mqa_prefill_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
                 for (int G = max(0, issued_v - kPfVSlots); G < issued_v; ++G) mbar_wait(v_full + 8 * (G % kPfVSlots), (G / kPfVSlots) & 1);
             }
         }
-    } else if (warp == kPfMmaWarp) {
-        // =============================================================== issuer of both products
-        if (lane == 0) {
-            constexpr uint32_t kIdescS = umma_idesc(128, 128, false, false);
-            constexpr uint32_t kIdescO = umma_idesc(128, 128, false, true);
-            bool ok = true;
-            int g = 0, qi = 0, c_done[2] = {0, 0};               // stages, units, and stages of each head so far
-            for (int round = 0, item; (item = pf_unit(round)) < n_items && ok; ++round) {
-                const PfItem it = pf_item(item, start, b, h, n, m_max);
-                if (it.n_kv == 0) continue;
-                const int n_act = it.n_act, n_kv = it.n_kv;
-                auto issue_s = [&](int w, int G) {              // S_w = Q_w K^T into its 128 columns
-                    const uint32_t k_s = k_ring + (G % kPfKSlots) * kPfTileBytes, qw = q_s + w * kPfTileBytes;
+    } else if (warp == kPfSWarp) {
+        // =============================================================== issuer of the logits: S = Q_w K^T, the heads in turn,
+        // each as soon as the ones before are in registers
+        constexpr uint32_t kIdescS = umma_idesc(128, 128, false, false);
+        bool ok = true;
+        int g = 0, qi = 0, n_s = 0;                              // stages, units and logits so far
+        for (int round = 0, item; (item = pf_unit(round)) < n_items && ok; ++round) {
+            const PfItem it = pf_item(item, start, b, h, n, m_max);
+            const int n_kv = __shfl_sync(0xffffffffu, it.n_kv, 0), n_act = it.n_act;
+            if (n_kv == 0) continue;
+            ok = warp_wait(q_full, qi & 1);
+            for (int j = 0; j < n_kv && ok; ++j, ++g) {
+                const int slot = g % kPfKSlots;
+                const uint32_t k_s = k_ring + slot * kPfTileBytes;
+                ok = warp_wait(k_full + 8 * slot, (g / kPfKSlots) & 1);
+                for (int w = 0; w < n_act && ok; ++w, ++n_s) {
+                    if (n_s > 0) ok = warp_wait(s_free, (n_s - 1) & 1);
+                    if (!ok) break;
+                    tc_fence_after();
+                    if (elect_one()) {
+                        const uint32_t qw = q_s + w * kPfTileBytes;
 #pragma unroll
-                    for (int ks = 0; ks < 8; ++ks) {            // 8 k-steps of 16 columns; 4 per 64-column box
-                        const uint32_t off = (ks >> 2) * kPfHalfBytes + (ks & 3) * 32;
-                        umma_ss(tmem_base + w * 128, umma_desc(qw + off, 16, 1024), umma_desc(k_s + off, 16, 1024), kIdescS, ks ? 1u : 0u);
-                    }
-                    tc_commit(s_ready + 8 * w);
-                };
-                auto issue_pv = [&](int w, int G, bool first) {  // O_w += P_w V: P from TMEM (bf16 pairs: 8 columns per 16 rows of V)
-                    const uint32_t v_s = v_ring + (G % kPfVSlots) * kPfTileBytes;
-                    for (int part = 0; part < (it.hilo ? 2 : 1); ++part) {
-#pragma unroll
-                        for (int kk = 0; kk < 8; ++kk)
-                            umma_ts(tmem_base + 256 + w * 128, tmem_base + w * 128 + (kk >> 1) * 32 + part * 16 + (kk & 1) * 8,
-                                    umma_desc(v_s + kk * 2048, kPfHalfBytes, 1024), kIdescO, (first && part == 0 && kk == 0) ? 0u : 1u);
-                    }
-                    tc_commit(pv_done + 8 * w);
-                };
-                ok = mbar_wait(q_full, qi & 1);
-                if (ok) ok = mbar_wait(k_full + 8 * (g % kPfKSlots), (g / kPfKSlots) & 1);
-                if (!ok) break;
-                tc_fence_after();
-                for (int w = 0; w < n_act; ++w) issue_s(w, g);
-                tc_commit(k_empty + 8 * (g % kPfKSlots));
-                if (n_kv == 1) tc_commit(q_empty);
-                for (int j = 0; j < n_kv && ok; ++j) {
-                    const bool more = j + 1 < n_kv;
-                    const int G = g + j;
-                    for (int w = 0; w < n_act && ok; ++w) {
-                        ok = mbar_wait(p_ready + 8 * w, (c_done[w] + j) & 1);
-                        if (ok && w == 0) ok = mbar_wait(v_full + 8 * (G % kPfVSlots), (G / kPfVSlots) & 1);
-                        if (ok && w == 0 && more) ok = mbar_wait(k_full + 8 * ((G + 1) % kPfKSlots), ((G + 1) / kPfKSlots) & 1);
-                        if (!ok) break;
-                        tc_fence_after();
-                        issue_pv(w, G, j == 0);
-                        if (w == n_act - 1) tc_commit(v_empty + 8 * (G % kPfVSlots));
-                        if (more) {
-                            issue_s(w, G + 1);
-                            if (w == n_act - 1) {
-                                tc_commit(k_empty + 8 * ((G + 1) % kPfKSlots));
-                                if (j + 2 == n_kv) tc_commit(q_empty);       // the unit's last logits are on their way
-                            }
+                        for (int ks = 0; ks < 8; ++ks) {         // 8 k-steps of 16 columns; 4 per 64-column box
+                            const uint32_t off = (ks >> 2) * kPfHalfBytes + (ks & 3) * 32;
+                            umma_ss(tmem_base, umma_desc(qw + off, 16, 1024), umma_desc(k_s + off, 16, 1024), kIdescS, ks ? 1u : 0u);
+                        }
+                        tc_commit(s_ready + 8 * w);
+                        if (w == n_act - 1) {
+                            tc_commit(k_empty + 8 * slot);
+                            if (j == n_kv - 1) tc_commit(q_empty);       // the unit's last logits are on their way
                         }
                     }
+                    __syncwarp();
                 }
-                g += n_kv;
-                ++qi;
-                for (int w = 0; w < n_act; ++w) c_done[w] += n_kv;
             }
-            if (!ok) atomicExch(&timed_out, 1);
+            ++qi;
         }
+        if (!ok && lane == 0) atomicExch(&timed_out, 1);
+    } else if (warp == kPfPvWarp) {
+        // =============================================================== issuer of O_w += P_w V: P from tensor memory (bf16 pairs: 8
+        // columns per 16 rows of V), both parts of it where there are two
+        constexpr uint32_t kIdescO = umma_idesc(128, 128, false, true);
+        bool ok = true;
+        int g = 0, n_p[2] = {0, 0};                              // stages and each head's weights so far
+        for (int round = 0, item; (item = pf_unit(round)) < n_items && ok; ++round) {
+            const PfItem it = pf_item(item, start, b, h, n, m_max);
+            const int n_kv = __shfl_sync(0xffffffffu, it.n_kv, 0), n_act = it.n_act, parts = __any_sync(0xffffffffu, it.hilo) ? 2 : 1;
+            for (int j = 0; j < n_kv && ok; ++j, ++g) {
+                const int slot = g % kPfVSlots;
+                const uint32_t v_s = v_ring + slot * kPfTileBytes;
+                ok = warp_wait(v_full + 8 * slot, (g / kPfVSlots) & 1);
+                for (int w = 0; w < n_act && ok; ++w) {
+                    for (int part = 0; part < parts && ok; ++part) {
+                        ok = warp_wait(p_ready + 8 * w, n_p[w] & 1);
+                        if (!ok) break;
+                        ++n_p[w];
+                        tc_fence_after();
+                        if (elect_one()) {
+#pragma unroll
+                            for (int kk = 0; kk < 8; ++kk)
+                                umma_ts(tmem_base + kPfTmemO + w * 128, tmem_base + kPfTmemP + w * 64 + kk * 8,
+                                        umma_desc(v_s + kk * 2048, kPfHalfBytes, 1024), kIdescO, (j == 0 && part == 0 && kk == 0) ? 0u : 1u);
+                            tc_commit(pv_done + 8 * w);
+                            if (w == n_act - 1 && part == parts - 1) tc_commit(v_empty + 8 * slot);
+                        }
+                        __syncwarp();
+                    }
+                }
+            }
+        }
+        if (!ok && lane == 0) atomicExch(&timed_out, 1);
     }
     } else {
         asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(kPfRegsSoftmax));
         // =============================================================== softmax warps: one thread per query row
         const int w = warp >> 2, quarter = warp & 3, r = quarter * 32 + lane;
         const uint32_t lane_base = tmem_base + ((uint32_t)(quarter * 32) << 16);
-        const uint32_t s_t = lane_base + w * 128, o_t = lane_base + 256 + w * 128;
+        const uint32_t p_t = lane_base + kPfTmemP + w * 64, o_t = lane_base + kPfTmemO + w * 128;
+        const uint32_t out_w = out_s + warp * kPfOutBytes;
         bool ok = true;
-        int g = 0, c_done = 0;                                   // stages of the CTA and of this head so far
+        int g = 0, n_s = 0, n_p = 0;                             // stages of the CTA, logits and weights of this head so far
         for (int round = 0, item; (item = pf_unit(round)) < n_items; ++round) {
             const PfItem it = pf_item(item, start, b, h, n, m_max);
             if (w >= it.n_act) { g += it.n_kv; continue; }       // (an odd head count: the unit has one head)
@@ -280,14 +307,18 @@ mqa_prefill_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
             float m = -INFINITY, l = 0.f;                        // reference maximum (log2 units), sum of weights
             for (int j = 0; j < it.n_kv; ++j) {
                 const int k0 = j * kPfRows;
-                if (ok) ok = mbar_wait(s_ready + 8 * w, (c_done + j) & 1);
+                if (ok) ok = mbar_wait(s_ready + 8 * w, n_s & 1);
+                ++n_s;
                 tc_fence_after();
                 const bool diag = k0 + kPfRows > lim_first;           // some position of the tile cannot see all of this stage
                 // ---- the row's 128 logits, read once and kept in registers.  The mask of Section 2.3 is applied
                 // by index, as a select: what lies behind a masked logit is never used.
                 uint32_t x[128];
-                tmem_ld_cols<128>(s_t, x);
+                tmem_ld_cols<128>(lane_base, x);
                 tmem_wait_ld();
+                tc_fence_before();
+                __syncwarp();
+                if (lane == 0) mbar_arrive(s_free);                   // the other head's logits may take their place
                 if (diag) {
 #pragma unroll
                     for (int i = 0; i < 128; ++i)
@@ -304,7 +335,7 @@ mqa_prefill_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
                     if (j > 0) {
                         const float f = fast_exp2(m - m_new);         // (m is finite from the first stage on)
                         l *= f;
-                        if (ok) ok = mbar_wait(pv_done + 8 * w, (c_done + j - 1) & 1);    // O holds the stages before this one
+                        if (ok) ok = mbar_wait(pv_done + 8 * w, (n_p - 1) & 1);           // O holds the stages before this one
                         tc_fence_after();
 #pragma unroll 1
                         for (int c = 0; c < 16; ++c) {
@@ -320,35 +351,26 @@ mqa_prefill_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
                 }
                 const unsigned long long neg_m2 = f2_pack(-m, -m), log2e2 = f2_pack(kLog2e, kLog2e);
                 unsigned long long sum2[2] = {0ull, 0ull};
+                // the weights stay in registers until the product before has read the ones in tensor memory
+                uint32_t hi[2][32];
                 if (it.hilo) {
 #pragma unroll
-                    for (int c = 0; c < 4; ++c) {
-                        uint32_t hi[16];
-#pragma unroll
-                        for (int i = 0; i < 16; ++i) {
-                            float a0, a1;
-                            f2_unpack(f2_fma(f2_pack(__uint_as_float(x[c * 32 + 2 * i]), __uint_as_float(x[c * 32 + 2 * i + 1])), log2e2, neg_m2), a0, a1);
-                            const float pa = fast_exp2(a0), pb = fast_exp2(a1);
-                            sum2[i & 1] = f2_add(sum2[i & 1], f2_pack(pa, pb));
-                            hi[i] = pack_bf16(pa, pb);
-                            x[c * 32 + i] = pack_bf16(pa - bf16_lo(hi[i]), pb - bf16_hi(hi[i]));
-                        }
-                        tmem_st16(s_t + c * 32, hi);
-                        tmem_st16(s_t + c * 32 + 16, *reinterpret_cast<uint32_t(*)[16]>(&x[c * 32]));
+                    for (int i = 0; i < 64; ++i) {
+                        float a0, a1;
+                        f2_unpack(f2_fma(f2_pack(__uint_as_float(x[2 * i]), __uint_as_float(x[2 * i + 1])), log2e2, neg_m2), a0, a1);
+                        const float pa = fast_exp2(a0), pb = fast_exp2(a1);
+                        sum2[i & 1] = f2_add(sum2[i & 1], f2_pack(pa, pb));
+                        hi[i >> 5][i & 31] = pack_bf16(pa, pb);
+                        x[i] = pack_bf16(pa - bf16_lo(hi[i >> 5][i & 31]), pb - bf16_hi(hi[i >> 5][i & 31]));
                     }
                 } else {
 #pragma unroll
-                    for (int c = 0; c < 4; ++c) {
-                        uint32_t hi[16];
-#pragma unroll
-                        for (int i = 0; i < 16; ++i) {
-                            float a0, a1;
-                            f2_unpack(f2_fma(f2_pack(__uint_as_float(x[c * 32 + 2 * i]), __uint_as_float(x[c * 32 + 2 * i + 1])), log2e2, neg_m2), a0, a1);
-                            const float pa = fast_exp2(a0), pb = fast_exp2(a1);
-                            sum2[i & 1] = f2_add(sum2[i & 1], f2_pack(pa, pb));
-                            hi[i] = pack_bf16(pa, pb);
-                        }
-                        tmem_st16(s_t + c * 32, hi);
+                    for (int i = 0; i < 64; ++i) {
+                        float a0, a1;
+                        f2_unpack(f2_fma(f2_pack(__uint_as_float(x[2 * i]), __uint_as_float(x[2 * i + 1])), log2e2, neg_m2), a0, a1);
+                        const float pa = fast_exp2(a0), pb = fast_exp2(a1);
+                        sum2[i & 1] = f2_add(sum2[i & 1], f2_pack(pa, pb));
+                        hi[i >> 5][i & 31] = pack_bf16(pa, pb);
                     }
                 }
                 {
@@ -356,6 +378,10 @@ mqa_prefill_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
                     f2_unpack(f2_add(sum2[0], sum2[1]), s0, s1);
                     l += s0 + s1;
                 }
+                if (n_p > 0 && ok) ok = mbar_wait(pv_done + 8 * w, (n_p - 1) & 1);
+                tc_fence_after();
+                tmem_st32(p_t, hi[0]);
+                tmem_st32(p_t + 32, hi[1]);
                 tmem_wait_st();
                 tc_fence_before();
                 if (w == 0 && j == it.n_kv - 1 && it.L < k0 + kPfRows) {
@@ -374,9 +400,21 @@ mqa_prefill_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
                 }
                 __syncwarp();
                 if (lane == 0) mbar_arrive(p_ready + 8 * w);
+                ++n_p;
+                if (it.hilo) {                                        // the remainders, once the first part's product has been made
+                    if (ok) ok = mbar_wait(pv_done + 8 * w, (n_p - 1) & 1);
+                    tc_fence_after();
+                    tmem_st32(p_t, *reinterpret_cast<uint32_t(*)[32]>(&x[0]));
+                    tmem_st32(p_t + 32, *reinterpret_cast<uint32_t(*)[32]>(&x[32]));
+                    tmem_wait_st();
+                    tc_fence_before();
+                    __syncwarp();
+                    if (lane == 0) mbar_arrive(p_ready + 8 * w);
+                    ++n_p;
+                }
             }
             // ---- the row of O, divided by the sum of its weights
-            if (ok) ok = mbar_wait(pv_done + 8 * w, (c_done + it.n_kv - 1) & 1);
+            if (ok) ok = mbar_wait(pv_done + 8 * w, (n_p - 1) & 1);
             tc_fence_after();
             const float inv = 1.f / l;
 #pragma unroll
@@ -384,23 +422,33 @@ mqa_prefill_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
                 uint32_t y[32];
                 tmem_ld32(o_t + c * 32, y);
                 tmem_wait_ld();
-                if (stored) {
+                // 32 columns of the warp's 32 rows through shared memory, so that they leave as 128-byte pieces (straight from
+                // here a store instruction would touch 32 rows, 16 bytes of each)
 #pragma unroll
-                    for (int i = 0; i < 32; i += 4)
-                        *reinterpret_cast<float4*>(dst + c * 32 + i) =
-                            make_float4(__uint_as_float(y[i]) * inv, __uint_as_float(y[i + 1]) * inv, __uint_as_float(y[i + 2]) * inv,
-                                        __uint_as_float(y[i + 3]) * inv);
+                for (int i = 0; i < 8; ++i)
+                    asm volatile("st.shared.v4.f32 [%0], {%1,%2,%3,%4};" ::"r"(out_w + lane * 128 + ((i ^ (lane & 7)) << 4)),
+                                 "f"(__uint_as_float(y[4 * i]) * inv), "f"(__uint_as_float(y[4 * i + 1]) * inv),
+                                 "f"(__uint_as_float(y[4 * i + 2]) * inv), "f"(__uint_as_float(y[4 * i + 3]) * inv) : "memory");
+                __syncwarp();
+#pragma unroll
+                for (int i = 0; i < 8; ++i) {
+                    const int rr = i * 4 + (lane >> 3), row = quarter * 32 + rr;
+                    float4 v;
+                    asm volatile("ld.shared.v4.f32 {%0,%1,%2,%3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w)
+                                 : "r"(out_w + rr * 128 + (((lane & 7) ^ (rr & 7)) << 4)) : "memory");
+                    if (p0 + row < n)
+                        *reinterpret_cast<float4*>(O + (size_t)(it.q_row0 + (long long)w * n + row) * kHeadDim + c * 32 + (lane & 7) * 4) = v;
                 }
+                __syncwarp();
             }
             tc_fence_before();                                   // (the next unit's first product overwrites O once its weights are in)
             g += it.n_kv;
-            c_done += it.n_kv;
         }
         if (!ok) atomicExch(&timed_out, 1);
     }
     tc_fence_before();
     __syncthreads();
-    if (warp == kPfMmaWarp) {
+    if (warp == kPfSWarp) {
         tc_fence_after();
         tmem_dealloc(tmem_base, 512);
     }
