@@ -13,13 +13,14 @@
 // The two softmax warpgroups take the stages in turn (warpgroup w: stages w, w + 2, ...), each with an S buffer, an
 // O accumulator, reference maxima and sums of its own -- two partial softmaxes over interleaved rows of the cache,
 // merged exactly at the end (the same recombination as between splits) -- so the logits of a stage are computed and
-// its weights formed while the other warpgroup's stage is multiplied with V.  TMEM: S_0, S_1, O_0, O_1 (512 columns).
+// its weights formed while the other warpgroup's stage is multiplied with V.  TMEM: one buffer of logits that the stages
+// use in turn, P_0, P_1, O_0, O_1 (512 columns; why they lie like this, and why two warps issue the products: prefill.cuh).
 // A CTA writes o itself when the sequence has one split, else a piece (maximum, sum, unnormalised rows) for the
 // second-pass kernel (combine.cuh).  Valid prefix: rows >= lens are never fetched except in a split's last stage,
 // where they are masked by index (select) and their V rows cleared in shared memory.
 //
-// Roles: warps 0-3 and 4-7 the two softmax warpgroups, warp 8 TMA producer, warp 9 MMA issuer (warps 10, 11 only
-// complete the third warpgroup, which hands most of its registers to the other two).  Every wait is bounded.
+// Roles: warps 0-3 and 4-7 the two softmax warpgroups, warp 8 TMA producer, warps 9 and 10 issue the products (warp 11 only
+// completes the third warpgroup, which hands most of its registers to the other two).  Every wait is bounded.
 #pragma once
 #include "prefill.cuh"
 
@@ -28,9 +29,9 @@ namespace mqa {
 constexpr int kWideRows = 128;                                 // query rows of the tile = cache rows per stage
 constexpr int kWideKSlots = 3, kWideVSlots = 3;
 constexpr int kWideThreads = 12 * 32;
-constexpr int kWideProducerWarp = 8, kWideMmaWarp = 9;
-// barriers: q_full, k_full/k_empty, v_full/v_empty per slot, s_ready[2], p_ready[2], pv_done[2]
-constexpr int kWideBarriers = 1 + 2 * kWideKSlots + 2 * kWideVSlots + 6;
+constexpr int kWideProducerWarp = 8, kWideSWarp = 9, kWidePvWarp = 10;
+// barriers: q_full, k_full/k_empty, v_full/v_empty per slot, s_ready[2], p_ready[2], pv_done[2], s_free
+constexpr int kWideBarriers = 1 + 2 * kWideKSlots + 2 * kWideVSlots + 7;
 constexpr int kWideSmemBytes = (1 + kWideKSlots + kWideVSlots) * kPfTileBytes + kWideBarriers * 8 + 16 + 1024 /* alignment slack */;
 static_assert(kWideSmemBytes + 1024 + 16 /* static */ <= 227 * 1024, "exceeds the shared memory of one SM");
 
@@ -41,7 +42,7 @@ mqa_decode_wide_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_c
                        float2* __restrict__ part_ml, float* __restrict__ part_acc, int32_t* __restrict__ status, int h,
                        int m_max, int chunk_rows, int n_splits, int len_bias, const FusedArgs fa, int32_t* __restrict__ lens_advance,
                        int withhold) {
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int warp = __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0), lane = threadIdx.x & 31;
     const int seq = blockIdx.x / n_splits, split = blockIdx.x % n_splits;
     const int row0 = blockIdx.y * kWideRows;                   // this CTA's first query row of the sequence (more than 128: grid.y tiles)
 
@@ -52,7 +53,7 @@ mqa_decode_wide_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_c
     const uint32_t bars = v_ring + kWideVSlots * kPfTileBytes;
     const uint32_t q_full = bars, k_full = bars + 8, k_empty = k_full + 8 * kWideKSlots, v_full = k_empty + 8 * kWideKSlots,
                    v_empty = v_full + 8 * kWideVSlots, s_ready = v_empty + 8 * kWideVSlots, p_ready = s_ready + 16,
-                   pv_done = p_ready + 16;
+                   pv_done = p_ready + 16, s_free = pv_done + 16;
     uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(base + (1 + kWideKSlots + kWideVSlots) * kPfTileBytes + kWideBarriers * 8);
     __shared__ int timed_out;
     __shared__ float2 ex_ml[kWideRows];                       // (maximum, sum) of warpgroup 1's rows, for the merge at the end
@@ -60,6 +61,7 @@ mqa_decode_wide_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_c
     if (threadIdx.x == 0) {
         prefetch_tensormap(&map_q); prefetch_tensormap(&map_k); prefetch_tensormap(&map_v);
         mbar_init(q_full, 1);
+        mbar_init(s_free, 4);
         for (int i = 0; i < kWideKSlots; ++i) { mbar_init(k_full + 8 * i, 1); mbar_init(k_empty + 8 * i, 1); }
         for (int i = 0; i < kWideVSlots; ++i) { mbar_init(v_full + 8 * i, 1); mbar_init(v_empty + 8 * i, 1); }
         for (int w = 0; w < 2; ++w) { mbar_init(s_ready + 8 * w, 1); mbar_init(p_ready + 8 * w, 4); mbar_init(pv_done + 8 * w, 1); }
@@ -67,14 +69,14 @@ mqa_decode_wide_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_c
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
     }
-    if (warp == kWideMmaWarp) {
+    if (warp == kWideSWarp) {
         tmem_alloc(smem_addr(tmem_slot), 512);
         tmem_relinquish();
     }
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
-    const uint32_t tmem_base = *tmem_slot;
+    const uint32_t tmem_base = __shfl_sync(0xffffffffu, *tmem_slot, 0);
 
     grid_dependency_wait();              // q, lens and the newest cache row may come from the kernel before
     grid_launch_dependents();
@@ -88,8 +90,8 @@ mqa_decode_wide_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_c
         atomicOr(status, raw < 0 ? kStatusAppendNegative : kStatusAppendFull);
     const int L = clamp_len(appended ? raw + 1 : biased_len(raw, m_max, len_bias), m_max, (split == 0 && blockIdx.y == 0 && threadIdx.x == 0) ? status : nullptr);
     const int r0 = split * chunk_rows, r1 = min(r0 + chunk_rows, L);           // this CTA's rows of the sequence's cache
-    const int n_kv = r1 > r0 ? (r1 - r0 + kWideRows - 1) / kWideRows : 0;      // stages
-    const bool hilo = L < kSingleRoundingMinRows;
+    const int n_kv = __shfl_sync(0xffffffffu, r1 > r0 ? (r1 - r0 + kWideRows - 1) / kWideRows : 0, 0);      // stages
+    const bool hilo = __any_sync(0xffffffffu, L < kSingleRoundingMinRows);
 
     if (warp >= 8) {
         asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(kPfRegsOther));
@@ -135,61 +137,67 @@ mqa_decode_wide_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_c
                     for (int j = max(0, issued_v - kWideVSlots); j < issued_v; ++j) mbar_wait(v_full + 8 * (j % kWideVSlots), (j / kWideVSlots) & 1);
                 }
             }
-        } else if (warp == kWideMmaWarp) {
-            // =========================================================== issuer of both products
-            if (lane == 0 && n_kv > 0) {
-                constexpr uint32_t kIdescS = umma_idesc(128, 128, false, false);
-                constexpr uint32_t kIdescO = umma_idesc(128, 128, false, true);
-                bool ok = mbar_wait(q_full, 0);
-                auto issue_s = [&](int j) {                     // S = Q K_j^T into the buffer of warpgroup j mod 2
-                    const uint32_t k_s = k_ring + (j % kWideKSlots) * kPfTileBytes;
+        } else if (warp == kWideSWarp) {
+            // =========================================================== issuer of the logits: S = Q K_j^T, each stage as soon as
+            // the one before is in registers
+            constexpr uint32_t kIdescS = umma_idesc(128, 128, false, false);
+            bool ok = n_kv == 0 || warp_wait(q_full, 0);
+            for (int j = 0; j < n_kv && ok; ++j) {
+                const int slot = j % kWideKSlots;
+                ok = warp_wait(k_full + 8 * slot, (j / kWideKSlots) & 1);
+                if (ok && j > 0) ok = warp_wait(s_free, (j - 1) & 1);
+                if (!ok) break;
+                tc_fence_after();
+                if (elect_one()) {
+                    const uint32_t k_s = k_ring + slot * kPfTileBytes;
 #pragma unroll
                     for (int ks = 0; ks < 8; ++ks) {            // 8 k-steps of 16 columns; 4 per 64-column box
                         const uint32_t off = (ks >> 2) * kPfHalfBytes + (ks & 3) * 32;
-                        umma_ss(tmem_base + (j & 1) * 128, umma_desc(q_s + off, 16, 1024), umma_desc(k_s + off, 16, 1024), kIdescS, ks ? 1u : 0u);
+                        umma_ss(tmem_base, umma_desc(q_s + off, 16, 1024), umma_desc(k_s + off, 16, 1024), kIdescS, ks ? 1u : 0u);
                     }
                     tc_commit(s_ready + 8 * (j & 1));
-                    tc_commit(k_empty + 8 * (j % kWideKSlots));
-                };
-                auto issue_pv = [&](int j) {                    // O_w += P V_j: P from TMEM (bf16 pairs: 8 columns per 16 rows of V)
-                    const uint32_t v_s = v_ring + (j % kWideVSlots) * kPfTileBytes;
-                    const int w = j & 1;
-                    for (int part = 0; part < (hilo ? 2 : 1); ++part) {
+                    tc_commit(k_empty + 8 * slot);
+                }
+                __syncwarp();
+            }
+            if (!ok && lane == 0) atomicExch(&timed_out, 1);
+        } else if (warp == kWidePvWarp) {
+            // =========================================================== issuer of O_w += P_w V_j: P from tensor memory (bf16 pairs: 8
+            // columns per 16 rows of V), both parts of it where there are two
+            constexpr uint32_t kIdescO = umma_idesc(128, 128, false, true);
+            bool ok = true;
+            int n_p[2] = {0, 0};
+            for (int j = 0; j < n_kv && ok; ++j) {
+                const int slot = j % kWideVSlots, w = j & 1;
+                const uint32_t v_s = v_ring + slot * kPfTileBytes;
+                ok = warp_wait(v_full + 8 * slot, (j / kWideVSlots) & 1);
+                for (int part = 0; part < (hilo ? 2 : 1) && ok; ++part) {
+                    ok = warp_wait(p_ready + 8 * w, n_p[w] & 1);
+                    if (!ok) break;
+                    ++n_p[w];
+                    tc_fence_after();
+                    if (elect_one()) {
 #pragma unroll
                         for (int kk = 0; kk < 8; ++kk)
-                            umma_ts(tmem_base + 256 + w * 128, tmem_base + w * 128 + part * 64 + kk * 8,
+                            umma_ts(tmem_base + kPfTmemO + w * 128, tmem_base + kPfTmemP + w * 64 + kk * 8,
                                     umma_desc(v_s + kk * 2048, kPfHalfBytes, 1024), kIdescO, (j < 2 && part == 0 && kk == 0) ? 0u : 1u);
+                        tc_commit(pv_done + 8 * w);
+                        if (part == (hilo ? 1 : 0)) tc_commit(v_empty + 8 * slot);
                     }
-                    tc_commit(pv_done + 8 * w);
-                    tc_commit(v_empty + 8 * (j % kWideVSlots));
-                };
-                for (int j = 0; j < 2 && j < n_kv && ok; ++j) {
-                    ok = mbar_wait(k_full + 8 * j, 0);
-                    if (!ok) break;
-                    tc_fence_after();
-                    issue_s(j);
+                    __syncwarp();
                 }
-                for (int j = 0; j < n_kv && ok; ++j) {
-                    ok = mbar_wait(p_ready + 8 * (j & 1), (j >> 1) & 1);
-                    if (ok) ok = mbar_wait(v_full + 8 * (j % kWideVSlots), (j / kWideVSlots) & 1);
-                    if (ok && j + 2 < n_kv) ok = mbar_wait(k_full + 8 * ((j + 2) % kWideKSlots), ((j + 2) / kWideKSlots) & 1);
-                    if (!ok) break;
-                    tc_fence_after();
-                    issue_pv(j);
-                    if (j + 2 < n_kv) issue_s(j + 2);           // the buffer these weights were in takes the logits of stage j + 2
-                }
-                if (!ok) atomicExch(&timed_out, 1);
             }
+            if (!ok && lane == 0) atomicExch(&timed_out, 1);
         }
     } else {
         asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(kPfRegsSoftmax));
         // =============================================================== softmax warpgroups: one thread per query row
         const int w = warp >> 2, quarter = warp & 3, r = quarter * 32 + lane;
         const uint32_t lane_base = tmem_base + ((uint32_t)(quarter * 32) << 16);
-        const uint32_t s_t = lane_base + w * 128, o_t = lane_base + 256 + w * 128;
+        const uint32_t p_t = lane_base + kPfTmemP + w * 64, o_t = lane_base + kPfTmemO + w * 128;
         float m = -INFINITY, l = 0.f;                                 // reference maximum (log2 units), sum of weights
         bool ok = true;
-        int last_phase = -1;                                          // phase of this warpgroup's last product
+        int n_p = 0;                                                  // products of this warpgroup's weights so far
         for (int j = w; j < n_kv; j += 2) {
             const int ph = j >> 1;
             const int valid = r1 - (r0 + j * kWideRows);              // rows of the stage inside this split's prefix (> 0)
@@ -197,8 +205,11 @@ mqa_decode_wide_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_c
             tc_fence_after();
             // ---- the row's 128 logits, read once and kept in registers; rows past the prefix masked by index (a select)
             uint32_t x[128];
-            tmem_ld_cols<128>(s_t, x);
+            tmem_ld_cols<128>(lane_base, x);
             tmem_wait_ld();
+            tc_fence_before();
+            __syncwarp();
+            if (lane == 0) mbar_arrive(s_free);                       // the next stage's logits may take their place
             if (valid < kWideRows) {
 #pragma unroll
                 for (int i = 0; i < 128; ++i)
@@ -217,7 +228,7 @@ mqa_decode_wide_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_c
                 if (ph > 0) {
                     const float f = fast_exp2(m - m_new);             // (m is finite from the warpgroup's first stage on)
                     l *= f;
-                    if (ok) ok = mbar_wait(pv_done + 8 * w, (ph - 1) & 1);   // O holds the warpgroup's stages before this one
+                    if (ok) ok = mbar_wait(pv_done + 8 * w, (n_p - 1) & 1);  // O holds the warpgroup's stages before this one
                     tc_fence_after();
 #pragma unroll 1
                     for (int c = 0; c < 16; ++c) {
@@ -231,40 +242,29 @@ mqa_decode_wide_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_c
                 }
                 m = m_new;
             }
-            // ---- P = exp2(S log2e - m) as bf16 pairs over the first 64 columns of S (hi) and, for a short prefix, their
-            // remainders over the other 64 (lo)
+            // ---- P = exp2(S log2e - m) as bf16 pairs (hi) and, for a short prefix, their remainders (lo)
             const unsigned long long neg_m2 = f2_pack(-m, -m), log2e2 = f2_pack(kLog2e, kLog2e);
             unsigned long long sum2[2] = {0ull, 0ull};
+            // the weights stay in registers until the product before has read the ones in tensor memory
+            uint32_t hi[2][32];
             if (hilo) {
 #pragma unroll
-                for (int c = 0; c < 4; ++c) {
-                    uint32_t hi[16];
-#pragma unroll
-                    for (int i = 0; i < 16; ++i) {
-                        float a0, a1;
-                        f2_unpack(f2_fma(f2_pack(__uint_as_float(x[c * 32 + 2 * i]), __uint_as_float(x[c * 32 + 2 * i + 1])), log2e2, neg_m2), a0, a1);
-                        const float pa = fast_exp2(a0), pb = fast_exp2(a1);
-                        sum2[i & 1] = f2_add(sum2[i & 1], f2_pack(pa, pb));
-                        hi[i] = pack_bf16(pa, pb);
-                        x[c * 32 + i] = pack_bf16(pa - bf16_lo(hi[i]), pb - bf16_hi(hi[i]));
-                    }
-                    tmem_st16(s_t + c * 16, hi);
+                for (int i = 0; i < 64; ++i) {
+                    float a0, a1;
+                    f2_unpack(f2_fma(f2_pack(__uint_as_float(x[2 * i]), __uint_as_float(x[2 * i + 1])), log2e2, neg_m2), a0, a1);
+                    const float pa = fast_exp2(a0), pb = fast_exp2(a1);
+                    sum2[i & 1] = f2_add(sum2[i & 1], f2_pack(pa, pb));
+                    hi[i >> 5][i & 31] = pack_bf16(pa, pb);
+                    x[i] = pack_bf16(pa - bf16_lo(hi[i >> 5][i & 31]), pb - bf16_hi(hi[i >> 5][i & 31]));
                 }
-#pragma unroll
-                for (int c = 0; c < 4; ++c) tmem_st16(s_t + 64 + c * 16, *reinterpret_cast<uint32_t(*)[16]>(&x[c * 32]));
             } else {
 #pragma unroll
-                for (int c = 0; c < 4; ++c) {
-                    uint32_t hi[16];
-#pragma unroll
-                    for (int i = 0; i < 16; ++i) {
-                        float a0, a1;
-                        f2_unpack(f2_fma(f2_pack(__uint_as_float(x[c * 32 + 2 * i]), __uint_as_float(x[c * 32 + 2 * i + 1])), log2e2, neg_m2), a0, a1);
-                        const float pa = fast_exp2(a0), pb = fast_exp2(a1);
-                        sum2[i & 1] = f2_add(sum2[i & 1], f2_pack(pa, pb));
-                        hi[i] = pack_bf16(pa, pb);
-                    }
-                    tmem_st16(s_t + c * 16, hi);
+                for (int i = 0; i < 64; ++i) {
+                    float a0, a1;
+                    f2_unpack(f2_fma(f2_pack(__uint_as_float(x[2 * i]), __uint_as_float(x[2 * i + 1])), log2e2, neg_m2), a0, a1);
+                    const float pa = fast_exp2(a0), pb = fast_exp2(a1);
+                    sum2[i & 1] = f2_add(sum2[i & 1], f2_pack(pa, pb));
+                    hi[i >> 5][i & 31] = pack_bf16(pa, pb);
                 }
             }
             {
@@ -272,6 +272,10 @@ mqa_decode_wide_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_c
                 f2_unpack(f2_add(sum2[0], sum2[1]), s0, s1);
                 l += s0 + s1;
             }
+            if (n_p > 0 && ok) ok = mbar_wait(pv_done + 8 * w, (n_p - 1) & 1);
+            tc_fence_after();
+            tmem_st32(p_t, hi[0]);
+            tmem_st32(p_t + 32, hi[1]);
             tmem_wait_st();
             tc_fence_before();
             if (valid < kWideRows) {
@@ -289,9 +293,23 @@ mqa_decode_wide_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_c
             }
             __syncwarp();
             if (lane == 0) mbar_arrive(p_ready + 8 * w);
-            last_phase = ph;
+            ++n_p;
+            if (hilo) {                                               // the remainders, once the first part's product has been made
+                if (ok) ok = mbar_wait(pv_done + 8 * w, (n_p - 1) & 1);
+                tc_fence_after();
+                tmem_st32(p_t, *reinterpret_cast<uint32_t(*)[32]>(&x[0]));
+                tmem_st32(p_t + 32, *reinterpret_cast<uint32_t(*)[32]>(&x[32]));
+                tmem_wait_st();
+                tc_fence_before();
+                __syncwarp();
+                if (lane == 0) mbar_arrive(p_ready + 8 * w);
+                ++n_p;
+            }
         }
-        if (last_phase >= 0 && ok) ok = mbar_wait(pv_done + 8 * w, last_phase & 1);
+        if (n_p > 0 && ok) ok = mbar_wait(pv_done + 8 * w, (n_p - 1) & 1);
+        // (the K ring is used below: a last stage that is warpgroup 0's must have its logits.  Its logits before those have
+        // been ready since before this warpgroup's last ones were issued, so the wait cannot be a phase early)
+        if (w == 1 && n_p > 0 && (n_kv & 1) && ok) ok = mbar_wait(s_ready, ((n_kv - 1) >> 1) & 1);
         tc_fence_after();
         // ---- the two warpgroups' partial results become one: warpgroup 1 leaves (maximum, sum) and its rows of O in
         // shared memory (the K ring: every S product has completed by now), warpgroup 0 merges and writes out
@@ -299,7 +317,7 @@ mqa_decode_wide_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_c
         if (w == 1) {
             if (n_kv > 0) {
                 ex_ml[r] = make_float2(m, l);
-                if (last_phase >= 0) {
+                if (n_p > 0) {
                     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");       // (the ring was the copy engine's and the tensor core's)
 #pragma unroll
                     for (int c = 0; c < 4; ++c) {
@@ -374,7 +392,7 @@ mqa_decode_wide_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_c
     }
     tc_fence_before();
     __syncthreads();
-    if (warp == kWideMmaWarp) {
+    if (warp == kWideSWarp) {
         tc_fence_after();
         tmem_dealloc(tmem_base, 512);
     }
