@@ -321,33 +321,39 @@ EncodeTiledFn encode_fn() {
     return f;
 }
 
-// A row-major bf16 matrix [rows][cols] fetched in boxes of box_rows rows x 64 columns (128-byte swizzle).
+// A row-major bf16 tensor [planes][rows][cols] fetched in boxes of box_planes x box_rows rows x 64 columns (128-byte swizzle).
 // A decoding loop asks for the same few maps at every step (the cache, the weights) and encoding one costs about a
 // microsecond of host time, so every thread keeps the maps it encoded last, by (address, shape, box): a map describes
 // nothing but those, so it stays valid whatever the memory holds.
-bool encode_matrix_map(CUtensorMap* map, const void* base, long long rows, long long cols, int box_rows) {
-    struct Entry { const void* base; long long rows, cols; int box_rows; bool used; CUtensorMap map; };
-    constexpr int kEntries = 32;
+bool encode_map(CUtensorMap* map, const void* base, long long planes, long long rows, long long cols, int box_planes, int box_rows) {
+    struct Entry { const void* base; long long planes, rows, cols; int box_planes, box_rows; bool used; CUtensorMap map; };
+    constexpr int kEntries = 64;
     thread_local Entry kept[kEntries] = {};
     size_t hash = reinterpret_cast<size_t>(base) >> 8;
     hash = (hash ^ (hash >> 7) ^ (size_t)rows * 31u ^ (size_t)cols * 131u ^ (size_t)box_rows * 7u) % kEntries;
     Entry& e = kept[hash];
-    if (e.used && e.base == base && e.rows == rows && e.cols == cols && e.box_rows == box_rows) {
+    if (e.used && e.base == base && e.planes == planes && e.rows == rows && e.cols == cols && e.box_planes == box_planes &&
+        e.box_rows == box_rows) {
         *map = e.map;
         return true;
     }
     EncodeTiledFn enc = encode_fn();
     if (!enc) return false;
-    const cuuint64_t dims[2] = {(cuuint64_t)cols, (cuuint64_t)rows};
-    const cuuint64_t strides[1] = {(cuuint64_t)cols * 2};
-    const cuuint32_t box[2] = {(cuuint32_t)kBoxCols, (cuuint32_t)box_rows};
-    const cuuint32_t elem[2] = {1, 1};
-    if (enc(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<void*>(base), dims, strides, box, elem,
+    const cuuint64_t dims[3] = {(cuuint64_t)cols, (cuuint64_t)rows, (cuuint64_t)planes};
+    const cuuint64_t strides[2] = {(cuuint64_t)cols * 2, (cuuint64_t)cols * (cuuint64_t)rows * 2};
+    const cuuint32_t box[3] = {(cuuint32_t)kBoxCols, (cuuint32_t)box_rows, (cuuint32_t)box_planes};
+    const cuuint32_t elem[3] = {1, 1, 1};
+    if (enc(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, planes > 0 ? 3 : 2, const_cast<void*>(base), dims, strides, box, elem,
             CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
             CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
         return false;
-    e.base = base; e.rows = rows; e.cols = cols; e.box_rows = box_rows; e.map = *map; e.used = true;
+    e.base = base; e.planes = planes; e.rows = rows; e.cols = cols; e.box_planes = box_planes; e.box_rows = box_rows; e.map = *map; e.used = true;
     return true;
+}
+
+// A matrix [rows][cols] in boxes of box_rows rows: a 2-D map.
+bool encode_matrix_map(CUtensorMap* map, const void* base, long long rows, long long cols, int box_rows) {
+    return encode_map(map, base, 0, rows, cols, 0, box_rows);
 }
 
 // The cache of one tensor (K or V) as a 2-D bf16 tensor [rows = b * m_max][128 columns], fetched in
@@ -1052,6 +1058,45 @@ static int check_prefill_dims(int b, int h, int n, int m_max, int k, int v) {
     return MQA_OK;
 }
 
+// The tiles of a sequence: of all heads x positions with at most 128 rows the one with the fewest tiles (rows past the last
+// position or head are work for nothing: with 128 positions of one head per tile, 16 positions of 32 heads would fill an eighth of
+// their rows); among equals the most positions, whose tiles share their last stages.
+static PfShape prefill_shape(int b, int h, int n, int m_max) {
+    PfShape sh = {};
+    sh.b = b; sh.h = h; sh.n = n; sh.m_max = m_max;
+    for (int heads = 1; heads <= kPfRows && heads <= h; ++heads) {
+        const int positions = kPfRows / heads < n ? kPfRows / heads : n;
+        const int head_blocks = (h + heads - 1) / heads;
+        const int tiles = (n + positions - 1) / positions * head_blocks;     // (at most 2 h n / 128 + h: checked with the sizes)
+        if (heads == 1 || tiles < sh.n_tiles) {
+            sh.positions = positions; sh.heads = heads; sh.head_blocks = head_blocks; sh.n_tiles = tiles;
+        }
+        if ((long long)sh.n_tiles * kPfRows < (long long)h * n + kPfRows) break;      // no shape has fewer
+    }
+    sh.n_units = (sh.n_tiles + 1) / 2;
+    sh.group = sh.head_blocks / 2 > 1 ? sh.head_blocks / 2 : 1;
+    sh.n_items = (sh.n_units + sh.group - 1) / sh.group * sh.group * b;
+    return sh;
+}
+
+// CTAs (one cluster) that share a unit's stages, where there are fewer units than SMs: by a model of the time.  Measured, us
+// for 1 / 2 / 4 / 8 CTAs per unit: 60 units of up to 24 stages 41.3 / 32.8 / 43.8 / 69.1 (4 do not fit at once); 64 of 16: 30.5 / 26.3 / 35.8;
+// 32 of 16: 28.8 / 25.6 / 20.1 / 45.4; 16 of 32: 53.3 / 38.1 / 25.4 / 29.4 (clusters of 8 do not fill every GPC); 1 of 17: 21.5 / 18.3 /
+// 12.6 / 9.9; 16 of 4: 16.5 / 18.8 / 31.2.
+static int prefill_split(const PfShape& sh, int rows, int sms) {
+    const double stage_us = 1.4, unit_us = 4.0, merge_us = 4.0;
+    const int stages = (rows + kPfRows - 1) / kPfRows;
+    if (sh.n_items > 2 * sms) return 1;
+    int best = 1;
+    double best_us = 0;
+    for (int ctas = 1; ctas <= kPfMaxSplit && ctas * 2 <= (stages > 2 ? stages : 2); ctas *= 2) {
+        const int slots = ctas == 8 ? sms / 16 : ctas == 4 ? sms * 9 / 40 : sms / ctas;
+        const double us = (double)((sh.n_items + slots - 1) / slots) * ((double)((stages + ctas - 1) / ctas) * stage_us + unit_us + (ctas > 1 ? merge_us : 0));
+        if (best_us == 0 || us < 0.93 * best_us) { best = ctas; best_us = us; }
+    }
+    return best;
+}
+
 size_t mqa_prefill_workspace_bytes(int b, int h, int n, int m_max, int k, int v) {
     return check_prefill_dims(b, h, n, m_max, k, v) == MQA_OK ? 16 : 0;     // (the kernel keeps everything on chip)
 }
@@ -1071,22 +1116,25 @@ int mqa_prefill_attention(const void* Q, const void* K, const void* V, const int
     int dev = 0;
     if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxDevices) { cudaGetLastError(); return MQA_ERR_CUDA; }
     if (!opt_in[dev].load(std::memory_order_acquire)) {
-        if (cudaFuncSetAttribute(mqa_prefill_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kPfSmemBytes) != cudaSuccess) {
+        if (cudaFuncSetAttribute(mqa_prefill_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, kPfSmemBytes) != cudaSuccess ||
+            cudaFuncSetAttribute(mqa_prefill_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, kPfSmemBytes) != cudaSuccess) {
             cudaGetLastError();
             return MQA_ERR_CUDA;
         }
         opt_in[dev].store(1, std::memory_order_release);
     }
-    // a unit of work per (tile of 128 positions, pair of heads, sequence); the last tile of a head may be partly filled.
-    // One CTA per SM walks the units, longest first.
-    const long long ctas = (long long)((n + kPfRows - 1) / kPfRows) * b * ((h + 1) / 2);
-    const unsigned grid = (unsigned)(ctas < sm_count() ? ctas : sm_count());
+    const PfShape sh = prefill_shape(b, h, n, m_max);
+    const int sms = sm_count(), ctas = prefill_split(sh, start ? m_max : n, sms);
     alignas(64) CUtensorMap map_q, map_k, map_v;
-    if (!encode_cache_map(&map_q, Q, (long long)b * h * n, kPfRows) || !encode_cache_map(&map_k, K, (long long)b * m_max, kPfRows) ||
-        !encode_cache_map(&map_v, V, (long long)b * m_max, kPfRows))
+    if (!encode_map(&map_q, Q, (long long)b * h, n, kHeadDim, sh.heads, sh.positions) ||
+        !encode_cache_map(&map_k, K, (long long)b * m_max, kPfRows) || !encode_cache_map(&map_v, V, (long long)b * m_max, kPfRows))
         return MQA_ERR_CUDA;
-    launch_dependent(mqa_prefill_kernel, grid, (unsigned)kPfThreads, (size_t)kPfSmemBytes, stream, map_q, map_k, map_v, start, O,
-                     status, b, h, n, m_max, (int)ctas);
+    if (ctas > 1)
+        launch_dependent_clusters((unsigned)ctas, mqa_prefill_kernel<true>, (unsigned)(sh.n_items * ctas), (unsigned)kPfThreads,
+                                  (size_t)kPfSmemBytes, stream, map_q, map_k, map_v, start, O, status, sh);
+    else
+        launch_dependent(mqa_prefill_kernel<false>, (unsigned)(sh.n_items < sms ? sh.n_items : sms), (unsigned)kPfThreads,
+                         (size_t)kPfSmemBytes, stream, map_q, map_k, map_v, start, O, status, sh);
     return launch_status();
 }
 

@@ -3,8 +3,9 @@
 // Section 2.3 for an autoregressive model.  This is the one part of the method whose arithmetic intensity is high:
 // every K/V row is used by all h heads and by every later position, so it runs against the tensor-core roofline.
 //
-// Shape of the work on sm_100a.  A CTA takes 128 consecutive positions of TWO heads of one sequence (multi-query: the
-// heads share K and V, so one staged K/V tile of 128 rows serves 256 query rows) and walks the cache rows up to its
+// Shape of the work on sm_100a.  A CTA takes TWO tiles of 128 query rows of one sequence, each 128 positions of a head or,
+// where that fills the tiles better, fewer positions of several heads (PfShape; "head" below stands for tile; multi-query:
+// the heads share K and V, so one staged K/V tile of 128 rows serves 256 query rows), and walks the cache rows up to their
 // last position in stages of 128:
 //     S_w   = Q_w K_j^T       tcgen05.mma, M = 128 query rows (TMEM lanes), N = 128 cache rows, fp32 in TMEM
 //     P_w   = exp2(S_w log2e - m)   one thread per query row: the row's maximum and sum need no other thread
@@ -28,8 +29,10 @@
 //
 // What bounds it: power.  A stage of both heads takes 2630 cycles (4400 before the logits had a buffer of their own and
 // the issuers were taken apart; the tensor cores need 2048, the exponentials 2048), and at that rate the card holds its
-// clock near 1.2 GHz.  32 x 32 heads x 4096 positions, in a loop: 5.15 ms -> 4.13 ms (1070 TFLOP/s); 5 x 9 heads x 333
-// positions: 50 -> 35 us.
+// clock near 1.2 GHz.  32 x 32 heads x 4096 positions, in a loop: 5.0 ms -> 4.13 ms (1070 TFLOP/s).  Where a call has fewer
+// units than the card has SMs it is the longest unit's chain of stages: those a cluster shares out (SPLIT).  5 x 9 heads x 333
+// positions over up to 3000 rows: 50 -> 35 us with the stages as above, 31 with tiles of 3 heads and two CTAs per unit; 5 x 2 x 108
+// over 2257: 36 -> 16; 7 x 22 x 200: 21 -> 13.6.
 // Every wait is bounded; a wait that runs out flags PIPELINE_TIMEOUT and the CTA drains and leaves.
 #pragma once
 #include "decode_umma.cuh"
@@ -43,6 +46,7 @@ constexpr int kPfKSlots = 2, kPfVSlots = 2;
 constexpr int kPfThreads = 12 * 32;                            // (warps 10 and 11 only complete the third warpgroup)
 constexpr int kPfProducerWarp = 8, kPfSWarp = 9, kPfPvWarp = 10;
 constexpr int kPfRegsSoftmax = 216, kPfRegsOther = 72;
+constexpr int kPfMaxSplit = 8;                                 // CTAs that share a unit's stages
 constexpr float kPfMaxLead = 8.f;                              // log2 units a logit may exceed its row's reference by
 // barriers: q_full, k_full/k_empty[2], v_full/v_empty[2], s_ready[2], p_ready[2], pv_done[2], s_free, q_empty
 constexpr int kPfBarriers = 1 + 2 * kPfKSlots + 2 * kPfVSlots + 6 + 2;
@@ -79,40 +83,106 @@ __device__ __forceinline__ float max3(float a, float b, float c) {
 // unit, so that a bounded wait runs out.
 __device__ int g_test_withhold = 0;
 
-// One unit of work: 128 positions of a pair of heads of one sequence.  Units are numbered ((n_tiles - 1 - position tile) *
-// b + sequence) * head pairs + pair, the longest first; CTA c takes units c, c + grid, c + 2 grid, ... one after the other
-// (a persistent kernel: barriers, tensor memory and the K/V rings are set up once, and the next unit's Q and first stages
-// are fetched, and its first logits computed, while the softmax warps still write the unit before out).
-struct PfItem {
-    int seq, p0, head0, n_act, raw, L, n_kv;
-    bool hilo;
-    long long q_row0;
+// A tile is `positions` consecutive positions of `heads` consecutive heads, positions * heads <= 128 rows: row r is position
+// r % positions of head r / positions (one box of Q as a [b h][n][128] tensor).  A sequence's tiles are numbered position
+// block by position block, the heads' blocks within it, and a unit of work is two tiles in a row.  Units go out in groups of
+// those that share a position block, the longest memories first, all sequences of a group after one another; CTA c takes
+// units c, 2 grid - 1 - c, ... one after the other (a persistent kernel: barriers, tensor memory and the K/V rings are set
+// up once, and the next unit's Q and first stages are fetched, and its first logits computed, while the softmax warps
+// still write the unit before out).
+struct PfShape {
+    int b, h, n, m_max;
+    int positions, heads;                 // of a tile
+    int head_blocks, n_tiles, n_units;    // of a sequence
+    int group;                            // units that go out together for one sequence
+    int n_items;
 };
-__device__ __forceinline__ PfItem pf_item(int item, const int32_t* __restrict__ start, int b, int h, int n, int m_max) {
+struct PfItem {
+    int seq, raw, L, n_kv;
+    int tile0, n_act;                     // its first tile, how many it has (the last unit of a sequence may have one)
+    bool hilo;
+};
+__device__ __forceinline__ int pf_position(const PfShape& sh, int tile) { return tile / sh.head_blocks * sh.positions; }   // the tile's first
+__device__ __forceinline__ int pf_head(const PfShape& sh, int tile) { return tile % sh.head_blocks * sh.heads; }
+__device__ __forceinline__ PfItem pf_item(int item, const int32_t* __restrict__ start, const PfShape& sh) {
     PfItem it;
-    const int pairs = (h + 1) >> 1, n_tiles = (n + kPfRows - 1) / kPfRows;
-    const int pair = item % pairs;
-    it.seq = (item / pairs) % b;
-    it.p0 = (n_tiles - 1 - item / (pairs * b)) * kPfRows;        // first query position of the tile
-    it.head0 = 2 * pair;
-    it.n_act = it.head0 + 1 < h ? 2 : 1;                         // heads of the unit (an odd head count leaves one alone)
-    it.raw = start ? __ldg(start + it.seq) : 0;
-    // rows of the memory the tile's last position sees (the last tile of a head may hold fewer than 128 positions: the
-    // rows after them are computed on whatever the Q tile holds there and never stored); a memory that would pass m_max
-    // is cut there
-    it.L = it.raw + min(it.p0 + kPfRows, n);
-    if (it.L > m_max) it.L = m_max;
-    const bool empty = it.raw < 0 || it.L <= 0;                  // nothing to look at: zeros (like a bad lens)
+    it.seq = (item / sh.group) % sh.b;
+    const int unit = sh.n_units - 1 - (item / (sh.group * sh.b) * sh.group + item % sh.group);
+    it.n_act = unit < 0 ? 0 : min(2, sh.n_tiles - 2 * unit);     // (the last group may be partly filled)
+    it.raw = start ? min(__ldg(start + it.seq), sh.m_max) : 0;
+    it.tile0 = 2 * unit;
+    // rows of the memory the unit's last position sees (rows of a tile past the last position or head are computed on
+    // whatever the Q tile holds there and never stored); a memory that would pass m_max is cut there
+    it.L = min(it.raw + min(pf_position(sh, it.tile0 + it.n_act - 1) + sh.positions, sh.n), sh.m_max);
+    const bool empty = it.n_act == 0 || it.raw < 0 || it.L <= 0; // nothing to look at: zeros (like a bad lens)
     it.n_kv = empty ? 0 : (it.L + kPfRows - 1) / kPfRows;        // stages
-    it.hilo = it.L < kSingleRoundingMinRows;
-    it.q_row0 = ((long long)it.seq * h + it.head0) * n + it.p0;  // row of head 0's first query in [b h n, 128]
+    // one rounding of the weights from the block of 128 positions on whose last one sees kSingleRoundingMinRows rows,
+    // whatever the tiles' shape
+    it.hilo = min(it.raw + min((pf_position(sh, it.tile0) & ~(kPfRows - 1)) + kPfRows, sh.n), sh.m_max) < kSingleRoundingMinRows;
     return it;
 }
+// The row of [b h n, 128] that row r of the unit's tile w is, or -1.
+__device__ __forceinline__ int pf_row(const PfItem& it, const PfShape& sh, int w, int r) {
+    const int hh = r / sh.positions, head = pf_head(sh, it.tile0 + w) + hh, pos = pf_position(sh, it.tile0 + w) + r - hh * sh.positions;
+    return hh < sh.heads && head < sh.h && pos < sh.n && w < it.n_act ? (it.seq * sh.h + head) * sh.n + pos : -1;
+}
+__device__ __forceinline__ void tma_load_3d(uint32_t dst, const CUtensorMap* map, int x, int y, int z, uint32_t bar) {
+    asm volatile(
+        "cp.async.bulk.tensor.3d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4}], [%5];"
+        ::"r"(dst), "l"(map), "r"(x), "r"(y), "r"(z), "r"(bar) : "memory");
+}
 
+// The rows warp, warp + 8 CTAS, ... of a unit, merged out of the CTAS shares (rank order) and stored: a warp per row, a lane 16
+// bytes of it.  All the remote loads of 16 / CTAS rows are in flight at once (row by row, a round trip each, the merge of
+// two shares took about 6 us).
+template <int CTAS>
+__device__ __forceinline__ void pf_merge(const PfItem& it, const PfShape& sh, float* __restrict__ O, uint32_t ml_s, uint32_t rows_s,
+                                         int row0, int lane) {
+    constexpr int R = 16 / CTAS;
+#pragma unroll 1
+    for (int i0 = row0; i0 < 2 * kPfRows; i0 += 8 * CTAS * R) {
+        int row[R];
+        float2 ml[R][CTAS];
+        float4 part[R][CTAS];
+#pragma unroll
+        for (int i = 0; i < R; ++i) {
+            const int rr = i0 + i * 8 * CTAS;                    // (2 * kPfRows is a multiple of 8 * CTAS * R)
+            row[i] = pf_row(it, sh, rr / kPfRows, rr % kPfRows);
+            if (row[i] < 0) continue;
+#pragma unroll
+            for (int c = 0; c < CTAS; ++c) {
+                ml[i][c] = cluster_ld_f2(cluster_map(ml_s + rr * 8, c));
+                part[i][c] = cluster_ld_f4(cluster_map(rows_s + rr * 512 + ((lane ^ (rr & 31)) << 4), c));
+            }
+        }
+#pragma unroll
+        for (int i = 0; i < R; ++i) {
+            if (row[i] < 0) continue;
+            float top = -INFINITY, den = 0.f;
+            float4 num = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+            for (int c = 0; c < CTAS; ++c) top = fmaxf(top, ml[i][c].x);
+#pragma unroll
+            for (int c = 0; c < CTAS; ++c) {
+                if (ml[i][c].x == -INFINITY) continue;           // nothing of this share is visible to the row (it may never have been written)
+                const float f = fast_exp2(ml[i][c].x - top);
+                den = fmaf(f, ml[i][c].y, den);
+                num.x = fmaf(f, part[i][c].x, num.x); num.y = fmaf(f, part[i][c].y, num.y);
+                num.z = fmaf(f, part[i][c].z, num.z); num.w = fmaf(f, part[i][c].w, num.w);
+            }
+            const float inv = it.n_kv > 0 ? 1.f / den : 0.f;
+            *reinterpret_cast<float4*>(O + (size_t)row[i] * kHeadDim + lane * 4) = make_float4(num.x * inv, num.y * inv, num.z * inv, num.w * inv);
+        }
+    }
+}
+
+// SPLIT: fewer units than SMs.  The CTAs of a cluster share a unit's stages, each a run of them, and merge their partial
+// softmaxes through distributed shared memory (rank order; the rows of the two tiles are shared out over the CTAs).
+template <bool SPLIT>
 __global__ void __launch_bounds__(kPfThreads, 1)
 mqa_prefill_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CUtensorMap map_k,
                    const __grid_constant__ CUtensorMap map_v, const int32_t* __restrict__ start, float* __restrict__ O,
-                   int32_t* __restrict__ status, int b, int h, int n, int m_max, int n_items) {
+                   int32_t* __restrict__ status, const PfShape sh) {
     const int warp = __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0), lane = threadIdx.x & 31;
 
     extern __shared__ uint8_t smem_raw[];
@@ -151,15 +221,20 @@ mqa_prefill_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
     grid_dependency_wait();              // Q, K, V and start may come from the kernel before
     grid_launch_dependents();
     // the units of this CTA: c, 2G - 1 - c, 2G + c, 4G - 1 - c, ... (G CTAs; the units come longest first, so taking them
-    // forwards and backwards in turn evens the CTAs' totals out)
+    // forwards and backwards in turn evens the CTAs' totals out); with SPLIT one unit per cluster
+    const int n_items = sh.n_items, ctas = SPLIT ? (int)cluster_size() : 1, rank = SPLIT ? (int)cluster_cta_rank() : 0;
     auto pf_unit = [&](int round) -> int {
         const int G = (int)gridDim.x, c = (int)blockIdx.x;
+        if (SPLIT) return round == 0 ? c / ctas : n_items;
         return round * G + ((round & 1) ? G - 1 - c : c);
     };
+    // this CTA's stages of a unit: [first, first + count)
+    auto first_stage = [&](int n_kv) { return SPLIT ? rank * n_kv / ctas : 0; };
+    auto count_stages = [&](int n_kv) { return SPLIT ? (rank + 1) * n_kv / ctas - rank * n_kv / ctas : n_kv; };
     if (start && threadIdx.x < 32) {
         // a start that is negative or leaves too little room is flagged once (its rows are zeros, or the memory is cut at m_max)
         bool bad = false;
-        for (int i = blockIdx.x * 32 + threadIdx.x; i < b; i += gridDim.x * 32) bad = bad || start[i] < 0 || start[i] + n > m_max;
+        for (int i = blockIdx.x * 32 + threadIdx.x; i < sh.b; i += gridDim.x * 32) bad = bad || start[i] < 0 || start[i] > sh.m_max - sh.n;
         if (bad && status) atomicOr(status, kStatusLenClamped);
     }
 
@@ -173,18 +248,20 @@ mqa_prefill_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
             int issued_k = 0, issued_v = 0, issued_q = 0;
             const bool withhold = blockIdx.x == 0 && *reinterpret_cast<volatile int*>(&g_test_withhold) != 0;
             for (int round = 0, item; (item = pf_unit(round)) < n_items && ok; ++round) {
-                const PfItem it = pf_item(item, start, b, h, n, m_max);
-                if (it.n_kv == 0) continue;
+                const PfItem it = pf_item(item, start, sh);
+                const int first = first_stage(it.n_kv), n_kv = count_stages(it.n_kv);
+                if (n_kv == 0) continue;
                 if (qi > 0) ok = mbar_wait(q_empty, (qi - 1) & 1);            // the unit before has read its Q for the last time
                 if (!ok) break;
-                mbar_expect_tx(q_full, it.n_act * kPfTileBytes);
+                mbar_expect_tx(q_full, it.n_act * sh.positions * sh.heads * kRowBytes);
                 for (int w = 0; w < it.n_act; ++w)
                     for (int half = 0; half < 2; ++half)
-                        tma_load_2d(q_s + w * kPfTileBytes + half * kPfHalfBytes, &map_q, half * kBoxCols, (int)(it.q_row0 + (long long)w * n), q_full);
+                        tma_load_3d(q_s + w * kPfTileBytes + half * kPfHalfBytes, &map_q, half * kBoxCols, pf_position(sh, it.tile0 + w),
+                                    it.seq * sh.h + pf_head(sh, it.tile0 + w), q_full);
                 issued_q = qi + 1;
-                for (int j = 0; j < it.n_kv && ok; ++j) {
+                for (int j = 0; j < n_kv && ok; ++j) {
                     const int G = g + j;
-                    const int y = it.seq * m_max + j * kPfRows;
+                    const int y = it.seq * sh.m_max + (first + j) * kPfRows;
                     const int ks = G % kPfKSlots, vs = G % kPfVSlots;
                     if (G >= kPfKSlots) ok = mbar_wait(k_empty + 8 * ks, ((G / kPfKSlots) - 1) & 1);
                     if (!ok) break;
@@ -199,7 +276,7 @@ mqa_prefill_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
                     if (!(withhold && G == 1)) tma_load_2d(v_ring + vs * kPfTileBytes + kPfHalfBytes, &map_v, kBoxCols, y, v_full + 8 * vs);
                     issued_v = G + 1;
                 }
-                g += it.n_kv;
+                g += n_kv;
                 ++qi;
             }
             if (!ok) {
@@ -217,8 +294,8 @@ mqa_prefill_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
         bool ok = true;
         int g = 0, qi = 0, n_s = 0;                              // stages, units and logits so far
         for (int round = 0, item; (item = pf_unit(round)) < n_items && ok; ++round) {
-            const PfItem it = pf_item(item, start, b, h, n, m_max);
-            const int n_kv = __shfl_sync(0xffffffffu, it.n_kv, 0), n_act = it.n_act;
+            const PfItem it = pf_item(item, start, sh);
+            const int n_kv = __shfl_sync(0xffffffffu, count_stages(it.n_kv), 0), n_act = it.n_act;
             if (n_kv == 0) continue;
             ok = warp_wait(q_full, qi & 1);
             for (int j = 0; j < n_kv && ok; ++j, ++g) {
@@ -255,8 +332,8 @@ mqa_prefill_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
         bool ok = true;
         int g = 0, n_p[2] = {0, 0};                              // stages and each head's weights so far
         for (int round = 0, item; (item = pf_unit(round)) < n_items && ok; ++round) {
-            const PfItem it = pf_item(item, start, b, h, n, m_max);
-            const int n_kv = __shfl_sync(0xffffffffu, it.n_kv, 0), n_act = it.n_act, parts = __any_sync(0xffffffffu, it.hilo) ? 2 : 1;
+            const PfItem it = pf_item(item, start, sh);
+            const int n_kv = __shfl_sync(0xffffffffu, count_stages(it.n_kv), 0), n_act = it.n_act, parts = __any_sync(0xffffffffu, it.hilo) ? 2 : 1;
             for (int j = 0; j < n_kv && ok; ++j, ++g) {
                 const int slot = g % kPfVSlots;
                 const uint32_t v_s = v_ring + slot * kPfTileBytes;
@@ -282,6 +359,7 @@ mqa_prefill_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
         }
         if (!ok && lane == 0) atomicExch(&timed_out, 1);
     }
+    if (SPLIT) cluster_sync();           // (the softmax warps' first one)
     } else {
         asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(kPfRegsSoftmax));
         // =============================================================== softmax warps: one thread per query row
@@ -292,21 +370,21 @@ mqa_prefill_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
         bool ok = true;
         int g = 0, n_s = 0, n_p = 0;                             // stages of the CTA, logits and weights of this head so far
         for (int round = 0, item; (item = pf_unit(round)) < n_items; ++round) {
-            const PfItem it = pf_item(item, start, b, h, n, m_max);
-            if (w >= it.n_act) { g += it.n_kv; continue; }       // (an odd head count: the unit has one head)
-            const int p0 = it.p0, raw = it.raw;
-            float* dst = O + (size_t)(it.q_row0 + (long long)w * n + r) * kHeadDim;
-            const bool stored = p0 + r < n;                      // (a position of this head)
-            if (it.n_kv == 0) {
-                if (stored)
-                    for (int i = 0; i < kHeadDim; i += 4) *reinterpret_cast<float4*>(dst + i) = make_float4(0.f, 0.f, 0.f, 0.f);
+            const PfItem it = pf_item(item, start, sh);
+            const int first = first_stage(it.n_kv), n_kv = count_stages(it.n_kv);
+            const int my_row = pf_row(it, sh, w, r);             // where this thread's row of O goes (-1: nowhere)
+            if (!SPLIT && w >= it.n_act) { g += n_kv; continue; }        // (the last unit of a sequence may have one tile)
+            if (!SPLIT && n_kv == 0) {
+                if (my_row >= 0)
+                    for (int i = 0; i < kHeadDim; i += 4) *reinterpret_cast<float4*>(O + (size_t)my_row * kHeadDim + i) = make_float4(0.f, 0.f, 0.f, 0.f);
                 continue;
             }
-            const int lim_first = min(raw + p0 + 1, it.L);       // rows the tile's first position sees
-            const int lim = min(raw + p0 + r + 1, it.L);         // rows this thread's position sees: >= 1
+            const int p0 = pf_position(sh, it.tile0 + w);
+            const int lim_first = min(it.raw + p0 + 1, it.L);            // rows the tile's first position sees
+            const int lim = min(it.raw + min(p0 + r % sh.positions, sh.n - 1) + 1, it.L);   // rows this thread's position sees: >= 1
             float m = -INFINITY, l = 0.f;                        // reference maximum (log2 units), sum of weights
-            for (int j = 0; j < it.n_kv; ++j) {
-                const int k0 = j * kPfRows;
+            for (int j = 0; j < (w < it.n_act ? n_kv : 0); ++j) {
+                const int k0 = (first + j) * kPfRows;
                 if (ok) ok = mbar_wait(s_ready + 8 * w, n_s & 1);
                 ++n_s;
                 tc_fence_after();
@@ -333,7 +411,8 @@ mqa_prefill_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
                 if (__any_sync(0xffffffffu, mx > m + kPfMaxLead)) {
                     const float m_new = fmaxf(m, mx);
                     if (j > 0) {
-                        const float f = fast_exp2(m - m_new);         // (m is finite from the first stage on)
+                        // (m is finite from the unit's first stage on; of a run of its stages a row may have seen nothing yet)
+                        const float f = SPLIT && m == m_new ? 1.f : fast_exp2(m - m_new);
                         l *= f;
                         if (ok) ok = mbar_wait(pv_done + 8 * w, (n_p - 1) & 1);           // O holds the stages before this one
                         tc_fence_after();
@@ -349,7 +428,8 @@ mqa_prefill_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
                     }
                     m = m_new;
                 }
-                const unsigned long long neg_m2 = f2_pack(-m, -m), log2e2 = f2_pack(kLog2e, kLog2e);
+                const float neg_m = SPLIT && m == -INFINITY ? 0.f : -m;
+                const unsigned long long neg_m2 = f2_pack(neg_m, neg_m), log2e2 = f2_pack(kLog2e, kLog2e);
                 unsigned long long sum2[2] = {0ull, 0ull};
                 // the weights stay in registers until the product before has read the ones in tensor memory
                 uint32_t hi[2][32];
@@ -384,7 +464,7 @@ mqa_prefill_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
                 tmem_st32(p_t + 32, hi[1]);
                 tmem_wait_st();
                 tc_fence_before();
-                if (w == 0 && j == it.n_kv - 1 && it.L < k0 + kPfRows) {
+                if (w == 0 && it.L < k0 + kPfRows) {
                     // the last stage runs past the memory: the tensor core would multiply the zero weights with
                     // whatever lies there (NaN * 0 = NaN), so those V rows are cleared first
                     const int vs = (g + j) % kPfVSlots;
@@ -413,6 +493,29 @@ mqa_prefill_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
                     ++n_p;
                 }
             }
+            if (SPLIT) {
+                // ---- this CTA's share: (maximum, sum) and rows of O into shared memory (the K and V rings, once both tiles'
+                // products are done), 16-byte pieces swizzled by row
+                if (n_p > 0 && ok) ok = mbar_wait(pv_done + 8 * w, (n_p - 1) & 1);
+                tc_fence_after();
+                named_barrier(1, 256);
+                asm volatile("st.shared.v2.f32 [%0], {%1,%2};" ::"r"(out_s + (w * 128 + r) * 8), "f"(m), "f"(l) : "memory");
+                if (n_p > 0) {
+                    const uint32_t ex_o = k_ring + (w * 128 + r) * 512;
+                    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");       // (the rings were the copy engine's and the tensor core's)
+#pragma unroll
+                    for (int c = 0; c < 4; ++c) {
+                        uint32_t y[32];
+                        tmem_ld32(o_t + c * 32, y);
+                        tmem_wait_ld();
+#pragma unroll
+                        for (int i = 0; i < 8; ++i)
+                            asm volatile("st.shared.v4.b32 [%0], {%1,%2,%3,%4};" ::"r"(ex_o + (((c * 8 + i) ^ (r & 31)) << 4)), "r"(y[4 * i]),
+                                         "r"(y[4 * i + 1]), "r"(y[4 * i + 2]), "r"(y[4 * i + 3]) : "memory");
+                    }
+                }
+                break;
+            }
             // ---- the row of O, divided by the sum of its weights
             if (ok) ok = mbar_wait(pv_done + 8 * w, (n_p - 1) & 1);
             tc_fence_after();
@@ -432,20 +535,28 @@ mqa_prefill_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
                 __syncwarp();
 #pragma unroll
                 for (int i = 0; i < 8; ++i) {
-                    const int rr = i * 4 + (lane >> 3), row = quarter * 32 + rr;
+                    const int rr = i * 4 + (lane >> 3), row = __shfl_sync(0xffffffffu, my_row, rr);
                     float4 v;
                     asm volatile("ld.shared.v4.f32 {%0,%1,%2,%3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w)
                                  : "r"(out_w + rr * 128 + (((lane & 7) ^ (rr & 7)) << 4)) : "memory");
-                    if (p0 + row < n)
-                        *reinterpret_cast<float4*>(O + (size_t)(it.q_row0 + (long long)w * n + row) * kHeadDim + c * 32 + (lane & 7) * 4) = v;
+                    if (row >= 0) *reinterpret_cast<float4*>(O + (size_t)row * kHeadDim + c * 32 + (lane & 7) * 4) = v;
                 }
                 __syncwarp();
             }
             tc_fence_before();                                   // (the next unit's first product overwrites O once its weights are in)
-            g += it.n_kv;
+            g += n_kv;
         }
         if (!ok) atomicExch(&timed_out, 1);
+        if (SPLIT) {
+            // (in here, where a thread has the registers for it)
+            cluster_sync();                                      // every CTA's rows are in its shared memory
+            const PfItem it = pf_item((int)blockIdx.x / ctas, start, sh);
+            if (ctas == 2) pf_merge<2>(it, sh, O, out_s, k_ring, warp + 8 * rank, lane);
+            else if (ctas == 4) pf_merge<4>(it, sh, O, out_s, k_ring, warp + 8 * rank, lane);
+            else pf_merge<8>(it, sh, O, out_s, k_ring, warp + 8 * rank, lane);
+        }
     }
+    if (SPLIT) cluster_sync();           // nobody leaves while its shared memory is being read
     tc_fence_before();
     __syncthreads();
     if (warp == kPfSWarp) {

@@ -123,6 +123,38 @@ def test_whole_tiles_match_oracle(b, h, n, m_max, start):
     run(b, h, n, m_max, start, seed=7 * b + h)
 
 
+@pytest.mark.parametrize("b,h,n,m_max,start", [
+    # tiles of several heads: rows past the last position, past the last head, a tile alone in its unit, more heads than rows
+    (2, 9, 45, 400, [0, 355]), (3, 20, 16, 1100, [1084, 0, 500]), (1, 33, 7, 64, [3]), (2, 128, 3, 40, [0, 37]), (1, 130, 2, 20, None),
+    (1, 6, 130, 130, None), (2, 7, 21, 1030, [1003, 1009]),
+    # few units: 2, 4 and 8 CTAs share a unit's stages; stages that some rows, or some CTAs, see nothing of
+    (5, 9, 333, 3000, [0, 2667, 100, 1300, 700]), (8, 16, 64, 2000, [0, 1, 63, 64, 127, 900, 1935, 1936]), (1, 4, 16, 2064, [2048]),
+    (1, 4, 16, 2064, [0]), (2, 3, 100, 1500, [1400, 130]), (1, 1, 1500, 1500, None), (3, 2, 128, 4096, [3968, 0, 895]),
+])
+def test_tile_shapes_and_shared_units(b, h, n, m_max, start):
+    run(b, h, n, m_max, start, seed=b + 3 * h + n)
+
+
+def test_shared_units_with_a_negative_start_and_one_past_the_memory():
+    """The same units shared by a cluster: nothing to look at gives zeros, a memory that would pass m_max is cut there."""
+    b, h, n, m_max = 3, 4, 16, 2064
+    gen = torch.Generator(device=DEV).manual_seed(41)
+    Q = wl.bf16_normal((b, h, n, 128), 128 ** -0.5, gen, DEV)
+    K = wl.bf16_normal((b, m_max, 128), 1.0, gen, DEV)
+    V = wl.bf16_normal((b, m_max, 128), 1.0, gen, DEV)
+    st = np.array([-5, m_max - 3, 1000], np.int32)
+    O = torch.full((b, h, n, 128), float("nan"), dtype=torch.float32, device=DEV)
+    status = torch.zeros(1, dtype=torch.int32, device=DEV)
+    mqa.mqa_prefill_attention(Q, K, V, O, torch.empty(16, dtype=torch.uint8, device=DEV), torch.from_numpy(st).to(DEV), status)
+    torch.cuda.synchronize()
+    assert int(status.item()) == binding.STATUS_LEN_CLAMPED
+    assert bool((O[0] == 0).all())
+    for t in range(n):
+        lens = np.clip(st + t + 1, 0, m_max).astype(np.int32)
+        ref = oracle.mqa_decode_step(wl.bits(Q[:, :, t].contiguous()), wl.bits(K), wl.bits(V), lens)
+        check_close(O[1:, :, t].cpu().numpy(), ref[1:], f"position {t}")
+
+
 def test_a_logit_far_above_every_earlier_one_in_a_long_memory():
     """A key row 300 times larger than the others, deep in a memory of more than 1024 rows, makes logits hundreds of
     units above (and below) everything before it: the rows' reference maxima move late and by a lot, and their
