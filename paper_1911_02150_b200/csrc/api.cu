@@ -368,7 +368,7 @@ template <int M_TILES, int EARLY = 0>
 int launch_mma(const Plan& p, const void* q, const void* K, const void* V, const int32_t* lens, float* o,
                float2* part_ml, float* part_acc, int32_t* status, int b, int h, int m_max, cudaStream_t stream, int len_bias,
                const void* k_new = nullptr, const void* v_new = nullptr, int32_t* lens_advance = nullptr,
-               bool withhold = false) {
+               int mode = 0) {
     using Cfg = MmaCfg<M_TILES>;
     auto kernel = mqa_decode_split_mma_kernel<M_TILES, EARLY>;
     constexpr int kSlot = (M_TILES - 1) * 3 + EARLY;
@@ -395,10 +395,13 @@ int launch_mma(const Plan& p, const void* q, const void* K, const void* V, const
     }
     launch_dependent(kernel, (unsigned)((size_t)b * p.n_splits), Cfg::kThreads, Cfg::kSmemBytes, stream, map_k, map_v,
                      map_k_big, map_v_big, static_cast<const uint32_t*>(q), lens, o, part_ml, part_acc, status, h, m_max, p.chunk_rows,
-                     p.n_splits, len_bias, fa, lens_advance, withhold ? 2 : 0);
+                     p.n_splits, len_bias, fa, lens_advance, mode);
     return cudaGetLastError() == cudaSuccess ? MQA_OK : MQA_ERR_CUDA;
 }
 
+// Sequences per SM up to which a window of several tiles gives each sequence a CTA of the fixed-split kernel (us per step, a warp per
+// sequence against that: 100 x 16 heads, window 200: 14.0 / 6.2; 290 x 8, window 64: 6.5 / 4.8; beyond two per SM it takes waves).
+constexpr int kLocalTeamSeqs = 2;
 constexpr int kLocalMaxWindow = 4096;         // the longest window the local step takes (a warp per sequence: decode_local.cuh)
 constexpr size_t kL2KeepBytes = 64u << 20;   // K and V together: half of the 126 MB L2
 constexpr int kEarlyTestWithhold = 1 << 8;    // rides on `early`: MQA_STEP_TEST_WITHHOLD_COPY
@@ -839,7 +842,7 @@ static int append_step_impl(const void* q, void* K, void* V, const void* k_new, 
         float* part_acc = alone ? nullptr : partials_acc(p, workspace);
         int32_t* move_lens = alone && advance ? lens : nullptr;
 #define MQA_MMA_STEP(TILES, EARLY) \
-    launch_mma<TILES, EARLY>(p, q, K, V, lens, o, part_ml, part_acc, status, b, h, m_max, stream, 0, k_new, v_new, move_lens, withhold)
+    launch_mma<TILES, EARLY>(p, q, K, V, lens, o, part_ml, part_acc, status, b, h, m_max, stream, 0, k_new, v_new, move_lens, withhold ? kMmaWithhold : 0)
         const int ahead = withhold ? 0 : early == kEarlyChained ? 1 : early == kEarlyAfterProjection ? 2 : 0;
         if (p.kernel == Kernel::kMma1)
             rc = ahead == 1 ? MQA_MMA_STEP(1, 1) : ahead == 2 ? MQA_MMA_STEP(1, 2) : MQA_MMA_STEP(1, 0);
@@ -876,26 +879,37 @@ int mqa_decode_local_step(const void* q, void* K, void* V, const void* k_new, co
     if (rc) return rc;
     if (!k_new || !v_new || !aligned16(k_new) || !aligned16(v_new)) return MQA_ERR_INVALID_ARG;
     if ((long long)b * window >= 0x7fffffffLL) return MQA_ERR_UNSUPPORTED;
-    if (window <= kLocalMaxWindow) {
-        // a warp per sequence: windows of a few tiles (the paper's is one), any number of heads
-        static std::atomic<int> opted[kMaxDevices];
-        int dev = 0;
-        if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxDevices) { cudaGetLastError(); return MQA_ERR_CUDA; }
-        if (!opted[dev].load(std::memory_order_acquire)) {
-            if (cudaFuncSetAttribute(mqa_decode_local_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kLocalSmemBytes) != cudaSuccess) {
-                cudaGetLastError();
-                return MQA_ERR_CUDA;
-            }
-            opted[dev].store(1, std::memory_order_release);
-        }
-        alignas(64) CUtensorMap map_k, map_v;
-        if (!encode_cache_map(&map_k, K, (long long)b * window) || !encode_cache_map(&map_v, V, (long long)b * window)) return MQA_ERR_CUDA;
-        launch_dependent(mqa_decode_local_kernel, (unsigned)((b + kLocalWarps - 1) / kLocalWarps), kLocalThreads, kLocalSmemBytes, stream,
-                         map_k, map_v, static_cast<const uint32_t*>(q), static_cast<const uint4*>(k_new), static_cast<const uint4*>(v_new),
-                         static_cast<uint4*>(K), static_cast<uint4*>(V), pos, o, status, b, h, window, advance ? 1 : 0);
-        return launch_status();
+    if (window > kLocalMaxWindow) return MQA_ERR_UNSUPPORTED;   // a window that long is the ordinary step's business
+    const int sms = sm_count();
+    if (window > kTileRows && h <= 32 && b <= kLocalTeamSeqs * sms) {
+        // few sequences, several tiles each: four warps to a sequence (and two head tiles side by side)
+        Plan p;
+        p.units = (size_t)b * h;
+        p.b = b; p.h = h;
+        p.n_splits = 1;
+        p.chunk_rows = (window + kTileRows - 1) / kTileRows * kTileRows;
+        auto launch = h <= 16 ? launch_mma<1, 0> : launch_mma<2, 0>;
+        return launch(p, q, K, V, pos, o, nullptr, nullptr, status, b, h, window, stream, 0, k_new, v_new, advance ? pos : nullptr, kMmaRing);
     }
-    return MQA_ERR_UNSUPPORTED;   // a window that long is the ordinary step's business
+    // a warp per sequence: windows of a few tiles (the paper's is one), any number of heads
+    static std::atomic<int> opted[kMaxDevices];
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxDevices) { cudaGetLastError(); return MQA_ERR_CUDA; }
+    if (!opted[dev].load(std::memory_order_acquire)) {
+        if (cudaFuncSetAttribute(mqa_decode_local_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, local_smem_bytes(kLocalMaxWarps, 2)) != cudaSuccess) {
+            cudaGetLastError();
+            return MQA_ERR_CUDA;
+        }
+        opted[dev].store(1, std::memory_order_release);
+    }
+    alignas(64) CUtensorMap map_k, map_v;
+    if (!encode_cache_map(&map_k, K, (long long)b * window) || !encode_cache_map(&map_v, V, (long long)b * window)) return MQA_ERR_CUDA;
+    const int stages = window <= kTileRows && h <= 16 ? 1 : 2;
+    const int each = (b + sms - 1) / sms, warps = each < kLocalMaxWarps ? each : kLocalMaxWarps;
+    launch_dependent(mqa_decode_local_kernel, (unsigned)((b + warps - 1) / warps), (unsigned)(warps * 32), (size_t)local_smem_bytes(warps, stages),
+                     stream, map_k, map_v, static_cast<const uint32_t*>(q), static_cast<const uint4*>(k_new), static_cast<const uint4*>(v_new),
+                     static_cast<uint4*>(K), static_cast<uint4*>(V), pos, o, status, b, h, window, advance ? 1 : 0, stages);
+    return launch_status();
 }
 
 size_t mqa_host_staging_bytes(int b, int h, int k, int v) {

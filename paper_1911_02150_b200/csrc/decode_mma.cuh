@@ -50,6 +50,7 @@ constexpr uint32_t kWaitRounds = 1u << 24;             // ... or after this many
 // The limit in force, in SM clock cycles (mqa_set_wait_limit_cycles: a test shortens it to see a wait run out).
 __device__ long long g_wait_limit_cycles = kWaitLimitCycles;
 constexpr int kSingleRoundingMinRows = 1024;            // prefixes this long feed P to the tensor cores in one bf16 rounding
+constexpr int kMmaWithhold = 2, kMmaRing = 4;           // bits of the fixed-split kernel's `mode`
 constexpr int kStreamMaxSeqs = 1024;                   // sequences the persistent kernel can index in shared memory
 
 // Ring depth must be a multiple of kRowWarps: tile i lives in stage i % kStages and belongs to
@@ -344,7 +345,9 @@ mqa_decode_split_mma_kernel(const __grid_constant__ CUtensorMap map_k, const __g
                             int32_t* __restrict__ status, int h, int m_max, int chunk_rows, int n_splits, int len_bias,
                             const FusedArgs fa, int32_t* __restrict__ lens_advance, int mode) {
     using Cfg = MmaCfg<M_TILES>;
-    const bool withhold = (mode & 2) != 0;                 // for tests: one copy is never started, so that a wait runs out (bit 0: unused)
+    const bool withhold = (mode & kMmaWithhold) != 0;      // for tests: one copy is never started, so that a wait runs out
+    // the cache is a ring of m_max rows (local attention) and lens counts the tokens so far: the new row goes to row lens % m_max
+    const bool ring = (mode & kMmaRing) != 0;
     constexpr int kStages = Cfg::kStages;
     const int seq = blockIdx.x / n_splits;
     const int split = blockIdx.x % n_splits;
@@ -446,16 +449,17 @@ mqa_decode_split_mma_kernel(const __grid_constant__ CUtensorMap map_k, const __g
     const int rw = warp / M_TILES;                         // which tiles (round-robin over kRowWarps)
     uint32_t qa[8][4];
     if (warp < Cfg::kConsumerWarps) load_q_fragments(qa, q, (size_t)seq, h, mt, lane);
-    const bool appended = fa.k_new != nullptr && raw >= 0 && raw < m_max;
-    const bool holds_new = appended && raw >= r0 && raw - r0 < chunk_rows;        // the new row is one of this split's
+    const bool appended = fa.k_new != nullptr && raw >= 0 && (ring || raw < m_max);
+    const int new_row = ring ? raw % m_max : raw;
+    const bool holds_new = appended && new_row >= r0 && new_row - r0 < chunk_rows;      // the new row is one of this split's
     if (fa.k_new != nullptr) {
         if (!appended && threadIdx.x == 0 && status) atomicOr(status, raw < 0 ? kStatusAppendNegative : kStatusAppendFull);
         if (holds_new && warp == 0) {
-            const size_t dst = ((size_t)seq * m_max + raw) * (kRowBytes / 16) + (lane & 15);
+            const size_t dst = ((size_t)seq * m_max + new_row) * (kRowBytes / 16) + (lane & 15);
             if (lane < 16) fa.K[dst] = row_piece; else fa.V[dst] = row_piece;
         }
     }
-    const int L = clamp_len(appended ? raw + 1 : biased_len(raw, m_max, len_bias), m_max,
+    const int L = clamp_len(appended ? min(raw, m_max - 1) + 1 : biased_len(raw, m_max, len_bias), m_max,
                             threadIdx.x == 0 ? status : nullptr);
     const int r1 = min(L, r0 + chunk_rows);
     if (r0 >= L) {                                         // nothing valid in this split (uniform)
@@ -500,9 +504,9 @@ mqa_decode_split_mma_kernel(const __grid_constant__ CUtensorMap map_k, const __g
             // a tile's K boxes, then its V boxes; in a copy of four tiles the tile is 32 of a box's 128 rows
             const uint32_t k_s = big ? stages_s + (i >> 2) * 4 * kStageBytes + (i & 3) * kBoxBytes : stages_s + s * kStageBytes;
             const uint32_t half = big ? 4 * kBoxBytes : kBoxBytes;
-            if (holds_new && (raw - r0) / kTileRows == i) {
+            if (holds_new && (new_row - r0) / kTileRows == i) {
                 // the new row into its place (with two head tiles both warps that read this tile write the same bytes)
-                const int row = (raw - r0) & (kTileRows - 1), c = lane & 7;
+                const int row = (new_row - r0) & (kTileRows - 1), c = lane & 7;
                 const uint32_t at = k_s + (lane >> 3) * half + row * 128 + ((c ^ (row & 7)) << 4);   // boxes: K, K, V, V
                 asm volatile("st.shared.v4.b32 [%0], {%1,%2,%3,%4};" ::"r"(at), "r"(row_piece.x), "r"(row_piece.y), "r"(row_piece.z),
                              "r"(row_piece.w) : "memory");

@@ -61,6 +61,37 @@ def test_local_attention_ring_equals_attention_over_the_last_window_rows(b, h, w
         assert np.array_equal(Kg[:, t % window], hist_k[:, t]) and np.array_equal(Vg[:, t % window], hist_v[:, t])
 
 
+@pytest.mark.parametrize("b,h,window,steps", [
+    (2, 17, 64, 130), (40, 16, 33, 70),          # four warps to a sequence: two head tiles; a tile of one row
+    (310, 8, 40, 90), (310, 20, 33, 70),         # a warp per sequence, two stages: two tiles; two passes over them
+    (1040, 5, 31, 40),                           # CTAs of seven warps, the last one partly filled, one stage
+    (150, 40, 32, 40),                           # three passes over one tile
+])
+def test_local_step_on_either_kernel(b, h, window, steps):
+    test_local_attention_ring_equals_attention_over_the_last_window_rows(b, h, window, steps)
+
+
+@pytest.mark.parametrize("b,window", [(6, 100), (320, 100)])
+def test_local_step_of_several_tiles_with_a_negative_position(b, window):
+    h = 8
+    inp = wl.make_inputs(b, h, window, "mqa", seed=4, device=DEV)
+    pos0 = np.resize(np.array([-3, 0, 31, 32, 99, 250], np.int32), b)
+    pos = torch.from_numpy(pos0).to(DEV)
+    Kh, Vh = wl.bits(inp["K"]).copy(), wl.bits(inp["V"]).copy()
+    o = torch.full((b, h, 128), float("nan"), dtype=torch.float32, device=DEV)
+    status = torch.zeros(1, dtype=torch.int32, device=DEV)
+    mqa.mqa_decode_local_step(inp["q"], inp["K"], inp["V"], inp["k_new"], inp["v_new"], pos, o, status)
+    torch.cuda.synchronize()
+    assert np.array_equal(pos.cpu().numpy(), np.where(pos0 < 0, pos0, pos0 + 1))
+    assert int(status.item()) == (binding.STATUS_APPEND_NEGATIVE_LEN | binding.STATUS_LEN_CLAMPED)
+    kn, vn = wl.bits(inp["k_new"]), wl.bits(inp["v_new"])
+    for s in np.nonzero(pos0 >= 0)[0]:
+        Kh[s, pos0[s] % window], Vh[s, pos0[s] % window] = kn[s], vn[s]
+    lens = np.clip(pos0 + 1, 0, window).astype(np.int32)
+    assert np.array_equal(wl.bits(inp["K"]), Kh) and np.array_equal(wl.bits(inp["V"]), Vh)
+    check_close(o.cpu().numpy(), oracle.mqa_decode_step(wl.bits(inp["q"]), Kh, Vh, np.maximum(lens, 0)), "local step")
+
+
 def test_local_step_without_advance_and_negative_position():
     b, h, window = 6, 8, 32
     inp = wl.make_inputs(b, h, window, "mqa", seed=2, device=DEV)
