@@ -408,7 +408,9 @@ mqa_prefill_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
 #pragma unroll
                 for (int i = 8; i < 64; ++i) mx8[i & 7] = max3(mx8[i & 7], __uint_as_float(x[2 * i]), __uint_as_float(x[2 * i + 1]));
                 const float mx = max3(max3(mx8[0], mx8[1], mx8[2]), max3(mx8[3], mx8[4], mx8[5]), fmaxf(mx8[6], mx8[7])) * kLog2e;
-                if (__any_sync(0xffffffffu, mx > m + kPfMaxLead)) {
+                // (a row that is nobody's does not count: its query is whatever shared memory held, and the moment at which a warp
+                // moves its references shows in the last bits of all of them)
+                if (__any_sync(0xffffffffu, my_row >= 0 && mx > m + kPfMaxLead)) {
                     const float m_new = fmaxf(m, mx);
                     if (j > 0) {
                         // (m is finite from the unit's first stage on; of a run of its stages a row may have seen nothing yet)
