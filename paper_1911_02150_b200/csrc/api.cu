@@ -473,6 +473,7 @@ int launch_umma_for(const Plan& p, const void* q, const void* K, const void* V, 
 
 int launch_status() { return cudaGetLastError() == cudaSuccess ? MQA_OK : MQA_ERR_CUDA; }
 
+template <int EARLY = 0>
 int launch_wide(const Plan& p, const void* q, const void* K, const void* V, const int32_t* lens, float* o, float2* part_ml,
                 float* part_acc, int32_t* status, int b, int h, int m_max, cudaStream_t stream, int len_bias,
                 const void* k_new = nullptr, const void* v_new = nullptr, int32_t* lens_advance = nullptr, bool withhold = false) {
@@ -487,7 +488,7 @@ int launch_wide(const Plan& p, const void* q, const void* K, const void* V, cons
     int dev = 0;
     if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxDevices) { cudaGetLastError(); return MQA_ERR_CUDA; }
     if (!opt_in[dev].load(std::memory_order_acquire)) {
-        if (cudaFuncSetAttribute(mqa_decode_wide_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kWideSmemBytes) != cudaSuccess) {
+        if (cudaFuncSetAttribute(mqa_decode_wide_kernel<EARLY>, cudaFuncAttributeMaxDynamicSharedMemorySize, kWideSmemBytes) != cudaSuccess) {
             cudaGetLastError();
             return MQA_ERR_CUDA;
         }
@@ -497,7 +498,7 @@ int launch_wide(const Plan& p, const void* q, const void* K, const void* V, cons
     if (!encode_cache_map(&map_q, q, (long long)b * h, kWideRows) || !encode_cache_map(&map_k, K, (long long)b * m_max, kWideRows) ||
         !encode_cache_map(&map_v, V, (long long)b * m_max, kWideRows))
         return MQA_ERR_CUDA;
-    launch_dependent_2d(mqa_decode_wide_kernel, (unsigned)((size_t)b * p.n_splits), (unsigned)((h + kWideRows - 1) / kWideRows),
+    launch_dependent_2d(mqa_decode_wide_kernel<EARLY>, (unsigned)((size_t)b * p.n_splits), (unsigned)((h + kWideRows - 1) / kWideRows),
                         (unsigned)kWideThreads, (size_t)kWideSmemBytes, stream, map_q,
                      map_k, map_v, lens, o, part_ml, part_acc, status, h, m_max, p.chunk_rows, p.n_splits, len_bias, fa, lens_advance,
                      withhold ? 1 : 0);
@@ -824,8 +825,10 @@ static int append_step_impl(const void* q, void* K, void* V, const void* k_new, 
         float* part_acc = partials_acc(p, workspace);
         // (one split and one tile of 128 rows: the CTA moves lens on itself)
         const bool alone = p.n_splits == 1 && h <= kWideRows;
-        rc = launch_wide(p, q, K, V, lens, o, part_ml, part_acc, status, b, h, m_max, stream, 0, k_new, v_new,
-                         alone && advance ? lens : nullptr, withhold);
+        const int ahead = withhold ? 0 : early == kEarlyChained ? 1 : early == kEarlyAfterProjection ? 2 : 0;
+        auto launch = ahead == 1 ? launch_wide<1> : ahead == 2 ? launch_wide<2> : launch_wide<0>;
+        rc = launch(p, q, K, V, lens, o, part_ml, part_acc, status, b, h, m_max, stream, 0, k_new, v_new,
+                    alone && advance ? lens : nullptr, withhold);
         if (rc || alone) return rc;
         if (p.n_splits == 1) {                                   // several row tiles read lens: moved on by a kernel of its own
             if (advance) launch_dependent(lens_advance_kernel, (unsigned)((b + 255) / 256), 256u, 0, stream, lens, b, m_max);

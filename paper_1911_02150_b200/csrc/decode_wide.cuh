@@ -36,6 +36,12 @@ constexpr int kWideSmemBytes = (1 + kWideKSlots + kWideVSlots) * kPfTileBytes + 
 static_assert(kWideSmemBytes + 1024 + 16 /* static */ <= 227 * 1024, "exceeds the shared memory of one SM");
 
 // grid: x = sequence * n_splits + split, y = tile of 128 query rows.  part_ml [b * h][n_splits], part_acc [b * h][n_splits][128] (combine.cuh).
+// EARLY: what is fetched before the wait for the kernel ahead -- 0 nothing; 1 (the caller's promise of a decoding loop) the
+// stages that lie wholly below the prefix's last rows by lens as it reads now, which is final or one short; 2 (behind the
+// library's own projection or host-input kernel: lens is final) the first stages whatever they hold.  In a loop of two
+// launches per step a CTA is on its SM, set up and idle, while the second pass of the step before runs
+// (8 x 16 heads x 4096 rows: 11.5 -> 11.0 us per step; 32 x 128 x 8192: 33.0 -> 32.1).
+template <int EARLY>
 __global__ void __launch_bounds__(kWideThreads, 1)
 mqa_decode_wide_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CUtensorMap map_k,
                        const __grid_constant__ CUtensorMap map_v, const int32_t* __restrict__ lens, float* __restrict__ o,
@@ -78,61 +84,98 @@ mqa_decode_wide_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_c
     tc_fence_after();
     const uint32_t tmem_base = __shfl_sync(0xffffffffu, *tmem_slot, 0);
 
+    const int r0 = split * chunk_rows;                         // this CTA's rows of the sequence's cache begin here
+    const bool producer = warp == kWideProducerWarp && lane == 0;
+    const uint64_t policy = l2_stream_policy(true);            // the cache is read once per step
+    constexpr int kAhead = kWideKSlots < kWideVSlots ? kWideKSlots : kWideVSlots;       // stages that the rings take without a wait
+    auto issue_k = [&](int j) {
+        const int ks = j % kWideKSlots, y = seq * m_max + r0 + j * kWideRows;
+        mbar_expect_tx(k_full + 8 * ks, kPfTileBytes);
+        tma_load_2d_hint(k_ring + ks * kPfTileBytes, &map_k, 0, y, k_full + 8 * ks, policy);
+        tma_load_2d_hint(k_ring + ks * kPfTileBytes + kPfHalfBytes, &map_k, kBoxCols, y, k_full + 8 * ks, policy);
+    };
+    auto issue_v = [&](int j) {
+        const int vs = j % kWideVSlots, y = seq * m_max + r0 + j * kWideRows;
+        mbar_expect_tx(v_full + 8 * vs, kPfTileBytes);
+        tma_load_2d_hint(v_ring + vs * kPfTileBytes, &map_v, 0, y, v_full + 8 * vs, policy);
+        // (for tests: one copy of the first CTA's second stage is never started, so that a wait runs out)
+        if (!(withhold && blockIdx.x == 0 && blockIdx.y == 0 && j == 1))
+            tma_load_2d_hint(v_ring + vs * kPfTileBytes + kPfHalfBytes, &map_v, kBoxCols, y, v_full + 8 * vs, policy);
+    };
+    int pre = 0, guess = 0;                                    // stages asked for so far (by the producer's thread)
+    if (EARLY != 0 && producer) {
+        guess = max(0, __ldcg(lens + seq));
+        // (2: rows in the prefix once the new one is in; 1: the step ahead writes row guess - 1 or row guess)
+        const int rows = min((EARLY == 2 ? min(guess + 1, m_max) : min(guess - 1, m_max)) - r0, chunk_rows);
+        const int ready = max(0, min(EARLY == 2 ? (rows + kWideRows - 1) / kWideRows : rows / kWideRows, kAhead));
+        for (; pre < ready; ++pre) { issue_k(pre); issue_v(pre); }
+    }
+
     grid_dependency_wait();              // q, lens and the newest cache row may come from the kernel before
     grid_launch_dependents();
-    // The append-and-attend step (fa.k_new given): the CTA whose rows hold row lens[seq] writes the new key/value row
-    // there before it fetches it (its producer warp: store, proxy fence, then the copies), every split attends over one
-    // row more, and lens moves on at the end -- here when the sequence has one split (lens_advance given), else in the
-    // second-pass kernel.
+    if (EARLY == 1 && producer) {        // the rows that the prefix has in any case
+        const int rows = min(min(guess + 1, m_max) - r0, chunk_rows);
+        const int sure = max(pre, min((rows + kWideRows - 1) / kWideRows, kAhead));
+        for (; pre < sure; ++pre) { issue_k(pre); issue_v(pre); }
+    }
+    // The append-and-attend step (fa.k_new given): the CTA whose rows hold row lens[seq] puts the new key/value row into its
+    // place in the landed stage (the warps that issue the products do) and stores it in the cache (its producer warp, with
+    // nobody waiting for it), every split attends over one row more, and lens moves on at the end -- here when the sequence
+    // has one split (lens_advance given), else in the second-pass kernel.
+    uint4 row_piece = make_uint4(0u, 0u, 0u, 0u);              // lanes 0-15: of the key row (S and producer warp), or the value row
+    if (fa.k_new != nullptr && warp >= kWideProducerWarp)      // (the producer warp's lanes 16-31 the value row)
+        row_piece = (warp == kWidePvWarp || (warp == kWideProducerWarp && lane >= 16) ? fa.v_new : fa.k_new)[(size_t)seq * (kRowBytes / 16) + (lane & 15)];
     const int raw = __ldcg(lens + seq);
     const bool appended = fa.k_new != nullptr && raw >= 0 && raw < m_max;
     if (fa.k_new != nullptr && !appended && split == 0 && blockIdx.y == 0 && threadIdx.x == 0 && status)
         atomicOr(status, raw < 0 ? kStatusAppendNegative : kStatusAppendFull);
     const int L = clamp_len(appended ? raw + 1 : biased_len(raw, m_max, len_bias), m_max, (split == 0 && blockIdx.y == 0 && threadIdx.x == 0) ? status : nullptr);
-    const int r0 = split * chunk_rows, r1 = min(r0 + chunk_rows, L);           // this CTA's rows of the sequence's cache
+    const int r1 = min(r0 + chunk_rows, L);                    // and end here
     const int n_kv = __shfl_sync(0xffffffffu, r1 > r0 ? (r1 - r0 + kWideRows - 1) / kWideRows : 0, 0);      // stages
     const bool hilo = __any_sync(0xffffffffu, L < kSingleRoundingMinRows);
+    const bool holds_new = appended && raw >= r0 && raw - r0 < chunk_rows;
+    const int new_stage = holds_new ? (raw - r0) / kWideRows : -1;
+    // the new row into a landed K or V stage, by a warp's lanes 0-15
+    auto place_row = [&](uint32_t stage_s) {
+        const int row = (raw - r0) % kWideRows;
+        if (lane < 16)
+            asm volatile("st.shared.v4.b32 [%0], {%1,%2,%3,%4};" ::"r"(stage_s + (lane >> 3) * kPfHalfBytes + row * 128 + (((lane & 7) ^ (row & 7)) << 4)),
+                         "r"(row_piece.x), "r"(row_piece.y), "r"(row_piece.z), "r"(row_piece.w) : "memory");
+        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");     // read by the tensor core
+        __syncwarp();
+    };
 
     if (warp >= 8) {
         asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(kPfRegsOther));
         if (warp == kWideProducerWarp) {
             // =========================================================== TMA producer
-            if (appended && raw >= split * chunk_rows && raw < (split + 1) * chunk_rows) {
-                const uint4 piece = (lane < 16 ? fa.k_new : fa.v_new)[(size_t)seq * (kRowBytes / 16) + (lane & 15)];
+            if (holds_new) {
                 const size_t at = ((size_t)seq * m_max + raw) * (kRowBytes / 16) + (lane & 15);
-                if (lane < 16) fa.K[at] = piece; else fa.V[at] = piece;
-                asm volatile("fence.proxy.async;" ::: "memory");    // the copy engine must see the row
-                __syncwarp();
+                if (lane < 16) fa.K[at] = row_piece; else fa.V[at] = row_piece;
             }
-            if (lane == 0 && n_kv > 0) {
+            if (lane == 0 && (n_kv > 0 || pre > 0)) {
                 bool ok = true;
-                mbar_expect_tx(q_full, kPfTileBytes);
-                for (int half = 0; half < 2; ++half)
-                    tma_load_2d(q_s + half * kPfHalfBytes, &map_q, half * kBoxCols, seq * h + row0, q_full);
-                const uint64_t policy = l2_stream_policy(true);     // the cache is read once per step
-                int issued_k = 0, issued_v = 0;
-                for (int j = 0; j < n_kv && ok; ++j) {
-                    const int y = seq * m_max + r0 + j * kWideRows;
-                    const int ks = j % kWideKSlots, vs = j % kWideVSlots;
-                    if (j >= kWideKSlots) ok = mbar_wait(k_empty + 8 * ks, ((j / kWideKSlots) - 1) & 1);
+                int issued_k = pre, issued_v = pre;
+                if (n_kv > 0) {
+                    mbar_expect_tx(q_full, kPfTileBytes);
+                    for (int half = 0; half < 2; ++half)
+                        tma_load_2d(q_s + half * kPfHalfBytes, &map_q, half * kBoxCols, seq * h + row0, q_full);
+                }
+                for (int j = pre; j < n_kv && ok; ++j) {
+                    if (j >= kWideKSlots) ok = mbar_wait(k_empty + 8 * (j % kWideKSlots), ((j / kWideKSlots) - 1) & 1);
                     if (!ok) break;
-                    mbar_expect_tx(k_full + 8 * ks, kPfTileBytes);
-                    tma_load_2d_hint(k_ring + ks * kPfTileBytes, &map_k, 0, y, k_full + 8 * ks, policy);
-                    tma_load_2d_hint(k_ring + ks * kPfTileBytes + kPfHalfBytes, &map_k, kBoxCols, y, k_full + 8 * ks, policy);
+                    issue_k(j);
                     issued_k = j + 1;
-                    if (j >= kWideVSlots) ok = mbar_wait(v_empty + 8 * vs, ((j / kWideVSlots) - 1) & 1);
+                    if (j >= kWideVSlots) ok = mbar_wait(v_empty + 8 * (j % kWideVSlots), ((j / kWideVSlots) - 1) & 1);
                     if (!ok) break;
-                    mbar_expect_tx(v_full + 8 * vs, kPfTileBytes);
-                    tma_load_2d_hint(v_ring + vs * kPfTileBytes, &map_v, 0, y, v_full + 8 * vs, policy);
-                    // (for tests: one copy of the first CTA's second stage is never started, so that a wait runs out)
-                    if (!(withhold && blockIdx.x == 0 && blockIdx.y == 0 && j == 1))
-                        tma_load_2d_hint(v_ring + vs * kPfTileBytes + kPfHalfBytes, &map_v, kBoxCols, y, v_full + 8 * vs, policy);
+                    issue_v(j);
                     issued_v = j + 1;
                 }
+                for (int j = n_kv; j < pre; ++j) ok = mbar_wait(k_full + 8 * j, 0) && mbar_wait(v_full + 8 * j, 0) && ok;   // (a broken promise)
                 if (!ok) {
                     // a wait ran out: the copies already started are given a bounded wait each before the CTA may leave
                     atomicExch(&timed_out, 1);
-                    mbar_wait(q_full, 0);
+                    if (n_kv > 0) mbar_wait(q_full, 0);
                     for (int j = max(0, issued_k - kWideKSlots); j < issued_k; ++j) mbar_wait(k_full + 8 * (j % kWideKSlots), (j / kWideKSlots) & 1);
                     for (int j = max(0, issued_v - kWideVSlots); j < issued_v; ++j) mbar_wait(v_full + 8 * (j % kWideVSlots), (j / kWideVSlots) & 1);
                 }
@@ -147,9 +190,10 @@ mqa_decode_wide_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_c
                 ok = warp_wait(k_full + 8 * slot, (j / kWideKSlots) & 1);
                 if (ok && j > 0) ok = warp_wait(s_free, (j - 1) & 1);
                 if (!ok) break;
+                const uint32_t k_s = k_ring + slot * kPfTileBytes;
+                if (j == new_stage) place_row(k_s);
                 tc_fence_after();
                 if (elect_one()) {
-                    const uint32_t k_s = k_ring + slot * kPfTileBytes;
 #pragma unroll
                     for (int ks = 0; ks < 8; ++ks) {            // 8 k-steps of 16 columns; 4 per 64-column box
                         const uint32_t off = (ks >> 2) * kPfHalfBytes + (ks & 3) * 32;
@@ -171,6 +215,7 @@ mqa_decode_wide_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_c
                 const int slot = j % kWideVSlots, w = j & 1;
                 const uint32_t v_s = v_ring + slot * kPfTileBytes;
                 ok = warp_wait(v_full + 8 * slot, (j / kWideVSlots) & 1);
+                if (ok && j == new_stage) place_row(v_s);
                 for (int part = 0; part < (hilo ? 2 : 1) && ok; ++part) {
                     ok = warp_wait(p_ready + 8 * w, n_p[w] & 1);
                     if (!ok) break;
