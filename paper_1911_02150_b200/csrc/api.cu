@@ -494,12 +494,12 @@ int launch_wide(const Plan& p, const void* q, const void* K, const void* V, cons
         }
         opt_in[dev].store(1, std::memory_order_release);
     }
-    alignas(64) CUtensorMap map_q, map_k, map_v;
-    if (!encode_cache_map(&map_q, q, (long long)b * h, kWideRows) || !encode_cache_map(&map_k, K, (long long)b * m_max, kWideRows) ||
+    alignas(64) CUtensorMap map_k, map_v;
+    if (!encode_cache_map(&map_k, K, (long long)b * m_max, kWideRows) ||
         !encode_cache_map(&map_v, V, (long long)b * m_max, kWideRows))
         return MQA_ERR_CUDA;
     launch_dependent_2d(mqa_decode_wide_kernel<EARLY>, (unsigned)((size_t)b * p.n_splits), (unsigned)((h + kWideRows - 1) / kWideRows),
-                        (unsigned)kWideThreads, (size_t)kWideSmemBytes, stream, map_q,
+                        (unsigned)kWideThreads, (size_t)kWideSmemBytes, stream, static_cast<const uint4*>(q),
                      map_k, map_v, lens, o, part_ml, part_acc, status, h, m_max, p.chunk_rows, p.n_splits, len_bias, fa, lens_advance,
                      withhold ? 1 : 0);
     return launch_status();
@@ -564,10 +564,13 @@ int run_combine(bool multi_query, const int32_t* lens, float* o, const void* wor
     // fused (the append-and-attend step of a sequence cut into fixed splits): the pass wrote a piece for every split,
     // the second pass does not look at lens and moves it on when asked to
     const int32_t* lens_read = fused ? nullptr : lens;
-    if (p.n_splits <= kCombineEager)
-        launch_dependent(combine_few_kernel, (unsigned)((p.units + kCombineFewWarps - 1) / kCombineFewWarps), (unsigned)(kCombineFewWarps * 32),
-                         0, stream, part_ml, part_acc, lens_read, o, h, m_max, p.chunk_rows, p.n_splits, len_bias,
-                         fused ? lens_advance : static_cast<int32_t*>(nullptr), p.units);
+    if (p.n_splits <= 32) {
+        // a warp per (sequence, head); with few of them each warp is a CTA of its own, so that they spread over the SMs
+        auto kernel = p.n_splits <= 8 ? combine_few_kernel<8> : p.n_splits <= 16 ? combine_few_kernel<16> : combine_few_kernel<32>;
+        const size_t warps = p.units > (size_t)8 * sm_count() ? kCombineFewWarps : 1;
+        launch_dependent(kernel, (unsigned)((p.units + warps - 1) / warps), (unsigned)(warps * 32), 0, stream, part_ml, part_acc, lens_read, o, h,
+                         m_max, p.chunk_rows, p.n_splits, len_bias, fused ? lens_advance : static_cast<int32_t*>(nullptr), p.units);
+    }
     else
         launch_dependent(combine_splits_kernel<4>, (unsigned)p.units, 4 * kHeadDim, 0, stream, part_ml, part_acc, lens_read, o, h,
                          m_max, p.chunk_rows, p.n_splits, len_bias, fused ? lens_advance : static_cast<int32_t*>(nullptr));

@@ -37,13 +37,15 @@ static_assert(kWideSmemBytes + 1024 + 16 /* static */ <= 227 * 1024, "exceeds th
 
 // grid: x = sequence * n_splits + split, y = tile of 128 query rows.  part_ml [b * h][n_splits], part_acc [b * h][n_splits][128] (combine.cuh).
 // EARLY: what is fetched before the wait for the kernel ahead -- 0 nothing; 1 (the caller's promise of a decoding loop) the
-// stages that lie wholly below the prefix's last rows by lens as it reads now, which is final or one short; 2 (behind the
-// library's own projection or host-input kernel: lens is final) the first stages whatever they hold.  In a loop of two
-// launches per step a CTA is on its SM, set up and idle, while the second pass of the step before runs
-// (8 x 16 heads x 4096 rows: 11.5 -> 11.0 us per step; 32 x 128 x 8192: 33.0 -> 32.1).
+// first stage, if it lies wholly below the prefix's last rows by lens as it reads now, which is final or one short (or else right
+// after the wait, if the prefix has its rows in any case); 2 (behind the library's own projection or host-input kernel: lens
+// is final) the first stages whatever they hold.  In a loop of two launches per step a CTA is on its SM, set up and idle, while
+// the second pass of the step before runs.  One stage and no more: q has to come next, and behind 28 MB of stages (three per
+// CTA) it took 4.7 us (us per step with 0 / 1 / 2 / 3 stages ahead: 32 x 128 rows x 8192: 30.3 / 30.4 / 31.8 / 32.1; 64 x 100 x 2048: 20.6 /
+// 19.8 / 21.0 / 21.8; 8 x 16 x 32768: 27.9 / 26.9 / 27.3 / 29.0; 8 x 16 x 4096: 11.5 / 9.6 / 9.9 / 9.6).
 template <int EARLY>
 __global__ void __launch_bounds__(kWideThreads, 1)
-mqa_decode_wide_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CUtensorMap map_k,
+mqa_decode_wide_kernel(const uint4* __restrict__ q, const __grid_constant__ CUtensorMap map_k,
                        const __grid_constant__ CUtensorMap map_v, const int32_t* __restrict__ lens, float* __restrict__ o,
                        float2* __restrict__ part_ml, float* __restrict__ part_acc, int32_t* __restrict__ status, int h,
                        int m_max, int chunk_rows, int n_splits, int len_bias, const FusedArgs fa, int32_t* __restrict__ lens_advance,
@@ -62,11 +64,11 @@ mqa_decode_wide_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_c
                    pv_done = p_ready + 16, s_free = pv_done + 16;
     uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(base + (1 + kWideKSlots + kWideVSlots) * kPfTileBytes + kWideBarriers * 8);
     __shared__ int timed_out;
-    __shared__ float2 ex_ml[kWideRows];                       // (maximum, sum) of warpgroup 1's rows, for the merge at the end
+    __shared__ float2 ex_ml[kWideRows];                       // (maximum, sum) of warpgroup 1's rows, then each row's two factors
 
     if (threadIdx.x == 0) {
-        prefetch_tensormap(&map_q); prefetch_tensormap(&map_k); prefetch_tensormap(&map_v);
-        mbar_init(q_full, 1);
+        prefetch_tensormap(&map_k); prefetch_tensormap(&map_v);
+        mbar_init(q_full, 8);
         mbar_init(s_free, 4);
         for (int i = 0; i < kWideKSlots; ++i) { mbar_init(k_full + 8 * i, 1); mbar_init(k_empty + 8 * i, 1); }
         for (int i = 0; i < kWideVSlots; ++i) { mbar_init(v_full + 8 * i, 1); mbar_init(v_empty + 8 * i, 1); }
@@ -87,7 +89,7 @@ mqa_decode_wide_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_c
     const int r0 = split * chunk_rows;                         // this CTA's rows of the sequence's cache begin here
     const bool producer = warp == kWideProducerWarp && lane == 0;
     const uint64_t policy = l2_stream_policy(true);            // the cache is read once per step
-    constexpr int kAhead = kWideKSlots < kWideVSlots ? kWideKSlots : kWideVSlots;       // stages that the rings take without a wait
+    constexpr int kAhead = EARLY == 1 ? 1 : kWideKSlots < kWideVSlots ? kWideKSlots : kWideVSlots;
     auto issue_k = [&](int j) {
         const int ks = j % kWideKSlots, y = seq * m_max + r0 + j * kWideRows;
         mbar_expect_tx(k_full + 8 * ks, kPfTileBytes);
@@ -156,11 +158,6 @@ mqa_decode_wide_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_c
             if (lane == 0 && (n_kv > 0 || pre > 0)) {
                 bool ok = true;
                 int issued_k = pre, issued_v = pre;
-                if (n_kv > 0) {
-                    mbar_expect_tx(q_full, kPfTileBytes);
-                    for (int half = 0; half < 2; ++half)
-                        tma_load_2d(q_s + half * kPfHalfBytes, &map_q, half * kBoxCols, seq * h + row0, q_full);
-                }
                 for (int j = pre; j < n_kv && ok; ++j) {
                     if (j >= kWideKSlots) ok = mbar_wait(k_empty + 8 * (j % kWideKSlots), ((j / kWideKSlots) - 1) & 1);
                     if (!ok) break;
@@ -175,7 +172,6 @@ mqa_decode_wide_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_c
                 if (!ok) {
                     // a wait ran out: the copies already started are given a bounded wait each before the CTA may leave
                     atomicExch(&timed_out, 1);
-                    if (n_kv > 0) mbar_wait(q_full, 0);
                     for (int j = max(0, issued_k - kWideKSlots); j < issued_k; ++j) mbar_wait(k_full + 8 * (j % kWideKSlots), (j / kWideKSlots) & 1);
                     for (int j = max(0, issued_v - kWideVSlots); j < issued_v; ++j) mbar_wait(v_full + 8 * (j % kWideVSlots), (j / kWideVSlots) & 1);
                 }
@@ -240,6 +236,29 @@ mqa_decode_wide_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_c
         const int w = warp >> 2, quarter = warp & 3, r = quarter * 32 + lane;
         const uint32_t lane_base = tmem_base + ((uint32_t)(quarter * 32) << 16);
         const uint32_t p_t = lane_base + kPfTmemP + w * 64, o_t = lane_base + kPfTmemO + w * 128;
+        // q, by the threads that have nothing else to do yet: 16 bytes a thread and turn, all its loads in flight, in the layout of
+        // a K-major operand with the 128-byte swizzle.  (A tensor copy waited for the producer to read lens, and queued behind
+        // the stages already asked for.)
+        const int n_rows = min(h - row0, kWideRows);                  // query rows of this tile
+        {
+            uint4 v[8];
+            const uint4* src = q + ((size_t)seq * h + row0) * (kRowBytes / 16);
+#pragma unroll
+            for (int i = 0; i < 8; ++i)
+                if (threadIdx.x + i * 256 < n_rows * 16) v[i] = __ldcg(src + threadIdx.x + i * 256);
+#pragma unroll
+            for (int i = 0; i < 8; ++i) {
+                const int item = threadIdx.x + i * 256, row = item >> 4, ch = item & 15;
+                if (item < n_rows * 16)
+                    asm volatile("st.shared.v4.b32 [%0], {%1,%2,%3,%4};" ::"r"(q_s + (ch >> 3) * kPfHalfBytes + row * 128 + (((ch & 7) ^ (row & 7)) << 4)),
+                                 "r"(v[i].x), "r"(v[i].y), "r"(v[i].z), "r"(v[i].w) : "memory");
+            }
+            asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+            __syncwarp();
+            if (lane == 0) mbar_arrive(q_full);
+        }
+        // a warp none of whose rows is one of the sequence's only keeps the barriers' counts
+        const bool idle = quarter * 32 >= n_rows, mine = r < n_rows;
         float m = -INFINITY, l = 0.f;                                 // reference maximum (log2 units), sum of weights
         bool ok = true;
         int n_p = 0;                                                  // products of this warpgroup's weights so far
@@ -248,81 +267,86 @@ mqa_decode_wide_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_c
             const int valid = r1 - (r0 + j * kWideRows);              // rows of the stage inside this split's prefix (> 0)
             if (ok) ok = mbar_wait(s_ready + 8 * w, ph & 1);
             tc_fence_after();
-            // ---- the row's 128 logits, read once and kept in registers; rows past the prefix masked by index (a select)
             uint32_t x[128];
-            tmem_ld_cols<128>(lane_base, x);
-            tmem_wait_ld();
-            tc_fence_before();
-            __syncwarp();
-            if (lane == 0) mbar_arrive(s_free);                       // the next stage's logits may take their place
-            if (valid < kWideRows) {
+            if (idle) {
+                if (lane == 0) mbar_arrive(s_free);
+                if (n_p > 0 && ok) ok = mbar_wait(pv_done + 8 * w, (n_p - 1) & 1);    // (the arrival below belongs to the next phase)
+            } else {
+                // ---- the row's 128 logits, read once and kept in registers; rows past the prefix masked by index (a select)
+                tmem_ld_cols<128>(lane_base, x);
+                tmem_wait_ld();
+                tc_fence_before();
+                __syncwarp();
+                if (lane == 0) mbar_arrive(s_free);                       // the next stage's logits may take their place
+                if (valid < kWideRows) {
 #pragma unroll
-                for (int i = 0; i < 128; ++i)
-                    if (i >= valid) x[i] = 0xff800000u;               // -inf
-            }
-            float mx8[8];
+                    for (int i = 0; i < 128; ++i)
+                        if (i >= valid) x[i] = 0xff800000u;               // -inf
+                }
+                float mx8[8];
 #pragma unroll
-            for (int i = 0; i < 8; ++i) mx8[i] = fmaxf(__uint_as_float(x[2 * i]), __uint_as_float(x[2 * i + 1]));
+                for (int i = 0; i < 8; ++i) mx8[i] = fmaxf(__uint_as_float(x[2 * i]), __uint_as_float(x[2 * i + 1]));
 #pragma unroll
-            for (int i = 8; i < 64; ++i) mx8[i & 7] = max3(mx8[i & 7], __uint_as_float(x[2 * i]), __uint_as_float(x[2 * i + 1]));
-            const float mx = max3(max3(mx8[0], mx8[1], mx8[2]), max3(mx8[3], mx8[4], mx8[5]), fmaxf(mx8[6], mx8[7])) * kLog2e;
-            if (__any_sync(0xffffffffu, mx > m + kPfMaxLead)) {
-                // ---- a row of this warp leads its reference by too much: every row of the warp moves its reference
-                // to its largest logit so far and rescales its sum and its row of O
-                const float m_new = fmaxf(m, mx);
-                if (ph > 0) {
-                    const float f = fast_exp2(m - m_new);             // (m is finite from the warpgroup's first stage on)
-                    l *= f;
-                    if (ok) ok = mbar_wait(pv_done + 8 * w, (n_p - 1) & 1);  // O holds the warpgroup's stages before this one
-                    tc_fence_after();
+                for (int i = 8; i < 64; ++i) mx8[i & 7] = max3(mx8[i & 7], __uint_as_float(x[2 * i]), __uint_as_float(x[2 * i + 1]));
+                const float mx = max3(max3(mx8[0], mx8[1], mx8[2]), max3(mx8[3], mx8[4], mx8[5]), fmaxf(mx8[6], mx8[7])) * kLog2e;
+                if (__any_sync(0xffffffffu, mine && mx > m + kPfMaxLead)) {  // (rows past the sequence's last hold no query)
+                    // ---- a row of this warp leads its reference by too much: every row of the warp moves its reference
+                    // to its largest logit so far and rescales its sum and its row of O
+                    const float m_new = fmaxf(m, mx);
+                    if (ph > 0) {
+                        const float f = fast_exp2(m - m_new);             // (m is finite from the warpgroup's first stage on)
+                        l *= f;
+                        if (ok) ok = mbar_wait(pv_done + 8 * w, (n_p - 1) & 1);  // O holds the warpgroup's stages before this one
+                        tc_fence_after();
 #pragma unroll 1
-                    for (int c = 0; c < 16; ++c) {
-                        uint32_t y[8];
-                        tmem_ld8(o_t + c * 8, y);
-                        tmem_wait_ld();
+                        for (int c = 0; c < 16; ++c) {
+                            uint32_t y[8];
+                            tmem_ld8(o_t + c * 8, y);
+                            tmem_wait_ld();
 #pragma unroll
-                        for (int i = 0; i < 8; ++i) y[i] = __float_as_uint(__uint_as_float(y[i]) * f);
-                        tmem_st8(o_t + c * 8, y);
+                            for (int i = 0; i < 8; ++i) y[i] = __float_as_uint(__uint_as_float(y[i]) * f);
+                            tmem_st8(o_t + c * 8, y);
+                        }
+                    }
+                    m = m_new;
+                }
+                // ---- P = exp2(S log2e - m) as bf16 pairs (hi) and, for a short prefix, their remainders (lo)
+                const unsigned long long neg_m2 = f2_pack(-m, -m), log2e2 = f2_pack(kLog2e, kLog2e);
+                unsigned long long sum2[2] = {0ull, 0ull};
+                // the weights stay in registers until the product before has read the ones in tensor memory
+                uint32_t hi[2][32];
+                if (hilo) {
+#pragma unroll
+                    for (int i = 0; i < 64; ++i) {
+                        float a0, a1;
+                        f2_unpack(f2_fma(f2_pack(__uint_as_float(x[2 * i]), __uint_as_float(x[2 * i + 1])), log2e2, neg_m2), a0, a1);
+                        const float pa = fast_exp2(a0), pb = fast_exp2(a1);
+                        sum2[i & 1] = f2_add(sum2[i & 1], f2_pack(pa, pb));
+                        hi[i >> 5][i & 31] = pack_bf16(pa, pb);
+                        x[i] = pack_bf16(pa - bf16_lo(hi[i >> 5][i & 31]), pb - bf16_hi(hi[i >> 5][i & 31]));
+                    }
+                } else {
+#pragma unroll
+                    for (int i = 0; i < 64; ++i) {
+                        float a0, a1;
+                        f2_unpack(f2_fma(f2_pack(__uint_as_float(x[2 * i]), __uint_as_float(x[2 * i + 1])), log2e2, neg_m2), a0, a1);
+                        const float pa = fast_exp2(a0), pb = fast_exp2(a1);
+                        sum2[i & 1] = f2_add(sum2[i & 1], f2_pack(pa, pb));
+                        hi[i >> 5][i & 31] = pack_bf16(pa, pb);
                     }
                 }
-                m = m_new;
-            }
-            // ---- P = exp2(S log2e - m) as bf16 pairs (hi) and, for a short prefix, their remainders (lo)
-            const unsigned long long neg_m2 = f2_pack(-m, -m), log2e2 = f2_pack(kLog2e, kLog2e);
-            unsigned long long sum2[2] = {0ull, 0ull};
-            // the weights stay in registers until the product before has read the ones in tensor memory
-            uint32_t hi[2][32];
-            if (hilo) {
-#pragma unroll
-                for (int i = 0; i < 64; ++i) {
-                    float a0, a1;
-                    f2_unpack(f2_fma(f2_pack(__uint_as_float(x[2 * i]), __uint_as_float(x[2 * i + 1])), log2e2, neg_m2), a0, a1);
-                    const float pa = fast_exp2(a0), pb = fast_exp2(a1);
-                    sum2[i & 1] = f2_add(sum2[i & 1], f2_pack(pa, pb));
-                    hi[i >> 5][i & 31] = pack_bf16(pa, pb);
-                    x[i] = pack_bf16(pa - bf16_lo(hi[i >> 5][i & 31]), pb - bf16_hi(hi[i >> 5][i & 31]));
+                {
+                    float s0, s1;
+                    f2_unpack(f2_add(sum2[0], sum2[1]), s0, s1);
+                    l += s0 + s1;
                 }
-            } else {
-#pragma unroll
-                for (int i = 0; i < 64; ++i) {
-                    float a0, a1;
-                    f2_unpack(f2_fma(f2_pack(__uint_as_float(x[2 * i]), __uint_as_float(x[2 * i + 1])), log2e2, neg_m2), a0, a1);
-                    const float pa = fast_exp2(a0), pb = fast_exp2(a1);
-                    sum2[i & 1] = f2_add(sum2[i & 1], f2_pack(pa, pb));
-                    hi[i >> 5][i & 31] = pack_bf16(pa, pb);
-                }
+                if (n_p > 0 && ok) ok = mbar_wait(pv_done + 8 * w, (n_p - 1) & 1);
+                tc_fence_after();
+                tmem_st32(p_t, hi[0]);
+                tmem_st32(p_t + 32, hi[1]);
+                tmem_wait_st();
+                tc_fence_before();
             }
-            {
-                float s0, s1;
-                f2_unpack(f2_add(sum2[0], sum2[1]), s0, s1);
-                l += s0 + s1;
-            }
-            if (n_p > 0 && ok) ok = mbar_wait(pv_done + 8 * w, (n_p - 1) & 1);
-            tc_fence_after();
-            tmem_st32(p_t, hi[0]);
-            tmem_st32(p_t + 32, hi[1]);
-            tmem_wait_st();
-            tc_fence_before();
             if (valid < kWideRows) {
                 // the stage runs past the prefix: the tensor core would multiply the zero weights with whatever lies
                 // there (NaN * 0 = NaN), so those V rows are cleared first
@@ -342,95 +366,77 @@ mqa_decode_wide_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_c
             if (hilo) {                                               // the remainders, once the first part's product has been made
                 if (ok) ok = mbar_wait(pv_done + 8 * w, (n_p - 1) & 1);
                 tc_fence_after();
-                tmem_st32(p_t, *reinterpret_cast<uint32_t(*)[32]>(&x[0]));
-                tmem_st32(p_t + 32, *reinterpret_cast<uint32_t(*)[32]>(&x[32]));
-                tmem_wait_st();
-                tc_fence_before();
+                if (!idle) {
+                    tmem_st32(p_t, *reinterpret_cast<uint32_t(*)[32]>(&x[0]));
+                    tmem_st32(p_t + 32, *reinterpret_cast<uint32_t(*)[32]>(&x[32]));
+                    tmem_wait_st();
+                    tc_fence_before();
+                }
                 __syncwarp();
                 if (lane == 0) mbar_arrive(p_ready + 8 * w);
                 ++n_p;
             }
         }
         if (n_p > 0 && ok) ok = mbar_wait(pv_done + 8 * w, (n_p - 1) & 1);
-        // (the K ring is used below: a last stage that is warpgroup 0's must have its logits.  Its logits before those have
-        // been ready since before this warpgroup's last ones were issued, so the wait cannot be a phase early)
-        if (w == 1 && n_p > 0 && (n_kv & 1) && ok) ok = mbar_wait(s_ready, ((n_kv - 1) >> 1) & 1);
+        // (Q and the K ring are used below: a last stage that is the other warpgroup's must have its logits.  That warpgroup's
+        // logits before those were ready before this one's last ones were issued, so the wait cannot be a phase early)
+        if (n_p > 0 && n_kv > 1 && ((n_kv - 1) & 1) != w && ok) ok = mbar_wait(s_ready + 8 * (w ^ 1), ((n_kv - 1) >> 1) & 1);
         tc_fence_after();
-        // ---- the two warpgroups' partial results become one: warpgroup 1 leaves (maximum, sum) and its rows of O in
-        // shared memory (the K ring: every S product has completed by now), warpgroup 0 merges and writes out
-        const uint32_t ex_o = k_ring + r * 512;                                        // [128][128] fp32, 16-byte pieces swizzled by row
-        if (w == 1) {
-            if (n_kv > 0) {
-                ex_ml[r] = make_float2(m, l);
-                if (n_p > 0) {
-                    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");       // (the ring was the copy engine's and the tensor core's)
-#pragma unroll
-                    for (int c = 0; c < 4; ++c) {
-                        uint32_t y[32];
-                        tmem_ld32(o_t + c * 32, y);
-                        tmem_wait_ld();
-#pragma unroll
-                        for (int i = 0; i < 32; i += 4)
-                            asm volatile("st.shared.v4.b32 [%0], {%1,%2,%3,%4};" ::"r"(ex_o + ((((c * 8 + (i >> 2)) ^ (r & 31)) << 4))),
-                                         "r"(y[i]), "r"(y[i + 1]), "r"(y[i + 2]), "r"(y[i + 3]) : "memory");
-                    }
-                }
-            }
-            named_barrier_arrive(1, 256);
-        } else {
-            named_barrier(1, 256);
-            // (the loads from tensor memory below are warp-wide instructions: every lane executes them, whether or not
-            // its row is one of the sequence's h query rows)
-            const bool stored = row0 + r < h;
-            const size_t unit = (size_t)seq * h + (stored ? row0 + r : 0);
-            if (n_kv == 0) {
-                // nothing of this split lies inside the prefix: zeros (one split, written below) or an empty piece
-                if (stored && n_splits > 1) part_ml[unit * n_splits + split] = make_float2(-INFINITY, 0.f);
-            } else {
-                const float2 other = ex_ml[r];
-                const bool two = other.x != -INFINITY;                                 // warpgroup 1 had a stage
-                const float top = fmaxf(m, other.x);
-                const float f0 = fast_exp2(m - top), f1 = two ? fast_exp2(other.x - top) : 0.f;
-                const float tot = f0 * l + f1 * other.y;
-                const float scale = n_splits == 1 ? 1.f / tot : 1.f;
-                const float g0 = f0 * scale, g1 = f1 * scale;
-                // the merged row goes back to shared memory, in place of warpgroup 1's: a thread's row is 512 bytes, and
-                // stored from here it would leave as 32 separate 16-byte pieces per instruction (measured: 4.7 us for the
-                // CTA's 64 KB); all eight warps then copy whole rows out, 512 contiguous bytes per instruction
-                float4* my_row = reinterpret_cast<float4*>(base + kPfTileBytes + r * 512);   // (plain accesses: the eight loads of a
-                                                                                            // block go out together, ahead of its stores)
+        // ---- the two warpgroups' partial results become one: each leaves (maximum, sum) and its rows of O in shared memory
+        // (warpgroup 0 where Q and the first K slot were, 1 in the other two; 16-byte pieces swizzled by row), then all eight
+        // warps merge whole rows on the way out, 512 contiguous bytes per instruction.
+        if (!idle) {
+            if (w == 1) ex_ml[r] = make_float2(m, l);
+            if (n_p > 0) {
+                const uint32_t ex_o = q_s + (w * kWideRows + r) * 512;
+                asm volatile("fence.proxy.async.shared::cta;" ::: "memory");           // (it was the copy engine's and the tensor core's)
 #pragma unroll
                 for (int c = 0; c < 4; ++c) {
                     uint32_t y[32];
                     tmem_ld32(o_t + c * 32, y);
-                    float4 u[8];
-#pragma unroll
-                    for (int i = 0; i < 8; ++i) u[i] = two ? my_row[(c * 8 + i) ^ (r & 31)] : make_float4(0.f, 0.f, 0.f, 0.f);
                     tmem_wait_ld();
 #pragma unroll
-                    for (int i = 0; i < 8; ++i) {
-                        float4 v;
-                        v.x = fmaf(u[i].x, g1, __uint_as_float(y[4 * i]) * g0);
-                        v.y = fmaf(u[i].y, g1, __uint_as_float(y[4 * i + 1]) * g0);
-                        v.z = fmaf(u[i].z, g1, __uint_as_float(y[4 * i + 2]) * g0);
-                        v.w = fmaf(u[i].w, g1, __uint_as_float(y[4 * i + 3]) * g0);
-                        my_row[(c * 8 + i) ^ (r & 31)] = v;
-                    }
+                    for (int i = 0; i < 32; i += 4)
+                        asm volatile("st.shared.v4.b32 [%0], {%1,%2,%3,%4};" ::"r"(ex_o + ((((c * 8 + (i >> 2)) ^ (r & 31)) << 4))),
+                                     "r"(y[i]), "r"(y[i + 1]), "r"(y[i + 2]), "r"(y[i + 3]) : "memory");
                 }
-                if (stored && n_splits > 1) part_ml[unit * n_splits + split] = make_float2(top, tot);
             }
         }
-        // ---- all eight warps: the CTA's rows from shared memory to o (one split) or to its piece
+        named_barrier(1, 256);
+        const bool two = n_kv > 1;                                                     // warpgroup 1 had a stage
+        if (w == 0 && mine) {
+            // (maximum, sum) of the row, and what each warpgroup's sums count for
+            float2 ml = make_float2(-INFINITY, 0.f);                                   // (nothing of this split inside the prefix: an empty piece)
+            if (n_kv > 0) {
+                const float2 other = ex_ml[r];
+                const float top = two ? fmaxf(m, other.x) : m;
+                const float f0 = fast_exp2(m - top), f1 = two ? fast_exp2(other.x - top) : 0.f;
+                ml = make_float2(top, f0 * l + (two ? f1 * other.y : 0.f));
+                const float scale = n_splits == 1 ? 1.f / ml.y : 1.f;
+                ex_ml[r] = make_float2(f0 * scale, f1 * scale);
+            }
+            if (n_splits > 1) part_ml[((size_t)seq * h + row0 + r) * n_splits + split] = ml;
+        }
         named_barrier(2, 256);
         if (n_kv > 0 || n_splits == 1) {
-            for (int item = threadIdx.x; item < kWideRows * 32; item += 256) {
-                const int row = item >> 5, c16 = item & 31;                             // (a warp: one row, its 32 pieces of 16 bytes)
-                if (row0 + row >= h) break;
+#pragma unroll 4
+            for (int i = 0; i < kWideRows / 8; ++i) {
+                const int row = warp + 8 * i;
+                if (row >= n_rows) break;
                 float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
-                if (n_kv > 0) v = reinterpret_cast<const float4*>(base + kPfTileBytes + row * 512)[c16 ^ (row & 31)];
+                if (n_kv > 0) {
+                    const float4* rows = reinterpret_cast<const float4*>(base);
+                    const float2 f = ex_ml[row];
+                    const float4 a = rows[row * 32 + (lane ^ (row & 31))];
+                    v = make_float4(a.x * f.x, a.y * f.x, a.z * f.x, a.w * f.x);
+                    if (two) {
+                        const float4 c = rows[(kWideRows + row) * 32 + (lane ^ (row & 31))];
+                        v.x = fmaf(c.x, f.y, v.x); v.y = fmaf(c.y, f.y, v.y); v.z = fmaf(c.z, f.y, v.z); v.w = fmaf(c.w, f.y, v.w);
+                    }
+                }
                 const size_t unit = (size_t)seq * h + row0 + row;
                 float* dst = n_splits == 1 ? o + unit * kHeadDim : part_acc + (unit * n_splits + split) * kHeadDim;
-                reinterpret_cast<float4*>(dst)[c16] = v;
+                reinterpret_cast<float4*>(dst)[lane] = v;
             }
         }
         if (!ok) atomicExch(&timed_out, 1);
