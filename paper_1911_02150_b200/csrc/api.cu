@@ -636,7 +636,7 @@ int launch_projections_in(const void* x, const void* P_q, const void* P_k, const
         !encode_matrix_map(&map_pv, P_v, d, kHeadDim, 128) || !encode_matrix_map(&map_x, x, b, d, NB))
         return MQA_ERR_CUDA;
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)(h + 2), (unsigned)parts, (unsigned)((b + 127) / 128));
+    cfg.gridDim = dim3((unsigned)(h + 2), (unsigned)parts, (unsigned)((b + NB - 1) / NB));
     cfg.blockDim = dim3(kProjThreads);
     cfg.dynamicSmemBytes = Cfg::kSmemBytes;
     cfg.stream = stream;
@@ -654,31 +654,45 @@ int launch_projections_in(const void* x, const void* P_q, const void* P_k, const
     return launch_status();
 }
 
-// CTAs (of one cluster) that share an input slab's d rows: as many as keep the kernel on half of the SMs.  A slab's rows are
-// a serial chain for one CTA, so a few CTAs per slab are quicker (per layer step, 1 / 2 / 4 / 8 CTAs per slab: 10 slabs of
-// 1024 rows 18.8 / 17.3 / 17.1 / 17.1 us; 4 slabs of 768 rows 29.1 / 28.1 / 27.6 / 26.8; 18 slabs of 2048 rows 22.1 / 19.8 / 18.0 /
-// 21.6), but the attention kernel behind it sets itself up and fetches its first stages on the SMs that this one leaves
-// free (34 slabs of 1024 rows in front of the streaming kernel 39.3 / 39.0 / 41.5 / 46.1; 34 of 2048: 26.3 / 24.3 / 27.8 / 31.0).
-int projection_parts(int b, int h, int d) {
-    const int slabs = (h + 2) * ((b + 127) / 128);
-    int parts = 1;
-    while (2 * parts <= kProjMaxParts && 2 * parts <= d / 128 && 4 * parts * slabs <= sm_count()) parts *= 2;
-    return parts;
+// How a projection is cut up: NB batch columns per tile (16, 32, 64 or 128) and the CTAs of a cluster that share the depth of the
+// product (the chunks of d rows of an input slab; the heads of an output tile).  By a model of a CTA's chain, in microseconds: its
+// activations (act_kb per batch column and chunk) at 60 KB/us, step_us per chunk (an output tile's chunk is a round trip for o), 0.4
+// per chunk of weights beyond those fetched ahead of the wait, and what the cluster exchanges, which is slow (SM to SM about
+// 24 KB/us per CTA).  Only cuts whose CTAs fit the SMs at once, in clusters
+// that fit the GPCs (of 8: about half of the SMs), count; the input projection keeps to about half of the SMs, where the attention kernel behind it
+// does not yet set itself up.  Measured, us per layer step, one fixed cut (128 columns; 16 heads' groups) against this one:
+// 128 x 8 heads x 1024 18.4 / 15.4; 200 x 16 x 1536 47.6 / 28.8; 256 x 8 x 2048 38.8 / 23.4; 8 x 32 x 2048 25.6 / 19.2; 1 x 16 x 2048 23.4 / 18.3.
+struct ProjectionCut { int nb, ctas; };
+ProjectionCut projection_cut(int b, int columns, int depth, double act_kb, double step_us, int most_ctas) {
+    ProjectionCut best = {128, 1};
+    double best_us = -1;
+    for (int nb = 16; nb <= 128 && (nb == 16 || nb < 2 * b); nb *= 2) {
+        const int batch_tiles = (b + nb - 1) / nb, rows = b < nb ? b : nb;
+        const int stages = nb == 128 ? ProjCfg<128>::kStages : nb == 64 ? ProjCfg<64>::kStages : ProjCfg<32>::kStages;
+        for (int ctas = 1; ctas <= kProjMaxCluster && ctas <= depth; ctas *= 2) {
+            const long long total = (long long)columns * batch_tiles * ctas;
+            const int each = (depth + ctas - 1) / ctas;
+            const double waves = total <= (ctas == 8 ? most_ctas * 5 / 9 : most_ctas) ? 1.0 : (double)total / most_ctas + 0.5;
+            const double us = waves * (3.0 + each * step_us + rows * each * act_kb / 60 + (each > stages ? (each - stages) * 0.4 : 0) +
+                                       (ctas > 1 ? 0.3 + rows * 0.5 * (ctas - 1) / ctas / 24 : 0));
+            if (best_us < 0 || us < best_us) { best = {nb, ctas}; best_us = us; }
+        }
+    }
+    return best;
 }
 
 // The output projection: the head groups of a (d tile, batch tile) are the CTAs of one thread-block cluster (see
-// project_out_kernel), so there are at most kProjMaxGroups of them, each with ceil(h / groups) heads.
+// project_out_kernel), each with ceil(h / ctas) heads.
 template <int NB>
-int launch_projection_out(const void* P_o, const float* o, float* y, int32_t* status, int b, int h, int d, cudaStream_t stream) {
+int launch_projection_out(const void* P_o, const float* o, float* y, int32_t* status, int b, int h, int d, int ctas, cudaStream_t stream) {
     using Cfg = ProjCfg<NB>;
     auto kernel = project_out_kernel<NB>;
     constexpr int kSlot = 4 + (NB == 16 ? 0 : (NB == 32 ? 1 : (NB == 64 ? 2 : 3)));
-    constexpr int kSmem = 2 * Cfg::kStageBytes + 256 + 1024;
+    constexpr int kSmem = Cfg::kSmemBytes;
     int dev = 0;
     if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxDevices) { cudaGetLastError(); return MQA_ERR_CUDA; }
     if (!g_proj_opt_in[dev][kSlot].load(std::memory_order_acquire)) {
-        if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmem) != cudaSuccess ||
-            (kProjMaxGroups > 8 && cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess)) {
+        if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmem) != cudaSuccess) {
             cudaGetLastError();
             return MQA_ERR_CUDA;
         }
@@ -686,10 +700,10 @@ int launch_projection_out(const void* P_o, const float* o, float* y, int32_t* st
     }
     alignas(64) CUtensorMap map_po;
     if (!encode_matrix_map(&map_po, P_o, (long long)h * d, kHeadDim, 128)) return MQA_ERR_CUDA;
-    const int heads_per_cta = (h + kProjMaxGroups - 1) / kProjMaxGroups;
+    const int heads_per_cta = (h + ctas - 1) / ctas;
     const int groups = (h + heads_per_cta - 1) / heads_per_cta;
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)(d / 128), (unsigned)groups, (unsigned)((b + 127) / 128));
+    cfg.gridDim = dim3((unsigned)(d / 128), (unsigned)groups, (unsigned)((b + NB - 1) / NB));
     cfg.blockDim = dim3(kProjThreads);
     cfg.dynamicSmemBytes = kSmem;
     cfg.stream = stream;
@@ -1023,24 +1037,25 @@ int mqa_layer_decode_step(const void* x, const void* P_q, const void* P_k, const
     void* k_new = base + w.k_new;
     void* v_new = base + w.v_new;
     float* o = reinterpret_cast<float*>(base + w.o);
-    const int nb = b >= 128 ? 128 : (b > 64 ? 128 : (b > 32 ? 64 : (b > 16 ? 32 : 16)));
-    const int parts = projection_parts(b, h, d);
+    const int sms = sm_count();
+    const ProjectionCut in = projection_cut(b, h + 2, d / 128, 0.25, 0.2, sms * 5 / 9);        // bf16 x
+    const ProjectionCut out = projection_cut(b, d / 128, h, 0.5, 0.45, sms * 8 / 9);            // fp32 o
     int rc;
-    switch (nb) {
-        case 16: rc = launch_projections_in<16>(x, P_q, P_k, P_v, q, k_new, v_new, status, b, h, d, parts, stream); break;
-        case 32: rc = launch_projections_in<32>(x, P_q, P_k, P_v, q, k_new, v_new, status, b, h, d, parts, stream); break;
-        case 64: rc = launch_projections_in<64>(x, P_q, P_k, P_v, q, k_new, v_new, status, b, h, d, parts, stream); break;
-        default: rc = launch_projections_in<128>(x, P_q, P_k, P_v, q, k_new, v_new, status, b, h, d, parts, stream); break;
+    switch (in.nb) {
+        case 16: rc = launch_projections_in<16>(x, P_q, P_k, P_v, q, k_new, v_new, status, b, h, d, in.ctas, stream); break;
+        case 32: rc = launch_projections_in<32>(x, P_q, P_k, P_v, q, k_new, v_new, status, b, h, d, in.ctas, stream); break;
+        case 64: rc = launch_projections_in<64>(x, P_q, P_k, P_v, q, k_new, v_new, status, b, h, d, in.ctas, stream); break;
+        default: rc = launch_projections_in<128>(x, P_q, P_k, P_v, q, k_new, v_new, status, b, h, d, in.ctas, stream); break;
     }
     if (rc) return rc;
     rc = append_step_impl(q, K, V, k_new, v_new, lens, advance ? MQA_STEP_ADVANCE : 0, o, base + w.step, w.total - w.step, status,
                           b, h, m_max, k, v, stream_, true);
     if (rc) return rc;
-    switch (nb) {
-        case 16: return launch_projection_out<16>(P_o, o, y, status, b, h, d, stream);
-        case 32: return launch_projection_out<32>(P_o, o, y, status, b, h, d, stream);
-        case 64: return launch_projection_out<64>(P_o, o, y, status, b, h, d, stream);
-        default: return launch_projection_out<128>(P_o, o, y, status, b, h, d, stream);
+    switch (out.nb) {
+        case 16: return launch_projection_out<16>(P_o, o, y, status, b, h, d, out.ctas, stream);
+        case 32: return launch_projection_out<32>(P_o, o, y, status, b, h, d, out.ctas, stream);
+        case 64: return launch_projection_out<64>(P_o, o, y, status, b, h, d, out.ctas, stream);
+        default: return launch_projection_out<128>(P_o, o, y, status, b, h, d, out.ctas, stream);
     }
 }
 

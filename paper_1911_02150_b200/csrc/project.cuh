@@ -16,18 +16,16 @@
 //                        P_o[head][128 d-rows of tile j x 128] (K-major A) * o[:, head, :]^T (K-major B, converted
 //                        from fp32 to bf16 by the CTA); the head groups of a tile are one thread-block cluster
 //
-// The CTAs of a cluster leave their sums in shared memory and add them up through distributed shared memory, each the
-// batch rows that fall to it, in rank order (no float atomics).
+// The CTAs of a cluster leave their sums in shared memory, send each other the batch rows that fall to each, and add them up
+// in rank order (no float atomics): SumShares.
 //
 // What bounds these kernels is latency: the weights are in flight before the kernel ahead has finished, and a CTA's work
-// after that is a chain of round trips (x or o, the products, the other CTAs' sums).  So a chain is cut into as many CTAs
-// as help (projection_parts in api.cu), and each of its links is one round trip: all of a head's o loads, and all the remote loads
-// of a row's sums, are in flight at once.  Measured on one B200, per layer step of 128 sequences, 8 heads, d = 1024, 128
-// rows: 24.7 -> 17.1 us, about 1 us of it from the attention step between them (the 4.7 MB of weights take 0.7 us
-// at the copy rate).
+// after that is a chain of round trips (x or o, the products, the other CTAs' sums), each made one round trip: all of a
+// head's o loads are in flight at once, another CTA's sums come in one copy.  How the chain is cut up over batch columns
+// and CTAs: projection_cut in api.cu, with what it measured.
 //
-// NB = batch columns of a tile (the batch rounded up to 16, 32, 64 or 128; larger batches take
-// several tiles of 128).  Every wait is bounded (mbar_wait); TMEM is freed on every path.
+// NB = batch columns of a tile (16, 32, 64 or 128; larger batches take several tiles).  Every wait is bounded (mbar_wait);
+// TMEM is freed on every path.
 #pragma once
 #include <cuda_bf16.h>
 
@@ -39,17 +37,19 @@ constexpr int kProjWorkWarps = 8;              // convert o, read the sums out, 
 constexpr int kProjTmaWarp = 8, kProjMmaWarp = 9;
 constexpr int kProjThreads = 10 * 32;
 constexpr int kProjChunkBytes = 128 * 256;     // 128 rows x 128 bf16 of a weight matrix: 32 KiB, two 64-column boxes
-constexpr int kProjMaxGroups = 16;             // project_out: head groups of a tile = CTAs of one cluster (16: the
-                                               // non-portable cluster size, which the B200 offers; two heads per CTA at h = 32)
-constexpr int kProjMaxParts = 8;               // project_in: CTAs (of one cluster) that share a slab's d rows
+constexpr int kProjMaxCluster = 8;             // CTAs that share the depth of a product
 
 template <int NB>
 struct ProjCfg {
     static_assert(NB == 16 || NB == 32 || NB == 64 || NB == 128, "batch columns of a tile");
     static constexpr int kActBytes = NB * 256;                 // NB rows x 128 bf16, two 64-column boxes
-    static constexpr int kStages = NB == 128 ? 3 : 4;
+    static constexpr int kStages = NB == 128 ? 2 : NB == 64 ? 3 : 4;
     static constexpr int kStageBytes = kProjChunkBytes + kActBytes;
-    static constexpr int kSmemBytes = kStages * kStageBytes + 256 /* barriers */ + 1024 /* alignment slack */;
+    static constexpr int kSumBytes = NB * 512;                 // a CTA's sums, [NB batch rows][128] fp32: where the stages were
+    static constexpr int kRecvBytes = (NB + kProjMaxCluster) * 512;     // the other CTAs' sums of this one's rows (whole rows, rounded up per CTA)
+    static constexpr int smem_bytes(int stages) { return stages * kStageBytes + kRecvBytes + 256 /* barriers */ + 1024 /* alignment slack */; }
+    static constexpr int kSmemBytes = smem_bytes(kStages);
+    static_assert(kSumBytes <= 2 * kStageBytes, "the sums take the stages' place");
     static constexpr int kTmemCols = NB < 32 ? 32 : NB;
     static_assert(kSmemBytes <= 227 * 1024, "exceeds the shared memory of one SM");
 };
@@ -70,22 +70,48 @@ __device__ __forceinline__ void leave_sums(uint32_t tmem, uint32_t dst, int warp
         for (int i = 0; i < CH; ++i)
             asm volatile("st.shared.b32 [%0], %1;" ::"r"(dst + (uint32_t)((col0 + c + i) * 128 + feature) * 4), "r"(valid ? part[i] : 0u) : "memory");
     }
+    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");   // (bulk copies read them)
 }
 
-// Batch row n of the tile, features lane * 4 .. + 3: the sums of all the cluster's CTAs, added up in rank order.  Every
-// remote load of a row is asked for before the first is used (one round trip through the cluster per row, not one per CTA).
-template <int MAX_CTAS>
-__device__ __forceinline__ float4 add_up_row(uint32_t sums, int n, int lane, int ctas) {
-    float4 part[MAX_CTAS];
-#pragma unroll
-    for (int g = 0; g < MAX_CTAS; ++g)
-        if (g < ctas) part[g] = cluster_ld_f4(cluster_map(sums + (uint32_t)(n * 128 + lane * 4) * 4, (uint32_t)g));
-    float4 sum = part[0];
-#pragma unroll
-    for (int g = 1; g < MAX_CTAS; ++g)
-        if (g < ctas) { sum.x += part[g].x; sum.y += part[g].y; sum.z += part[g].z; sum.w += part[g].w; }
-    return sum;
+// ---- the sums of a cluster's CTAs, added up: CTA r of C takes the batch rows [r * per, (r + 1) * per) of the tile.  Every CTA
+// sends each other one the rows that fall to it as ONE bulk copy from shared memory to shared memory (SM to SM, signalled on the
+// receiver's mbarrier; a place of its own per sender) and adds up what it has and what it gets, in rank order.  Read by
+// 16-byte remote loads instead, between two cluster barriers, the 64 KB that a CTA needs took 3.2 to 3.9 us at 128 batch
+// columns; this 2.3 to 3.1 (SM to SM a CTA
+// gets about 24 KB/us), and at 16 batch columns 1.0 in place of 1.6.
+__device__ __forceinline__ void send_rows(uint32_t dst, uint32_t src, uint32_t bytes, uint32_t bar) {      // dst and bar: cluster addresses
+    asm volatile("cp.async.bulk.shared::cluster.shared::cta.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
+                 ::"r"(dst), "r"(src), "r"(bytes), "r"(bar) : "memory");
 }
+struct SumShares {
+    int rank, ctas, rows, per;            // rows: of the tile; per: of a CTA (the last ones may have fewer)
+    __device__ __forceinline__ int count(int r) const { return max(0, min(per, rows - r * per)); }
+    // by one thread, before the cluster barrier that tells the others that this CTA's barrier is in place
+    __device__ __forceinline__ void expect(uint32_t bar) const { mbar_expect_tx(bar, (uint32_t)((ctas - 1) * count(rank)) * 512); }
+    // by one warp, once this CTA's sums lie in its shared memory
+    __device__ __forceinline__ void send(uint32_t sums, uint32_t recv, uint32_t bar, int lane) const {
+        const int to = lane;              // (a cluster has at most kProjMaxCluster CTAs)
+        if (to < ctas && to != rank && count(to) > 0)
+            send_rows(cluster_map(recv + (uint32_t)(rank * per) * 512, to), sums + (uint32_t)(to * per) * 512, (uint32_t)count(to) * 512, cluster_map(bar, to));
+    }
+    // row i of this CTA's, features lane * 4 .. + 3
+    __device__ __forceinline__ float4 add_up(uint32_t sums, uint32_t recv, int i, int lane) const {
+        float4 sum = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll 4
+        for (int g = 0; g < ctas; ++g) {
+            const uint32_t at = (g == rank ? sums + (uint32_t)(rank * per + i) * 512 : recv + (uint32_t)(g * per + i) * 512) + lane * 16;
+            float4 v;
+            asm volatile("ld.shared.v4.f32 {%0,%1,%2,%3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "r"(at) : "memory");
+            sum.x += v.x; sum.y += v.y; sum.z += v.z; sum.w += v.w;
+        }
+        return sum;
+    }
+};
+__device__ __forceinline__ void cluster_arrive() {
+    __syncwarp();
+    asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+}
+__device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
 
 template <int NB>
 __global__ void __launch_bounds__(kProjThreads, 1)
@@ -95,7 +121,7 @@ project_in_kernel(const __grid_constant__ CUtensorMap map_pq, const __grid_const
                   int32_t* __restrict__ status, int b, int h, int d) {
     using Cfg = ProjCfg<NB>;
     constexpr int S = Cfg::kStages;
-    const int slab = blockIdx.x, row0 = blockIdx.z * 128;          // weight slab; first batch row of this tile
+    const int slab = blockIdx.x, row0 = blockIdx.z * NB;          // weight slab; first batch row of this tile
     const int part = blockIdx.y, parts = gridDim.y;                // this CTA's part of the slab's d rows: one cluster per slab
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int chunk0 = part * (d / 128) / parts;                   // chunks of 128 rows [chunk0, chunk0 + n_chunks)
@@ -104,7 +130,10 @@ project_in_kernel(const __grid_constant__ CUtensorMap map_pq, const __grid_const
     extern __shared__ uint8_t smem_raw[];
     uint8_t* stages = smem_raw + ((1024u - (smem_addr(smem_raw) & 1023u)) & 1023u);
     const uint32_t stages_s = smem_addr(stages);
-    const uint32_t full_s = stages_s + S * Cfg::kStageBytes, empty_s = full_s + S * 8, done_s = empty_s + S * 8;
+    const uint32_t recv_s = stages_s + S * Cfg::kStageBytes;       // the other CTAs' sums of this one's batch rows
+    const uint32_t full_s = recv_s + Cfg::kRecvBytes, empty_s = full_s + S * 8, done_s = empty_s + S * 8, recv_bar = done_s + 8;
+    const int rows = min(NB, b - row0);
+    const SumShares shares{part, parts, rows, (rows + parts - 1) / parts};
     __shared__ uint32_t tmem_slot;
     __shared__ int timed_out, issued;
 
@@ -131,8 +160,10 @@ project_in_kernel(const __grid_constant__ CUtensorMap map_pq, const __grid_const
         issued = 0;
         for (int s = 0; s < S; ++s) { mbar_init(full_s + s * 8, 2); mbar_init(empty_s + s * 8, 1); }
         mbar_init(done_s, 1);
+        mbar_init(recv_bar, 1);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+        if (parts > 1) shares.expect(recv_bar);
         for (int c = 0; c < n_chunks && c < S; ++c) issue_weights(c);
     }
     if (warp == kProjMmaWarp) { tmem_alloc(smem_addr(&tmem_slot), Cfg::kTmemCols); tmem_relinquish(); }
@@ -140,6 +171,7 @@ project_in_kernel(const __grid_constant__ CUtensorMap map_pq, const __grid_const
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem = tmem_slot;
+    if (parts > 1) cluster_sync();   // every CTA's barrier is in place
     grid_dependency_wait();          // x may come from the kernel before this one
     grid_launch_dependents();
 
@@ -193,30 +225,32 @@ project_in_kernel(const __grid_constant__ CUtensorMap map_pq, const __grid_const
         if (status) atomicOr(status, kStatusPipelineTimeout);
     }
     __syncthreads();
-    if (parts > 1) cluster_sync();   // every part's sums are in its shared memory
+    if (parts > 1) {
+        if (warp == 0) shares.send(stages_s, recv_s, recv_bar, lane);
+        if (!mbar_wait(recv_bar, 0)) { if (status && lane == 0) atomicOr(status, kStatusPipelineTimeout); mbar_wait(recv_bar, 0); }
+        cluster_arrive();            // what the others send has landed
+    }
     {
         __nv_bfloat16* out = slab < h ? q + (size_t)slab * 128 : (slab == h ? k_new : v_new);
         const size_t stride = slab < h ? (size_t)h * 128 : 128;
-        for (int n = part + parts * warp; n < NB && row0 + n < b; n += parts * (kProjThreads / 32)) {
-            const float4 v = add_up_row<kProjMaxParts>(stages_s, n, lane, parts);
-            *reinterpret_cast<uint2*>(out + (size_t)(row0 + n) * stride + lane * 4) = make_uint2(pack_bf16(v.x, v.y), pack_bf16(v.z, v.w));
+        for (int i = warp; i < shares.count(part); i += kProjThreads / 32) {
+            const float4 v = shares.add_up(stages_s, recv_s, i, lane);
+            *reinterpret_cast<uint2*>(out + (size_t)(row0 + part * shares.per + i) * stride + lane * 4) = make_uint2(pack_bf16(v.x, v.y), pack_bf16(v.z, v.w));
         }
     }
-    if (parts > 1) cluster_sync();   // nobody leaves while its shared memory is being read
+    if (parts > 1) cluster_wait();   // nobody leaves while its sums are on their way
     if (warp == kProjMmaWarp) { tc_fence_after(); tmem_dealloc(tmem, Cfg::kTmemCols); }
 }
 
-// The head groups of one (d tile, batch tile) form one thread-block cluster (gridDim.y CTAs, at most 16): each CTA
-// accumulates Y^T over its heads in TMEM, leaves it in its shared memory, and after a cluster barrier every CTA adds up,
-// in group order, the batch rows that fall to it (row n to CTA n mod cluster size) out of all the CTAs' shared memory
-// and stores them to y.  No partial sums pass through global memory and no float atomics are used.
+// The head groups of one (d tile, batch tile) form one thread-block cluster (gridDim.y CTAs): each CTA accumulates Y^T over its
+// heads in TMEM, and the cluster adds the sums up.  No partial sums pass through global memory and no float atomics are used.
 template <int NB>
 __global__ void __launch_bounds__(kProjThreads, 1)
 project_out_kernel(const __grid_constant__ CUtensorMap map_po, const float* __restrict__ o, float* __restrict__ y,
                    int32_t* __restrict__ status, int b, int h, int d, int heads_per_cta) {
     using Cfg = ProjCfg<NB>;
-    constexpr int S = 2;                                           // ring of two stages: a head's weights and its o tile
-    const int tile = blockIdx.x, group = blockIdx.y, row0 = blockIdx.z * 128;
+    constexpr int S = Cfg::kStages;                                // a stage: a head's weights and its o tile
+    const int tile = blockIdx.x, group = blockIdx.y, row0 = blockIdx.z * NB;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int head0 = group * heads_per_cta;
     const int n_heads = max(0, min(heads_per_cta, h - head0));
@@ -224,7 +258,10 @@ project_out_kernel(const __grid_constant__ CUtensorMap map_po, const float* __re
     extern __shared__ uint8_t smem_raw[];
     uint8_t* stages = smem_raw + ((1024u - (smem_addr(smem_raw) & 1023u)) & 1023u);
     const uint32_t stages_s = smem_addr(stages);
-    const uint32_t w_full = stages_s + S * Cfg::kStageBytes, o_full = w_full + S * 8, empty_s = o_full + S * 8, done_s = empty_s + S * 8;
+    const uint32_t recv_s = stages_s + S * Cfg::kStageBytes;       // the other CTAs' sums of this one's batch rows
+    const uint32_t w_full = recv_s + Cfg::kRecvBytes, o_full = w_full + S * 8, empty_s = o_full + S * 8, done_s = empty_s + S * 8, recv_bar = done_s + 8;
+    const int rows = min(NB, b - row0), n_groups = gridDim.y;
+    const SumShares shares{group, n_groups, rows, (rows + n_groups - 1) / n_groups};
     __shared__ uint32_t tmem_slot;
     __shared__ int timed_out, issued;
 
@@ -234,8 +271,10 @@ project_out_kernel(const __grid_constant__ CUtensorMap map_po, const float* __re
         issued = 0;
         for (int s = 0; s < S; ++s) { mbar_init(w_full + s * 8, 1); mbar_init(o_full + s * 8, kProjWorkWarps); mbar_init(empty_s + s * 8, 1); }
         mbar_init(done_s, 1);
+        mbar_init(recv_bar, 1);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+        shares.expect(recv_bar);
     }
     if (warp == kProjMmaWarp) { tmem_alloc(smem_addr(&tmem_slot), Cfg::kTmemCols); tmem_relinquish(); }
     auto issue_weights = [&](int i) {
@@ -254,6 +293,7 @@ project_out_kernel(const __grid_constant__ CUtensorMap map_po, const float* __re
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem = tmem_slot;
+    cluster_sync();                  // every CTA's barrier is in place
     grid_dependency_wait();          // o comes from the kernel before this one
     grid_launch_dependents();
 
@@ -329,13 +369,12 @@ project_out_kernel(const __grid_constant__ CUtensorMap map_po, const float* __re
         if (status) atomicOr(status, kStatusPipelineTimeout);
     }
     __syncthreads();
-    cluster_sync();                  // every group's Y^T is in its shared memory
-    const int rank = (int)cluster_cta_rank(), n_groups = (int)cluster_size();
-    for (int n = rank + n_groups * warp; n < NB && row0 + n < b; n += n_groups * (kProjThreads / 32)) {
-        const float4 sum = add_up_row<kProjMaxGroups>(stages_s, n, lane, n_groups);
-        *reinterpret_cast<float4*>(y + (size_t)(row0 + n) * d + (size_t)tile * 128 + lane * 4) = sum;
-    }
-    cluster_sync();                  // nobody leaves while its shared memory is being read
+    if (warp == 0) shares.send(stages_s, recv_s, recv_bar, lane);
+    if (!mbar_wait(recv_bar, 0)) { if (status && lane == 0) atomicOr(status, kStatusPipelineTimeout); mbar_wait(recv_bar, 0); }
+    cluster_arrive();                // what the others send has landed
+    for (int i = warp; i < shares.count(group); i += kProjThreads / 32)
+        *reinterpret_cast<float4*>(y + (size_t)(row0 + group * shares.per + i) * d + (size_t)tile * 128 + lane * 4) = shares.add_up(stages_s, recv_s, i, lane);
+    cluster_wait();                  // nobody leaves while its sums are on their way
     if (warp == kProjMmaWarp) { tc_fence_after(); tmem_dealloc(tmem, Cfg::kTmemCols); }
 }
 

@@ -98,10 +98,12 @@ def test_layer_step_matches_oracle(b, h, d, m_max):
 
 
 @pytest.mark.parametrize("b,h,d,m_max", [
-    (3, 1, 1024, 130),        # eight CTAs share an input slab's d rows
-    (17, 5, 640, 130),        # five chunks over four CTAs; a batch that is no multiple of a tile
-    (70, 32, 896, 96),        # seven chunks over two; 128 batch columns of which 70 count
-    (129, 2, 128, 64),        # one chunk; a second batch tile of one sequence
+    (3, 1, 1024, 130),        # one head: an output tile's CTA has no cluster, an input slab's has
+    (17, 5, 640, 130),        # five chunks and five heads over clusters that do not divide them
+    (70, 32, 896, 96),        # a last batch tile partly filled
+    (129, 2, 128, 64),        # one chunk of depth; a last batch tile of one sequence
+    (250, 16, 1024, 40),      # batch tiles of 64 and more, clusters of two
+    (120, 3, 2048, 33),       # sixteen chunks
 ])
 def test_input_slabs_shared_by_a_cluster(b, h, d, m_max):
     """...and prefixes that end at every place of a tile, for the small steps that fetch their cache rows before the
