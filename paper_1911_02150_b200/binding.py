@@ -128,33 +128,35 @@ def alloc_workspace(b: int, h: int, m_max: int, device, k: int = 128, v: int = 1
     return torch.empty(max(n, 16), dtype=torch.uint8, device=device)
 
 
-class _OnDevice:
-    """`with` block that makes a tensor's device current only when it is not already (the common case costs nothing)."""
-    __slots__ = ("ctx",)
+# The current stream's handle without a Stream object around it (a microsecond per call, of a call that takes ten).
+_raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None)
 
-    def __init__(self, device):
-        idx = device.index if device.index is not None else torch.cuda.current_device()
-        self.ctx = None if idx == torch.cuda.current_device() else torch.cuda.device(idx)
 
-    def __enter__(self):
-        if self.ctx is not None:
-            self.ctx.__enter__()
+def _stream_of(device, stream) -> int:
+    """The handle of `stream`, or of the stream that is current on `device`."""
+    if stream is not None:
+        return stream.cuda_stream
+    if _raw_stream is not None and device.index is not None:
+        return _raw_stream(device.index)
+    return torch.cuda.current_stream(device).cuda_stream
 
-    def __exit__(self, *exc):
-        if self.ctx is not None:
-            self.ctx.__exit__(*exc)
+
+def _call(fn, device, *args) -> int:
+    """The C call with the tensors' device current (made current only when it is not already)."""
+    idx = device.index
+    if idx is None or idx == torch.cuda.current_device():
+        return fn(*args)
+    with torch.cuda.device(idx):
+        return fn(*args)
 
 
 def _ptr(t: Optional[torch.Tensor]):
-    return None if t is None else ctypes.c_void_p(t.data_ptr())
-
-
-def _stream(stream) -> ctypes.c_void_p:
-    s = torch.cuda.current_stream() if stream is None else stream
-    return ctypes.c_void_p(s.cuda_stream)
+    return None if t is None else t.data_ptr()
 
 
 def _need(t: torch.Tensor, dtype, shape, name: str):
+    if isinstance(t, torch.Tensor) and t.dtype is dtype and t.is_cuda and t.shape == shape and t.is_contiguous():
+        return
     if not isinstance(t, torch.Tensor) or not t.is_cuda:
         raise TypeError(f"{name} must be a CUDA tensor")
     if t.dtype != dtype:
@@ -206,16 +208,15 @@ def kv_cache_append(K, V, k_new, v_new, lens, advance: bool = True, status=None,
         new_shape = (b, kvh, k)
     v = V.shape[-1]
     _need(K, torch.bfloat16, K.shape, "K")
-    _need(V, torch.bfloat16, tuple(K.shape[:-1]) + (v,), "V")
+    _need(V, torch.bfloat16, K.shape[:-1] + (v,), "V")
     _need(k_new, torch.bfloat16, new_shape, "k_new")
     _need(v_new, torch.bfloat16, new_shape[:-1] + (v,), "v_new")
     _need(lens, torch.int32, (b,), "lens")
     if status is not None:
         _need(status, torch.int32, (1,), "status")
-    with _OnDevice(K.device):
-        rc = lib().kv_cache_append(_ptr(K), _ptr(V), _ptr(k_new), _ptr(v_new), _ptr(lens), int(bool(advance)),
-                                   _ptr(status), b, kvh, m_max, k, v, _stream(stream))
-    _check(rc, "kv_cache_append")
+    device = K.device
+    _check(_call(lib().kv_cache_append, device, _ptr(K), _ptr(V), _ptr(k_new), _ptr(v_new), _ptr(lens), int(bool(advance)),
+                 _ptr(status), b, kvh, m_max, k, v, _stream_of(device, stream)), "kv_cache_append")
 
 
 def _step(name: str, multi_query: bool, q, K, V, lens, o, workspace, status, stream, phase: str):
@@ -230,12 +231,12 @@ def _step(name: str, multi_query: bool, q, K, V, lens, o, workspace, status, str
     if status is not None:
         _need(status, torch.int32, (1,), "status")
     ws_ptr, ws_bytes = (None, 0) if workspace is None else (_ptr(workspace), workspace.numel() * workspace.element_size())
-    with _OnDevice(q.device):
-        if phase == "combine":
-            rc = getattr(lib(), name)(_ptr(lens), _ptr(o), ws_ptr, ws_bytes, b, h, m_max, k, v, _stream(stream))
-        else:
-            rc = getattr(lib(), name)(_ptr(q), _ptr(K), _ptr(V), _ptr(lens), _ptr(o), ws_ptr, ws_bytes,
-                                      _ptr(status), b, h, m_max, k, v, _stream(stream))
+    device = q.device
+    fn, on = getattr(lib(), name), _stream_of(device, stream)
+    if phase == "combine":
+        rc = _call(fn, device, _ptr(lens), _ptr(o), ws_ptr, ws_bytes, b, h, m_max, k, v, on)
+    else:
+        rc = _call(fn, device, _ptr(q), _ptr(K), _ptr(V), _ptr(lens), _ptr(o), ws_ptr, ws_bytes, _ptr(status), b, h, m_max, k, v, on)
     _check(rc, name)
     return o
 
@@ -285,10 +286,8 @@ def mqa_decode_step_noalloc(q, K, V, lens, o, status=None, stream=None):
     _need(o, torch.float32, (b, h, v), "o")
     if status is not None:
         _need(status, torch.int32, (1,), "status")
-    with _OnDevice(q.device):
-        rc = lib().mqa_decode_step_noalloc(_ptr(q), _ptr(K), _ptr(V), _ptr(lens), _ptr(o), _ptr(status),
-                                           b, h, m_max, k, v, _stream(stream))
-    _check(rc, "mqa_decode_step_noalloc")
+    _check(_call(lib().mqa_decode_step_noalloc, q.device, _ptr(q), _ptr(K), _ptr(V), _ptr(lens), _ptr(o), _ptr(status),
+                 b, h, m_max, k, v, _stream_of(q.device, stream)), "mqa_decode_step_noalloc")
     return o
 
 
@@ -305,11 +304,10 @@ def _append_step_args(q, K, V, k_new, v_new, lens, o, workspace, status, advance
     _need(o, torch.float32, (b, h, v), "o")
     if status is not None:
         _need(status, torch.int32, (1,), "status")
-    s = torch.cuda.current_stream(q.device) if stream is None else stream
     return (q.data_ptr(), K.data_ptr(), V.data_ptr(), k_new.data_ptr(), v_new.data_ptr(), lens.data_ptr(),
             _step_flags(advance, chained, withhold_copy), o.data_ptr(), None if workspace is None else workspace.data_ptr(),
             0 if workspace is None else workspace.numel() * workspace.element_size(),
-            None if status is None else status.data_ptr(), b, h, m_max, k, v, s.cuda_stream)
+            None if status is None else status.data_ptr(), b, h, m_max, k, v, _stream_of(q.device, stream))
 
 
 def mqa_decode_append_step(q, K, V, k_new, v_new, lens, o, workspace=None, status=None, advance: bool = True, stream=None,
@@ -321,9 +319,7 @@ def mqa_decode_append_step(q, K, V, k_new, v_new, lens, o, workspace=None, statu
     the cache, ``lens`` or the workspace (a decoding loop); the kernel then starts on the cache before the
     kernel ahead of it has finished."""
     args = _append_step_args(q, K, V, k_new, v_new, lens, o, workspace, status, advance, stream, chained, withhold_copy)
-    with _OnDevice(q.device):
-        rc = lib().mqa_decode_append_step(*args)
-    _check(rc, "mqa_decode_append_step")
+    _check(_call(lib().mqa_decode_append_step, q.device, *args), "mqa_decode_append_step")
     return o
 
 
@@ -381,12 +377,9 @@ def mqa_layer_decode_step(x, P_q, P_k, P_v, P_o, K, V, lens, y, workspace, statu
     _need(y, torch.float32, (b, d), "y")
     if status is not None:
         _need(status, torch.int32, (1,), "status")
-    with _OnDevice(x.device):
-        rc = lib().mqa_layer_decode_step(_ptr(x), _ptr(P_q), _ptr(P_k), _ptr(P_v), _ptr(P_o), _ptr(K), _ptr(V), _ptr(lens),
-                                         int(bool(advance)), _ptr(y), _ptr(workspace),
-                                         workspace.numel() * workspace.element_size(), _ptr(status),
-                                         b, h, d, m_max, k, v, _stream(stream))
-    _check(rc, "mqa_layer_decode_step")
+    _check(_call(lib().mqa_layer_decode_step, x.device, _ptr(x), _ptr(P_q), _ptr(P_k), _ptr(P_v), _ptr(P_o), _ptr(K), _ptr(V), _ptr(lens),
+                 int(bool(advance)), _ptr(y), _ptr(workspace), workspace.numel() * workspace.element_size(), _ptr(status),
+                 b, h, d, m_max, k, v, _stream_of(x.device, stream)), "mqa_layer_decode_step")
     return y
 
 
@@ -404,10 +397,8 @@ def mqa_decode_local_step(q, K, V, k_new, v_new, pos, o, status=None, advance: b
     _need(o, torch.float32, (b, h, v), "o")
     if status is not None:
         _need(status, torch.int32, (1,), "status")
-    with _OnDevice(q.device):
-        rc = lib().mqa_decode_local_step(_ptr(q), _ptr(K), _ptr(V), _ptr(k_new), _ptr(v_new), _ptr(pos), int(bool(advance)),
-                                         _ptr(o), _ptr(status), b, h, window, k, v, _stream(stream))
-    _check(rc, "mqa_decode_local_step")
+    _check(_call(lib().mqa_decode_local_step, q.device, _ptr(q), _ptr(K), _ptr(V), _ptr(k_new), _ptr(v_new), _ptr(pos),
+                 int(bool(advance)), _ptr(o), _ptr(status), b, h, window, k, v, _stream_of(q.device, stream)), "mqa_decode_local_step")
     return o
 
 
@@ -429,12 +420,9 @@ def mqa_prefill_attention(Q, K, V, O, workspace, start=None, status=None, stream
         _need(start, torch.int32, (b,), "start")
     if status is not None:
         _need(status, torch.int32, (1,), "status")
-    s = torch.cuda.current_stream(Q.device) if stream is None else stream
-    with _OnDevice(Q.device):
-        rc = lib().mqa_prefill_attention(Q.data_ptr(), K.data_ptr(), V.data_ptr(), None if start is None else start.data_ptr(),
-                                         O.data_ptr(), workspace.data_ptr(), workspace.numel() * workspace.element_size(),
-                                         None if status is None else status.data_ptr(), b, h, n, m_max, k, v, s.cuda_stream)
-    _check(rc, "mqa_prefill_attention")
+    _check(_call(lib().mqa_prefill_attention, Q.device, _ptr(Q), _ptr(K), _ptr(V), _ptr(start), _ptr(O), _ptr(workspace),
+                 workspace.numel() * workspace.element_size(), _ptr(status), b, h, n, m_max, k, v, _stream_of(Q.device, stream)),
+           "mqa_prefill_attention")
     return O
 
 
@@ -455,11 +443,10 @@ def _host_step_args(q_host, k_new_host, v_new_host, o_host, K, V, lens, staging,
     _need(lens, torch.int32, (b,), "lens")
     if status is not None:
         _need(status, torch.int32, (1,), "status")
-    s = torch.cuda.current_stream(K.device) if stream is None else stream
     return (q_host.data_ptr(), k_new_host.data_ptr(), v_new_host.data_ptr(), o_host.data_ptr(), K.data_ptr(), V.data_ptr(),
             lens.data_ptr(), _step_flags(advance, chained), staging.data_ptr(), staging.numel() * staging.element_size(),
             None if workspace is None else workspace.data_ptr(), 0 if workspace is None else workspace.numel() * workspace.element_size(),
-            None if status is None else status.data_ptr(), b, h, m_max, k, v, s.cuda_stream)
+            None if status is None else status.data_ptr(), b, h, m_max, k, v, _stream_of(K.device, stream))
 
 
 def mqa_decode_append_step_host(q_host, k_new_host, v_new_host, o_host, K, V, lens, staging, workspace=None, status=None,
@@ -468,9 +455,7 @@ def mqa_decode_append_step_host(q_host, k_new_host, v_new_host, o_host, K, V, le
     asynchronous copies); ``staging`` is a device uint8 tensor of ``host_staging_bytes(b, h)`` bytes.  Nothing is
     synchronised: wait on the stream before reading ``o_host``."""
     args = _host_step_args(q_host, k_new_host, v_new_host, o_host, K, V, lens, staging, workspace, status, advance, stream, chained)
-    with _OnDevice(K.device):
-        rc = lib().mqa_decode_append_step_host(*args)
-    _check(rc, "mqa_decode_append_step_host")
+    _check(_call(lib().mqa_decode_append_step_host, K.device, *args), "mqa_decode_append_step_host")
     return o_host
 
 
