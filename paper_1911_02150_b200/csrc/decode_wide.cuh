@@ -218,10 +218,12 @@ mqa_decode_wide_kernel(const uint4* __restrict__ q, const __grid_constant__ CUte
                     ++n_p[w];
                     tc_fence_after();
                     if (elect_one()) {
+                        // one rounding: the stage's 128 rows; hi and lo: 64 of them, twice over
+                        const uint32_t v_p = v_s + part * 4 * 2048;
 #pragma unroll
                         for (int kk = 0; kk < 8; ++kk)
                             umma_ts(tmem_base + kPfTmemO + w * 128, tmem_base + kPfTmemP + w * 64 + kk * 8,
-                                    umma_desc(v_s + kk * 2048, kPfHalfBytes, 1024), kIdescO, (j < 2 && part == 0 && kk == 0) ? 0u : 1u);
+                                    umma_desc(v_p + (hilo ? kk & 3 : kk) * 2048, kPfHalfBytes, 1024), kIdescO, (j < 2 && part == 0 && kk == 0) ? 0u : 1u);
                         tc_commit(pv_done + 8 * w);
                         if (part == (hilo ? 1 : 0)) tc_commit(v_empty + 8 * slot);
                     }
@@ -267,10 +269,30 @@ mqa_decode_wide_kernel(const uint4* __restrict__ q, const __grid_constant__ CUte
             const int valid = r1 - (r0 + j * kWideRows);              // rows of the stage inside this split's prefix (> 0)
             if (ok) ok = mbar_wait(s_ready + 8 * w, ph & 1);
             tc_fence_after();
+            auto clear_v = [&]() {
+                if (valid < kWideRows) {
+                    // the stage runs past the prefix: the tensor core would multiply the zero weights with whatever lies
+                    // there (NaN * 0 = NaN), so those V rows are cleared first
+                    const int vs = j % kWideVSlots;
+                    if (ok) ok = mbar_wait(v_full + 8 * vs, (j / kWideVSlots) & 1);
+                    const uint32_t v_s = v_ring + vs * kPfTileBytes;
+                    for (int i = r; i < (kWideRows - valid) * 16; i += 128) {
+                        const int vrow = valid + (i >> 4), ch = i & 15;
+                        const uint32_t a = v_s + (ch >> 3) * kPfHalfBytes + vrow * 128 + ((ch & 7) << 4);
+                        asm volatile("st.shared.v4.b32 [%0], {%1,%1,%1,%1};" ::"r"(a), "r"(0u) : "memory");
+                    }
+                    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+                }
+            };
             uint32_t x[128];
             if (idle) {
                 if (lane == 0) mbar_arrive(s_free);
-                if (n_p > 0 && ok) ok = mbar_wait(pv_done + 8 * w, (n_p - 1) & 1);    // (the arrival below belongs to the next phase)
+                clear_v();
+                for (int part = 0; part < (hilo ? 2 : 1); ++part, ++n_p) {
+                    if (n_p > 0 && ok) ok = mbar_wait(pv_done + 8 * w, (n_p - 1) & 1);    // (the arrival below belongs to the next phase)
+                    __syncwarp();
+                    if (lane == 0) mbar_arrive(p_ready + 8 * w);
+                }
             } else {
                 // ---- the row's 128 logits, read once and kept in registers; rows past the prefix masked by index (a select)
                 tmem_ld_cols<128>(lane_base, x);
@@ -313,19 +335,37 @@ mqa_decode_wide_kernel(const uint4* __restrict__ q, const __grid_constant__ CUte
                 // ---- P = exp2(S log2e - m) as bf16 pairs (hi) and, for a short prefix, their remainders (lo)
                 const unsigned long long neg_m2 = f2_pack(-m, -m), log2e2 = f2_pack(kLog2e, kLog2e);
                 unsigned long long sum2[2] = {0ull, 0ull};
+                clear_v();
                 // the weights stay in registers until the product before has read the ones in tensor memory
-                uint32_t hi[2][32];
+                auto give = [&](const uint32_t (&p0)[32], const uint32_t (&p1)[32]) {
+                    if (n_p > 0 && ok) ok = mbar_wait(pv_done + 8 * w, (n_p - 1) & 1);
+                    tc_fence_after();
+                    tmem_st32(p_t, p0);
+                    tmem_st32(p_t + 32, p1);
+                    tmem_wait_st();
+                    tc_fence_before();
+                    __syncwarp();
+                    if (lane == 0) mbar_arrive(p_ready + 8 * w);
+                    ++n_p;
+                };
                 if (hilo) {
+                    // hi and lo parts of half of the stage's rows at a time: the first half's product runs under the other's exponentials
 #pragma unroll
-                    for (int i = 0; i < 64; ++i) {
-                        float a0, a1;
-                        f2_unpack(f2_fma(f2_pack(__uint_as_float(x[2 * i]), __uint_as_float(x[2 * i + 1])), log2e2, neg_m2), a0, a1);
-                        const float pa = fast_exp2(a0), pb = fast_exp2(a1);
-                        sum2[i & 1] = f2_add(sum2[i & 1], f2_pack(pa, pb));
-                        hi[i >> 5][i & 31] = pack_bf16(pa, pb);
-                        x[i] = pack_bf16(pa - bf16_lo(hi[i >> 5][i & 31]), pb - bf16_hi(hi[i >> 5][i & 31]));
+                    for (int half = 0; half < 2; ++half) {
+                        uint32_t hi[32], lo[32];
+#pragma unroll
+                        for (int i = 0; i < 32; ++i) {
+                            float a0, a1;
+                            f2_unpack(f2_fma(f2_pack(__uint_as_float(x[64 * half + 2 * i]), __uint_as_float(x[64 * half + 2 * i + 1])), log2e2, neg_m2), a0, a1);
+                            const float pa = fast_exp2(a0), pb = fast_exp2(a1);
+                            sum2[i & 1] = f2_add(sum2[i & 1], f2_pack(pa, pb));
+                            hi[i] = pack_bf16(pa, pb);
+                            lo[i] = pack_bf16(pa - bf16_lo(hi[i]), pb - bf16_hi(hi[i]));
+                        }
+                        give(hi, lo);
                     }
                 } else {
+                    uint32_t hi[2][32];
 #pragma unroll
                     for (int i = 0; i < 64; ++i) {
                         float a0, a1;
@@ -334,47 +374,13 @@ mqa_decode_wide_kernel(const uint4* __restrict__ q, const __grid_constant__ CUte
                         sum2[i & 1] = f2_add(sum2[i & 1], f2_pack(pa, pb));
                         hi[i >> 5][i & 31] = pack_bf16(pa, pb);
                     }
+                    give(hi[0], hi[1]);
                 }
                 {
                     float s0, s1;
                     f2_unpack(f2_add(sum2[0], sum2[1]), s0, s1);
                     l += s0 + s1;
                 }
-                if (n_p > 0 && ok) ok = mbar_wait(pv_done + 8 * w, (n_p - 1) & 1);
-                tc_fence_after();
-                tmem_st32(p_t, hi[0]);
-                tmem_st32(p_t + 32, hi[1]);
-                tmem_wait_st();
-                tc_fence_before();
-            }
-            if (valid < kWideRows) {
-                // the stage runs past the prefix: the tensor core would multiply the zero weights with whatever lies
-                // there (NaN * 0 = NaN), so those V rows are cleared first
-                const int vs = j % kWideVSlots;
-                if (ok) ok = mbar_wait(v_full + 8 * vs, (j / kWideVSlots) & 1);
-                const uint32_t v_s = v_ring + vs * kPfTileBytes;
-                for (int i = r; i < (kWideRows - valid) * 16; i += 128) {
-                    const int vrow = valid + (i >> 4), ch = i & 15;
-                    const uint32_t a = v_s + (ch >> 3) * kPfHalfBytes + vrow * 128 + ((ch & 7) << 4);
-                    asm volatile("st.shared.v4.b32 [%0], {%1,%1,%1,%1};" ::"r"(a), "r"(0u) : "memory");
-                }
-                asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-            }
-            __syncwarp();
-            if (lane == 0) mbar_arrive(p_ready + 8 * w);
-            ++n_p;
-            if (hilo) {                                               // the remainders, once the first part's product has been made
-                if (ok) ok = mbar_wait(pv_done + 8 * w, (n_p - 1) & 1);
-                tc_fence_after();
-                if (!idle) {
-                    tmem_st32(p_t, *reinterpret_cast<uint32_t(*)[32]>(&x[0]));
-                    tmem_st32(p_t + 32, *reinterpret_cast<uint32_t(*)[32]>(&x[32]));
-                    tmem_wait_st();
-                    tc_fence_before();
-                }
-                __syncwarp();
-                if (lane == 0) mbar_arrive(p_ready + 8 * w);
-                ++n_p;
             }
         }
         if (n_p > 0 && ok) ok = mbar_wait(pv_done + 8 * w, (n_p - 1) & 1);

@@ -18,8 +18,8 @@
 // head was a chain logits - softmax - product - logits; two heads' chains side by side left the tensor cores and the
 // exponentials half idle.)  The reference maximum of a row moves only when the row's largest logit leads it by more than
 // kPfMaxLead (then O_w's row is rescaled in TMEM by the row's own thread); P is bounded by 2^kPfMaxLead.
-// Rows of a tile whose memory is shorter than 1024 rows feed P as bf16 hi + lo parts (two products, one after the other
-// out of the same columns), like the decoding kernels, so that the rounding of few large weights stays inside the
+// Rows of a tile whose memory is shorter than 1024 rows feed P as bf16 hi + lo parts (two products, of half of the
+// stage's rows each), like the decoding kernels, so that the rounding of few large weights stays inside the
 // tolerance.
 //
 // Roles: warps 0-3 softmax of head 0, warps 4-7 softmax of head 1, warp 8 TMA producer, warp 9 issues the logits'
@@ -327,7 +327,7 @@ mqa_prefill_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
         if (!ok && lane == 0) atomicExch(&timed_out, 1);
     } else if (warp == kPfPvWarp) {
         // =============================================================== issuer of O_w += P_w V: P from tensor memory (bf16 pairs: 8
-        // columns per 16 rows of V), both parts of it where there are two
+        // columns per 16 rows of V), in two parts where the weights have a hi and a lo one
         constexpr uint32_t kIdescO = umma_idesc(128, 128, false, true);
         bool ok = true;
         int g = 0, n_p[2] = {0, 0};                              // stages and each head's weights so far
@@ -345,10 +345,12 @@ mqa_prefill_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
                         ++n_p[w];
                         tc_fence_after();
                         if (elect_one()) {
+                            // one rounding: the stage's 128 rows; hi and lo: 64 of them, twice over
+                            const uint32_t v_p = v_s + part * 4 * 2048;
 #pragma unroll
                             for (int kk = 0; kk < 8; ++kk)
                                 umma_ts(tmem_base + kPfTmemO + w * 128, tmem_base + kPfTmemP + w * 64 + kk * 8,
-                                        umma_desc(v_s + kk * 2048, kPfHalfBytes, 1024), kIdescO, (j == 0 && part == 0 && kk == 0) ? 0u : 1u);
+                                        umma_desc(v_p + (parts == 2 ? kk & 3 : kk) * 2048, kPfHalfBytes, 1024), kIdescO, (j == 0 && part == 0 && kk == 0) ? 0u : 1u);
                             tc_commit(pv_done + 8 * w);
                             if (w == n_act - 1 && part == parts - 1) tc_commit(v_empty + 8 * slot);
                         }
@@ -433,39 +435,6 @@ mqa_prefill_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
                 const float neg_m = SPLIT && m == -INFINITY ? 0.f : -m;
                 const unsigned long long neg_m2 = f2_pack(neg_m, neg_m), log2e2 = f2_pack(kLog2e, kLog2e);
                 unsigned long long sum2[2] = {0ull, 0ull};
-                // the weights stay in registers until the product before has read the ones in tensor memory
-                uint32_t hi[2][32];
-                if (it.hilo) {
-#pragma unroll
-                    for (int i = 0; i < 64; ++i) {
-                        float a0, a1;
-                        f2_unpack(f2_fma(f2_pack(__uint_as_float(x[2 * i]), __uint_as_float(x[2 * i + 1])), log2e2, neg_m2), a0, a1);
-                        const float pa = fast_exp2(a0), pb = fast_exp2(a1);
-                        sum2[i & 1] = f2_add(sum2[i & 1], f2_pack(pa, pb));
-                        hi[i >> 5][i & 31] = pack_bf16(pa, pb);
-                        x[i] = pack_bf16(pa - bf16_lo(hi[i >> 5][i & 31]), pb - bf16_hi(hi[i >> 5][i & 31]));
-                    }
-                } else {
-#pragma unroll
-                    for (int i = 0; i < 64; ++i) {
-                        float a0, a1;
-                        f2_unpack(f2_fma(f2_pack(__uint_as_float(x[2 * i]), __uint_as_float(x[2 * i + 1])), log2e2, neg_m2), a0, a1);
-                        const float pa = fast_exp2(a0), pb = fast_exp2(a1);
-                        sum2[i & 1] = f2_add(sum2[i & 1], f2_pack(pa, pb));
-                        hi[i >> 5][i & 31] = pack_bf16(pa, pb);
-                    }
-                }
-                {
-                    float s0, s1;
-                    f2_unpack(f2_add(sum2[0], sum2[1]), s0, s1);
-                    l += s0 + s1;
-                }
-                if (n_p > 0 && ok) ok = mbar_wait(pv_done + 8 * w, (n_p - 1) & 1);
-                tc_fence_after();
-                tmem_st32(p_t, hi[0]);
-                tmem_st32(p_t + 32, hi[1]);
-                tmem_wait_st();
-                tc_fence_before();
                 if (w == 0 && it.L < k0 + kPfRows) {
                     // the last stage runs past the memory: the tensor core would multiply the zero weights with
                     // whatever lies there (NaN * 0 = NaN), so those V rows are cleared first
@@ -480,19 +449,50 @@ mqa_prefill_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
                     }
                     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
                 }
-                __syncwarp();
-                if (lane == 0) mbar_arrive(p_ready + 8 * w);
-                ++n_p;
-                if (it.hilo) {                                        // the remainders, once the first part's product has been made
-                    if (ok) ok = mbar_wait(pv_done + 8 * w, (n_p - 1) & 1);
+                // the weights stay in registers until the product before has read the ones in tensor memory
+                auto give = [&](const uint32_t (&p0)[32], const uint32_t (&p1)[32]) {
+                    if (n_p > 0 && ok) ok = mbar_wait(pv_done + 8 * w, (n_p - 1) & 1);
                     tc_fence_after();
-                    tmem_st32(p_t, *reinterpret_cast<uint32_t(*)[32]>(&x[0]));
-                    tmem_st32(p_t + 32, *reinterpret_cast<uint32_t(*)[32]>(&x[32]));
+                    tmem_st32(p_t, p0);
+                    tmem_st32(p_t + 32, p1);
                     tmem_wait_st();
                     tc_fence_before();
                     __syncwarp();
                     if (lane == 0) mbar_arrive(p_ready + 8 * w);
                     ++n_p;
+                };
+                if (it.hilo) {
+                    // hi and lo parts of half of the stage's rows at a time: the first half's product runs under the other's exponentials
+#pragma unroll
+                    for (int half = 0; half < 2; ++half) {
+                        uint32_t hi[32], lo[32];
+#pragma unroll
+                        for (int i = 0; i < 32; ++i) {
+                            float a0, a1;
+                            f2_unpack(f2_fma(f2_pack(__uint_as_float(x[64 * half + 2 * i]), __uint_as_float(x[64 * half + 2 * i + 1])), log2e2, neg_m2), a0, a1);
+                            const float pa = fast_exp2(a0), pb = fast_exp2(a1);
+                            sum2[i & 1] = f2_add(sum2[i & 1], f2_pack(pa, pb));
+                            hi[i] = pack_bf16(pa, pb);
+                            lo[i] = pack_bf16(pa - bf16_lo(hi[i]), pb - bf16_hi(hi[i]));
+                        }
+                        give(hi, lo);
+                    }
+                } else {
+                    uint32_t hi[2][32];
+#pragma unroll
+                    for (int i = 0; i < 64; ++i) {
+                        float a0, a1;
+                        f2_unpack(f2_fma(f2_pack(__uint_as_float(x[2 * i]), __uint_as_float(x[2 * i + 1])), log2e2, neg_m2), a0, a1);
+                        const float pa = fast_exp2(a0), pb = fast_exp2(a1);
+                        sum2[i & 1] = f2_add(sum2[i & 1], f2_pack(pa, pb));
+                        hi[i >> 5][i & 31] = pack_bf16(pa, pb);
+                    }
+                    give(hi[0], hi[1]);
+                }
+                {
+                    float s0, s1;
+                    f2_unpack(f2_add(sum2[0], sum2[1]), s0, s1);
+                    l += s0 + s1;
                 }
             }
             if (SPLIT) {
