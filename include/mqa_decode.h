@@ -154,7 +154,7 @@ int mha_decode_step(const void* q, const void* K, const void* V, const int32_t* 
  *                     lens on by one), and so do projections, a sampler, copies of q; other caches, o
  *                     and the workspace may be written freely.  The first step after something else
  *                     filled the cache (a prefill kernel) must not carry the flag.  With the promise
- *                     the persistent kernel starts fetching the cache, except each prefix's last rows,
+ *                     the step's kernel starts fetching the cache, except each prefix's last rows,
  *                     while the kernel before it is still finishing, and reads q, the new rows, lens
  *                     and the workspace only after that kernel has completed.  What it fetches early
  *                     goes by lens as it reads then; should lens have moved by the time it may rely on
@@ -299,8 +299,8 @@ size_t mqa_host_staging_bytes(int b, int h, int k, int v);
  *   K, V              [b, window, k], [b, window, v] bf16, read-write
  *   pos               [b] int32: tokens of the sequence before this step (0 for the first); advance != 0: pos[b] += 1
  *   o                 [b, h, v] fp32, written;  status optional (APPEND_NEGATIVE_LEN for pos[b] < 0: no row, zeros)
- * One launch; no workspace.  One warp per sequence, eight sequences per CTA, any number of heads (16 at a time),
- * windows of up to 4096 rows (the paper's is 32; MQA_ERR_UNSUPPORTED beyond).
+ * One launch; no workspace.  One warp per sequence, or four for windows of several 32-row tiles and few sequences; any number
+ * of heads, windows of up to 4096 rows (the paper's is 32; MQA_ERR_UNSUPPORTED beyond).
  */
 int mqa_decode_local_step(const void* q, void* K, void* V, const void* k_new, const void* v_new, int32_t* pos,
                           int advance, float* o, int32_t* status, int b, int h, int window, int k, int v,
@@ -322,8 +322,8 @@ int mqa_decode_local_step(const void* q, void* K, void* V, const void* k_new, co
  * cores in bf16 with fp32 accumulation; q, k_new and v_new are rounded to bf16 where the step and the cache
  * take them, o is rounded to bf16 as an operand of the output product; y is summed over head groups in a fixed
  * order (no float atomics: results are reproducible bit for bit).  Kernels: projections in, the step (one
- * launch for large batches), projection out (its head groups are one thread-block cluster of up to 16 CTAs, which
- * sum y through distributed shared memory).
+ * launch for large batches), projection out (CTAs that share a product's depth are
+ * one thread-block cluster and add their sums up through distributed shared memory).
  */
 int mqa_layer_decode_step(const void* x, const void* P_q, const void* P_k, const void* P_v, const void* P_o,
                           void* K, void* V, int32_t* lens, int advance, float* y,
@@ -347,11 +347,12 @@ size_t mqa_layer_workspace_bytes(int b, int h, int d, int m_max, int k, int v);
  *          for that sequence (zeros) and flagged LEN_CLAMPED, like a bad lens.
  *   O      [b, h, n, v] fp32, written           status   optional; LEN_CLAMPED, PIPELINE_TIMEOUT
  *   workspace   at least mqa_prefill_workspace_bytes(b, h, n, m_max, k, v) bytes (see below).
- * One launch of a persistent kernel made for this form (mqa_prefill_kernel: a CTA per SM walks the units of work).  A
- * unit is 128 consecutive positions of two heads of a sequence -- the heads share K and V, so each staged 128-row K/V tile serves 256 query rows -- with the query
- * rows as the rows of the tensor-core tiles (one thread owns one query row's logits, maximum and sum), the weights
- * handed to the second product through tensor memory, and cache rows beyond a tile's last position never fetched.
- * Any n >= 1 (the last tile of a head may be partly filled); k = v = 128 (MQA_ERR_UNSUPPORTED otherwise, and for
+ * One launch of a kernel made for this form (mqa_prefill_kernel).  A unit of work is two tiles of up to 128 query rows of a
+ * sequence, each some positions of some heads -- the heads share K and V, so each staged 128-row K/V tile serves 256 query rows --
+ * with the query rows as the rows of the tensor-core tiles (one thread owns one query row's logits, maximum and sum), the weights
+ * handed to the second product through tensor memory, and cache rows beyond a unit's last position never fetched.  A CTA per
+ * SM walks the units; a call with few units gives each a thread-block cluster, whose CTAs share the cache rows out.
+ * Any n >= 1 (a tile may be partly filled); k = v = 128 (MQA_ERR_UNSUPPORTED otherwise, and for
  * n > m_max).  A memory that would pass m_max (start[b] + n > m_max) is cut at m_max and flagged LEN_CLAMPED.  The
  * workspace is not touched by the present kernel; the argument stays in the interface (pass at least
  * mqa_prefill_workspace_bytes() bytes, which is small and non-zero for supported sizes, 0 otherwise).

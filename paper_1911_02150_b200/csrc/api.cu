@@ -1126,6 +1126,7 @@ static int prefill_split(const PfShape& sh, int rows, int sms) {
     double best_us = 0;
     for (int ctas = 1; ctas <= kPfMaxSplit && ctas * 2 <= (stages > 2 ? stages : 2); ctas *= 2) {
         const int slots = ctas == 8 ? sms / 16 : ctas == 4 ? sms * 9 / 40 : sms / ctas;
+        if (slots < 1) break;
         const double us = (double)((sh.n_items + slots - 1) / slots) * ((double)((stages + ctas - 1) / ctas) * stage_us + unit_us + (ctas > 1 ? merge_us : 0));
         if (best_us == 0 || us < 0.93 * best_us) { best = ctas; best_us = us; }
     }
