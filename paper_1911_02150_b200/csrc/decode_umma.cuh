@@ -48,7 +48,7 @@ constexpr int kUmmaProducerWarp = 8, kUmmaSWarp = 9, kUmmaPvWarp = 10;
 constexpr int kUmmaThreads = 11 * 32;
 // virtual tiles in front of each sequence on the line: what crossing from one sequence to the next costs this kernel
 constexpr int kUmmaBoundaryPenalty = 8;
-constexpr int kGuessL2Stages = 2;                                // stages asked into L2 on a guess, beyond those the rings take
+constexpr int kGuessL2Stages = 3;                                // stages asked into L2 on a guess, beyond those the rings take
 constexpr float kMaxLead = 16.f;                                 // log2 units a logit may exceed the reference maximum by
 
 template <int HP>
@@ -609,7 +609,7 @@ mqa_decode_stream_umma_kernel(const __grid_constant__ CUtensorMap map_k, const _
                         issue_stage(g0.s, u, g0.hi, pre_issued);
                     if (before && lensfree) {
                         // and the stages after those are asked into L2 (measured at 32 sequences x 8192 rows on 128
-                        // CTAs: 26.9 us per step without, 26.2 / 26.0 / 26.5 / 27.2 us with 1 / 2 / 3 / 4 stages)
+                        // CTAs: 27.0 us per step without, 26.4 / 25.9 / 25.7 us with 1 / 2 / 3 stages)
                         int u = g0.lo + pre_issued * ust;
                         for (int p = 0; p < kGuessL2Stages && (u + kSubs) * kTileRows <= stop_row && u + kSubs <= g0.hi; ++p, u += ust) {
                             tma_prefetch_l2_2d((lane >> 1) ? &map_v : &map_k, (lane & 1) * kBoxCols, g0.s * m_max + u * kTileRows);
