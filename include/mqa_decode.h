@@ -350,8 +350,10 @@ size_t mqa_layer_workspace_bytes(int b, int h, int d, int m_max, int k, int v);
  * One launch of a kernel made for this form (mqa_prefill_kernel).  A unit of work is two tiles of up to 128 query rows of a
  * sequence, each some positions of some heads -- the heads share K and V, so each staged 128-row K/V tile serves 256 query rows --
  * with the query rows as the rows of the tensor-core tiles (one thread owns one query row's logits, maximum and sum), the weights
- * handed to the second product through tensor memory, and cache rows beyond a unit's last position never fetched.  A CTA per
- * SM walks the units; a call with few units gives each a thread-block cluster, whose CTAs share the cache rows out.
+ * handed to the second product through tensor memory, and cache rows beyond a tile's last position never multiplied.  A CTA per
+ * SM walks the units; a call with few units gives each a thread-block cluster, whose CTAs share the cache rows out.  (Masked
+ * logits are selected away by index; the weights of a tile's later positions are zeros that are multiplied, so a NaN or Inf in a V
+ * row reaches the up to 127 positions before it that share its tile, and no others.)
  * Any n >= 1 (a tile may be partly filled); k = v = 128 (MQA_ERR_UNSUPPORTED otherwise, and for
  * n > m_max).  A memory that would pass m_max (start[b] + n > m_max) is cut at m_max and flagged LEN_CLAMPED.  The
  * workspace is not touched by the present kernel; the argument stays in the interface (pass at least

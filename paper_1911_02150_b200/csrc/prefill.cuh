@@ -100,10 +100,17 @@ struct PfShape {
 struct PfItem {
     int seq, raw, L, n_kv;
     int tile0, n_act;                     // its first tile, how many it has (the last unit of a sequence may have one)
+    int L0, n_kv0;                        // L and n_kv of the first tile alone (its positions may be earlier than the second's)
     bool hilo;
 };
 __device__ __forceinline__ int pf_position(const PfShape& sh, int tile) { return tile / sh.head_blocks * sh.positions; }   // the tile's first
 __device__ __forceinline__ int pf_head(const PfShape& sh, int tile) { return tile % sh.head_blocks * sh.heads; }
+// A tile goes no further than its own last position: a weight of zero does not silence a V row that is not finite, so what
+// the unit's other tile sees beyond that must not enter its products.  The first tile of a unit may end earlier, by stages,
+// and inside its last stage by rows: of that stage the whole steps of 16 rows below L0 are multiplied as they lie, and the step
+// that L0 falls into from a copy whose rows from L0 on are zeros (pf_cut).  (The copy is made by the warp that issues those products: made
+// by the softmax warps it cost every stage of every call 2 %, by way of their registers.)  What it costs: 5 x 9 heads x 333
+// positions over up to 3000 rows 29.5 -> 30.0 us.  Inside a tile, a later position's row still reaches the earlier ones.
 __device__ __forceinline__ PfItem pf_item(int item, const int32_t* __restrict__ start, const PfShape& sh) {
     PfItem it;
     it.seq = (item / sh.group) % sh.b;
@@ -116,11 +123,15 @@ __device__ __forceinline__ PfItem pf_item(int item, const int32_t* __restrict__ 
     it.L = min(it.raw + min(pf_position(sh, it.tile0 + it.n_act - 1) + sh.positions, sh.n), sh.m_max);
     const bool empty = it.n_act == 0 || it.raw < 0 || it.L <= 0; // nothing to look at: zeros (like a bad lens)
     it.n_kv = empty ? 0 : (it.L + kPfRows - 1) / kPfRows;        // stages
+    it.L0 = min(it.raw + min(pf_position(sh, it.tile0) + sh.positions, sh.n), sh.m_max);
+    it.n_kv0 = empty ? 0 : (it.L0 + kPfRows - 1) / kPfRows;
     // one rounding of the weights from the block of 128 positions on whose last one sees kSingleRoundingMinRows rows,
     // whatever the tiles' shape
     it.hilo = min(it.raw + min((pf_position(sh, it.tile0) & ~(kPfRows - 1)) + kPfRows, sh.n), sh.m_max) < kSingleRoundingMinRows;
     return it;
 }
+// Rows of the first tile's last stage that are its own, if the unit's other tile sees more of them; else 0.
+__device__ __forceinline__ int pf_cut(const PfItem& it) { return it.L0 < it.L ? it.L0 & (kPfRows - 1) : 0; }
 // The row of [b h n, 128] that row r of the unit's tile w is, or -1.
 __device__ __forceinline__ int pf_row(const PfItem& it, const PfShape& sh, int w, int r) {
     const int hh = r / sh.positions, head = pf_head(sh, it.tile0 + w) + hh, pos = pf_position(sh, it.tile0 + w) + r - hh * sh.positions;
@@ -231,6 +242,8 @@ mqa_prefill_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
     // this CTA's stages of a unit: [first, first + count)
     auto first_stage = [&](int n_kv) { return SPLIT ? rank * n_kv / ctas : 0; };
     auto count_stages = [&](int n_kv) { return SPLIT ? (rank + 1) * n_kv / ctas - rank * n_kv / ctas : n_kv; };
+    // how many of them the unit's first tile has
+    auto count_stages0 = [&](const PfItem& it) { return SPLIT ? max(0, min(count_stages(it.n_kv), it.n_kv0 - first_stage(it.n_kv))) : it.n_kv0; };
     if (start && threadIdx.x < 32) {
         // a start that is negative or leaves too little room is flagged once (its rows are zeros, or the memory is cut at m_max)
         bool bad = false;
@@ -296,13 +309,15 @@ mqa_prefill_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
         for (int round = 0, item; (item = pf_unit(round)) < n_items && ok; ++round) {
             const PfItem it = pf_item(item, start, sh);
             const int n_kv = __shfl_sync(0xffffffffu, count_stages(it.n_kv), 0), n_act = it.n_act;
+            const int n_kv0 = __shfl_sync(0xffffffffu, count_stages0(it), 0);
             if (n_kv == 0) continue;
             ok = warp_wait(q_full, qi & 1);
             for (int j = 0; j < n_kv && ok; ++j, ++g) {
                 const int slot = g % kPfKSlots;
                 const uint32_t k_s = k_ring + slot * kPfTileBytes;
                 ok = warp_wait(k_full + 8 * slot, (g / kPfKSlots) & 1);
-                for (int w = 0; w < n_act && ok; ++w, ++n_s) {
+                for (int w = 0; w < n_act && ok; ++w) {
+                    if (w == 0 && j >= n_kv0) continue;
                     if (n_s > 0) ok = warp_wait(s_free, (n_s - 1) & 1);
                     if (!ok) break;
                     tc_fence_after();
@@ -320,6 +335,7 @@ mqa_prefill_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
                         }
                     }
                     __syncwarp();
+                    ++n_s;
                 }
             }
             ++qi;
@@ -334,25 +350,62 @@ mqa_prefill_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
         for (int round = 0, item; (item = pf_unit(round)) < n_items && ok; ++round) {
             const PfItem it = pf_item(item, start, sh);
             const int n_kv = __shfl_sync(0xffffffffu, count_stages(it.n_kv), 0), n_act = it.n_act, parts = __any_sync(0xffffffffu, it.hilo) ? 2 : 1;
+            const int n_kv0 = __shfl_sync(0xffffffffu, count_stages0(it), 0);
+            // (the stage that is cut, counted from this CTA's first one: with SPLIT it may be another CTA's.  A reduction over the
+            // warp leaves its result where the issue of a product can test it: 0.4 us less for a unit than with a shuffle)
+            const int cut = __reduce_max_sync(0xffffffffu, pf_cut(it)), cut_j = cut > 0 ? it.n_kv0 - 1 - first_stage(it.n_kv) : -1;
             for (int j = 0; j < n_kv && ok; ++j, ++g) {
                 const int slot = g % kPfVSlots;
                 const uint32_t v_s = v_ring + slot * kPfTileBytes;
                 ok = warp_wait(v_full + 8 * slot, (g / kPfVSlots) & 1);
                 for (int w = 0; w < n_act && ok; ++w) {
+                    if (w == 0 && j >= n_kv0) continue;
+                    const bool whole = __all_sync(0xffffffffu, w > 0 || j != cut_j);
+                    if (!whole && (cut & 15)) {
+                        // the 16 rows that the first tile ends in, zeros from its end on, to the place where its softmax warps hand O out
+                        // (with those of the unit before they are through once this stage's weights are there)
+                        if (!SPLIT) ok = warp_wait(p_ready, n_p[0] & 1);
+                        uint4 v[8];
+#pragma unroll
+                        for (int i = 0; i < 8; ++i) {            // 16-byte pieces, eight to a row of a 64-column half
+                            const int at = (i >> 2) * kPfHalfBytes + ((cut & ~15) + (i & 3) * 4) * 128 + lane * 16;
+                            asm volatile("ld.shared.v4.b32 {%0,%1,%2,%3}, [%4];" : "=r"(v[i].x), "=r"(v[i].y), "=r"(v[i].z), "=r"(v[i].w) : "r"(v_s + at) : "memory");
+                        }
+#pragma unroll
+                        for (int i = 0; i < 8; ++i) {
+                            if ((i & 3) * 4 + (lane >> 3) >= (cut & 15)) v[i] = make_uint4(0u, 0u, 0u, 0u);
+                            asm volatile("st.shared.v4.b32 [%0], {%1,%2,%3,%4};" ::"r"(out_s + (i * 32 + lane) * 16), "r"(v[i].x), "r"(v[i].y), "r"(v[i].z), "r"(v[i].w) : "memory");
+                        }
+                        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+                        __syncwarp();
+                    }
                     for (int part = 0; part < parts && ok; ++part) {
                         ok = warp_wait(p_ready + 8 * w, n_p[w] & 1);
                         if (!ok) break;
                         ++n_p[w];
                         tc_fence_after();
-                        if (elect_one()) {
-                            // one rounding: the stage's 128 rows; hi and lo: 64 of them, twice over
-                            const uint32_t v_p = v_s + part * 4 * 2048;
+                        if (whole) {
+                            if (elect_one()) {
+                                // one rounding: the stage's 128 rows; hi and lo: 64 of them, twice over
+                                const uint32_t v_p = v_s + part * 4 * 2048;
 #pragma unroll
-                            for (int kk = 0; kk < 8; ++kk)
-                                umma_ts(tmem_base + kPfTmemO + w * 128, tmem_base + kPfTmemP + w * 64 + kk * 8,
-                                        umma_desc(v_p + (parts == 2 ? kk & 3 : kk) * 2048, kPfHalfBytes, 1024), kIdescO, (j == 0 && part == 0 && kk == 0) ? 0u : 1u);
-                            tc_commit(pv_done + 8 * w);
-                            if (w == n_act - 1 && part == parts - 1) tc_commit(v_empty + 8 * slot);
+                                for (int kk = 0; kk < 8; ++kk)
+                                    umma_ts(tmem_base + kPfTmemO + w * 128, tmem_base + kPfTmemP + w * 64 + kk * 8,
+                                            umma_desc(v_p + (parts == 2 ? kk & 3 : kk) * 2048, kPfHalfBytes, 1024), kIdescO, (j == 0 && part == 0 && kk == 0) ? 0u : 1u);
+                                tc_commit(pv_done + 8 * w);
+                                if (w == n_act - 1 && part == parts - 1) tc_commit(v_empty + 8 * slot);
+                            }
+                        } else if (elect_one()) {
+                            // the first tile's last stage, up to its last row (the other tile has the stage too)
+#pragma unroll
+                            for (int kk = 0; kk < 8; ++kk) {
+                                const int row = (parts == 2 ? part * 4 + (kk & 3) : kk) * 16;
+                                if (row < cut)
+                                    umma_ts(tmem_base + kPfTmemO, tmem_base + kPfTmemP + kk * 8,
+                                            row + 16 > cut ? umma_desc(out_s, 2048, 1024) : umma_desc(v_s + row * 128, kPfHalfBytes, 1024),
+                                            kIdescO, (j == 0 && part == 0 && kk == 0) ? 0u : 1u);
+                            }
+                            tc_commit(pv_done);
                         }
                         __syncwarp();
                     }
@@ -385,7 +438,9 @@ mqa_prefill_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
             const int lim_first = min(it.raw + p0 + 1, it.L);            // rows the tile's first position sees
             const int lim = min(it.raw + min(p0 + r % sh.positions, sh.n - 1) + 1, it.L);   // rows this thread's position sees: >= 1
             float m = -INFINITY, l = 0.f;                        // reference maximum (log2 units), sum of weights
-            for (int j = 0; j < (w < it.n_act ? n_kv : 0); ++j) {
+            const int n_own = w == 0 ? count_stages0(it) : w < it.n_act ? n_kv : 0;      // stages of this tile
+            const bool clears = w == (it.n_kv0 == it.n_kv ? 0 : 1);                      // the first tile to see the unit's last stage
+            for (int j = 0; j < n_own; ++j) {
                 const int k0 = (first + j) * kPfRows;
                 if (ok) ok = mbar_wait(s_ready + 8 * w, n_s & 1);
                 ++n_s;
@@ -435,7 +490,7 @@ mqa_prefill_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
                 const float neg_m = SPLIT && m == -INFINITY ? 0.f : -m;
                 const unsigned long long neg_m2 = f2_pack(neg_m, neg_m), log2e2 = f2_pack(kLog2e, kLog2e);
                 unsigned long long sum2[2] = {0ull, 0ull};
-                if (w == 0 && it.L < k0 + kPfRows) {
+                if (clears && it.L < k0 + kPfRows) {
                     // the last stage runs past the memory: the tensor core would multiply the zero weights with
                     // whatever lies there (NaN * 0 = NaN), so those V rows are cleared first
                     const int vs = (g + j) % kPfVSlots;

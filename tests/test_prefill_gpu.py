@@ -239,3 +239,40 @@ def test_a_memory_that_would_pass_m_max_is_cut_there_and_flagged():
         lens = np.minimum(st + t + 1, m_max).astype(np.int32)
         ref = oracle.mqa_decode_step(wl.bits(Q[:, :, t].contiguous()), wl.bits(K), wl.bits(V), lens)
         check_close(Oh[:, :, t], ref, f"position {t}")
+
+
+def attend(Q, K, V, start):
+    """O of the batched form as it comes, whatever the inputs hold."""
+    b, h, n, _ = Q.shape
+    O = torch.empty(b, h, n, 128, dtype=torch.float32, device=DEV)
+    status = torch.zeros(1, dtype=torch.int32, device=DEV)
+    mqa.mqa_prefill_attention(Q, K, V, O, torch.empty(16, dtype=torch.uint8, device=DEV),
+                              None if start is None else torch.tensor(start, dtype=torch.int32, device=DEV), status)
+    torch.cuda.synchronize()
+    assert int(status.item()) == 0
+    return O
+
+
+@pytest.mark.parametrize("b,h,n,m_max,start,positions", [
+    # the two tiles of a unit begin at different positions: an odd number of tiles side by side at each position
+    (1, 1, 256, 256, None, 128), (300, 1, 256, 260, None, 128), (3, 1, 500, 900, [0, 37, 399], 128), (1, 1, 256, 2048, [1003], 128),
+    (2, 9, 333, 1000, [100, 3], 42), (40, 9, 84, 84, None, 42), (1, 9, 333, 3000, [2001], 42), (60, 9, 333, 340, None, 42),
+])
+def test_rows_of_later_positions_do_not_reach_the_tiles_before_them(b, h, n, m_max, start, positions):
+    """NaN and Inf in V rows from the first position of a tile on: the tiles before it are the same to the last bit, those
+    positions themselves are not finite where the row is not."""
+    gen = torch.Generator(device=DEV).manual_seed(n + h)
+    Q = wl.bf16_normal((b, h, n, 128), 128 ** -0.5, gen, DEV)
+    K = wl.bf16_normal((b, m_max, 128), 1.0, gen, DEV)
+    V = wl.bf16_normal((b, m_max, 128), 1.0, gen, DEV)
+    clean = attend(Q, K, V, start)
+    assert bool(torch.isfinite(clean).all())
+    at = torch.tensor([0] * b if start is None else start, device=DEV)[:, None]
+    for first in range(positions, n, positions):
+        bad = V.clone()
+        later = torch.arange(m_max, device=DEV)[None] >= at + first
+        bad[..., ::2].masked_fill_(later[..., None], float("nan"))
+        bad[..., 1::2].masked_fill_(later[..., None], float("inf"))
+        O = attend(Q, K, bad, start)
+        assert torch.equal(O[:, :, :first].view(torch.int32), clean[:, :, :first].view(torch.int32)), f"rows from position {first} on"
+        assert bool(torch.isnan(O[:, :, first:, ::2]).all()) and not bool(torch.isfinite(O[:, :, first:]).any())
