@@ -175,7 +175,9 @@ __device__ __forceinline__ void pf_merge(const PfItem& it, const PfShape& sh, fl
             for (int c = 0; c < CTAS; ++c) top = fmaxf(top, ml[i][c].x);
 #pragma unroll
             for (int c = 0; c < CTAS; ++c) {
-                if (ml[i][c].x == -INFINITY) continue;           // nothing of this share is visible to the row (it may never have been written)
+                // a share of which the row sees nothing (it may never have been written).  Its maximum does not tell: that of a
+                // share whose logits are all NaN is -inf too, and its sum is NaN
+                if (ml[i][c].y == 0.f) continue;
                 const float f = fast_exp2(ml[i][c].x - top);
                 den = fmaf(f, ml[i][c].y, den);
                 num.x = fmaf(f, part[i][c].x, num.x); num.y = fmaf(f, part[i][c].y, num.y);

@@ -276,3 +276,24 @@ def test_rows_of_later_positions_do_not_reach_the_tiles_before_them(b, h, n, m_m
         O = attend(Q, K, bad, start)
         assert torch.equal(O[:, :, :first].view(torch.int32), clean[:, :, :first].view(torch.int32)), f"rows from position {first} on"
         assert bool(torch.isnan(O[:, :, first:, ::2]).all()) and not bool(torch.isfinite(O[:, :, first:]).any())
+
+
+@pytest.mark.parametrize("b,h,n,m_max,start", [
+    (1, 4, 16, 2064, 2048), (1, 4, 16, 2064, 1500), (2, 9, 100, 1500, 1400), (1, 3, 128, 1000, 700), (200, 4, 128, 512, 384),
+])
+def test_a_memory_whose_rows_are_partly_nan_gives_nan(b, h, n, m_max, start):
+    """A position that sees a key row of NaN has no finite output, wherever the row lies: also where all that one of several
+    CTAs sees of the memory is such rows (and where a position sees nothing else at all)."""
+    gen = torch.Generator(device=DEV).manual_seed(m_max)
+    Q = wl.bf16_normal((b, h, n, 128), 128 ** -0.5, gen, DEV)
+    K = wl.bf16_normal((b, m_max, 128), 1.0, gen, DEV)
+    V = wl.bf16_normal((b, m_max, 128), 1.0, gen, DEV)
+    for rows in (slice(start // 2, start), slice(0, start // 2), slice(0, start), slice(0, start + n), slice(start // 3, start // 3 + 1)):
+        bad = K.clone()
+        bad[:, rows] = float("nan")
+        assert bool(torch.isnan(attend(Q, bad, V, [start] * b)).all()), f"rows {rows}"
+    bad = K.clone()
+    bad[:, start + n // 2] = float("nan")                  # a row that only the later positions see
+    O, clean = attend(Q, bad, V, [start] * b), attend(Q, K, V, [start] * b)
+    assert bool(torch.isnan(O[:, :, n // 2:]).all())
+    assert torch.equal(O[:, :, : n // 2].view(torch.int32), clean[:, :, : n // 2].view(torch.int32))
