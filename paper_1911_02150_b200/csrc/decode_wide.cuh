@@ -316,7 +316,7 @@ mqa_decode_wide_kernel(const uint4* __restrict__ q, const __grid_constant__ CUte
                     // to its largest logit so far and rescales its sum and its row of O
                     const float m_new = fmaxf(m, mx);
                     if (ph > 0) {
-                        const float f = fast_exp2(m - m_new);             // (m is finite from the warpgroup's first stage on)
+                        const float f = m == m_new ? 1.f : fast_exp2(m - m_new);     // (m = -inf while all logits were)
                         l *= f;
                         if (ok) ok = mbar_wait(pv_done + 8 * w, (n_p - 1) & 1);  // O holds the warpgroup's stages before this one
                         tc_fence_after();
@@ -333,7 +333,8 @@ mqa_decode_wide_kernel(const uint4* __restrict__ q, const __grid_constant__ CUte
                     m = m_new;
                 }
                 // ---- P = exp2(S log2e - m) as bf16 pairs (hi) and, for a short prefix, their remainders (lo)
-                const unsigned long long neg_m2 = f2_pack(-m, -m), log2e2 = f2_pack(kLog2e, kLog2e);
+                const float neg_m = m == -INFINITY ? 0.f : -m;            // (nothing but logits of -inf so far: weights of zero)
+                const unsigned long long neg_m2 = f2_pack(neg_m, neg_m), log2e2 = f2_pack(kLog2e, kLog2e);
                 unsigned long long sum2[2] = {0ull, 0ull};
                 clear_v();
                 // the weights stay in registers until the product before has read the ones in tensor memory
@@ -416,7 +417,8 @@ mqa_decode_wide_kernel(const uint4* __restrict__ q, const __grid_constant__ CUte
             if (n_kv > 0) {
                 const float2 other = ex_ml[r];
                 const float top = two ? fmaxf(m, other.x) : m;
-                const float f0 = fast_exp2(m - top), f1 = two ? fast_exp2(other.x - top) : 0.f;
+                // (a share of logits that are all -inf has that maximum and a sum of 0)
+                const float f0 = m == top ? 1.f : fast_exp2(m - top), f1 = !two ? 0.f : other.x == top ? 1.f : fast_exp2(other.x - top);
                 ml = make_float2(top, f0 * l + (two ? f1 * other.y : 0.f));
                 const float scale = n_splits == 1 ? 1.f / ml.y : 1.f;
                 ex_ml[r] = make_float2(f0 * scale, f1 * scale);

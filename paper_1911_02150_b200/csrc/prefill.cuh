@@ -472,8 +472,8 @@ mqa_prefill_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
                 if (__any_sync(0xffffffffu, my_row >= 0 && mx > m + kPfMaxLead)) {
                     const float m_new = fmaxf(m, mx);
                     if (j > 0) {
-                        // (m is finite from the unit's first stage on; of a run of its stages a row may have seen nothing yet)
-                        const float f = SPLIT && m == m_new ? 1.f : fast_exp2(m - m_new);
+                        // (a row whose logits have all been -inf, or which has seen nothing yet of a run of stages, has m = -inf)
+                        const float f = m == m_new ? 1.f : fast_exp2(m - m_new);
                         l *= f;
                         if (ok) ok = mbar_wait(pv_done + 8 * w, (n_p - 1) & 1);           // O holds the stages before this one
                         tc_fence_after();
@@ -489,7 +489,7 @@ mqa_prefill_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
                     }
                     m = m_new;
                 }
-                const float neg_m = SPLIT && m == -INFINITY ? 0.f : -m;
+                const float neg_m = m == -INFINITY ? 0.f : -m;      // (weights of zero)
                 const unsigned long long neg_m2 = f2_pack(neg_m, neg_m), log2e2 = f2_pack(kLog2e, kLog2e);
                 unsigned long long sum2[2] = {0ull, 0ull};
                 if (clears && it.L < k0 + kPfRows) {

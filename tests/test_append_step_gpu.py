@@ -238,3 +238,21 @@ def test_bound_step_gives_what_the_call_gives():
     assert torch.equal(inp["K"].view(torch.int16), K2.view(torch.int16)) and torch.equal(inp["V"].view(torch.int16), V2.view(torch.int16))
     with pytest.raises(TypeError):
         mqa.AppendStep(inp["q"].float(), K2, V2, inp["k_new"], inp["v_new"], lens_b, o_b, ws)
+
+
+@pytest.mark.parametrize("b,h,m_max", [(5, 40, 700), (3, 96, 2600), (160, 33, 600), (2, 130, 1500)])
+def test_logits_of_minus_infinity_weigh_nothing_with_many_query_rows(b, h, m_max):
+    """Key rows whose logit is -inf for every query row: whole 128-row stages of them, the first, the second (the other softmax
+    warps' first) and all but the last rows."""
+    inp = wl.make_inputs(b, h, m_max, "mqa", seed=m_max, device=DEV)
+    inp["q"][..., 0] = inp["q"][..., 0].abs() + 0.125
+    lens = torch.full((b,), m_max - 1, dtype=torch.int32, device=DEV)
+    ws, status = mqa.alloc_workspace(b, h, m_max, DEV), torch.zeros(1, dtype=torch.int32, device=DEV)
+    for rows in (slice(128, 256), slice(0, 128), slice(0, 384), slice(130, 500), slice(0, m_max - 2)):
+        K, o = inp["K"].clone(), torch.empty(b, h, 128, dtype=torch.float32, device=DEV)
+        K[:, rows, 0] = -float("inf")
+        mqa.mqa_decode_append_step(inp["q"], K, inp["V"], inp["k_new"], inp["v_new"], lens, o, ws, status, advance=False)
+        torch.cuda.synchronize()
+        assert int(status.item()) == 0
+        ref = torch.softmax(inp["q"].double() @ K.double().transpose(1, 2), -1) @ inp["V"].double()    # (the new row is in K and V by now)
+        check_close(o.cpu().numpy(), ref.cpu().numpy(), f"rows {rows}")

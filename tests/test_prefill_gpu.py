@@ -297,3 +297,26 @@ def test_a_memory_whose_rows_are_partly_nan_gives_nan(b, h, n, m_max, start):
     O, clean = attend(Q, bad, V, [start] * b), attend(Q, K, V, [start] * b)
     assert bool(torch.isnan(O[:, :, n // 2:]).all())
     assert torch.equal(O[:, :, : n // 2].view(torch.int32), clean[:, :, : n // 2].view(torch.int32))
+
+
+@pytest.mark.parametrize("b,h,n,m_max,start", [
+    (1, 4, 16, 2064, 2048), (2, 9, 100, 1500, 1400), (200, 2, 128, 640, 512), (150, 4, 128, 1300, 1172),
+])
+def test_logits_of_minus_infinity_weigh_nothing(b, h, n, m_max, start):
+    """Key rows whose logit is -inf for every query: whole stages of them, first, in the middle and last."""
+    gen = torch.Generator(device=DEV).manual_seed(m_max)
+    Q = wl.bf16_normal((b, h, n, 128), 128 ** -0.5, gen, DEV)
+    Q[..., 0] = Q[..., 0].abs() + 0.125
+    K = wl.bf16_normal((b, m_max, 128), 1.0, gen, DEV)
+    V = wl.bf16_normal((b, m_max, 128), 1.0, gen, DEV)
+    for rows in (slice(0, 128), slice(0, 300), slice(128, 384), slice(start // 2, start), slice(128, start)):
+        K2 = K.clone()
+        K2[:, rows, 0] = -float("inf")
+        O = attend(Q, K2, V, [start] * b)
+        s = Q[0].double() @ K2[0].double().T
+        hidden = torch.arange(m_max, device=DEV)[None] > start + torch.arange(n, device=DEV)[:, None]
+        ref = torch.softmax(s.masked_fill(hidden, -float("inf")), -1) @ V[0].double()
+        check_close(O[0].cpu().numpy(), ref.cpu().numpy(), f"rows {rows}")
+    K2 = K.clone()
+    K2[..., 0] = -float("inf")                             # nothing else: 0 / 0
+    assert bool(torch.isnan(attend(Q, K2, V, [start] * b)).all())
