@@ -16,7 +16,7 @@ kv_cache_append_kernel(uint4* __restrict__ K, uint4* __restrict__ V,
     const int bi = blockIdx.x;
     grid_dependency_wait();          // lens may come from the kernel before this one
     grid_launch_dependents();        // the step that follows may set itself up; it waits before reading
-    const int row = lens[bi];
+    const int row = __ldcg(lens + bi);
     if (row < 0 || row >= m_max) {   // uniform over the CTA
         if (threadIdx.x == 0 && status)
             atomicOr(status, row < 0 ? kStatusAppendNegative : kStatusAppendFull);
@@ -29,7 +29,7 @@ kv_cache_append_kernel(uint4* __restrict__ K, uint4* __restrict__ V,
     for (int g = warp; g < kv_heads; g += kAppendThreads / 32) {
         const size_t src = ((size_t)bi * kv_heads + g) * kVecPerRow + vec;
         const size_t dst = (((size_t)bi * kv_heads + g) * m_max + row) * kVecPerRow + vec;
-        if (is_v) V[dst] = v_new[src]; else K[dst] = k_new[src];
+        if (is_v) V[dst] = __ldcg(v_new + src); else K[dst] = __ldcg(k_new + src);
     }
     if (advance) {
         __syncthreads();             // every warp has read lens[bi] before it moves

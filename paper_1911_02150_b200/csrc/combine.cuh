@@ -103,7 +103,7 @@ combine_splits_kernel(const float2* __restrict__ part_ml, const float* __restric
     // the CTA of a sequence's first head may move it on (lens_advance: the append-and-attend step)
     int live = n_splits;
     if (lens != nullptr) {
-        int L = biased_len(lens[u / h], m_max, len_bias);
+        int L = biased_len(__ldcg(lens + u / h), m_max, len_bias);
         L = L < 0 ? 0 : (L > m_max ? m_max : L);
         live = (L + chunk_rows - 1) / chunk_rows;
         if (live > n_splits) live = n_splits;
@@ -141,7 +141,7 @@ combine_few_kernel(const float2* __restrict__ part_ml, const float* __restrict__
     if (u >= units) return;
     int live = n_splits;
     if (lens != nullptr) {
-        int L = biased_len(lens[seq], m_max, len_bias);
+        int L = biased_len(__ldcg(lens + seq), m_max, len_bias);
         L = L < 0 ? 0 : (L > m_max ? m_max : L);
         live = (L + chunk_rows - 1) / chunk_rows;
         if (live > n_splits) live = n_splits;

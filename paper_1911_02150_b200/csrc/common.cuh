@@ -24,10 +24,10 @@ __device__ __forceinline__ float fast_exp2(float x) {
     return y;
 }
 
-// 16-byte read-only global load that does not allocate in L1 (each cache byte is used once).
+// 16-byte global load that does not allocate in L1 (each cache byte is used once).
 __device__ __forceinline__ uint4 ldg_stream(const void* p) {
     uint4 r;
-    asm volatile("ld.global.nc.L1::no_allocate.v4.u32 {%0,%1,%2,%3}, [%4];"
+    asm volatile("ld.global.L1::no_allocate.v4.u32 {%0,%1,%2,%3}, [%4];"
                  : "=r"(r.x), "=r"(r.y), "=r"(r.z), "=r"(r.w) : "l"(p));
     return r;
 }
@@ -39,6 +39,10 @@ __device__ __forceinline__ uint4 ldg_stream(const void* p) {
 // here waits first and lets its dependents start afterwards: with second-pass kernels that let
 // theirs start before their own wait, a decoding loop of four kernels per step gave results that
 // differed from run to run.
+// So a kernel may be resident while the one ahead of it still writes what it will read, and none of that is read-only for
+// its lifetime: memory that a kernel ahead may have written (lens, positions, q, new rows, o, pieces, the cache) is read after the
+// wait with ordinary loads or __ldcg, never with a read-only one (__ldg; a plain load through a const __restrict__ pointer becomes
+// one too, so those pointers have no __restrict__), which need not see the write.
 __device__ __forceinline__ void grid_dependency_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void grid_launch_dependents() { asm volatile("griddepcontrol.launch_dependents;"); }
 

@@ -29,7 +29,7 @@ static_assert(local_smem_bytes(kLocalMaxWarps, 2) <= 227 * 1024, "exceeds the sh
 
 __global__ void __launch_bounds__(kLocalMaxWarps * 32, 1)
 mqa_decode_local_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_constant__ CUtensorMap map_v,
-                        const uint32_t* __restrict__ q, const uint4* __restrict__ k_new, const uint4* __restrict__ v_new,
+                        const uint32_t* q, const uint4* __restrict__ k_new, const uint4* __restrict__ v_new,
                         uint4* __restrict__ K, uint4* __restrict__ V, int32_t* __restrict__ pos, float* __restrict__ o,
                         int32_t* __restrict__ status, int b, int h, int window, int advance, int stages) {
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, warps = blockDim.x >> 5;
@@ -65,8 +65,8 @@ mqa_decode_local_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_
     };
     // the first tile, the new row's pieces (lanes 0-15 the key row, 16-31 the value row), q and pos are in flight together
     issue(0, 0);
-    const uint4 row_piece = (lane < 16 ? k_new : v_new)[(size_t)seq * (kRowBytes / 16) + (lane & 15)];
-    const int raw = pos[seq];
+    const uint4 row_piece = __ldcg((lane < 16 ? k_new : v_new) + (size_t)seq * (kRowBytes / 16) + (lane & 15));
+    const int raw = __ldcg(pos + seq);
     uint32_t qa[8][4];
     load_q_fragments(qa, q, (size_t)seq, h, 0, lane);
     const size_t units = (size_t)seq * h;

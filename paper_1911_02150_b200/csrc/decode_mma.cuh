@@ -203,7 +203,7 @@ struct WarpState {
 
 // Q fragments (A operand, 16 heads x 128 columns) of head tile mt of sequence seq, straight from
 // global memory; heads >= h are zero.
-__device__ __forceinline__ void load_q_fragments(uint32_t (&qa)[8][4], const uint32_t* __restrict__ q, size_t seq,
+__device__ __forceinline__ void load_q_fragments(uint32_t (&qa)[8][4], const uint32_t* q, size_t seq,
                                                  int h, int mt, int lane) {
     const int g = lane >> 2, t4 = lane & 3;
     const int head0 = mt * 16 + g, head1 = head0 + 8;
@@ -212,10 +212,10 @@ __device__ __forceinline__ void load_q_fragments(uint32_t (&qa)[8][4], const uin
 #pragma unroll
     for (int ks = 0; ks < 8; ++ks) {
         const int w0 = ks * 8 + t4;                    // 32-bit word: columns ks*16 + t4*2 + {0,1}
-        qa[ks][0] = head0 < h ? __ldg(q0 + w0) : 0u;
-        qa[ks][1] = head1 < h ? __ldg(q1 + w0) : 0u;
-        qa[ks][2] = head0 < h ? __ldg(q0 + w0 + 4) : 0u;   // columns + 8
-        qa[ks][3] = head1 < h ? __ldg(q1 + w0 + 4) : 0u;
+        qa[ks][0] = head0 < h ? q0[w0] : 0u;
+        qa[ks][1] = head1 < h ? q1[w0] : 0u;
+        qa[ks][2] = head0 < h ? q0[w0 + 4] : 0u;   // columns + 8
+        qa[ks][3] = head1 < h ? q1[w0 + 4] : 0u;
     }
 }
 
@@ -340,7 +340,7 @@ template <int M_TILES, int EARLY = 0>
 __global__ void __launch_bounds__(MmaCfg<M_TILES>::kThreads, MmaCfg<M_TILES>::kMinBlocks)
 mqa_decode_split_mma_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_constant__ CUtensorMap map_v,
                             const __grid_constant__ CUtensorMap map_k_big, const __grid_constant__ CUtensorMap map_v_big,
-                            const uint32_t* __restrict__ q, const int32_t* __restrict__ lens,
+                            const uint32_t* q, const int32_t* lens,
                             float* __restrict__ o, float2* __restrict__ part_ml, float* __restrict__ part_acc,
                             int32_t* __restrict__ status, int h, int m_max, int chunk_rows, int n_splits, int len_bias,
                             const FusedArgs fa, int32_t* __restrict__ lens_advance, int mode) {

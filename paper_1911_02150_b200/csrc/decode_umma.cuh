@@ -437,7 +437,7 @@ mqa_decode_stream_umma_kernel(const __grid_constant__ CUtensorMap map_k, const _
     // made visible to the copy engine) before the stage that contains it is fetched.
     auto row_load = [&](int s) -> uint4 {
         const uint4* src = (lane < 16 ? fa.k_new : fa.v_new) + (size_t)s * (kRowBytes / 16) + (lane & 15);
-        return __ldg(src);
+        return __ldcg(src);
     };
     auto row_store = [&](int s, int new_row, uint4 value) {
         uint4* dst = (lane < 16 ? fa.K : fa.V) + ((size_t)s * m_max + new_row) * (kRowBytes / 16) + (lane & 15);

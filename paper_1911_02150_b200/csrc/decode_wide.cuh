@@ -126,7 +126,7 @@ mqa_decode_wide_kernel(const uint4* __restrict__ q, const __grid_constant__ CUte
     // has one split (lens_advance given), else in the second-pass kernel.
     uint4 row_piece = make_uint4(0u, 0u, 0u, 0u);              // lanes 0-15: of the key row (S and producer warp), or the value row
     if (fa.k_new != nullptr && warp >= kWideProducerWarp)      // (the producer warp's lanes 16-31 the value row)
-        row_piece = (warp == kWidePvWarp || (warp == kWideProducerWarp && lane >= 16) ? fa.v_new : fa.k_new)[(size_t)seq * (kRowBytes / 16) + (lane & 15)];
+        row_piece = __ldcg((warp == kWidePvWarp || (warp == kWideProducerWarp && lane >= 16) ? fa.v_new : fa.k_new) + (size_t)seq * (kRowBytes / 16) + (lane & 15));
     const int raw = __ldcg(lens + seq);
     const bool appended = fa.k_new != nullptr && raw >= 0 && raw < m_max;
     if (fa.k_new != nullptr && !appended && split == 0 && blockIdx.y == 0 && threadIdx.x == 0 && status)

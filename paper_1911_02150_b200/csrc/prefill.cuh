@@ -111,12 +111,12 @@ __device__ __forceinline__ int pf_head(const PfShape& sh, int tile) { return til
 // that L0 falls into from a copy whose rows from L0 on are zeros (pf_cut).  (The copy is made by the warp that issues those products: made
 // by the softmax warps it cost every stage of every call 2 %, by way of their registers.)  What it costs: 5 x 9 heads x 333
 // positions over up to 3000 rows 29.5 -> 30.0 us.  Inside a tile, a later position's row still reaches the earlier ones.
-__device__ __forceinline__ PfItem pf_item(int item, const int32_t* __restrict__ start, const PfShape& sh) {
+__device__ __forceinline__ PfItem pf_item(int item, const int32_t* start, const PfShape& sh) {
     PfItem it;
     it.seq = (item / sh.group) % sh.b;
     const int unit = sh.n_units - 1 - (item / (sh.group * sh.b) * sh.group + item % sh.group);
     it.n_act = unit < 0 ? 0 : min(2, sh.n_tiles - 2 * unit);     // (the last group may be partly filled)
-    it.raw = start ? min(__ldg(start + it.seq), sh.m_max) : 0;
+    it.raw = start ? min(start[it.seq], sh.m_max) : 0;
     it.tile0 = 2 * unit;
     // rows of the memory the unit's last position sees (rows of a tile past the last position or head are computed on
     // whatever the Q tile holds there and never stored); a memory that would pass m_max is cut there
@@ -194,7 +194,7 @@ __device__ __forceinline__ void pf_merge(const PfItem& it, const PfShape& sh, fl
 template <bool SPLIT>
 __global__ void __launch_bounds__(kPfThreads, 1)
 mqa_prefill_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CUtensorMap map_k,
-                   const __grid_constant__ CUtensorMap map_v, const int32_t* __restrict__ start, float* __restrict__ O,
+                   const __grid_constant__ CUtensorMap map_v, const int32_t* start, float* __restrict__ O,
                    int32_t* __restrict__ status, const PfShape sh) {
     const int warp = __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0), lane = threadIdx.x & 31;
 
@@ -249,7 +249,10 @@ mqa_prefill_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
     if (start && threadIdx.x < 32) {
         // a start that is negative or leaves too little room is flagged once (its rows are zeros, or the memory is cut at m_max)
         bool bad = false;
-        for (int i = blockIdx.x * 32 + threadIdx.x; i < sh.b; i += gridDim.x * 32) bad = bad || start[i] < 0 || start[i] > sh.m_max - sh.n;
+        for (int i = blockIdx.x * 32 + threadIdx.x; i < sh.b; i += gridDim.x * 32) {
+            const int first = start[i];
+            bad = bad || first < 0 || first > sh.m_max - sh.n;
+        }
         if (bad && status) atomicOr(status, kStatusLenClamped);
     }
 

@@ -341,7 +341,7 @@ project_out_kernel(const __grid_constant__ CUtensorMap map_po, const float* __re
             for (int k = 0; k < NB / kProjWorkWarps; ++k) {
                 const int n = warp + k * kProjWorkWarps;
                 v[k] = make_float4(0.f, 0.f, 0.f, 0.f);
-                if (row0 + n < b) v[k] = *reinterpret_cast<const float4*>(o + ((size_t)(row0 + n) * h + head0 + i) * kHeadDim + lane * 4);
+                if (row0 + n < b) v[k] = __ldcg(reinterpret_cast<const float4*>(o + ((size_t)(row0 + n) * h + head0 + i) * kHeadDim + lane * 4));
             }
             if (i >= S && ok) ok = mbar_wait(empty_s + st * 8, ((i / S) - 1) & 1);   // the product that read this tile is done
             const uint32_t o_s = stages_s + st * Cfg::kStageBytes + kProjChunkBytes + (lane >> 4) * (Cfg::kActBytes / 2) + (lane & 1) * 8;

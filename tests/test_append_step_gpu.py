@@ -256,3 +256,36 @@ def test_logits_of_minus_infinity_weigh_nothing_with_many_query_rows(b, h, m_max
         assert int(status.item()) == 0
         ref = torch.softmax(inp["q"].double() @ K.double().transpose(1, 2), -1) @ inp["V"].double()    # (the new row is in K and V by now)
         check_close(o.cpu().numpy(), ref.cpu().numpy(), f"rows {rows}")
+
+
+@pytest.mark.parametrize("b,h,m_max", [
+    (70, 8, 128), (40, 16, 1000), (8, 32, 600),        # fixed splits: one, and several
+    (64, 40, 300), (9, 100, 2000),                     # many rows: one split, several
+    (40, 16, 1500), (300, 8, 1024),                    # the streaming kernel
+])
+def test_a_loop_of_steps_back_to_back_equals_steps_one_at_a_time(b, h, m_max):
+    """60 tokens, each step behind the one before with nothing waited for, its inputs put into the same buffers; 32
+    sequences' lengths share a line of memory and every step moves them all.  The caches and lengths are the same, o to the last bit."""
+    steps = 60
+    inp = wl.make_inputs(b, h, m_max, "mqa", seed=b + m_max, device=DEV)
+    gen = torch.Generator(device=DEV).manual_seed(h)
+    q, kn, vn = (wl.bf16_normal((steps, *s), std, gen, DEV) for s, std in (((b, h, 128), 128 ** -0.5), ((b, 128), 1.0), ((b, 128), 1.0)))
+    lens0 = torch.from_numpy(np.random.default_rng(b).integers(0, m_max - steps // 2, size=b).astype(np.int32)).to(DEV)
+    results = []
+    for apart in (False, True):
+        K, V, lens = inp["K"].clone(), inp["V"].clone(), lens0.clone()
+        ws, status = mqa.alloc_workspace(b, h, m_max, DEV), torch.zeros(1, dtype=torch.int32, device=DEV)
+        o = torch.full((steps, b, h, 128), float("nan"), dtype=torch.float32, device=DEV)
+        qb, kb, vb = q[0].clone(), kn[0].clone(), vn[0].clone()
+        torch.cuda.synchronize()
+        for t in range(steps):
+            for buf, src in ((qb, q), (kb, kn), (vb, vn)):
+                buf.copy_(src[t])
+            mqa.mqa_decode_append_step(qb, K, V, kb, vb, lens, o[t], ws, status, chained=not apart and t > 0)
+            if apart:
+                torch.cuda.synchronize()
+        torch.cuda.synchronize()
+        results.append((o, K, V, lens, status))
+    for name, x, y in zip(("o", "K", "V", "lens", "status"), *results):
+        assert torch.equal(x.view(torch.uint8), y.view(torch.uint8)), name
+    assert bool(torch.isfinite(results[0][0]).all())
