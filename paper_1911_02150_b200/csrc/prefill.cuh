@@ -116,7 +116,7 @@ __device__ __forceinline__ PfItem pf_item(int item, const int32_t* start, const 
     it.seq = (item / sh.group) % sh.b;
     const int unit = sh.n_units - 1 - (item / (sh.group * sh.b) * sh.group + item % sh.group);
     it.n_act = unit < 0 ? 0 : min(2, sh.n_tiles - 2 * unit);     // (the last group may be partly filled)
-    it.raw = start ? min(start[it.seq], sh.m_max) : 0;
+    it.raw = start ? min(__ldcg(start + it.seq), sh.m_max) : 0;
     it.tile0 = 2 * unit;
     // rows of the memory the unit's last position sees (rows of a tile past the last position or head are computed on
     // whatever the Q tile holds there and never stored); a memory that would pass m_max is cut there
@@ -250,7 +250,7 @@ mqa_prefill_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
         // a start that is negative or leaves too little room is flagged once (its rows are zeros, or the memory is cut at m_max)
         bool bad = false;
         for (int i = blockIdx.x * 32 + threadIdx.x; i < sh.b; i += gridDim.x * 32) {
-            const int first = start[i];
+            const int first = __ldcg(start + i);
             bad = bad || first < 0 || first > sh.m_max - sh.n;
         }
         if (bad && status) atomicOr(status, kStatusLenClamped);
