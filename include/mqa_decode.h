@@ -158,7 +158,7 @@ int mha_decode_step(const void* q, const void* K, const void* V, const int32_t* 
  *                     while the kernel before it is still finishing, and reads q, the new rows, lens
  *                     and the workspace only after that kernel has completed.  What it fetches early
  *                     goes by lens as it reads then; should lens have moved by the time it may rely on
- *                     it, it fetches again.
+ *                     it, it fetches again, or lets what it fetched too much land and ignores it.
  *                     MQA_STEP_TEST_WRONG_GUESS (4), for tests, with MQA_STEP_CHAINED: the early fetch is
  *                     deliberately the wrong one, so that this recovery runs; results are unchanged.
  *                     MQA_STEP_TEST_WITHHOLD_COPY (8), for tests: one on-chip copy of the first CTA is never

@@ -476,7 +476,7 @@ int launch_status() { return cudaGetLastError() == cudaSuccess ? MQA_OK : MQA_ER
 template <int EARLY = 0>
 int launch_wide(const Plan& p, const void* q, const void* K, const void* V, const int32_t* lens, float* o, float2* part_ml,
                 float* part_acc, int32_t* status, int b, int h, int m_max, cudaStream_t stream, int len_bias,
-                const void* k_new = nullptr, const void* v_new = nullptr, int32_t* lens_advance = nullptr, bool withhold = false) {
+                const void* k_new = nullptr, const void* v_new = nullptr, int32_t* lens_advance = nullptr, int mode = 0) {
     FusedArgs fa = {};
     if (k_new) {
         fa.k_new = static_cast<const uint4*>(k_new);
@@ -501,7 +501,7 @@ int launch_wide(const Plan& p, const void* q, const void* K, const void* V, cons
     launch_dependent_2d(mqa_decode_wide_kernel<EARLY>, (unsigned)((size_t)b * p.n_splits), (unsigned)((h + kWideRows - 1) / kWideRows),
                         (unsigned)kWideThreads, (size_t)kWideSmemBytes, stream, static_cast<const uint4*>(q),
                      map_k, map_v, lens, o, part_ml, part_acc, status, h, m_max, p.chunk_rows, p.n_splits, len_bias, fa, lens_advance,
-                     withhold ? 1 : 0);
+                     mode);
     return launch_status();
 }
 
@@ -833,6 +833,9 @@ static int append_step_impl(const void* q, void* K, void* V, const void* k_new, 
         if (rc) return rc;
         return run_combine(true, lens, o, workspace, workspace_bytes, b, h, m_max, k, v, stream, 0, advance ? lens : nullptr);
     }
+    // what the fixed-split and the many-rows kernel fetch ahead of the wait (their EARLY), and the testing flags
+    const int ahead = early >= kEarlyChained ? 1 : early == kEarlyAfterProjection ? 2 : 0;
+    const int mode = (withhold ? kMmaWithhold : 0) | (early == kEarlyChainedWrongGuess ? kMmaWrongGuess : 0);
     // other plans: the same step as separate launches.  Without `advance` the append leaves lens alone and
     // the step is told that a sequence which took a row has one more row than lens says.
     if (p.kernel == Kernel::kWide) {
@@ -842,10 +845,9 @@ static int append_step_impl(const void* q, void* K, void* V, const void* k_new, 
         float* part_acc = partials_acc(p, workspace);
         // (one split and one tile of 128 rows: the CTA moves lens on itself)
         const bool alone = p.n_splits == 1 && h <= kWideRows;
-        const int ahead = withhold ? 0 : early == kEarlyChained ? 1 : early == kEarlyAfterProjection ? 2 : 0;
         auto launch = ahead == 1 ? launch_wide<1> : ahead == 2 ? launch_wide<2> : launch_wide<0>;
         rc = launch(p, q, K, V, lens, o, part_ml, part_acc, status, b, h, m_max, stream, 0, k_new, v_new,
-                    alone && advance ? lens : nullptr, withhold);
+                    alone && advance ? lens : nullptr, mode);
         if (rc || alone) return rc;
         if (p.n_splits == 1) {                                   // several row tiles read lens: moved on by a kernel of its own
             if (advance) launch_dependent(lens_advance_kernel, (unsigned)((b + 255) / 256), 256u, 0, stream, lens, b, m_max);
@@ -862,8 +864,7 @@ static int append_step_impl(const void* q, void* K, void* V, const void* k_new, 
         float* part_acc = alone ? nullptr : partials_acc(p, workspace);
         int32_t* move_lens = alone && advance ? lens : nullptr;
 #define MQA_MMA_STEP(TILES, EARLY) \
-    launch_mma<TILES, EARLY>(p, q, K, V, lens, o, part_ml, part_acc, status, b, h, m_max, stream, 0, k_new, v_new, move_lens, withhold ? kMmaWithhold : 0)
-        const int ahead = withhold ? 0 : early == kEarlyChained ? 1 : early == kEarlyAfterProjection ? 2 : 0;
+    launch_mma<TILES, EARLY>(p, q, K, V, lens, o, part_ml, part_acc, status, b, h, m_max, stream, 0, k_new, v_new, move_lens, mode)
         if (p.kernel == Kernel::kMma1)
             rc = ahead == 1 ? MQA_MMA_STEP(1, 1) : ahead == 2 ? MQA_MMA_STEP(1, 2) : MQA_MMA_STEP(1, 0);
         else

@@ -50,7 +50,7 @@ constexpr uint32_t kWaitRounds = 1u << 24;             // ... or after this many
 // The limit in force, in SM clock cycles (mqa_set_wait_limit_cycles: a test shortens it to see a wait run out).
 __device__ long long g_wait_limit_cycles = kWaitLimitCycles;
 constexpr int kSingleRoundingMinRows = 1024;            // prefixes this long feed P to the tensor cores in one bf16 rounding
-constexpr int kMmaWithhold = 2, kMmaRing = 4;           // bits of the fixed-split kernel's `mode`
+constexpr int kMmaWithhold = 2, kMmaRing = 4, kMmaWrongGuess = 8;     // bits of the fixed-split kernel's `mode` (and of the many-rows kernel's)
 constexpr int kStreamMaxSeqs = 1024;                   // sequences the persistent kernel can index in shared memory
 
 // Ring depth must be a multiple of kRowWarps: tile i lives in stage i % kStages and belongs to
@@ -431,7 +431,8 @@ mqa_decode_split_mma_kernel(const __grid_constant__ CUtensorMap map_k, const __g
     if (EARLY == 1 && producer) {
         // the rest of the rows there can be (lens is at most one more than it was, and takes a row): a surplus tile is left to
         // land and ignored
-        const int rows = min(min(max(guess, 0) + 2, m_max) - r0, chunk_rows);
+        // (for tests, MQA_STEP_TEST_WRONG_GUESS: four tiles more than there can be)
+        const int rows = min(min(max(guess, 0) + 2 + ((mode & kMmaWrongGuess) != 0 ? 4 * kTileRows : 0), m_max) - r0, chunk_rows);
         const int most = max(pre, min((rows + kTileRows - 1) / kTileRows, kStages));
         for (; pre < most; ++pre) issue_tile(pre);
     }

@@ -49,7 +49,7 @@ mqa_decode_wide_kernel(const uint4* __restrict__ q, const __grid_constant__ CUte
                        const __grid_constant__ CUtensorMap map_v, const int32_t* __restrict__ lens, float* __restrict__ o,
                        float2* __restrict__ part_ml, float* __restrict__ part_acc, int32_t* __restrict__ status, int h,
                        int m_max, int chunk_rows, int n_splits, int len_bias, const FusedArgs fa, int32_t* __restrict__ lens_advance,
-                       int withhold) {
+                       int mode) {
     const int warp = __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0), lane = threadIdx.x & 31;
     const int seq = blockIdx.x / n_splits, split = blockIdx.x % n_splits;
     const int row0 = blockIdx.y * kWideRows;                   // this CTA's first query row of the sequence (more than 128: grid.y tiles)
@@ -101,7 +101,7 @@ mqa_decode_wide_kernel(const uint4* __restrict__ q, const __grid_constant__ CUte
         mbar_expect_tx(v_full + 8 * vs, kPfTileBytes);
         tma_load_2d_hint(v_ring + vs * kPfTileBytes, &map_v, 0, y, v_full + 8 * vs, policy);
         // (for tests: one copy of the first CTA's second stage is never started, so that a wait runs out)
-        if (!(withhold && blockIdx.x == 0 && blockIdx.y == 0 && j == 1))
+        if (!((mode & kMmaWithhold) != 0 && blockIdx.x == 0 && blockIdx.y == 0 && j == 1))
             tma_load_2d_hint(v_ring + vs * kPfTileBytes + kPfHalfBytes, &map_v, kBoxCols, y, v_full + 8 * vs, policy);
     };
     int pre = 0, guess = 0;                                    // stages asked for so far (by the producer's thread)
@@ -115,8 +115,8 @@ mqa_decode_wide_kernel(const uint4* __restrict__ q, const __grid_constant__ CUte
 
     grid_dependency_wait();              // q, lens and the newest cache row may come from the kernel before
     grid_launch_dependents();
-    if (EARLY == 1 && producer) {        // the rows that the prefix has in any case
-        const int rows = min(min(guess + 1, m_max) - r0, chunk_rows);
+    if (EARLY == 1 && producer) {        // the rows that the prefix has in any case (for tests, MQA_STEP_TEST_WRONG_GUESS: a stage more)
+        const int rows = min(min(guess + 1 + ((mode & kMmaWrongGuess) != 0 ? kWideRows : 0), m_max) - r0, chunk_rows);
         const int sure = max(pre, min((rows + kWideRows - 1) / kWideRows, kAhead));
         for (; pre < sure; ++pre) { issue_k(pre); issue_v(pre); }
     }

@@ -30,6 +30,8 @@ def check_close(got, ref, what):
     (6, 8, 300, False),         # fixed-split kernel, one CTA per sequence
     (20, 96, 2048, False),      # many query rows: the kernel with the query rows as tile rows, pieces and a second pass
     (160, 40, 700, False),      # the same kernel, one split per sequence
+    (20, 96, 2048, True), (160, 40, 700, True),                 # ... with a stage fetched ahead of the wait
+    (6, 8, 300, True), (8, 24, 1000, True), (8, 24, 1000, False),   # fixed splits, one and several, with tiles ahead of it and without
 ])
 def test_a_wait_that_runs_out_is_reported_and_leaves_nothing_behind(b, h, m_max, chained):
     inp = wl.make_inputs(b, h, m_max, "mqa", seed=77, device=DEV)
@@ -64,6 +66,39 @@ def test_a_wait_that_runs_out_is_reported_and_leaves_nothing_behind(b, h, m_max,
         assert np.array_equal(lens.cpu().numpy(), lens_h)
         check_close(o.cpu().numpy(), ref, f"call {rnd} after the timed-out one")
     assert np.array_equal(wl.bits(inp["K"]), Kh) and np.array_equal(wl.bits(inp["V"]), Vh)
+
+
+@pytest.mark.parametrize("b,h,m_max", [(6, 8, 300), (8, 24, 1000), (20, 96, 2048), (160, 40, 700)])
+def test_copies_ahead_of_the_wait_behind_the_host_inputs_that_run_out(b, h, m_max):
+    """The same flag through the host-buffer step, where the attention kernel fetches all that its stages hold before its wait."""
+    inp = wl.make_inputs(b, h, m_max, "mqa", seed=78, device=DEV)
+    lens0 = np.full(b, m_max - 1, np.int32)
+    Kh, Vh, lens_h = wl.bits(inp["K"]).copy(), wl.bits(inp["V"]).copy(), lens0.copy()
+    oracle.kv_cache_append(Kh, Vh, wl.bits(inp["k_new"]), wl.bits(inp["v_new"]), lens_h, True)
+    ref = oracle.mqa_decode_step(wl.bits(inp["q"]), Kh, Vh, lens_h)
+    lens = torch.from_numpy(lens0).to(DEV)
+    status = torch.zeros(1, dtype=torch.int32, device=DEV)
+    host = [inp[n].cpu().pin_memory() for n in ("q", "k_new", "v_new")]
+    o = torch.zeros(b, h, 128, dtype=torch.float32).pin_memory()
+    staging = torch.empty(mqa.host_staging_bytes(b, h), dtype=torch.uint8, device=DEV)
+    ws = mqa.alloc_workspace(b, h, m_max, DEV)
+    args = list(binding._host_step_args(*host, o, inp["K"], inp["V"], lens, staging, ws, status, False, None, False))
+    flags = 7                                        # (the position of `advance` in mqa_decode_append_step_host)
+    assert args[flags] == 0
+    args[flags] = binding.STEP_TEST_WITHHOLD_COPY
+    try:
+        mqa.set_wait_limit_cycles(SHORT_LIMIT)
+        assert binding.lib().mqa_decode_append_step_host(*args) == 0
+        torch.cuda.synchronize()
+    finally:
+        mqa.set_wait_limit_cycles(0)
+    assert int(status.item()) & binding.STATUS_PIPELINE_TIMEOUT
+    status.zero_()
+    o.fill_(float("nan"))
+    mqa.mqa_decode_append_step_host(*host, o, inp["K"], inp["V"], lens, staging, ws, status, advance=True)
+    torch.cuda.synchronize()
+    assert int(status.item()) == 0 and np.array_equal(lens.cpu().numpy(), lens_h)
+    check_close(o.numpy(), ref, "the call after the timed-out one")
 
 
 def test_the_batched_form_reports_a_wait_that_runs_out_and_is_correct_again_afterwards():
