@@ -46,6 +46,7 @@ mqa_decode_local_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
     }
     __syncwarp();
+    const bool withhold = seq == 0 && test_withhold();       // for tests: one copy of sequence 0's second tile is never started
     grid_dependency_wait();          // pos, q, the rings and the new row may come from the kernel before
     grid_launch_dependents();
     if (seq >= b) return;            // (the whole warp: nothing is in flight)
@@ -60,7 +61,7 @@ mqa_decode_local_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_
             tma_load_2d(dst, &map_k, 0, y, bar);
             tma_load_2d(dst + kBoxBytes, &map_k, kBoxCols, y, bar);
             tma_load_2d(dst + 2 * kBoxBytes, &map_v, 0, y, bar);
-            tma_load_2d(dst + 3 * kBoxBytes, &map_v, kBoxCols, y, bar);
+            if (!(withhold && i == 1)) tma_load_2d(dst + 3 * kBoxBytes, &map_v, kBoxCols, y, bar);
         }
     };
     // the first tile, the new row's pieces (lanes 0-15 the key row, 16-31 the value row), q and pos are in flight together

@@ -49,6 +49,9 @@ constexpr long long kWaitLimitCycles = 2000000000ll;   // every mbarrier wait gi
 constexpr uint32_t kWaitRounds = 1u << 24;             // ... or after this many polling rounds
 // The limit in force, in SM clock cycles (mqa_set_wait_limit_cycles: a test shortens it to see a wait run out).
 __device__ long long g_wait_limit_cycles = kWaitLimitCycles;
+// For tests (mqa_set_test_withhold_copy): when non-zero, the kernels of the calls that take no flags never start one copy.
+__device__ int g_test_withhold = 0;
+__device__ __forceinline__ bool test_withhold() { return *reinterpret_cast<volatile int*>(&g_test_withhold) != 0; }
 constexpr int kSingleRoundingMinRows = 1024;            // prefixes this long feed P to the tensor cores in one bf16 rounding
 constexpr int kMmaWithhold = 2, kMmaRing = 4, kMmaWrongGuess = 8;     // bits of the fixed-split kernel's `mode` (and of the many-rows kernel's)
 constexpr int kStreamMaxSeqs = 1024;                   // sequences the persistent kernel can index in shared memory

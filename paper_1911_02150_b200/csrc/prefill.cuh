@@ -79,10 +79,6 @@ __device__ __forceinline__ float max3(float a, float b, float c) {
     return d;
 }
 
-// For tests (mqa_set_test_withhold_copy): when non-zero, CTA 0 never starts one copy of the second stage of its first
-// unit, so that a bounded wait runs out.
-__device__ int g_test_withhold = 0;
-
 // A tile is `positions` consecutive positions of `heads` consecutive heads, positions * heads <= 128 rows: row r is position
 // r % positions of head r / positions (one box of Q as a [b h][n][128] tensor).  A sequence's tiles are numbered position
 // block by position block, the heads' blocks within it, and a unit of work is two tiles in a row.  Units go out in groups of
@@ -264,7 +260,8 @@ mqa_prefill_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
             bool ok = true;
             int g = 0, qi = 0;                                   // stages and units so far (they number the barriers' phases)
             int issued_k = 0, issued_v = 0, issued_q = 0;
-            const bool withhold = blockIdx.x == 0 && *reinterpret_cast<volatile int*>(&g_test_withhold) != 0;
+            // (for tests: CTA 0 never starts one copy of the second stage of its first unit)
+            const bool withhold = blockIdx.x == 0 && test_withhold();
             for (int round = 0, item; (item = pf_unit(round)) < n_items && ok; ++round) {
                 const PfItem it = pf_item(item, start, sh);
                 const int first = first_stage(it.n_kv), n_kv = count_stages(it.n_kv);

@@ -171,6 +171,8 @@ project_in_kernel(const __grid_constant__ CUtensorMap map_pq, const __grid_const
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem = tmem_slot;
+    // for tests: the first CTA keeps its sums to itself, so that the others of its cluster wait for them in vain
+    const bool withhold = blockIdx.x == 0 && part == 0 && row0 == 0 && test_withhold();
     if (parts > 1) cluster_sync();   // every CTA's barrier is in place
     grid_dependency_wait();          // x may come from the kernel before this one
     grid_launch_dependents();
@@ -226,7 +228,7 @@ project_in_kernel(const __grid_constant__ CUtensorMap map_pq, const __grid_const
     }
     __syncthreads();
     if (parts > 1) {
-        if (warp == 0) shares.send(stages_s, recv_s, recv_bar, lane);
+        if (warp == 0 && !withhold) shares.send(stages_s, recv_s, recv_bar, lane);
         if (!mbar_wait(recv_bar, 0)) { if (status && lane == 0) atomicOr(status, kStatusPipelineTimeout); mbar_wait(recv_bar, 0); }
         cluster_arrive();            // what the others send has landed
     }
@@ -293,6 +295,7 @@ project_out_kernel(const __grid_constant__ CUtensorMap map_po, const float* __re
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem = tmem_slot;
+    const bool withhold = tile == 0 && group == 0 && row0 == 0 && test_withhold();     // (as in project_in_kernel)
     cluster_sync();                  // every CTA's barrier is in place
     grid_dependency_wait();          // o comes from the kernel before this one
     grid_launch_dependents();
@@ -369,7 +372,7 @@ project_out_kernel(const __grid_constant__ CUtensorMap map_po, const float* __re
         if (status) atomicOr(status, kStatusPipelineTimeout);
     }
     __syncthreads();
-    if (warp == 0) shares.send(stages_s, recv_s, recv_bar, lane);
+    if (warp == 0 && !withhold) shares.send(stages_s, recv_s, recv_bar, lane);
     if (!mbar_wait(recv_bar, 0)) { if (status && lane == 0) atomicOr(status, kStatusPipelineTimeout); mbar_wait(recv_bar, 0); }
     cluster_arrive();                // what the others send has landed
     for (int i = warp; i < shares.count(group); i += kProjThreads / 32)

@@ -101,13 +101,17 @@ def test_copies_ahead_of_the_wait_behind_the_host_inputs_that_run_out(b, h, m_ma
     check_close(o.numpy(), ref, "the call after the timed-out one")
 
 
-def test_the_batched_form_reports_a_wait_that_runs_out_and_is_correct_again_afterwards():
-    b, h, n, m_max = 3, 4, 512, 600
+@pytest.mark.parametrize("b,h,n,m_max,starts", [
+    (3, 4, 512, 600, [88, 0, 31]),              # one CTA per unit
+    (1, 4, 16, 2064, [2048]),                   # a cluster of CTAs per unit: the others go on to the merge
+    (5, 9, 333, 3000, [2667, 0, 100, 1300, 700]),
+])
+def test_the_batched_form_reports_a_wait_that_runs_out_and_is_correct_again_afterwards(b, h, n, m_max, starts):
     gen = torch.Generator(device=DEV).manual_seed(4)
     Q = wl.bf16_normal((b, h, n, 128), 128 ** -0.5, gen, DEV)
     K = wl.bf16_normal((b, m_max, 128), 1.0, gen, DEV)
     V = wl.bf16_normal((b, m_max, 128), 1.0, gen, DEV)
-    st = np.array([88, 0, 31], np.int32)
+    st = np.array(starts, np.int32)
     start = torch.from_numpy(st).to(DEV)
     O = torch.zeros(b, h, n, 128, dtype=torch.float32, device=DEV)
     ws = torch.empty(max(16, mqa.prefill_workspace_bytes(b, h, n, m_max)), dtype=torch.uint8, device=DEV)
@@ -128,3 +132,56 @@ def test_the_batched_form_reports_a_wait_that_runs_out_and_is_correct_again_afte
     assert int(status.item()) == 0
     ref = oracle.mqa_batched_attention(wl.bits(Q), wl.bits(K), wl.bits(V), st)
     check_close(O.cpu().numpy(), ref, "the call after the timed-out one")
+
+
+@pytest.mark.parametrize("b,h,window", [(320, 8, 100), (310, 20, 33), (150, 40, 32)])
+def test_the_local_step_reports_a_wait_that_runs_out(b, h, window):
+    """A warp per sequence, the copy of its second tile (or of its second pass over the only one) never complete."""
+    inp = wl.make_inputs(b, h, window, "mqa", seed=5, device=DEV)
+    pos0 = np.full(b, window + 3, np.int32)
+    pos = torch.from_numpy(pos0).to(DEV)
+    o = torch.zeros(b, h, 128, dtype=torch.float32, device=DEV)
+    status = torch.zeros(1, dtype=torch.int32, device=DEV)
+    step = lambda: mqa.mqa_decode_local_step(inp["q"], inp["K"], inp["V"], inp["k_new"], inp["v_new"], pos, o, status)
+    try:
+        mqa.set_wait_limit_cycles(SHORT_LIMIT)
+        mqa.set_test_withhold_copy(True)
+        step()
+        torch.cuda.synchronize()                     # the kernel came back by itself
+    finally:
+        mqa.set_test_withhold_copy(False)
+        mqa.set_wait_limit_cycles(0)
+    assert int(status.item()) == binding.STATUS_PIPELINE_TIMEOUT
+    assert np.array_equal(pos.cpu().numpy(), pos0 + (np.arange(b) > 0))          # (the sequence that gave up stays where it was)
+    status.zero_()
+    pos.copy_(torch.from_numpy(pos0))
+    step()
+    torch.cuda.synchronize()
+    assert int(status.item()) == 0
+    check_close(o.cpu().numpy(), oracle.mqa_decode_step(wl.bits(inp["q"]), wl.bits(inp["K"]), wl.bits(inp["V"]), np.full(b, window, np.int32)), "the call after it")
+
+
+@pytest.mark.parametrize("b,h,d,m_max", [(17, 5, 640, 130), (128, 8, 1024, 64), (3, 1, 1024, 130)])
+def test_the_projections_report_sums_that_do_not_come(b, h, d, m_max):
+    gen = torch.Generator(device=DEV).manual_seed(b)
+    x, P_q, P_k, P_v, P_o, K, V = (wl.bf16_normal(s, std, gen, DEV) for s, std in (
+        ((b, d), 1.0), ((h, d, 128), (d * 128) ** -0.5), ((d, 128), d ** -0.5), ((d, 128), d ** -0.5), ((h, d, 128), (h * 128) ** -0.5),
+        ((b, m_max, 128), 1.0), ((b, m_max, 128), 1.0)))
+    lens = torch.full((b,), m_max // 2, dtype=torch.int32, device=DEV)
+    ws, status = mqa.alloc_layer_workspace(b, h, d, m_max, DEV), torch.zeros(1, dtype=torch.int32, device=DEV)
+    results = []
+    for withhold in (False, True, False):
+        y = torch.full((b, d), float("nan"), dtype=torch.float32, device=DEV)
+        status.zero_()
+        try:
+            if withhold:
+                mqa.set_wait_limit_cycles(SHORT_LIMIT)
+                mqa.set_test_withhold_copy(True)
+            mqa.mqa_layer_decode_step(x, P_q, P_k, P_v, P_o, K, V, lens, y, ws, status, advance=False)
+            torch.cuda.synchronize()                 # every kernel came back by itself
+        finally:
+            mqa.set_test_withhold_copy(False)
+            mqa.set_wait_limit_cycles(0)
+        assert int(status.item()) == (binding.STATUS_PIPELINE_TIMEOUT if withhold else 0)
+        results.append(y)
+    assert bool(torch.isfinite(results[0]).all()) and torch.equal(results[0], results[2])
