@@ -104,6 +104,19 @@ def test_new_row_at_the_edges_of_tiles_and_splits(h, m_max, chained):
     run(len(lens), h, m_max, lens, True, seed=h + m_max, chained=chained)
 
 
+@pytest.mark.parametrize("chained", [False, True, "wrong-guess"])
+@pytest.mark.parametrize("h,m_max", [(40, 700), (96, 2600), (130, 1500), (33, 260)])
+def test_new_row_at_the_edges_of_stages_and_splits_with_many_query_rows(h, m_max, chained):
+    """The many-rows kernel does so in stages of 128 rows: rows either side of every edge of a stage and of a split, with one row
+    tile and two, several splits and one."""
+    chunk = mqa.plan_splits(True, 32, h, m_max)[1]
+    edges = {0, 128, 256, m_max, *(chunk * i for i in range(1, 5)), chunk + 128}
+    lens = sorted({min(m_max - 1, max(0, e + x)) for e in edges for x in (-2, -1, 0, 1)})[:32]
+    lens = (lens + [m_max - 1] * 32)[:32]
+    assert mqa.plan_splits(True, len(lens), h, m_max)[1] == chunk
+    run(len(lens), h, m_max, lens, True, seed=h + m_max, chained=chained)
+
+
 def test_append_step_full_and_negative_sequences_take_no_row():
     b, h, m_max = 48, 16, 1024
     lens = lens_mix(b, m_max, seed=5)
