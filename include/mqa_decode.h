@@ -334,6 +334,13 @@ int mqa_layer_decode_step(const void* x, const void* P_q, const void* P_k, const
 size_t mqa_layer_workspace_bytes(int b, int h, int d, int m_max, int k, int v);
 
 /*
+ * mqa_layer_cut -- how mqa_layer_decode_step cuts its projections up for these sizes on the current device: cut[0], cut[2] the batch
+ * columns of a tile (16, 32, 64 or 128) and cut[1], cut[3] the CTAs that share a product's depth, going in and coming out.
+ * Informational; host-only.
+ */
+int mqa_layer_cut(int b, int h, int d, int cut[4]);
+
+/*
  * mqa_prefill_attention -- the three attention lines of the batched multi-query function of Section 3
  * (MultiqueryAttentionBatched: logits = einsum(bhnk,bmk->bhnm), weights = softmax(logits + mask),
  * O = einsum(bhnm,bmv->bhnv)) for n query positions per sequence at once, under the mask that Section 2.3

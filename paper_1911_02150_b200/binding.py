@@ -27,7 +27,7 @@ EXPORTS = (
     "mha_decode_step_split", "mha_decode_step_combine",
     "mqa_workspace_bytes", "mqa_plan_splits", "mqa_plan_kernel_name", "mqa_set_wait_limit_cycles", "mqa_set_test_withhold_copy", "mqa_prefill_attention", "mqa_prefill_workspace_bytes", "mqa_status_string", "mqa_decode_step_noalloc",
     "mqa_decode_append_step", "mqa_append_step_launches",
-    "mqa_layer_decode_step", "mqa_layer_workspace_bytes", "mqa_decode_local_step",
+    "mqa_layer_decode_step", "mqa_layer_workspace_bytes", "mqa_layer_cut", "mqa_decode_local_step",
     "mqa_decode_append_step_host", "mqa_host_staging_bytes",
 )
 
@@ -76,6 +76,8 @@ def lib() -> ctypes.CDLL:
         L.mqa_host_staging_bytes.restype = sz
         L.mqa_layer_workspace_bytes.argtypes = [I, I, I, I, I, I]
         L.mqa_layer_workspace_bytes.restype = sz
+        L.mqa_layer_cut.argtypes = [I, I, I, ctypes.POINTER(I)]
+        L.mqa_layer_cut.restype = I
         L.mqa_workspace_bytes.argtypes = [I, I, I, I, I]
         L.mqa_workspace_bytes.restype = sz
         L.mqa_plan_splits.argtypes = [I, I, I, I, I, I, ctypes.POINTER(I)]
@@ -354,6 +356,13 @@ class AppendStep:
 
 def layer_workspace_bytes(b: int, h: int, d: int, m_max: int, k: int = 128, v: int = 128) -> int:
     return int(lib().mqa_layer_workspace_bytes(b, h, d, m_max, k, v))
+
+
+def layer_cut(b: int, h: int, d: int):
+    """(batch columns of a tile, CTAs that share the depth) of the layer step's input projection and of its output projection."""
+    cut = (ctypes.c_int * 4)()
+    _check(lib().mqa_layer_cut(b, h, d, cut), "mqa_layer_cut")
+    return (cut[0], cut[1]), (cut[2], cut[3])
 
 
 def alloc_layer_workspace(b: int, h: int, d: int, m_max: int, device) -> torch.Tensor:

@@ -658,8 +658,8 @@ int launch_projections_in(const void* x, const void* P_q, const void* P_k, const
 // product (the chunks of d rows of an input slab; the heads of an output tile).  By a model of a CTA's chain, in microseconds: its
 // activations (act_kb per batch column and chunk) at 60 KB/us, step_us per chunk (an output tile's chunk is a round trip for o), 0.4
 // per chunk of weights beyond those fetched ahead of the wait, and what the cluster exchanges, which is slow (SM to SM about
-// 24 KB/us per CTA).  Only cuts whose CTAs fit the SMs at once, in clusters
-// that fit the GPCs (of 8: about half of the SMs), count; the input projection keeps to about half of the SMs, where the attention kernel behind it
+// 24 KB/us per CTA).  A cut whose CTAs do not fit the SMs at once, or whose clusters do not fit the GPCs (of 8: about half of the
+// SMs), is charged by its number of waves, total / most_ctas + 0.5; the input projection has about half of the SMs, where the attention kernel behind it
 // does not yet set itself up.  Measured, us per layer step, one fixed cut (128 columns; 16 heads' groups) against this one:
 // 128 x 8 heads x 1024 18.4 / 15.4; 200 x 16 x 1536 47.6 / 28.8; 256 x 8 x 2048 38.8 / 23.4; 8 x 32 x 2048 25.6 / 19.2; 1 x 16 x 2048 23.4 / 18.3.
 struct ProjectionCut { int nb, ctas; };
@@ -680,6 +680,9 @@ ProjectionCut projection_cut(int b, int columns, int depth, double act_kb, doubl
     }
     return best;
 }
+
+ProjectionCut input_cut(int b, int h, int d) { return projection_cut(b, h + 2, d / 128, 0.25, 0.2, sm_count() * 5 / 9); }       // bf16 x
+ProjectionCut output_cut(int b, int h, int d) { return projection_cut(b, d / 128, h, 0.5, 0.45, sm_count() * 8 / 9); }           // fp32 o
 
 // The output projection: the head groups of a (d tile, batch tile) are the CTAs of one thread-block cluster (see
 // project_out_kernel), each with ceil(h / ctas) heads.
@@ -1021,6 +1024,13 @@ size_t mqa_layer_workspace_bytes(int b, int h, int d, int m_max, int k, int v) {
     return layer_workspace(b, h, d, m_max).total;
 }
 
+int mqa_layer_cut(int b, int h, int d, int cut[4]) {
+    if (!cut || !dims_ok(b, h, 1) || d <= 0 || d % 128 != 0) return MQA_ERR_INVALID_ARG;
+    const ProjectionCut in = input_cut(b, h, d), out = output_cut(b, h, d);
+    cut[0] = in.nb; cut[1] = in.ctas; cut[2] = out.nb; cut[3] = out.ctas;
+    return MQA_OK;
+}
+
 int mqa_layer_decode_step(const void* x, const void* P_q, const void* P_k, const void* P_v, const void* P_o, void* K, void* V,
                           int32_t* lens, int advance, float* y, void* workspace, size_t workspace_bytes, int32_t* status,
                           int b, int h, int d, int m_max, int k, int v, mqa_stream_t stream_) {
@@ -1038,9 +1048,7 @@ int mqa_layer_decode_step(const void* x, const void* P_q, const void* P_k, const
     void* k_new = base + w.k_new;
     void* v_new = base + w.v_new;
     float* o = reinterpret_cast<float*>(base + w.o);
-    const int sms = sm_count();
-    const ProjectionCut in = projection_cut(b, h + 2, d / 128, 0.25, 0.2, sms * 5 / 9);        // bf16 x
-    const ProjectionCut out = projection_cut(b, d / 128, h, 0.5, 0.45, sms * 8 / 9);            // fp32 o
+    const ProjectionCut in = input_cut(b, h, d), out = output_cut(b, h, d);
     int rc;
     switch (in.nb) {
         case 16: rc = launch_projections_in<16>(x, P_q, P_k, P_v, q, k_new, v_new, status, b, h, d, in.ctas, stream); break;

@@ -53,6 +53,15 @@ def test_step_flags_are_checked_before_any_launch(L):
     assert rc == binding.ERR_INVALID_ARG
 
 
+def test_layer_cut(L):
+    for b, h, d in ((1, 1, 128), (128, 8, 1024), (256, 128, 2048), (65, 32, 256)):
+        for columns, ctas in binding.layer_cut(b, h, d):
+            assert columns in (16, 32, 64, 128) and ctas in (1, 2, 4, 8)
+    for bad in ((0, 8, 128), (1, 0, 128), (1, 8, 0), (1, 8, 100)):
+        with pytest.raises(binding.MqaError):
+            binding.layer_cut(*bad)
+
+
 def test_status_strings(L):
     seen = {binding.status_string(c) for c in range(0, 5)}
     assert len(seen) == 5

@@ -84,8 +84,8 @@ CASES = [
     (32, 32, 1024, 2048),     # the headline shapes: persistent kernel, one launch for the step
     (40, 16, 512, 1500),
     (8, 8, 256, 300),         # small: fixed-split kernel
-    (130, 8, 384, 1100),      # two batch tiles of 128 (the second nearly empty)
-    (64, 33, 512, 1200),      # an odd head count: the last head group of the output projection holds one head
+    (130, 8, 384, 1100),      # batch tiles whose last one holds two sequences, going in and coming out
+    (64, 33, 512, 1200),      # an odd head count: the last head group of the output projection has fewer heads than the others
 ]
 
 
@@ -102,13 +102,30 @@ def test_layer_step_matches_oracle(b, h, d, m_max):
     (17, 5, 640, 130),        # five chunks and five heads over clusters that do not divide them
     (70, 32, 896, 96),        # a last batch tile partly filled
     (129, 2, 128, 64),        # one chunk of depth; a last batch tile of one sequence
-    (250, 16, 1024, 40),      # batch tiles of 64 and more, clusters of two
+    (250, 16, 1024, 40),      # batch tiles of 128 going in and 64 coming out
     (120, 3, 2048, 33),       # sixteen chunks
+    (28, 40, 256, 900), (28, 130, 128, 300),      # the many-rows kernel behind the projection
 ])
 def test_input_slabs_shared_by_a_cluster(b, h, d, m_max):
     """...and prefixes that end at every place of a tile, for the small steps that fetch their cache rows before the
     projection has finished."""
     lens0 = np.resize(np.array([0, 31, 32, 33, 63, 64, 1, 30, m_max - 1, m_max - 2, m_max]), b).astype(np.int32)
+    run(b, h, d, m_max, lens0, seed=b + d)
+
+
+@pytest.mark.parametrize("b,h,d,m_max,going_in,coming_out", [
+    (33, 24, 640, 100, (64, 2), (64, 8)), (65, 32, 256, 64, (64, 1), (16, 8)),
+    (33, 3, 1664, 100, (64, 8), (16, 2)),         # thirteen chunks of depth over eight CTAs; a last head group of one head
+    (32, 9, 256, 70, (16, 1), (16, 8)),           # five head groups asked of eight CTAs, the last of one head
+    (8, 100, 128, 60, (16, 1), (16, 8)),          # 102 slabs: more CTAs than the input projection's share of the SMs
+    (40, 17, 384, 64, (16, 1), (16, 8)), (70, 32, 896, 96, (128, 2), (128, 8)), (250, 16, 1024, 40, (128, 2), (64, 4)),
+    (120, 3, 2048, 33, (32, 4), (16, 1)), (3, 1, 1024, 130, (16, 8), (16, 1)),
+])
+def test_every_cut_of_the_projections(b, h, d, m_max, going_in, coming_out):
+    """Tiles of 16, 32, 64 and 128 batch columns, one to eight CTAs to a product's depth; the cuts are those of 148 SMs."""
+    if torch.cuda.get_device_properties(0).multi_processor_count == 148:
+        assert mqa.layer_cut(b, h, d) == (going_in, coming_out)
+    lens0 = np.resize(np.array([0, 31, 32, 33, 1, m_max - 1, m_max - 2, m_max]), b).astype(np.int32)
     run(b, h, d, m_max, lens0, seed=b + d)
 
 
