@@ -134,7 +134,7 @@ int mha_decode_step(const void* q, const void* K, const void* V, const int32_t* 
  * (Section 3) in a single call: the new token's key/value row is concatenated to each
  * sequence's cache at row lens[b] (as kv_cache_append does), then the h heads attend over
  * the lens[b] + 1 rows (as mqa_decode_step does).  For batches large enough for the persistent
- * kernel (h <= 64) the whole step is one launch: the CTA that streams a sequence's last tile
+ * kernel (h <= 32) the whole step is one launch: the CTA that streams a sequence's last tile
  * writes the new row before it fetches that tile, the pieces of a sequence are merged by the
  * CTA that finishes the last one, and lens is advanced once every CTA has read it.  Other
  * sizes run the same step as separate launches (mqa_append_step_launches tells how many).

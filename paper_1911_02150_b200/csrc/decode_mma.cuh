@@ -165,8 +165,9 @@ __device__ __forceinline__ void named_barrier_arrive(int id, int threads) {
 }
 
 // The append-and-attend step: the kernel that owns a sequence's last tile also writes the new token's key
-// and value row (row lens[b]) into the cache before it fetches that tile, so the step attends over
-// lens[b] + 1 rows without a separate append launch.
+// and value row (row lens[b]) into the cache, so the step attends over lens[b] + 1 rows without a separate append
+// launch.  The streaming kernel writes it before it fetches that tile; the fixed-split and the many-rows kernel put it
+// into its place in the landed tile and write the cache with nobody waiting for it.
 struct FusedArgs {
     const uint4* k_new;      // [b, 128] bf16 rows as 16-byte words; null = nothing to append
     const uint4* v_new;

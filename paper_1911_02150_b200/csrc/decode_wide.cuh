@@ -5,12 +5,12 @@
 // The streaming kernel (decode_umma.cuh) puts the cache rows on the TMEM lanes and the heads on the columns, which is
 // right for a few heads (N = 16 .. 32) but makes the softmax a cross-thread affair; from 64 query rows on that kernel
 // is bound by its softmax warps, not by HBM.  Here a CTA holds all the sequence's query rows as ONE 128-row Q tile
-// (rows past h belong to the next sequence or read as zero: computed, never stored) and walks a fixed split of the
+// (rows past h are whatever shared memory held: computed, never stored) and walks a fixed split of the
 // sequence's cache rows in stages of 128:
 //     S   = Q K_j^T        tcgen05.mma, M = 128 query rows (TMEM lanes), N = 128 cache rows, fp32 in TMEM
 //     P   = exp2(S log2e - m)   one thread per query row: the row's maximum and sum need no other thread
-//     O  += P V_j          tcgen05.mma with A = P read from TMEM (bf16 pairs written over S), B = V_j (MN-major)
-// The two softmax warpgroups take the stages in turn (warpgroup w: stages w, w + 2, ...), each with an S buffer, an
+//     O  += P V_j          tcgen05.mma with A = P read from TMEM (bf16 pairs in columns of their own), B = V_j (MN-major)
+// The two softmax warpgroups take the stages in turn (warpgroup w: stages w, w + 2, ...), each with weights, an
 // O accumulator, reference maxima and sums of its own -- two partial softmaxes over interleaved rows of the cache,
 // merged exactly at the end (the same recombination as between splits) -- so the logits of a stage are computed and
 // its weights formed while the other warpgroup's stage is multiplied with V.  TMEM: one buffer of logits that the stages
@@ -20,7 +20,9 @@
 // where they are masked by index (select) and their V rows cleared in shared memory.
 //
 // Roles: warps 0-3 and 4-7 the two softmax warpgroups, warp 8 TMA producer, warps 9 and 10 issue the products (warp 11 only
-// completes the third warpgroup, which hands most of its registers to the other two).  Every wait is bounded.
+// completes the third warpgroup, which hands most of its registers to the other two).  The compiler may give a thread 168
+// registers, whatever the softmax warps have in the end, and keeps 2 to 8 values of theirs in local memory (EARLY 0, 1, 2: 32, 8, 20
+// bytes of spills).  Every wait is bounded.
 #pragma once
 #include "prefill.cuh"
 

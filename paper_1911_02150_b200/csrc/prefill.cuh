@@ -43,7 +43,7 @@ constexpr int kPfRows = 128;                                   // query position
 constexpr int kPfTileBytes = kPfRows * kRowBytes;              // 32 KiB: 128 rows x 128 bf16, two 64-column boxes
 constexpr int kPfHalfBytes = kPfTileBytes / 2;
 constexpr int kPfKSlots = 2, kPfVSlots = 2;
-constexpr int kPfThreads = 12 * 32;                            // (warps 10 and 11 only complete the third warpgroup)
+constexpr int kPfThreads = 12 * 32;                            // (warp 11 only completes the third warpgroup)
 constexpr int kPfProducerWarp = 8, kPfSWarp = 9, kPfPvWarp = 10;
 constexpr int kPfRegsSoftmax = 216, kPfRegsOther = 72;
 constexpr int kPfMaxSplit = 8;                                 // CTAs that share a unit's stages
