@@ -30,7 +30,8 @@ constexpr int kCombineEager = 8;
 constexpr int kCombineManyGroups = 5;
 
 // Merge `n` pieces of one (sequence, head).  ml_of(i) / acc_of(i) give piece i's (max, sum) and the address of
-// its 128 accumulators; a piece whose max is -inf is skipped entirely (it may never have been written).
+// its 128 accumulators; a piece whose max is -inf is skipped entirely (its accumulators may never have been written), unless its
+// sum is NaN: then all its logits were, and so is the result.
 template <int kCombineShape, typename MlOf, typename AccOf>
 __device__ __forceinline__ void merge_pieces(int n, MlOf ml_of, AccOf acc_of, float* __restrict__ out) {
     constexpr int kCombineGroups = kCombineShape >= 4 ? 4 : 1;
@@ -54,7 +55,9 @@ __device__ __forceinline__ void merge_pieces(int n, MlOf ml_of, AccOf acc_of, fl
     float top = -INFINITY;
     for (int i = 0; i < n; ++i) top = fmaxf(top, m_s[i]);
     if (top == -INFINITY) {                                // nothing but empty pieces: the empty prefix gives zeros
-        if (g == 0) out[c] = 0.f;
+        float sum = 0.f;                                   // (or NaN, if that is what all the logits were)
+        for (int i = 0; i < n; ++i) sum += l_s[i];
+        if (g == 0) out[c] = sum;
         return;
     }
     float num = 0.f, den = 0.f;
@@ -63,7 +66,7 @@ __device__ __forceinline__ void merge_pieces(int n, MlOf ml_of, AccOf acc_of, fl
         const int i = g + e * kCombineGroups;
         if (i < n) {
             const float w = fast_exp2(m_s[i] - top);
-            if (w != 0.f) { den = fmaf(w, l_s[i], den); num = fmaf(w, a[e], num); }   // never multiply an unwritten slot
+            if (w != 0.f || isnan(l_s[i])) { den = fmaf(w, l_s[i], den); num = fmaf(w, a[e], num); }   // never multiply an unwritten slot
         }
     }
     for (int i0 = g + kCombineEager * kCombineGroups; i0 < n; i0 += kCombineEager * kCombineGroups) {
@@ -77,7 +80,7 @@ __device__ __forceinline__ void merge_pieces(int n, MlOf ml_of, AccOf acc_of, fl
             const int i = i0 + e * kCombineGroups;
             if (i < n) {
                 const float w = fast_exp2(m_s[i] - top);
-                if (w != 0.f) { den = fmaf(w, l_s[i], den); num = fmaf(w, a[e], num); }
+                if (w != 0.f || isnan(l_s[i])) { den = fmaf(w, l_s[i], den); num = fmaf(w, a[e], num); }
             }
         }
     }
@@ -164,14 +167,13 @@ combine_few_kernel(const float2* __restrict__ part_ml, const float* __restrict__
         const int raw = lens_advance[seq];
         if (raw >= 0 && raw < m_max) lens_advance[seq] = raw + 1;
     }
-    float top = -INFINITY;
+    float top = -INFINITY, den = 0.f;                  // (den: 0, or NaN if some piece's sum is)
 #pragma unroll
-    for (int i = 0; i < PIECES; ++i) top = fmaxf(top, ml[i].x);
+    for (int i = 0; i < PIECES; ++i) { top = fmaxf(top, ml[i].x); den = fmaf(0.f, ml[i].y, den); }
     if (live == 0 || top == -INFINITY) {               // the empty prefix, or nothing but empty pieces: zeros
-        *out = make_float4(0.f, 0.f, 0.f, 0.f);
+        *out = make_float4(den, den, den, den);        // (or NaN, if that is what all the logits were)
         return;
     }
-    float den = 0.f;
     float4 num = make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll
     for (int i = 0; i < PIECES; ++i) {

@@ -1116,7 +1116,7 @@ mqa_decode_stream_umma_kernel(const __grid_constant__ CUtensorMap map_k, const _
                     }
 #pragma unroll
                     for (int c = 0; c < 8; ++c) {
-                        if (ml[c0 + c].x == -INFINITY) continue;  // an empty piece (its sums were never written) is skipped, not multiplied
+                        if (ml[c0 + c].x == -INFINITY && ml[c0 + c].y == 0.f) continue;  // an empty piece (its sums were never written) is skipped, not multiplied
                         const float w = fast_exp2(ml[c0 + c].x - top);
                         den = fmaf(w, ml[c0 + c].y, den);
                         num.x = fmaf(w, a[c].x, num.x); num.y = fmaf(w, a[c].y, num.y);

@@ -302,3 +302,31 @@ def test_a_loop_of_steps_back_to_back_equals_steps_one_at_a_time(b, h, m_max):
     for name, x, y in zip(("o", "K", "V", "lens", "status"), *results):
         assert torch.equal(x.view(torch.uint8), y.view(torch.uint8)), name
     assert bool(torch.isfinite(results[0][0]).all())
+
+
+@pytest.mark.parametrize("variant,b,h,m_max", [
+    ("mqa", 70, 8, 128), ("mqa", 40, 16, 1000), ("mqa", 8, 32, 600),            # fixed splits: one, and several
+    ("mqa", 64, 40, 300), ("mqa", 9, 100, 2000), ("mqa", 2, 130, 1500), ("mqa", 1, 16, 20000),   # many rows: one split, several, dozens
+    ("mqa", 40, 16, 1500), ("mqa", 32, 32, 2048), ("mqa", 300, 8, 1024),        # streaming: merged in the kernel, by clusters, mostly whole
+    ("mha", 3, 4, 700), ("mha", 1, 2, 40000),
+])
+def test_a_prefix_whose_rows_are_partly_nan_gives_nan(variant, b, h, m_max):
+    """Whatever pieces the prefix is cut into, and where all the logits of some of them, or of all, are NaN: never a finite
+    result made of the others, nor the empty prefix's zeros."""
+    inp = wl.make_inputs(b, h, m_max, variant, seed=m_max + h, device=DEV)
+    L = m_max - 3
+    lens = torch.full((b,), L, dtype=torch.int32, device=DEV)
+    ws, status = mqa.alloc_workspace(b, h, m_max, DEV), torch.zeros(1, dtype=torch.int32, device=DEV)
+    step = mqa.mqa_decode_step if variant == "mqa" else mqa.mha_decode_step
+    for rows in (slice(0, L), slice(L // 2, L), slice(0, L // 2), slice(L // 3, 2 * L // 3), slice(L - 1, L), slice(7, 8)):
+        K, o = inp["K"].clone(), torch.zeros(b, h, 128, dtype=torch.float32, device=DEV)
+        K[..., rows, :] = float("nan")
+        step(inp["q"], K, inp["V"], lens, o, ws, status)
+        torch.cuda.synchronize()
+        assert bool(torch.isnan(o).all()), f"step, rows {rows}: {int((~torch.isnan(o)).sum())} elements are not NaN"
+        if variant == "mqa":
+            o.zero_()
+            mqa.mqa_decode_append_step(inp["q"], K, inp["V"], inp["k_new"], inp["v_new"], lens, o, ws, status, advance=False)
+            torch.cuda.synchronize()
+            assert bool(torch.isnan(o).all()), f"append step, rows {rows}: {int((~torch.isnan(o)).sum())} elements are not NaN"
+    assert int(status.item()) == 0
