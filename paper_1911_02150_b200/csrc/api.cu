@@ -44,6 +44,11 @@ int sm_count() {
 
 enum class Kernel { kSimt, kMma1, kMma2, kUmma, kWide };
 constexpr int kMergeInKernelMaxPieces = 10;
+// Fixed splits of up to kMmaMaxCluster per sequence are one thread-block cluster that merges the pieces itself: one launch in place
+// of two.  Measured, us per step called directly (the second launch is 2 of the host's) / in a graph: 1 x 16 heads x 512 rows 6.9 / 5.1 ->
+// 4.8 / 4.9; 4 x 16 x 1000 7.6 / 5.3 -> 5.2 / 5.1; 1 x 32 x 600 8.0 / 7.5 -> 6.9 / 6.7; 30 x 8 x 900 7.9 / 7.1 -> 6.8 / 6.5.  Two pieces
+// (256 to 383 rows) keep the second pass: the launch counts of that plan are relied on.
+constexpr int kMmaMinCluster = 3;
 constexpr int kMaxClusterCtas = 4;            // a sequence's CTAs as one thread-block cluster.  Measured per step: clusters of 8
                                               // (16 sequences x 16384 rows) 43 us against 29 us without, clusters of 16
                                               // (8 x 32768) 43 against 30: too few of them fit the GPCs at once
@@ -57,6 +62,7 @@ struct Plan {
     int grid = 0;         // persistent kernel: number of CTAs
     Kernel kernel = Kernel::kSimt;
     bool merge_in_kernel = false;   // tcgen05 plan: pieces merged by the CTA that delivers a sequence's last one (single launch)
+    bool cluster = false;           // fixed-split plan: the splits of a sequence are a thread-block cluster that merges them (single launch)
     bool stream() const { return kernel == Kernel::kUmma; }
 };
 
@@ -113,6 +119,7 @@ Plan plan_mma(int b, int h, int m_max) {
             p.chunk_rows = chunk;
         }
     }
+    p.cluster = p.n_splits >= kMmaMinCluster && p.n_splits <= kMmaMaxCluster;
     return p;
 }
 
@@ -362,20 +369,21 @@ bool encode_cache_map(CUtensorMap* map, const void* base, long long rows, int bo
     return encode_matrix_map(map, base, rows, kHeadDim, box_rows);
 }
 
-std::atomic<int> g_smem_opt_in[kMaxDevices][6];
+std::atomic<int> g_smem_opt_in[kMaxDevices][12];
 
-template <int M_TILES, int EARLY = 0>
+template <int M_TILES, int EARLY = 0, bool CLUSTER = false>
 int launch_mma(const Plan& p, const void* q, const void* K, const void* V, const int32_t* lens, float* o,
                float2* part_ml, float* part_acc, int32_t* status, int b, int h, int m_max, cudaStream_t stream, int len_bias,
                const void* k_new = nullptr, const void* v_new = nullptr, int32_t* lens_advance = nullptr,
                int mode = 0) {
     using Cfg = MmaCfg<M_TILES>;
-    auto kernel = mqa_decode_split_mma_kernel<M_TILES, EARLY>;
-    constexpr int kSlot = (M_TILES - 1) * 3 + EARLY;
+    auto kernel = mqa_decode_split_mma_kernel<M_TILES, EARLY, CLUSTER>;
+    constexpr int kSlot = ((M_TILES - 1) * 3 + EARLY) * 2 + (CLUSTER ? 1 : 0);
+    constexpr int kSmem = CLUSTER ? Cfg::kSmemBytesCluster : Cfg::kSmemBytes;
     int dev = 0;
     if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxDevices) { cudaGetLastError(); return MQA_ERR_CUDA; }
     if (!g_smem_opt_in[dev][kSlot].load(std::memory_order_acquire)) {
-        if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, Cfg::kSmemBytes) != cudaSuccess) {
+        if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmem) != cudaSuccess) {
             cudaGetLastError();
             return MQA_ERR_CUDA;
         }
@@ -393,7 +401,7 @@ int launch_mma(const Plan& p, const void* q, const void* K, const void* V, const
         fa.K = static_cast<uint4*>(const_cast<void*>(K));
         fa.V = static_cast<uint4*>(const_cast<void*>(V));
     }
-    launch_dependent(kernel, (unsigned)((size_t)b * p.n_splits), Cfg::kThreads, Cfg::kSmemBytes, stream, map_k, map_v,
+    launch_dependent_clusters(CLUSTER ? (unsigned)p.n_splits : 1u, kernel, (unsigned)((size_t)b * p.n_splits), Cfg::kThreads, kSmem, stream, map_k, map_v,
                      map_k_big, map_v_big, static_cast<const uint32_t*>(q), lens, o, part_ml, part_acc, status, h, m_max, p.chunk_rows,
                      p.n_splits, len_bias, fa, lens_advance, mode);
     return cudaGetLastError() == cudaSuccess ? MQA_OK : MQA_ERR_CUDA;
@@ -519,10 +527,11 @@ int run_split(bool multi_query, const void* q, const void* K, const void* V, con
     float2* part_ml = partials_ml(workspace);
     float* part_acc = partials_acc(p, workspace);
     if (p.kernel == Kernel::kWide) return launch_wide(p, q, K, V, lens, o, part_ml, part_acc, status, b, h, m_max, stream, len_bias);
-    if (p.kernel == Kernel::kMma1)
-        return launch_mma<1>(p, q, K, V, lens, o, part_ml, part_acc, status, b, h, m_max, stream, len_bias);
-    if (p.kernel == Kernel::kMma2)
-        return launch_mma<2>(p, q, K, V, lens, o, part_ml, part_acc, status, b, h, m_max, stream, len_bias);
+    if (p.kernel == Kernel::kMma1 || p.kernel == Kernel::kMma2) {
+        auto launch = p.kernel == Kernel::kMma1 ? (merge_in_kernel ? launch_mma<1, 0, true> : launch_mma<1, 0>)
+                                                : (merge_in_kernel ? launch_mma<2, 0, true> : launch_mma<2, 0>);
+        return launch(p, q, K, V, lens, o, part_ml, part_acc, status, b, h, m_max, stream, len_bias, nullptr, nullptr, nullptr, 0);
+    }
     const unsigned grid = (unsigned)(p.units * (size_t)p.n_splits);
     launch_dependent(decode_split_simt_kernel, grid, kSimtThreads, 0, stream, static_cast<const uint4*>(q),
                      static_cast<const uint4*>(K), static_cast<const uint4*>(V), lens, o, part_ml, part_acc, status, h,
@@ -580,8 +589,12 @@ int run_combine(bool multi_query, const int32_t* lens, float* o, const void* wor
 int run_step(bool multi_query, const void* q, const void* K, const void* V, const int32_t* lens, float* o,
              void* workspace, size_t workspace_bytes, int32_t* status,
              int b, int h, int m_max, int k, int v, cudaStream_t stream) {
-    // the tcgen05 plan is a single launch: the CTA that delivers the last piece of a sequence merges the pieces
-    const bool one_launch = dims_ok(b, h, m_max) && make_plan(multi_query, b, h, m_max).merge_in_kernel;
+    // a single launch where the kernel merges the pieces itself
+    bool one_launch = false;
+    if (dims_ok(b, h, m_max)) {
+        const Plan p = make_plan(multi_query, b, h, m_max);
+        one_launch = p.merge_in_kernel || p.cluster;
+    }
     int rc = run_split(multi_query, q, K, V, lens, o, workspace, workspace_bytes, status, b, h, m_max, k, v, stream, 0,
                        one_launch);
     if (rc || one_launch) return rc;
@@ -862,12 +875,13 @@ static int append_step_impl(const void* q, void* K, void* V, const void* k_new, 
         // one CTA per sequence writes the row, attends and moves lens on, all in one launch; of several splits the CTA whose
         // rows hold the new one writes it and the second pass moves lens on.  What is fetched ahead of the wait: EARLY in
         // decode_mma.cuh.
-        const bool alone = p.n_splits == 1;
+        const bool alone = p.n_splits == 1 || p.cluster;
         float2* part_ml = alone ? nullptr : partials_ml(workspace);
         float* part_acc = alone ? nullptr : partials_acc(p, workspace);
         int32_t* move_lens = alone && advance ? lens : nullptr;
 #define MQA_MMA_STEP(TILES, EARLY) \
-    launch_mma<TILES, EARLY>(p, q, K, V, lens, o, part_ml, part_acc, status, b, h, m_max, stream, 0, k_new, v_new, move_lens, mode)
+    (p.cluster ? launch_mma<TILES, EARLY, true> : launch_mma<TILES, EARLY>)(p, q, K, V, lens, o, part_ml, part_acc, status, b, h, m_max, stream, 0, \
+                                                                             k_new, v_new, move_lens, mode)
         if (p.kernel == Kernel::kMma1)
             rc = ahead == 1 ? MQA_MMA_STEP(1, 1) : ahead == 2 ? MQA_MMA_STEP(1, 2) : MQA_MMA_STEP(1, 0);
         else
@@ -1079,7 +1093,7 @@ int mqa_append_step_launches(int b, int h, int m_max, int k, int v) {
     if (!dims_ok(b, h, m_max) || k != kHeadDim || v != kHeadDim) return 0;
     const Plan p = make_plan(true, b, h, m_max);
     if (p.merge_in_kernel) return 1;                   // append, pass, merge and lens advance in one kernel
-    if ((p.kernel == Kernel::kMma1 || p.kernel == Kernel::kMma2) && p.n_splits == 1) return 1;   // one CTA per sequence does it all
+    if ((p.kernel == Kernel::kMma1 || p.kernel == Kernel::kMma2) && (p.n_splits == 1 || p.cluster)) return 1;   // one CTA or cluster per sequence does it all
     if (p.stream()) return 2;                          // pass with the append inside, second pass
     if (p.kernel == Kernel::kMma1 || p.kernel == Kernel::kMma2) return 2;   // fixed splits: the same two
     if (p.kernel == Kernel::kWide) return p.n_splits == 1 && h <= kWideRows ? 1 : 2;

@@ -54,6 +54,7 @@ __device__ int g_test_withhold = 0;
 __device__ __forceinline__ bool test_withhold() { return *reinterpret_cast<volatile int*>(&g_test_withhold) != 0; }
 constexpr int kSingleRoundingMinRows = 1024;            // prefixes this long feed P to the tensor cores in one bf16 rounding
 constexpr int kMmaWithhold = 2, kMmaRing = 4, kMmaWrongGuess = 8;     // bits of the fixed-split kernel's `mode` (and of the many-rows kernel's)
+constexpr int kMmaMaxCluster = 8;                       // splits of a sequence that may be one thread-block cluster
 constexpr int kStreamMaxSeqs = 1024;                   // sequences the persistent kernel can index in shared memory
 
 // Ring depth must be a multiple of kRowWarps: tile i lives in stage i % kStages and belongs to
@@ -67,6 +68,10 @@ struct MmaCfg {                                        // fixed-split kernel
     static constexpr int kStages = (M_TILES == 1) ? 4 : 12;
     static_assert(kStages % kRowWarps == 0, "a stage must always be consumed by the same warp");
     static constexpr int kSmemBytes = kStages * kStageBytes + 1024 /* alignment slack */ + 256 /* barriers */;
+    // with the splits of a sequence as one cluster: what the others send of this CTA's heads, rows of 128 and (maximum, sum) pairs
+    static constexpr int kRecvRows = M_TILES * 16 + kMmaMaxCluster;
+    static constexpr int kSmemBytesCluster = kSmemBytes + kRecvRows * (kHeadDim * 4 + 8);
+    static_assert(2 * kStages * 8 + 8 <= 256 && kSmemBytesCluster + 64 /* static */ <= 227 * 1024, "exceeds the shared memory of one SM");
     static constexpr int kMinBlocks = (M_TILES == 1) ? 2 : 1;
 };
 
@@ -339,8 +344,13 @@ __device__ __forceinline__ void consume_tile(WarpState& st, const uint32_t (&qa)
 //           prefix's last rows are fetched ahead of the wait and the rest right behind it, without waiting for lens
 //        2  behind this library's input projection (or the host step's input kernel), which has waited for everything
 //           that writes the cache and lens: lens is final, and all the tiles are fetched ahead of the wait
+// CLUSTER  the splits of a sequence are the CTAs of one thread-block cluster (rank = split) and merge their pieces: CTA r gets
+//        heads [r per, (r + 1) per) from all of them, 16 bytes per thread straight from the registers that the merge of the
+//        row-warps leaves them in into the receiver's shared memory, counted on its mbarrier.  Nothing through global memory, no
+//        second launch, the same bits as the second pass.  (Instances of their own: as a run-time flag the code cost the paper's
+//        step, which does not run it, 0.1 us.)
 // =============================================================================================
-template <int M_TILES, int EARLY = 0>
+template <int M_TILES, int EARLY = 0, bool CLUSTER = false>
 __global__ void __launch_bounds__(MmaCfg<M_TILES>::kThreads, MmaCfg<M_TILES>::kMinBlocks)
 mqa_decode_split_mma_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_constant__ CUtensorMap map_v,
                             const __grid_constant__ CUtensorMap map_k_big, const __grid_constant__ CUtensorMap map_v_big,
@@ -364,6 +374,8 @@ mqa_decode_split_mma_kernel(const __grid_constant__ CUtensorMap map_k, const __g
     uint64_t* bars = reinterpret_cast<uint64_t*>(stages + kStages * kStageBytes);   // full[kStages], empty[kStages]
     const uint32_t stages_s = smem_addr(stages);
     const uint32_t full_s = smem_addr(bars), empty_s = full_s + kStages * 8;
+    const int per = CLUSTER ? (h + n_splits - 1) / n_splits : 1, own_heads = max(0, min(per, h - split * per));   // CTA r merges heads [r per, (r + 1) per)
+    const uint32_t recv_bar = full_s + 2 * kStages * 8, recv_s = full_s + 256, recv_ml = recv_s + Cfg::kRecvRows * kHeadDim * 4;
     __shared__ int timed_out, issued;   // a wait ran out; tiles (or groups of four) whose copies were started
 
     // set up by the thread that issues the copies (it may issue some before the first CTA-wide barrier)
@@ -374,6 +386,10 @@ mqa_decode_split_mma_kernel(const __grid_constant__ CUtensorMap map_k, const __g
         for (int s = 0; s < kStages; ++s) {
             mbar_init(full_s + s * 8, 1);                  // the producer's arrive + the TMA bytes
             mbar_init(empty_s + s * 8, M_TILES);           // one arrive per warp that read the tile
+        }
+        if (CLUSTER) {
+            mbar_init(recv_bar, 1);
+            mbar_expect_tx(recv_bar, (uint32_t)((n_splits - 1) * own_heads * (kHeadDim * 4 + 8)));
         }
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
@@ -429,6 +445,7 @@ mqa_decode_split_mma_kernel(const __grid_constant__ CUtensorMap map_k, const __g
         }
     }
     __syncthreads();
+    if (CLUSTER) cluster_arrive();   // this CTA's barrier is in place
     // everything above overlaps the tail of the kernel before this one
     grid_dependency_wait();          // lens, q and the newest cache row may come from the kernel before
     grid_launch_dependents();
@@ -467,7 +484,7 @@ mqa_decode_split_mma_kernel(const __grid_constant__ CUtensorMap map_k, const __g
     const int L = clamp_len(appended ? min(raw, m_max - 1) + 1 : biased_len(raw, m_max, len_bias), m_max,
                             threadIdx.x == 0 ? status : nullptr);
     const int r1 = min(L, r0 + chunk_rows);
-    if (r0 >= L) {                                         // nothing valid in this split (uniform)
+    if (r0 >= L && !CLUSTER) {                             // nothing valid in this split (uniform)
         if (n_splits == 1)                                 // L == 0: the empty prefix gives zeros
             for (int i = threadIdx.x; i < h * kHeadDim; i += Cfg::kThreads) o[(size_t)seq * h * kHeadDim + i] = 0.f;
         else                                               // an empty piece, for a second pass that does not look at lens
@@ -476,7 +493,7 @@ mqa_decode_split_mma_kernel(const __grid_constant__ CUtensorMap map_k, const __g
         for (int i = 0; i < pre; ++i) mbar_wait(full_s + i * 8, 0);   // copies already started land before the CTA leaves
         return;
     }
-    const int n_tiles = (r1 - r0 + kTileRows - 1) / kTileRows;
+    const int n_tiles = max(0, (r1 - r0 + kTileRows - 1) / kTileRows);      // (0: a cluster's CTA with nothing but an empty piece)
     const bool big = in_groups(n_tiles);
 
     WarpState st;
@@ -541,7 +558,7 @@ mqa_decode_split_mma_kernel(const __grid_constant__ CUtensorMap map_k, const __g
             if (status) atomicOr(status, kStatusPipelineTimeout);
         }
         __syncthreads();
-        return;
+        if (!CLUSTER) return;            // (the others of a cluster wait for this CTA's piece, whatever it holds)
     }
 
     // ---- merge the kRowWarps warps of each head tile through shared memory (stages are free now)
@@ -589,6 +606,7 @@ mqa_decode_split_mma_kernel(const __grid_constant__ CUtensorMap map_k, const __g
         sm_w[threadIdx.x * 8 + kRowWarps + 1] = den;
     }
     __syncthreads();
+    if (CLUSTER) cluster_wait();         // (arrived at the start: every CTA's barrier is in place)
     // then 16 bytes of a head's 128 outputs per thread and round
     for (int idx = threadIdx.x; idx < h * (kHeadDim / 4); idx += Cfg::kThreads) {
         const int head = idx >> 5, c4 = idx & 31;
@@ -606,11 +624,70 @@ mqa_decode_split_mma_kernel(const __grid_constant__ CUtensorMap map_k, const __g
         if (n_splits == 1) {
             const float inv = 1.f / wts[kRowWarps + 1];
             *reinterpret_cast<float4*>(o + unit * kHeadDim + c4 * 4) = make_float4(num.x * inv, num.y * inv, num.z * inv, num.w * inv);
+        } else if (CLUSTER) {
+            const int to = head / per, row = split * per + head - to * per;      // (the heads of a warp's lanes are one)
+            const uint32_t at = recv_s + row * (kHeadDim * 4) + c4 * 16, at_ml = recv_ml + row * 8;
+            const float2 ml = make_float2(wts[kRowWarps], wts[kRowWarps + 1]);
+            if (to == split) {
+                asm volatile("st.shared.v4.f32 [%0], {%1,%2,%3,%4};" ::"r"(at), "f"(num.x), "f"(num.y), "f"(num.z), "f"(num.w) : "memory");
+                if (c4 == 0) asm volatile("st.shared.v2.f32 [%0], {%1,%2};" ::"r"(at_ml), "f"(ml.x), "f"(ml.y) : "memory");
+            } else {
+                cluster_send_f4(cluster_map(at, to), num, cluster_map(recv_bar, to));
+                if (c4 == 0) cluster_send_f2(cluster_map(at_ml, to), ml, cluster_map(recv_bar, to));
+            }
         } else {
             const size_t slot = unit * n_splits + split;
             *reinterpret_cast<float4*>(part_acc + slot * kHeadDim + c4 * 4) = num;
             if (c4 == 0) part_ml[slot] = make_float2(wts[kRowWarps], wts[kRowWarps + 1]);
         }
+    }
+    if (CLUSTER) {
+        // ---- this CTA's heads: the pieces of all splits, merged in split order with the arithmetic of the second pass
+        // (combine_few_kernel): the same bits
+        cluster_arrive();                // (this CTA's pieces are on their way, and it has read lens)
+        __syncthreads();                 // its own piece is in place
+        const bool got = mbar_wait(recv_bar, 0);
+        for (int idx = threadIdx.x; idx < own_heads * (kHeadDim / 4); idx += Cfg::kThreads) {
+            const int i = idx >> 5, c4 = idx & 31;
+            float2 ml[kMmaMaxCluster];
+            float4 a[kMmaMaxCluster];
+            float top = -INFINITY, den = 0.f;                  // (den: 0, or NaN if some piece's sum is)
+#pragma unroll
+            for (int s = 0; s < kMmaMaxCluster; ++s) {
+                if (s >= n_splits) break;
+                const int row = s * per + i;
+                asm volatile("ld.shared.v2.f32 {%0,%1}, [%2];" : "=f"(ml[s].x), "=f"(ml[s].y) : "r"(recv_ml + row * 8) : "memory");
+                asm volatile("ld.shared.v4.f32 {%0,%1,%2,%3}, [%4];" : "=f"(a[s].x), "=f"(a[s].y), "=f"(a[s].z), "=f"(a[s].w)
+                             : "r"(recv_s + row * (kHeadDim * 4) + c4 * 16) : "memory");
+                top = fmaxf(top, ml[s].x);
+                den = fmaf(0.f, ml[s].y, den);
+            }
+            float4* out = reinterpret_cast<float4*>(o + ((size_t)seq * h + split * per + i) * kHeadDim) + c4;
+            if (top == -INFINITY) {                            // the empty prefix: zeros (or NaN, if that is what all the logits were)
+                *out = make_float4(den, den, den, den);
+                continue;
+            }
+            float4 num = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+            for (int s = 0; s < kMmaMaxCluster; ++s) {
+                if (s >= n_splits) break;
+                const float w = fast_exp2(ml[s].x - top);
+                if (w != 0.f) {
+                    den = fmaf(w, ml[s].y, den);
+                    num.x = fmaf(w, a[s].x, num.x); num.y = fmaf(w, a[s].y, num.y);
+                    num.z = fmaf(w, a[s].z, num.z); num.w = fmaf(w, a[s].w, num.w);
+                }
+            }
+            *out = make_float4(num.x / den, num.y / den, num.z / den, num.w / den);
+        }
+        cluster_wait();                  // everybody's pieces have been sent
+        if (!got) {
+            // a wait ran out: what is still on its way here gets another bounded one before this CTA's shared memory goes
+            mbar_wait(recv_bar, 0);
+            if (threadIdx.x == 0 && status) atomicOr(status, kStatusPipelineTimeout);
+        }
+        if (lens_advance && appended && split == 0 && threadIdx.x == 0) lens_advance[seq] = raw + 1;
+        return;
     }
     if (lens_advance && appended && threadIdx.x == 0) lens_advance[seq] = raw + 1;   // every thread read lens[seq] barriers ago
 }

@@ -228,42 +228,6 @@ __device__ __forceinline__ unsigned int ctrl_arrive(unsigned long long* word, un
     return 0xffffffffu;                                    // never seen; the caller then does not merge
 }
 
-// ---- thread-block cluster helpers (the pieces of a sequence, and the head groups of the output projection, are summed
-// through distributed shared memory)
-__device__ __forceinline__ uint32_t cluster_cta_rank() {
-    uint32_t r;
-    asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
-    return r;
-}
-__device__ __forceinline__ uint32_t cluster_size() {
-    uint32_t n;
-    asm volatile("mov.u32 %0, %%cluster_nctarank;" : "=r"(n));
-    return n;
-}
-// every thread of every CTA of the cluster, the same number of times on every path: what a CTA wrote to its shared
-// memory before is visible to the others after
-__device__ __forceinline__ void cluster_sync() {
-    __syncwarp();                    // the aligned forms want the whole warp at the same instruction
-    asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
-    asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
-}
-// The address, in the cluster's shared window, of this CTA's shared address `local` in the CTA of rank `rank`.
-__device__ __forceinline__ uint32_t cluster_map(uint32_t local, uint32_t rank) {
-    uint32_t remote;
-    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(remote) : "r"(local), "r"(rank));
-    return remote;
-}
-__device__ __forceinline__ float4 cluster_ld_f4(uint32_t addr) {
-    float4 v;
-    asm volatile("ld.shared::cluster.v4.f32 {%0,%1,%2,%3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "r"(addr) : "memory");
-    return v;
-}
-__device__ __forceinline__ float2 cluster_ld_f2(uint32_t addr) {
-    float2 v;
-    asm volatile("ld.shared::cluster.v2.f32 {%0,%1}, [%2];" : "=f"(v.x), "=f"(v.y) : "r"(addr) : "memory");
-    return v;
-}
-
 // Barrier over `threads` threads that also ORs a predicate over them.
 __device__ __forceinline__ bool named_barrier_or(int id, int threads, bool pred) {
     uint32_t out;

@@ -400,3 +400,36 @@ def test_the_many_rows_step_the_bench_times_at_full_size(rows):
         oracle.kv_cache_append(Kh, Vh, wl.bits(s["k_new"]), wl.bits(s["v_new"]), lens_h, True)
         assert np.array_equal(wl.bits(s["K"]), Kh) and np.array_equal(wl.bits(s["V"]), Vh)
         check_close(o.cpu().numpy(), oracle.mqa_decode_step(wl.bits(s["q"]), Kh, Vh, lens_h), f"many rows ({rows}) at the bench's size")
+
+
+@pytest.mark.parametrize("chained", [False, True])
+@pytest.mark.parametrize("h,m_max", [(1, 384), (8, 512), (16, 1000), (17, 900), (32, 1000), (23, 500)])
+def test_splits_of_a_sequence_merged_in_a_cluster(h, m_max, chained):
+    """Short caches in three to eight fixed splits: one launch, the splits of a sequence a cluster.  Lengths at the edges of tiles
+    and splits (splits that hold nothing, more CTAs than heads), in a loop of steps against the oracle; and the step without
+    an append against its two phases on their own, bit for bit."""
+    n, chunk = mqa.plan_splits(True, 12, h, m_max)
+    assert 3 <= n <= 8 and mqa.append_step_launches(12, h, m_max) == 1
+    lens0 = np.array([0, 1, 30, 31, 32, chunk - 1, chunk, chunk + 1, 2 * chunk - 2, m_max - 3, m_max - 2, m_max // 2], np.int32)
+    b = len(lens0)
+    inp = wl.make_inputs(b, h, m_max, "mqa", seed=h + m_max, device=DEV)
+    wl.poison_tail(inp["K"], lens0); wl.poison_tail(inp["V"], lens0)
+    lens_t, status = torch.from_numpy(lens0).to(DEV), torch.zeros(1, dtype=torch.int32, device=DEV)
+    ws = mqa.alloc_workspace(b, h, m_max, DEV)
+    whole, phases = (torch.full((b, h, 128), float("nan"), dtype=torch.float32, device=DEV) for _ in range(2))
+    mqa.mqa_decode_step(inp["q"], inp["K"], inp["V"], lens_t, whole, ws, status)
+    mqa.mqa_decode_step_split(inp["q"], inp["K"], inp["V"], lens_t, phases, ws, status)
+    mqa.mqa_decode_step_combine(inp["q"], inp["K"], inp["V"], lens_t, phases, ws, status)
+    torch.cuda.synchronize()
+    check_close(whole.cpu().numpy(), oracle.mqa_decode_step(wl.bits(inp["q"]), wl.bits(inp["K"]), wl.bits(inp["V"]), lens0), "step")
+    assert torch.equal(whole.view(torch.int32), phases.view(torch.int32))
+    Kh, Vh, lens_h = wl.bits(inp["K"]), wl.bits(inp["V"]), lens0.copy()
+    o = torch.full((b, h, 128), float("nan"), dtype=torch.float32, device=DEV)
+    for t in range(2):
+        mqa.mqa_decode_append_step(inp["q"], inp["K"], inp["V"], inp["k_new"], inp["v_new"], lens_t, o, ws, status, chained=chained and t > 0)
+        oracle.kv_cache_append(Kh, Vh, wl.bits(inp["k_new"]), wl.bits(inp["v_new"]), lens_h, True)
+        torch.cuda.synchronize()
+        check_close(o.cpu().numpy(), oracle.mqa_decode_step(wl.bits(inp["q"]), Kh, Vh, lens_h), f"append step {t}")
+        assert np.array_equal(lens_t.cpu().numpy(), lens_h)
+    assert int(status.item()) == 0
+    assert np.array_equal(wl.bits(inp["K"]), Kh) and np.array_equal(wl.bits(inp["V"]), Vh)
