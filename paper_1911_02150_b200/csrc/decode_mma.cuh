@@ -67,7 +67,8 @@ struct MmaCfg {                                        // fixed-split kernel
     static constexpr int kThreads = (kConsumerWarps + 1) * 32;
     static constexpr int kStages = (M_TILES == 1) ? 4 : 12;
     static_assert(kStages % kRowWarps == 0, "a stage must always be consumed by the same warp");
-    static constexpr int kSmemBytes = kStages * kStageBytes + 1024 /* alignment slack */ + 256 /* barriers */;
+    static constexpr int kQBytes = M_TILES * 16 * kRowBytes;
+    static constexpr int kSmemBytes = kStages * kStageBytes + kQBytes + 1024 /* alignment slack */ + 256 /* barriers */;
     // with the splits of a sequence as one cluster: what the others send of this CTA's heads, rows of 128 and (maximum, sum) pairs
     static constexpr int kRecvRows = M_TILES * 16 + kMmaMaxCluster;
     static constexpr int kSmemBytesCluster = kSmemBytes + kRecvRows * (kHeadDim * 4 + 8);
@@ -228,6 +229,42 @@ __device__ __forceinline__ void load_q_fragments(uint32_t (&qa)[8][4], const uin
     }
 }
 
+// Query rows on their way to the A operands: by way of shared memory, in the layout of a cache tile (two 64-column boxes of
+// ROWS rows, 128-byte swizzle), so that a row is read from global memory once per CTA, 16 bytes per lane, and a warp's
+// fragments come with eight ldmatrix.  (Straight into the fragments every warp had 32 loads of 4 bytes per lane, eight rows to
+// a load, and the load unit took them one after the other.  us per step: 1 x 32 heads x 128 rows 4.93 -> 4.32, 1 x 32 x 600 7.4 ->
+// 6.0 (with the cluster), the loop of 128 x 32 heads to 128 rows 5.59 -> 5.11, the paper's, of 8 heads, 3.81 -> 3.77.)
+// Rows >= h are zero.  Called by THREADS threads.
+template <int ROWS, int THREADS>
+struct QueryRows {
+    static constexpr int kPieces = (ROWS * (kRowBytes / 16) + THREADS - 1) / THREADS;
+    uint4 v[kPieces];
+    __device__ __forceinline__ void load(const uint32_t* q, size_t row0, int rows, int tid) {
+        const uint4* src = reinterpret_cast<const uint4*>(q) + row0 * (kRowBytes / 16);
+#pragma unroll
+        for (int i = 0; i < kPieces; ++i) {
+            const int item = tid + i * THREADS;
+            v[i] = make_uint4(0u, 0u, 0u, 0u);
+            if (item < rows * (kRowBytes / 16)) v[i] = src[item];
+        }
+    }
+    __device__ __forceinline__ void store(uint32_t dst, int tid) const {
+#pragma unroll
+        for (int i = 0; i < kPieces; ++i) {
+            const int item = tid + i * THREADS, row = item >> 4, ch = item & 15;
+            if (item < ROWS * (kRowBytes / 16))
+                asm volatile("st.shared.v4.b32 [%0], {%1,%2,%3,%4};" ::"r"(dst + (ch >> 3) * (ROWS * 128) + row * 128 + (((ch & 7) ^ (row & 7)) << 4)),
+                             "r"(v[i].x), "r"(v[i].y), "r"(v[i].z), "r"(v[i].w) : "memory");
+        }
+    }
+};
+// The fragments of 16 query rows at `rows_s` (a multiple of 8 rows into a box; boxes half_stride apart).
+__device__ __forceinline__ void load_q_fragments(uint32_t (&qa)[8][4], uint32_t rows_s, uint32_t half_stride, const LaneOffsets& off) {
+#pragma unroll
+    for (int ks = 0; ks < 8; ++ks)
+        ldmatrix_x4(rows_s + off.v[ks & 3] + (ks >> 2) * half_stride, qa[ks][0], qa[ks][1], qa[ks][2], qa[ks][3]);
+}
+
 // One 32-row tile (cache rows row0 .. row0+31 of the sequence, of which rows < r1 are valid) for
 // 16 heads: S = Q K^T, online softmax update, O += P V.
 // HILO: feed P to the tensor cores as bf16 hi + lo parts (weights good to ~2^-17) instead of one
@@ -371,8 +408,8 @@ mqa_decode_split_mma_kernel(const __grid_constant__ CUtensorMap map_k, const __g
     extern __shared__ uint8_t smem_raw[];
     // 1 KiB alignment in the shared window: the 128-byte swizzle repeats every 8 rows x 128 bytes
     uint8_t* stages = smem_raw + ((1024u - (smem_addr(smem_raw) & 1023u)) & 1023u);
-    uint64_t* bars = reinterpret_cast<uint64_t*>(stages + kStages * kStageBytes);   // full[kStages], empty[kStages]
-    const uint32_t stages_s = smem_addr(stages);
+    uint64_t* bars = reinterpret_cast<uint64_t*>(stages + kStages * kStageBytes + Cfg::kQBytes);   // full[kStages], empty[kStages]
+    const uint32_t stages_s = smem_addr(stages), q_s = stages_s + kStages * kStageBytes;
     const uint32_t full_s = smem_addr(bars), empty_s = full_s + kStages * 8;
     const int per = CLUSTER ? (h + n_splits - 1) / n_splits : 1, own_heads = max(0, min(per, h - split * per));   // CTA r merges heads [r per, (r + 1) per)
     const uint32_t recv_bar = full_s + 2 * kStages * 8, recv_s = full_s + 256, recv_ml = recv_s + Cfg::kRecvRows * kHeadDim * 4;
@@ -469,8 +506,11 @@ mqa_decode_split_mma_kernel(const __grid_constant__ CUtensorMap map_k, const __g
     const int raw = lens[seq];
     const int mt = warp % M_TILES;                         // which 16-head tile this warp serves
     const int rw = warp / M_TILES;                         // which tiles (round-robin over kRowWarps)
-    uint32_t qa[8][4];
-    if (warp < Cfg::kConsumerWarps) load_q_fragments(qa, q, (size_t)seq, h, mt, lane);
+    QueryRows<M_TILES * 16, Cfg::kConsumerWarps * 32> rows_q;
+    if (warp < Cfg::kConsumerWarps) {
+        rows_q.load(q, (size_t)seq * h, h, threadIdx.x);
+        rows_q.store(q_s, threadIdx.x);
+    }
     const bool appended = fa.k_new != nullptr && raw >= 0 && (ring || raw < m_max);
     const int new_row = ring ? raw % m_max : raw;
     const bool holds_new = appended && new_row >= r0 && new_row - r0 < chunk_rows;      // the new row is one of this split's
@@ -518,6 +558,9 @@ mqa_decode_split_mma_kernel(const __grid_constant__ CUtensorMap map_k, const __g
         st.reset();
         LaneOffsets off;
         off.init(lane);
+        uint32_t qa[8][4];
+        named_barrier(1, Cfg::kConsumerWarps * 32);        // the query rows are in place
+        load_q_fragments(qa, q_s + mt * 16 * 128, M_TILES * 16 * 128, off);
         bool ok = true;
         for (int i = rw; i < n_tiles; i += kRowWarps) {
             const int s = i % kStages;
