@@ -929,12 +929,13 @@ int mqa_decode_local_step(const void* q, void* K, void* V, const void* k_new, co
         auto launch = h <= 16 ? launch_mma<1, 0> : launch_mma<2, 0>;
         return launch(p, q, K, V, pos, o, nullptr, nullptr, status, b, h, window, stream, 0, k_new, v_new, advance ? pos : nullptr, kMmaRing);
     }
-    // a warp per sequence: windows of a few tiles (the paper's is one), any number of heads
+    // a warp per sequence: windows of a few tiles, any number of heads; and of one tile (the paper's) with up to 16
     static std::atomic<int> opted[kMaxDevices];
     int dev = 0;
     if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxDevices) { cudaGetLastError(); return MQA_ERR_CUDA; }
     if (!opted[dev].load(std::memory_order_acquire)) {
-        if (cudaFuncSetAttribute(mqa_decode_local_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, local_smem_bytes(kLocalMaxWarps, 2)) != cudaSuccess) {
+        if (cudaFuncSetAttribute(mqa_decode_local_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, local_smem_bytes(kLocalMaxWarps)) != cudaSuccess ||
+            cudaFuncSetAttribute(mqa_decode_local_tile_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, local_tile_smem_bytes(kLocalMaxWarps)) != cudaSuccess) {
             cudaGetLastError();
             return MQA_ERR_CUDA;
         }
@@ -942,11 +943,12 @@ int mqa_decode_local_step(const void* q, void* K, void* V, const void* k_new, co
     }
     alignas(64) CUtensorMap map_k, map_v;
     if (!encode_cache_map(&map_k, K, (long long)b * window) || !encode_cache_map(&map_v, V, (long long)b * window)) return MQA_ERR_CUDA;
-    const int stages = window <= kTileRows && h <= 16 ? 1 : 2;
+    const bool tile = window <= kTileRows && h <= 16;
     const int each = (b + sms - 1) / sms, warps = each < kLocalMaxWarps ? each : kLocalMaxWarps;
-    launch_dependent(mqa_decode_local_kernel, (unsigned)((b + warps - 1) / warps), (unsigned)(warps * 32), (size_t)local_smem_bytes(warps, stages),
-                     stream, map_k, map_v, static_cast<const uint32_t*>(q), static_cast<const uint4*>(k_new), static_cast<const uint4*>(v_new),
-                     static_cast<uint4*>(K), static_cast<uint4*>(V), pos, o, status, b, h, window, advance ? 1 : 0, stages);
+    launch_dependent(tile ? mqa_decode_local_tile_kernel : mqa_decode_local_kernel, (unsigned)((b + warps - 1) / warps), (unsigned)(warps * 32),
+                     (size_t)(tile ? local_tile_smem_bytes(warps) : local_smem_bytes(warps)), stream, map_k, map_v, static_cast<const uint4*>(q),
+                     static_cast<const uint4*>(k_new), static_cast<const uint4*>(v_new), static_cast<uint4*>(K), static_cast<uint4*>(V), pos, o, status,
+                     b, h, window, advance ? 1 : 0);
     return launch_status();
 }
 

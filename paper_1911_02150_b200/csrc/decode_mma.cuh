@@ -127,6 +127,11 @@ __device__ __forceinline__ void tma_load_2d_hint(uint32_t dst, const CUtensorMap
 __device__ __forceinline__ void tma_prefetch_l2_2d(const CUtensorMap* map, int x, int y) {
     asm volatile("cp.async.bulk.prefetch.tensor.2d.L2.global.tile [%0, {%1, %2}];" ::"l"(map), "r"(x), "r"(y) : "memory");
 }
+// The same for `bytes` (a multiple of 16) at a 16-byte aligned address.  L2 is where every write of the kernels ahead goes through: what
+// they write after this is seen by whoever reads the bytes through L2 afterwards, so it may be asked for ahead of the wait for them.
+__device__ __forceinline__ void prefetch_l2(const void* p, uint32_t bytes) {
+    asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(p), "r"(bytes) : "memory");
+}
 // Policy for data that is read once (read_once): its lines are the first to go, so that a pass over a cache larger
 // than L2 does not push out what every launch needs again (q, lens, the workspace, the kernel's own code and
 // parameters).  Otherwise the ordinary policy: a cache that fits in L2 is found there by the next step.
@@ -211,24 +216,6 @@ struct WarpState {
     }
 };
 
-// Q fragments (A operand, 16 heads x 128 columns) of head tile mt of sequence seq, straight from
-// global memory; heads >= h are zero.
-__device__ __forceinline__ void load_q_fragments(uint32_t (&qa)[8][4], const uint32_t* q, size_t seq,
-                                                 int h, int mt, int lane) {
-    const int g = lane >> 2, t4 = lane & 3;
-    const int head0 = mt * 16 + g, head1 = head0 + 8;
-    const uint32_t* q0 = q + (seq * h + head0) * (kHeadDim / 2);
-    const uint32_t* q1 = q + (seq * h + head1) * (kHeadDim / 2);
-#pragma unroll
-    for (int ks = 0; ks < 8; ++ks) {
-        const int w0 = ks * 8 + t4;                    // 32-bit word: columns ks*16 + t4*2 + {0,1}
-        qa[ks][0] = head0 < h ? q0[w0] : 0u;
-        qa[ks][1] = head1 < h ? q1[w0] : 0u;
-        qa[ks][2] = head0 < h ? q0[w0 + 4] : 0u;   // columns + 8
-        qa[ks][3] = head1 < h ? q1[w0 + 4] : 0u;
-    }
-}
-
 // Query rows on their way to the A operands: by way of shared memory, in the layout of a cache tile (two 64-column boxes of
 // ROWS rows, 128-byte swizzle), so that a row is read from global memory once per CTA, 16 bytes per lane, and a warp's
 // fragments come with eight ldmatrix.  (Straight into the fragments every warp had 32 loads of 4 bytes per lane, eight rows to
@@ -258,6 +245,33 @@ struct QueryRows {
         }
     }
 };
+// The same fragments without shared memory, for a warp that has its query rows to itself: 16 bytes per lane and load, then the
+// four lanes that share a row swap words (4 x 4 at a time).
+__device__ __forceinline__ void load_q_fragments(uint32_t (&qa)[8][4], const uint4* q, size_t row0, int rows, int lane) {
+    const int g = lane >> 2, t4 = lane & 3;
+    uint4 v[2][4];
+#pragma unroll
+    for (int r = 0; r < 2; ++r)
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            v[r][j] = make_uint4(0u, 0u, 0u, 0u);
+            if (g + 8 * r < rows) v[r][j] = q[(row0 + g + 8 * r) * (kRowBytes / 16) + 4 * j + t4];
+        }
+    const bool odd = (t4 & 1) != 0, upper = (t4 & 2) != 0;
+#pragma unroll
+    for (int r = 0; r < 2; ++r)
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            const uint4 a = v[r][j];                            // piece 4 j + t4 of the row
+            const uint32_t s0 = __shfl_xor_sync(0xffffffffu, odd ? a.x : a.y, 1), s1 = __shfl_xor_sync(0xffffffffu, odd ? a.z : a.w, 1);
+            const uint32_t b0 = odd ? s0 : a.x, b1 = odd ? a.y : s0, b2 = odd ? s1 : a.z, b3 = odd ? a.w : s1;
+            const uint32_t s2 = __shfl_xor_sync(0xffffffffu, upper ? b0 : b2, 2), s3 = __shfl_xor_sync(0xffffffffu, upper ? b1 : b3, 2);
+            qa[2 * j][r] = upper ? s2 : b0;                     // word t4 of pieces 4 j, 4 j + 1, 4 j + 2, 4 j + 3
+            qa[2 * j][2 + r] = upper ? s3 : b1;
+            qa[2 * j + 1][r] = upper ? b2 : s2;
+            qa[2 * j + 1][2 + r] = upper ? b3 : s3;
+        }
+}
 // The fragments of 16 query rows at `rows_s` (a multiple of 8 rows into a box; boxes half_stride apart).
 __device__ __forceinline__ void load_q_fragments(uint32_t (&qa)[8][4], uint32_t rows_s, uint32_t half_stride, const LaneOffsets& off) {
 #pragma unroll
@@ -265,20 +279,14 @@ __device__ __forceinline__ void load_q_fragments(uint32_t (&qa)[8][4], uint32_t 
         ldmatrix_x4(rows_s + off.v[ks & 3] + (ks >> 2) * half_stride, qa[ks][0], qa[ks][1], qa[ks][2], qa[ks][3]);
 }
 
-// One 32-row tile (cache rows row0 .. row0+31 of the sequence, of which rows < r1 are valid) for
-// 16 heads: S = Q K^T, online softmax update, O += P V.
-// HILO: feed P to the tensor cores as bf16 hi + lo parts (weights good to ~2^-17) instead of one
-// bf16 rounding (2^-9 per weight).  One rounding is enough once the prefix is long: the output
-// is then an average over many rows, of size ~1/sqrt(rows), and so is the rounding error.
+// The parts of a 32-row tile's work (cache rows row0 .. row0+31 of the sequence, of which rows < r1 are valid) for 16 heads.
 // half_stride: bytes between the box holding columns 0..63 and the box holding columns 64..127.
-template <bool HILO>
-__device__ __forceinline__ void consume_tile(WarpState& st, const uint32_t (&qa)[8][4], const LaneOffsets& off,
-                                             uint32_t k_s, uint32_t v_s, uint32_t half_stride, int row0, int r1, int lane) {
-    const int t4 = lane & 3;
-    const bool ragged = row0 + kTileRows > r1;
 
-    // S = Q K^T: 4 n-tiles of 8 rows, 8 k-steps of 16 columns
-    float sc[4][4];
+// S = Q K^T in log2 units, masked by index, and each head's largest logit
+__device__ __forceinline__ void tile_logits(float (&sc)[4][4], float (&top)[2], const uint32_t (&qa)[8][4], const LaneOffsets& off,
+                                            uint32_t k_s, uint32_t half_stride, int row0, int r1, bool ragged, int lane) {
+    const int t4 = lane & 3;
+    // 4 n-tiles of 8 rows, 8 k-steps of 16 columns
 #pragma unroll
     for (int nt = 0; nt < 4; ++nt) sc[nt][0] = sc[nt][1] = sc[nt][2] = sc[nt][3] = 0.f;
 #pragma unroll
@@ -292,8 +300,7 @@ __device__ __forceinline__ void consume_tile(WarpState& st, const uint32_t (&qa)
             mma_bf16(sc[np * 2 + 1], qa[ks], b2, b3);
         }
     }
-    // scale to log2 units, mask by index, row maxima
-    float top[2] = {-INFINITY, -INFINITY};
+    top[0] = top[1] = -INFINITY;
 #pragma unroll
     for (int nt = 0; nt < 4; ++nt) {
 #pragma unroll
@@ -308,6 +315,59 @@ __device__ __forceinline__ void consume_tile(WarpState& st, const uint32_t (&qa)
         top[r] = fmaxf(top[r], __shfl_xor_sync(0xffffffffu, top[r], 1));
         top[r] = fmaxf(top[r], __shfl_xor_sync(0xffffffffu, top[r], 2));
     }
+}
+
+// P = exp2(S - m) as A-fragments of the two 16-row k-steps, in bf16 hi and (HILO) lo parts: weights good to ~2^-17 instead of one
+// rounding (2^-9 per weight); their sums are added to l
+template <bool HILO>
+__device__ __forceinline__ void tile_weights(uint32_t (&p_hi)[2][4], uint32_t (&p_lo)[2][4], float (&l)[2], const float (&sc)[4][4], const float (&m)[2]) {
+#pragma unroll
+    for (int nt = 0; nt < 4; ++nt) {
+        float p[4];
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            p[j] = fast_exp2(sc[nt][j] - m[j >> 1]);        // exactly 1 at the maximum, 0 when masked
+            l[j >> 1] += p[j];
+        }
+        const uint32_t hi01 = pack_bf16(p[0], p[1]), hi23 = pack_bf16(p[2], p[3]);
+        const int kk = nt >> 1, hf = (nt & 1) * 2;          // A regs: {g,k}, {g+8,k}, {g,k+8}, {g+8,k+8}
+        p_hi[kk][hf] = hi01; p_hi[kk][hf + 1] = hi23;
+        if (HILO) {
+            p_lo[kk][hf] = pack_bf16(p[0] - bf16_lo(hi01), p[1] - bf16_hi(hi01));
+            p_lo[kk][hf + 1] = pack_bf16(p[2] - bf16_lo(hi23), p[3] - bf16_hi(hi23));
+        }
+    }
+}
+
+// O += P V for one 16-row k-step kk and one pair vp of 8-column n-tiles; keep_lo, keep_hi: masks of the rows (see tile_row_masks)
+template <bool HILO>
+__device__ __forceinline__ void tile_product(float (&acc0)[4], float (&acc1)[4], const uint32_t (&p_hi)[4], const uint32_t (&p_lo)[4], const LaneOffsets& off,
+                                             uint32_t v_s, uint32_t half_stride, int kk, int vp, bool ragged, uint32_t keep_lo, uint32_t keep_hi) {
+    uint32_t b0, b1, b2, b3;
+    ldmatrix_x4_trans(v_s + off.v[vp & 3] + (vp >> 2) * half_stride + kk * 2048, b0, b1, b2, b3);
+    if (ragged) { b0 &= keep_lo; b1 &= keep_hi; b2 &= keep_lo; b3 &= keep_hi; }
+    mma_bf16(acc0, p_hi, b0, b1);
+    mma_bf16(acc1, p_hi, b2, b3);
+    if (HILO) {
+        mma_bf16(acc0, p_lo, b0, b1);
+        mma_bf16(acc1, p_lo, b2, b3);
+    }
+}
+// The V rows of k-step kk that lie past r1 are zeroed in the fragments (a ragged tile): rows ra, ra + 1 in b0 and b2, ra + 8, ra + 9 in b1 and b3.
+__device__ __forceinline__ void tile_row_masks(uint32_t& keep_lo, uint32_t& keep_hi, int row0, int r1, int kk, int lane) {
+    const int ra = row0 + kk * 16 + (lane & 3) * 2;
+    keep_lo = (ra < r1 ? 0x0000ffffu : 0u) | (ra + 1 < r1 ? 0xffff0000u : 0u);
+    keep_hi = (ra + 8 < r1 ? 0x0000ffffu : 0u) | (ra + 9 < r1 ? 0xffff0000u : 0u);
+}
+
+// One tile for a warp that has more of them: S = Q K^T, online softmax update, O += P V.  One rounding of the weights (HILO false) is
+// enough once the prefix is long: the output is then an average over many rows, of size ~1/sqrt(rows), and so is the rounding error.
+template <bool HILO>
+__device__ __forceinline__ void consume_tile(WarpState& st, const uint32_t (&qa)[8][4], const LaneOffsets& off,
+                                             uint32_t k_s, uint32_t v_s, uint32_t half_stride, int row0, int r1, int lane) {
+    const bool ragged = row0 + kTileRows > r1;
+    float sc[4][4], top[2];
+    tile_logits(sc, top, qa, off, k_s, half_stride, row0, r1, ragged, lane);
     // a new maximum rescales what has been accumulated; most tiles do not bring one
     if (__any_sync(0xffffffffu, top[0] > st.m[0] || top[1] > st.m[1])) {
         float rescale[2];
@@ -324,45 +384,15 @@ __device__ __forceinline__ void consume_tile(WarpState& st, const uint32_t (&qa)
             st.acc[vt][2] *= rescale[1]; st.acc[vt][3] *= rescale[1];
         }
     }
-    // P = exp2(S - max) as bf16 hi + lo A-fragments for the two 16-row k-steps
     uint32_t p_hi[2][4], p_lo[2][4];
-#pragma unroll
-    for (int nt = 0; nt < 4; ++nt) {
-        float p[4];
-#pragma unroll
-        for (int j = 0; j < 4; ++j) {
-            p[j] = fast_exp2(sc[nt][j] - st.m[j >> 1]);     // exactly 1 at the maximum, 0 when masked
-            st.l[j >> 1] += p[j];
-        }
-        const uint32_t hi01 = pack_bf16(p[0], p[1]), hi23 = pack_bf16(p[2], p[3]);
-        const int kk = nt >> 1, hf = (nt & 1) * 2;          // A regs: {g,k}, {g+8,k}, {g,k+8}, {g+8,k+8}
-        p_hi[kk][hf] = hi01; p_hi[kk][hf + 1] = hi23;
-        if (HILO) {
-            p_lo[kk][hf] = pack_bf16(p[0] - bf16_lo(hi01), p[1] - bf16_hi(hi01));
-            p_lo[kk][hf + 1] = pack_bf16(p[2] - bf16_lo(hi23), p[3] - bf16_hi(hi23));
-        }
-    }
-    // O += P V : 2 k-steps of 16 rows x 16 n-tiles of 8 columns
+    tile_weights<HILO>(p_hi, p_lo, st.l, sc, st.m);
 #pragma unroll
     for (int kk = 0; kk < 2; ++kk) {
-        uint32_t keep_lo = 0xffffffffu, keep_hi = 0xffffffffu;   // per-register row masks (ragged tile)
-        if (ragged) {
-            const int ra = row0 + kk * 16 + t4 * 2;              // rows held by b0/b2: ra, ra+1; b1/b3: +8
-            keep_lo = (ra < r1 ? 0x0000ffffu : 0u) | (ra + 1 < r1 ? 0xffff0000u : 0u);
-            keep_hi = (ra + 8 < r1 ? 0x0000ffffu : 0u) | (ra + 9 < r1 ? 0xffff0000u : 0u);
-        }
+        uint32_t keep_lo = 0xffffffffu, keep_hi = 0xffffffffu;
+        if (ragged) tile_row_masks(keep_lo, keep_hi, row0, r1, kk, lane);
 #pragma unroll
-        for (int vp = 0; vp < 8; ++vp) {                         // pairs of 8-column n-tiles
-            uint32_t b0, b1, b2, b3;
-            ldmatrix_x4_trans(v_s + off.v[vp & 3] + (vp >> 2) * half_stride + kk * 2048, b0, b1, b2, b3);
-            if (ragged) { b0 &= keep_lo; b1 &= keep_hi; b2 &= keep_lo; b3 &= keep_hi; }
-            mma_bf16(st.acc[vp * 2], p_hi[kk], b0, b1);
-            mma_bf16(st.acc[vp * 2 + 1], p_hi[kk], b2, b3);
-            if (HILO) {
-                mma_bf16(st.acc[vp * 2], p_lo[kk], b0, b1);
-                mma_bf16(st.acc[vp * 2 + 1], p_lo[kk], b2, b3);
-            }
-        }
+        for (int vp = 0; vp < 8; ++vp)                           // pairs of 8-column n-tiles
+            tile_product<HILO>(st.acc[vp * 2], st.acc[vp * 2 + 1], p_hi[kk], p_lo[kk], off, v_s, half_stride, kk, vp, ragged, keep_lo, keep_hi);
     }
 }
 

@@ -71,6 +71,13 @@ def test_local_step_on_either_kernel(b, h, window, steps):
     test_local_attention_ring_equals_attention_over_the_last_window_rows(b, h, window, steps)
 
 
+@pytest.mark.parametrize("b,h,window,steps", [(1039, 1, 3, 9), (300, 16, 32, 66), (9, 9, 17, 40), (2, 8, 2, 7)])
+def test_local_step_of_one_tile(b, h, window, steps):
+    """Windows of one 32-row tile: small and odd ones, one head and sixteen, a last CTA partly filled; a call asks its window
+    into L2 while the call before, which writes a row of it, may still run."""
+    test_local_attention_ring_equals_attention_over_the_last_window_rows(b, h, window, steps)
+
+
 @pytest.mark.parametrize("b,window", [(6, 100), (320, 100)])
 def test_local_step_of_several_tiles_with_a_negative_position(b, window):
     h = 8

@@ -161,6 +161,11 @@ def test_the_local_step_reports_a_wait_that_runs_out(b, h, window):
     check_close(o.cpu().numpy(), oracle.mqa_decode_step(wl.bits(inp["q"]), wl.bits(inp["K"]), wl.bits(inp["V"]), np.full(b, window, np.int32)), "the call after it")
 
 
+@pytest.mark.parametrize("b,h,window", [(300, 8, 32), (5, 16, 20)])
+def test_the_local_step_of_one_tile_reports_a_wait_that_runs_out(b, h, window):
+    test_the_local_step_reports_a_wait_that_runs_out(b, h, window)
+
+
 @pytest.mark.parametrize("b,h,d,m_max", [(17, 5, 640, 130), (128, 8, 1024, 64), (3, 1, 1024, 130)])
 def test_the_projections_report_sums_that_do_not_come(b, h, d, m_max):
     gen = torch.Generator(device=DEV).manual_seed(b)
