@@ -651,7 +651,8 @@ int launch_projections_in(const void* x, const void* P_q, const void* P_k, const
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)(h + 2), (unsigned)parts, (unsigned)((b + NB - 1) / NB));
     cfg.blockDim = dim3(kProjThreads);
-    cfg.dynamicSmemBytes = Cfg::kSmemBytes;
+    const int chunks = (d / 128 + parts - 1) / parts, stages = chunks < Cfg::kStages ? chunks : Cfg::kStages;
+    cfg.dynamicSmemBytes = Cfg::smem_bytes(stages);
     cfg.stream = stream;
     cudaLaunchAttribute attr[2];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
@@ -663,7 +664,7 @@ int launch_projections_in(const void* x, const void* P_q, const void* P_k, const
     cfg.attrs = attr;
     cfg.numAttrs = parts > 1 ? 2 : 1;
     cudaLaunchKernelEx(&cfg, kernel, map_pq, map_pk, map_pv, map_x, static_cast<__nv_bfloat16*>(q),
-                       static_cast<__nv_bfloat16*>(k_new), static_cast<__nv_bfloat16*>(v_new), status, b, h, d);
+                       static_cast<__nv_bfloat16*>(k_new), static_cast<__nv_bfloat16*>(v_new), status, b, h, d, stages);
     return launch_status();
 }
 
@@ -704,11 +705,10 @@ int launch_projection_out(const void* P_o, const float* o, float* y, int32_t* st
     using Cfg = ProjCfg<NB>;
     auto kernel = project_out_kernel<NB>;
     constexpr int kSlot = 4 + (NB == 16 ? 0 : (NB == 32 ? 1 : (NB == 64 ? 2 : 3)));
-    constexpr int kSmem = Cfg::kSmemBytes;
     int dev = 0;
     if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxDevices) { cudaGetLastError(); return MQA_ERR_CUDA; }
     if (!g_proj_opt_in[dev][kSlot].load(std::memory_order_acquire)) {
-        if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmem) != cudaSuccess) {
+        if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, Cfg::kSmemBytes) != cudaSuccess) {
             cudaGetLastError();
             return MQA_ERR_CUDA;
         }
@@ -721,7 +721,8 @@ int launch_projection_out(const void* P_o, const float* o, float* y, int32_t* st
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)(d / 128), (unsigned)groups, (unsigned)((b + NB - 1) / NB));
     cfg.blockDim = dim3(kProjThreads);
-    cfg.dynamicSmemBytes = kSmem;
+    const int stages = heads_per_cta < Cfg::kStages ? heads_per_cta : Cfg::kStages;
+    cfg.dynamicSmemBytes = Cfg::smem_bytes(stages);
     cfg.stream = stream;
     cudaLaunchAttribute attr[2];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
@@ -732,7 +733,7 @@ int launch_projection_out(const void* P_o, const float* o, float* y, int32_t* st
     attr[1].val.clusterDim.z = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 2;
-    cudaLaunchKernelEx(&cfg, kernel, map_po, o, y, status, b, h, d, heads_per_cta);
+    cudaLaunchKernelEx(&cfg, kernel, map_po, o, y, status, b, h, d, heads_per_cta, stages);
     return launch_status();
 }
 

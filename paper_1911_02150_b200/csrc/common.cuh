@@ -79,6 +79,11 @@ __device__ __forceinline__ void cluster_arrive() {
     __syncwarp();                    // the aligned forms want the whole warp at the same instruction
     asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
 }
+// (without the release: where the barrier only keeps CTAs from leaving, and what was written is known to have arrived)
+__device__ __forceinline__ void cluster_arrive_relaxed() {
+    __syncwarp();
+    asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory");
+}
 __device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
 __device__ __forceinline__ void cluster_sync() { cluster_arrive(); cluster_wait(); }
 // The address, in the cluster's shared window, of this CTA's shared address `local` in the CTA of rank `rank`.

@@ -49,7 +49,7 @@ struct ProjCfg {
     static constexpr int kRecvBytes = (NB + kProjMaxCluster) * 512;     // the other CTAs' sums of this one's rows (whole rows, rounded up per CTA)
     static constexpr int smem_bytes(int stages) { return stages * kStageBytes + kRecvBytes + 256 /* barriers */ + 1024 /* alignment slack */; }
     static constexpr int kSmemBytes = smem_bytes(kStages);
-    static_assert(kSumBytes <= 2 * kStageBytes, "the sums take the stages' place");
+    static_assert(kSumBytes <= kStageBytes, "the sums take the first stage's place");
     static constexpr int kTmemCols = NB < 32 ? 32 : NB;
     static_assert(kSmemBytes <= 227 * 1024, "exceeds the shared memory of one SM");
 };
@@ -112,9 +112,8 @@ __global__ void __launch_bounds__(kProjThreads, 1)
 project_in_kernel(const __grid_constant__ CUtensorMap map_pq, const __grid_constant__ CUtensorMap map_pk,
                   const __grid_constant__ CUtensorMap map_pv, const __grid_constant__ CUtensorMap map_x,
                   __nv_bfloat16* __restrict__ q, __nv_bfloat16* __restrict__ k_new, __nv_bfloat16* __restrict__ v_new,
-                  int32_t* __restrict__ status, int b, int h, int d) {
-    using Cfg = ProjCfg<NB>;
-    constexpr int S = Cfg::kStages;
+                  int32_t* __restrict__ status, int b, int h, int d, const int S) {
+    using Cfg = ProjCfg<NB>;                                      // (S stages, as many as a CTA has chunks, at most Cfg::kStages)
     const int slab = blockIdx.x, row0 = blockIdx.z * NB;          // weight slab; first batch row of this tile
     const int part = blockIdx.y, parts = gridDim.y;                // this CTA's part of the slab's d rows: one cluster per slab
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -224,7 +223,7 @@ project_in_kernel(const __grid_constant__ CUtensorMap map_pq, const __grid_const
     if (parts > 1) {
         if (warp == 0 && !withhold) shares.send(stages_s, recv_s, recv_bar, lane);
         if (!mbar_wait(recv_bar, 0)) { if (status && lane == 0) atomicOr(status, kStatusPipelineTimeout); mbar_wait(recv_bar, 0); }
-        cluster_arrive();            // what the others send has landed
+        cluster_arrive_relaxed();    // what the others send has landed
     }
     {
         __nv_bfloat16* out = slab < h ? q + (size_t)slab * 128 : (slab == h ? k_new : v_new);
@@ -243,9 +242,8 @@ project_in_kernel(const __grid_constant__ CUtensorMap map_pq, const __grid_const
 template <int NB>
 __global__ void __launch_bounds__(kProjThreads, 1)
 project_out_kernel(const __grid_constant__ CUtensorMap map_po, const float* __restrict__ o, float* __restrict__ y,
-                   int32_t* __restrict__ status, int b, int h, int d, int heads_per_cta) {
-    using Cfg = ProjCfg<NB>;
-    constexpr int S = Cfg::kStages;                                // a stage: a head's weights and its o tile
+                   int32_t* __restrict__ status, int b, int h, int d, int heads_per_cta, const int S) {
+    using Cfg = ProjCfg<NB>;                                       // a stage: a head's weights and its o tile (S of them, as in project_in_kernel)
     const int tile = blockIdx.x, group = blockIdx.y, row0 = blockIdx.z * NB;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int head0 = group * heads_per_cta;
@@ -368,7 +366,7 @@ project_out_kernel(const __grid_constant__ CUtensorMap map_po, const float* __re
     __syncthreads();
     if (warp == 0 && !withhold) shares.send(stages_s, recv_s, recv_bar, lane);
     if (!mbar_wait(recv_bar, 0)) { if (status && lane == 0) atomicOr(status, kStatusPipelineTimeout); mbar_wait(recv_bar, 0); }
-    cluster_arrive();                // what the others send has landed
+    cluster_arrive_relaxed();        // what the others send has landed
     for (int i = warp; i < shares.count(group); i += kProjThreads / 32)
         *reinterpret_cast<float4*>(y + (size_t)(row0 + group * shares.per + i) * d + (size_t)tile * 128 + lane * 4) = shares.add_up(stages_s, recv_s, i, lane);
     cluster_wait();                  // nobody leaves while its sums are on their way
