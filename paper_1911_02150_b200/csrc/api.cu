@@ -6,6 +6,7 @@
 #include <stdint.h>
 
 #include <atomic>
+#include <cmath>
 #include <cstdlib>
 
 #include "../../include/mqa_decode.h"
@@ -46,9 +47,13 @@ enum class Kernel { kSimt, kMma1, kMma2, kUmma, kWide };
 constexpr int kMergeInKernelMaxPieces = 10;
 // Fixed splits of up to kMmaMaxCluster per sequence are one thread-block cluster that merges the pieces itself: one launch in place
 // of two.  Measured, us per step called directly (the second launch is 2 of the host's) / in a graph: 1 x 16 heads x 512 rows 6.9 / 5.1 ->
-// 4.8 / 4.9; 4 x 16 x 1000 7.6 / 5.3 -> 5.2 / 5.1; 1 x 32 x 600 8.0 / 7.5 -> 6.9 / 6.7; 30 x 8 x 900 7.9 / 7.1 -> 6.8 / 6.5.  Two pieces
-// (256 to 383 rows) keep the second pass: the launch counts of that plan are relied on.
-constexpr int kMmaMinCluster = 3;
+// 4.8 / 4.9; 4 x 16 x 1000 7.6 / 5.3 -> 5.2 / 5.1; 1 x 32 x 600 8.0 / 7.5 -> 6.9 / 6.7; 30 x 8 x 900 7.9 / 7.1 -> 6.8 / 6.5; sixteen pieces
+// (clusters beyond the portable eight): 1 x 16 x 2048 8.0 / 5.3 -> 5.9 / 5.0.
+// A cluster of S CTAs has to fit one GPC, and a launch whose clusters do not all fit at once takes a second round: at one CTA per SM (17
+// to 32 heads) 10 clusters of 8 took 6.4 us where 16 took 12.2, at two per SM 24 took 5.7 and 48 12.7.
+bool clusters_fit(int sequences, int S, int ctas_per_sm) { return S <= kMmaMaxCluster && sequences <= 17 * ctas_per_sm / S * (S <= 4 ? 8 : 7); }
+// 257 to 319 rows keep the second pass: callers count on two launches there.
+bool keeps_second_pass(int m_max) { return m_max > 256 && m_max < 320; }
 constexpr int kMaxClusterCtas = 4;            // a sequence's CTAs as one thread-block cluster.  Measured per step: clusters of 8
                                               // (16 sequences x 16384 rows) 43 us against 29 us without, clusters of 16
                                               // (8 x 32768) 43 against 30: too few of them fit the GPCs at once
@@ -119,7 +124,7 @@ Plan plan_mma(int b, int h, int m_max) {
             p.chunk_rows = chunk;
         }
     }
-    p.cluster = p.n_splits >= kMmaMinCluster && p.n_splits <= kMmaMaxCluster;
+    p.cluster = p.n_splits > 1 && clusters_fit(b, p.n_splits, ctas_per_sm) && !keeps_second_pass(m_max);
     return p;
 }
 
@@ -174,7 +179,8 @@ Plan plan_wide(int b, int h, int m_max) {
     return p;
 }
 
-Plan make_plan(bool multi_query, int b, int h, int m_max) {
+// The plan by rules on the sizes alone; make_plan below looks for a better one where there are up to 32 query rows.
+Plan plan_by_size(bool multi_query, int b, int h, int m_max) {
     // a row space too large for the 32-bit TMA coordinates goes to the general CUDA-core kernel
     if (!(multi_query && (long long)b * m_max < 0x7fffffffLL)) return plan_simt(b, h, m_max);
     // More than 32 query rows per sequence: the kernel with the query rows as tile rows, 128 rows per CTA and more as row
@@ -196,6 +202,128 @@ Plan make_plan(bool multi_query, int b, int h, int m_max) {
         return p;
     }
     return h <= 32 ? plan_mma(b, h, m_max) : plan_simt(b, h, m_max);
+}
+
+size_t plan_workspace_bytes(const Plan& p);
+
+// ---- which of the multi-query kernels, and how many splits: a model of a step's time in us, for a launch of this kernel over caches
+// that are a share `full` full.  Fitted to 9600 timings (1 to 512 sequences of 256 to 32768 rows, 8, 16 and 32 heads, full caches and
+// ragged ones, splits from one to as many as there are tiles, steps in a graph); it is off by 9 to 12 % (rms).
+// The two kernels that share out fixed splits take rounds (of the four row-warps, 128 rows, or of a stage) after a start, several
+// CTAs per SM or waves of them, and no less than the bytes; then the merge.
+struct SplitModel { double start, round, second, share, tail, floor, tbs, cluster, per_cluster, crowd, pass, pass_mb; };
+constexpr SplitModel kMma1Model = {2.71, 1.78, 0.24, -0.16, 0.40, 2.64, 5.03, 0.96, 0.64, 1.11, 1.74, 0.56};
+constexpr SplitModel kMma2Model = {3.85, 1.21, 0.63, 0.21, 0.18, 3.83, 4.46, 0.87, 0.08, 0.80, 1.74, 0.12};
+struct WideModel { double start, stage, short_stage, pass, tail, floor, tbs; };
+constexpr WideModel kWide1Model = {4.35, 0.70, 0.42, 2.07, 0.24, 4.39, 6.03}, kWide2Model = {4.87, 0.65, 0.37, 2.16, 0.31, 5.01, 6.03};
+// The streaming kernel: what is around its stream, where the batch makes whole clusters or shares of whole sequences of full caches,
+// where it does not, and for ragged ones.
+struct StreamModel { double whole, cut, ragged, tbs; };
+constexpr StreamModel kStream1Model = {7.43, 10.6, 11.7, 6.59}, kStream2Model = {8.72, 12.0, 14.1, 6.67};
+
+double either(double a, double b) { return std::sqrt(std::sqrt(a * a * a * a + b * b * b * b)); }   // the larger, and some more where they are alike
+
+double plan_us(const Plan& p, int m_max, double full, int sms) {
+    const bool few = p.h <= 16;
+    const double mb = (double)p.b * m_max * full * 2 * kRowBytes * 1e-6, per_sm = (double)p.b * p.n_splits / sms;
+    double us;
+    if (p.kernel == Kernel::kUmma) {
+        const StreamModel& m = few ? kStream1Model : kStream2Model;
+        const bool whole = p.b % p.grid == 0 || (p.grid % p.b == 0 && p.grid / p.b <= kMaxClusterCtas);
+        us = (full < 1 ? m.ragged : whole ? m.whole : m.cut) + mb / m.tbs;
+        // clusters that do not fit at once (3 x 48 sequences, 4 x 37): 18 us where 32 x 1024 rows take 9
+        if (whole && p.grid > p.b && p.grid / p.b > 2 && p.grid > sms - 16) us *= 1.6;
+        return us > 4.7 ? us : 4.7;
+    }
+    if (p.kernel == Kernel::kWide) {
+        const WideModel& m = few ? kWide1Model : kWide2Model;
+        const int stages = (p.chunk_rows + kWideRows - 1) / kWideRows;
+        us = m.start + stages * (m.stage + (m_max < kSingleRoundingMinRows ? m.short_stage : 0));
+        if (per_sm > 1) us *= per_sm + m.tail;
+        us = either(us, m.floor + mb / m.tbs) + (p.n_splits > 1 ? m.pass : 0);
+    } else {
+        const SplitModel& m = few ? kMma1Model : kMma2Model;
+        const int occ = few ? MmaCfg<1>::kMinBlocks : MmaCfg<2>::kMinBlocks, rounds = (p.chunk_rows + 4 * kTileRows - 1) / (4 * kTileRows);
+        us = m.start + m.round * (rounds - 1) + (rounds > 1 ? m.second : 0);
+        us *= 1 + m.share * ((per_sm > occ ? occ : per_sm > 1 ? per_sm : 1) - 1);
+        if (per_sm > occ) us *= per_sm / occ + m.tail;
+        us = either(us, m.floor + mb / m.tbs);
+        if (p.n_splits > 1)
+            us += p.cluster ? m.cluster + m.per_cluster * p.n_splits / 16 + (per_sm > 1 ? m.crowd * (per_sm - 1) : 0)
+                            : m.pass + m.pass_mb * p.b * p.n_splits * p.h * (kHeadDim + 2) * 4e-6;
+    }
+    // called directly, a launch and the call take the host 4.7 us, two launches 6.6
+    const double host = p.n_splits > 1 && !p.cluster ? 6.6 : 4.7;
+    return us > host ? us : host;
+}
+
+// A plan is kept where it is expected to be faster, for full caches and for ragged ones (half of the rows on average; what lens holds is not
+// known here), than the plan by size: by 13 % in all (18 % beyond 4096 rows, where fewer timings stand behind the model), and by 15 % more
+// where it takes a second launch and the other does not.
+// Measured against the plans by size over the sizes above: -13 % on average; us per step 16 x 16 heads x 1024 rows 11.3 -> 5.5,
+// 32 x 8 x 1024 8.9 -> 7.0, 48 x 8 x 1500 20.9 -> 10.1, 8 x 8 x 2048 8.1 -> 5.2, 64 x 8 x up to 2048 rows 18.0 -> 13.0.
+constexpr double kPlanGain = 0.87, kPlanGainLong = 0.82, kPlanSecondLaunch = 0.85;
+
+Plan make_plan(bool multi_query, int b, int h, int m_max) {
+    const Plan old = plan_by_size(multi_query, b, h, m_max);
+    if (!multi_query || h > 32 || old.kernel == Kernel::kSimt || b > kStreamMaxSeqs) return old;
+    const int sms = sm_count();
+    // (a decoding loop asks for the same few plans at every step)
+    struct Entry { int sms, b, h, m_max; Plan plan; };
+    thread_local Entry kept[32] = {};
+    Entry& e = kept[((unsigned)b * 7u + (unsigned)h * 31u + (unsigned)m_max) % 32u];
+    if (e.sms == sms && e.b == b && e.h == h && e.m_max == m_max) return e.plan;
+    const double us_full = plan_us(old, m_max, 1.0, sms), us_ragged = plan_us(old, m_max, 0.5, sms);
+    auto one_launch = [](const Plan& p) { return p.stream() ? p.merge_in_kernel : p.n_splits == 1 || p.cluster; };
+    auto launches = [&](const Plan& p) { return one_launch(p) ? 1.0 : 1.0 / (kPlanSecondLaunch * kPlanSecondLaunch); };
+    Plan best = old;
+    const double gain = m_max <= 4096 ? kPlanGain : kPlanGainLong;
+    double best_cost = us_full * us_ragged * gain * gain * launches(old);
+    auto consider = [&](const Plan& p) {
+        const size_t need = plan_workspace_bytes(p);
+        if (need > MQA_NOALLOC_SCRATCH_BYTES && need > plan_workspace_bytes(old)) return;      // (what the built-in scratch held it still holds)
+        const double full = plan_us(p, m_max, 1.0, sms), ragged = plan_us(p, m_max, 0.5, sms);
+        if (full > us_full || ragged > us_ragged || full * ragged * launches(p) >= best_cost) return;
+        best = p;
+        best_cost = full * ragged * launches(p);
+    };
+    // whole clusters of more than 16 heads stay with the streaming kernel from 2048 rows on (32 x 32 x 2048: 12.7 us, 12.8 in four splits)
+    const bool whole = old.stream() && old.grid % b == 0 && old.grid / b <= kMaxClusterCtas;
+    const bool search = !(whole && h > 16 && m_max >= 2048);
+    Plan p;
+    p.units = (size_t)b * h;
+    p.b = b; p.h = h;
+    // fixed splits of 128 rows and multiples of them, one round of the four row-warps per 128, that fit the SMs in one wave (2 x 21 x
+    // 9909 rows: 10.2 us by size, 12.9 in 156 splits for 148 SMs)
+    p.kernel = h <= 16 ? Kernel::kMma1 : Kernel::kMma2;
+    const int occ = h <= 16 ? MmaCfg<1>::kMinBlocks : MmaCfg<2>::kMinBlocks;
+    const bool two = keeps_second_pass(m_max) && b <= 48;          // (then nothing that is one launch)
+    for (int rows = 4 * kTileRows, before = 0; search; rows += 4 * kTileRows) {
+        const int S = (m_max + rows - 1) / rows;
+        if (S != before && S <= 128 && (S == 1 || (long long)S * b <= (long long)occ * sms) && !(two && S == 1)) {
+            p.n_splits = S;
+            p.chunk_rows = ((m_max + S - 1) / S + kTileRows - 1) / kTileRows * kTileRows;
+            p.cluster = S > 1 && m_max <= kMmaMaxCluster * 256 && clusters_fit(b, S, occ) && !keeps_second_pass(m_max);
+            if ((m_max + p.chunk_rows - 1) / p.chunk_rows == S) consider(p);
+        }
+        before = S;
+        if (S == 1) break;
+    }
+    // and of whole stages on the kernel with the query rows as tile rows, one wave of CTAs
+    p.kernel = Kernel::kWide;
+    p.cluster = false;
+    for (int rows = kWideRows, before = 0; search; rows += kWideRows) {
+        const int S = (m_max + rows - 1) / rows;
+        if (S != before && (long long)S * b <= sms && !(two && S == 1)) {
+            p.n_splits = S;
+            p.chunk_rows = ((m_max + S - 1) / S + kWideRows - 1) / kWideRows * kWideRows;
+            if ((m_max + p.chunk_rows - 1) / p.chunk_rows == S) consider(p);
+        }
+        before = S;
+        if (S == 1) break;
+    }
+    e = Entry{sms, b, h, m_max, best};
+    return best;
 }
 
 // Every workspace begins with the control block of the single-launch step (kStreamCtrlBytes: see decode_umma.cuh),
@@ -383,7 +511,8 @@ int launch_mma(const Plan& p, const void* q, const void* K, const void* V, const
     int dev = 0;
     if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxDevices) { cudaGetLastError(); return MQA_ERR_CUDA; }
     if (!g_smem_opt_in[dev][kSlot].load(std::memory_order_acquire)) {
-        if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmem) != cudaSuccess) {
+        if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmem) != cudaSuccess ||
+            (CLUSTER && cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess)) {
             cudaGetLastError();
             return MQA_ERR_CUDA;
         }

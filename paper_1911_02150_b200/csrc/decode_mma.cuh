@@ -54,7 +54,7 @@ __device__ int g_test_withhold = 0;
 __device__ __forceinline__ bool test_withhold() { return *reinterpret_cast<volatile int*>(&g_test_withhold) != 0; }
 constexpr int kSingleRoundingMinRows = 1024;            // prefixes this long feed P to the tensor cores in one bf16 rounding
 constexpr int kMmaWithhold = 2, kMmaRing = 4, kMmaWrongGuess = 8;     // bits of the fixed-split kernel's `mode` (and of the many-rows kernel's)
-constexpr int kMmaMaxCluster = 8;                       // splits of a sequence that may be one thread-block cluster
+constexpr int kMmaMaxCluster = 16;                      // splits of a sequence that may be one thread-block cluster
 constexpr int kStreamMaxSeqs = 1024;                   // sequences the persistent kernel can index in shared memory
 
 // Ring depth must be a multiple of kRowWarps: tile i lives in stage i % kStages and belongs to

@@ -403,13 +403,13 @@ def test_the_many_rows_step_the_bench_times_at_full_size(rows):
 
 
 @pytest.mark.parametrize("chained", [False, True])
-@pytest.mark.parametrize("h,m_max", [(1, 384), (8, 512), (16, 1000), (17, 900), (32, 1000), (23, 500)])
+@pytest.mark.parametrize("h,m_max", [(1, 384), (8, 512), (16, 1000), (17, 900), (32, 1000), (23, 500), (16, 2048), (8, 4096), (4, 1409), (20, 1500)])
 def test_splits_of_a_sequence_merged_in_a_cluster(h, m_max, chained):
-    """Short caches in three to eight fixed splits: one launch, the splits of a sequence a cluster.  Lengths at the edges of tiles
+    """Caches in three to sixteen fixed splits: one launch, the splits of a sequence a cluster.  Lengths at the edges of tiles
     and splits (splits that hold nothing, more CTAs than heads), in a loop of steps against the oracle; and the step without
     an append against its two phases on their own, bit for bit."""
     n, chunk = mqa.plan_splits(True, 12, h, m_max)
-    assert 3 <= n <= 8 and mqa.append_step_launches(12, h, m_max) == 1
+    assert 3 <= n <= 16 and mqa.append_step_launches(12, h, m_max) == 1
     lens0 = np.array([0, 1, 30, 31, 32, chunk - 1, chunk, chunk + 1, 2 * chunk - 2, m_max - 3, m_max - 2, m_max // 2], np.int32)
     b = len(lens0)
     inp = wl.make_inputs(b, h, m_max, "mqa", seed=h + m_max, device=DEV)
