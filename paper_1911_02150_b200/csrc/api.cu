@@ -756,6 +756,60 @@ LayerWorkspace layer_workspace(int b, int h, int d, int m_max) {
     return w;
 }
 
+// How a projection is cut up: NB batch columns per tile (16, 32, 64 or 128) and the CTAs of a cluster that share the depth of the
+// product (the chunks of d rows of an input slab; the heads of an output tile).  By a model of a CTA's chain, in microseconds: its
+// activations (act_kb per batch column and chunk) at 60 KB/us, step_us per chunk (an output tile's chunk is a round trip for o), 0.4
+// per chunk of weights beyond those fetched ahead of the wait, and what the cluster exchanges, which is slow (SM to SM about
+// 24 KB/us per CTA).  A cut whose CTAs do not fit the SMs at once, or whose clusters do not fit the GPCs (of 8: about half of the
+// SMs), is charged by its number of waves, total / most_ctas + 0.5; the input projection has about half of the SMs, where the attention kernel behind it
+// does not yet set itself up.  Measured, us per layer step, one fixed cut (128 columns; 16 heads' groups) against this one:
+// 128 x 8 heads x 1024 18.4 / 15.4; 200 x 16 x 1536 47.6 / 28.8; 256 x 8 x 2048 38.8 / 23.4; 8 x 32 x 2048 25.6 / 19.2; 1 x 16 x 2048 23.4 / 18.3.
+// A CTA takes the shared memory of as many stages as it has chunks, so where the chunks of a CTA are few, two CTAs fit an SM and the
+// weights are on their way while the kernel ahead still runs.  So a cut that leaves a CTA four chunks or more is halved once more where
+// a second look, fitted to all cuts of 14 layer steps, finds that 5 % better (a chunk 0.38, activations at 25 KB/us, SM to SM 23.5, and
+// two thirds of the SMs, times two where two fit); and clusters of 8 that do not all fit at once become clusters of 4.  us per layer step,
+// without and with both: 128 x 8 x 1024 14.7 / 13.4; 256 x 32 x 2048 39.8 / 35.6; 8 x 32 x 2048 24.4 / 21.1; 1 x 16 x 2048 17.4 / 16.4; 7 x
+// 11 x 1920 13.8 / 13.4.
+struct ProjectionCut { int nb, ctas; };
+int projection_stages(int nb, int chunks) {
+    const int most = nb == 128 ? ProjCfg<128>::kStages : nb == 64 ? ProjCfg<64>::kStages : ProjCfg<32>::kStages;
+    return chunks < most ? chunks : most;
+}
+bool two_projections_fit(int nb, int chunks) {
+    const int s = projection_stages(nb, chunks);
+    const int bytes = nb == 128 ? ProjCfg<128>::smem_bytes(s) : nb == 64 ? ProjCfg<64>::smem_bytes(s) : nb == 32 ? ProjCfg<32>::smem_bytes(s) : ProjCfg<16>::smem_bytes(s);
+    return 2 * (bytes + 1024 + 16) <= 228 * 1024;
+}
+ProjectionCut projection_cut(int b, int columns, int depth, double act_kb, double step_us, int most_ctas) {
+    ProjectionCut best = {128, 1};
+    double best_us = -1;
+    for (int nb = 16; nb <= 128 && (nb == 16 || nb < 2 * b); nb *= 2) {
+        const int batch_tiles = (b + nb - 1) / nb, rows = b < nb ? b : nb;
+        const int stages = nb == 128 ? ProjCfg<128>::kStages : nb == 64 ? ProjCfg<64>::kStages : ProjCfg<32>::kStages;
+        for (int ctas = 1; ctas <= kProjMaxCluster && ctas <= depth; ctas *= 2) {
+            const long long total = (long long)columns * batch_tiles * ctas;
+            const int each = (depth + ctas - 1) / ctas;
+            const double waves = total <= (ctas == 8 ? most_ctas * 5 / 9 : most_ctas) ? 1.0 : (double)total / most_ctas + 0.5;
+            const double us = waves * (3.0 + each * step_us + rows * each * act_kb / 60 + (each > stages ? (each - stages) * 0.4 : 0) +
+                                       (ctas > 1 ? 0.3 + rows * 0.5 * (ctas - 1) / ctas / 24 : 0));
+            if (best_us < 0 || us < best_us) { best = {nb, ctas}; best_us = us; }
+        }
+    }
+    const int batch_tiles = (b + best.nb - 1) / best.nb, rows = b < best.nb ? b : best.nb, each = (depth + best.ctas - 1) / best.ctas;
+    if (best.ctas == 8 && columns * batch_tiles > (two_projections_fit(best.nb, each) ? 28 : 14)) return {best.nb, 4};
+    auto second_look = [&](int ctas) {
+        const int chunks = (depth + ctas - 1) / ctas;
+        const bool two = two_projections_fit(best.nb, chunks);
+        const double total = (double)columns * batch_tiles * ctas, slots = sm_count() * (two ? 2 : 1) * 0.66 * (ctas < 8 ? 1 : two ? 0.65 : 0.95);
+        return (total <= slots ? 1.0 : total / slots) * (3.1 + chunks * 0.38 + rows * chunks * act_kb / 24.8 + rows * 0.5 * (ctas - 1) / ctas / 23.5);
+    };
+    if (each >= 4 && best.ctas * 2 <= kProjMaxCluster && second_look(best.ctas * 2) < 0.95 * second_look(best.ctas)) best.ctas *= 2;
+    return best;
+}
+
+ProjectionCut input_cut(int b, int h, int d) { return projection_cut(b, h + 2, d / 128, 0.25, 0.2, sm_count() * 5 / 9); }       // bf16 x
+ProjectionCut output_cut(int b, int h, int d) { return projection_cut(b, d / 128, h, 0.5, 0.45, sm_count() * 8 / 9); }           // fp32 o
+
 std::atomic<int> g_proj_opt_in[kMaxDevices][8];
 
 template <int NB>
@@ -780,7 +834,7 @@ int launch_projections_in(const void* x, const void* P_q, const void* P_k, const
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)(h + 2), (unsigned)parts, (unsigned)((b + NB - 1) / NB));
     cfg.blockDim = dim3(kProjThreads);
-    const int chunks = (d / 128 + parts - 1) / parts, stages = chunks < Cfg::kStages ? chunks : Cfg::kStages;
+    const int stages = projection_stages(NB, (d / 128 + parts - 1) / parts);
     cfg.dynamicSmemBytes = Cfg::smem_bytes(stages);
     cfg.stream = stream;
     cudaLaunchAttribute attr[2];
@@ -796,36 +850,6 @@ int launch_projections_in(const void* x, const void* P_q, const void* P_k, const
                        static_cast<__nv_bfloat16*>(k_new), static_cast<__nv_bfloat16*>(v_new), status, b, h, d, stages);
     return launch_status();
 }
-
-// How a projection is cut up: NB batch columns per tile (16, 32, 64 or 128) and the CTAs of a cluster that share the depth of the
-// product (the chunks of d rows of an input slab; the heads of an output tile).  By a model of a CTA's chain, in microseconds: its
-// activations (act_kb per batch column and chunk) at 60 KB/us, step_us per chunk (an output tile's chunk is a round trip for o), 0.4
-// per chunk of weights beyond those fetched ahead of the wait, and what the cluster exchanges, which is slow (SM to SM about
-// 24 KB/us per CTA).  A cut whose CTAs do not fit the SMs at once, or whose clusters do not fit the GPCs (of 8: about half of the
-// SMs), is charged by its number of waves, total / most_ctas + 0.5; the input projection has about half of the SMs, where the attention kernel behind it
-// does not yet set itself up.  Measured, us per layer step, one fixed cut (128 columns; 16 heads' groups) against this one:
-// 128 x 8 heads x 1024 18.4 / 15.4; 200 x 16 x 1536 47.6 / 28.8; 256 x 8 x 2048 38.8 / 23.4; 8 x 32 x 2048 25.6 / 19.2; 1 x 16 x 2048 23.4 / 18.3.
-struct ProjectionCut { int nb, ctas; };
-ProjectionCut projection_cut(int b, int columns, int depth, double act_kb, double step_us, int most_ctas) {
-    ProjectionCut best = {128, 1};
-    double best_us = -1;
-    for (int nb = 16; nb <= 128 && (nb == 16 || nb < 2 * b); nb *= 2) {
-        const int batch_tiles = (b + nb - 1) / nb, rows = b < nb ? b : nb;
-        const int stages = nb == 128 ? ProjCfg<128>::kStages : nb == 64 ? ProjCfg<64>::kStages : ProjCfg<32>::kStages;
-        for (int ctas = 1; ctas <= kProjMaxCluster && ctas <= depth; ctas *= 2) {
-            const long long total = (long long)columns * batch_tiles * ctas;
-            const int each = (depth + ctas - 1) / ctas;
-            const double waves = total <= (ctas == 8 ? most_ctas * 5 / 9 : most_ctas) ? 1.0 : (double)total / most_ctas + 0.5;
-            const double us = waves * (3.0 + each * step_us + rows * each * act_kb / 60 + (each > stages ? (each - stages) * 0.4 : 0) +
-                                       (ctas > 1 ? 0.3 + rows * 0.5 * (ctas - 1) / ctas / 24 : 0));
-            if (best_us < 0 || us < best_us) { best = {nb, ctas}; best_us = us; }
-        }
-    }
-    return best;
-}
-
-ProjectionCut input_cut(int b, int h, int d) { return projection_cut(b, h + 2, d / 128, 0.25, 0.2, sm_count() * 5 / 9); }       // bf16 x
-ProjectionCut output_cut(int b, int h, int d) { return projection_cut(b, d / 128, h, 0.5, 0.45, sm_count() * 8 / 9); }           // fp32 o
 
 // The output projection: the head groups of a (d tile, batch tile) are the CTAs of one thread-block cluster (see
 // project_out_kernel), each with ceil(h / ctas) heads.
@@ -850,7 +874,7 @@ int launch_projection_out(const void* P_o, const float* o, float* y, int32_t* st
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)(d / 128), (unsigned)groups, (unsigned)((b + NB - 1) / NB));
     cfg.blockDim = dim3(kProjThreads);
-    const int stages = heads_per_cta < Cfg::kStages ? heads_per_cta : Cfg::kStages;
+    const int stages = projection_stages(NB, heads_per_cta);
     cfg.dynamicSmemBytes = Cfg::smem_bytes(stages);
     cfg.stream = stream;
     cudaLaunchAttribute attr[2];
