@@ -1287,27 +1287,31 @@ static PfShape prefill_shape(int b, int h, int n, int m_max) {
         }
         if ((long long)sh.n_tiles * kPfRows < (long long)h * n + kPfRows) break;      // no shape has fewer
     }
-    sh.n_units = (sh.n_tiles + 1) / 2;
-    sh.group = sh.head_blocks / 2 > 1 ? sh.head_blocks / 2 : 1;
-    sh.n_items = (sh.n_units + sh.group - 1) / sh.group * sh.group * b;
     return sh;
 }
+// The units of work: two tiles each, or one (mqa_prefill_tile_kernel).
+static void prefill_units(PfShape& sh, int tiles) {
+    sh.n_units = (sh.n_tiles + tiles - 1) / tiles;
+    sh.group = sh.head_blocks / tiles > 1 ? sh.head_blocks / tiles : 1;
+    sh.n_items = (sh.n_units + sh.group - 1) / sh.group * sh.group * sh.b;
+}
 
-// CTAs (one cluster) that share a unit's stages, where there are fewer units than SMs: by a model of the time.  Measured, us
-// for 1 / 2 / 4 / 8 CTAs per unit: 60 units of up to 24 stages 41.3 / 32.8 / 43.8 / 69.1 (4 do not fit at once); 64 of 16: 30.5 / 26.3 / 35.8;
-// 32 of 16: 28.8 / 25.6 / 20.1 / 45.4; 16 of 32: 53.3 / 38.1 / 25.4 / 29.4 (clusters of 8 do not fill every GPC); 1 of 17: 21.5 / 18.3 /
-// 12.6 / 9.9; 16 of 4: 16.5 / 18.8 / 31.2.
-static int prefill_split(const PfShape& sh, int rows, int sms) {
-    const double stage_us = 1.4, unit_us = 4.0, merge_us = 4.0;
+// Which kernel, by a model of the time in us: 0 for two tiles to a CTA (persistent, one CTA per SM), else the CTAs of a cluster that share
+// one tile's stages.  Measured, us for two tiles / one tile by 1 / 2 / 4 / 8 CTAs: 120 tiles of up to 24 stages 37.8 / 25.6 / 35.7 (they do not
+// fit at once); 64 of 32: 51.1 / 32.3 / 23.6 / 29.9; 10 of 12: 21.6 / 16.5 / 15.6 / 13.6 / 12.3; 1 of 16: 19.5 / 16.6 / 14.1 / 11.5 / 10.4; 240 of 3:
+// 14.2 / 20.2; 256 of 16: 28.2 / 35.6.  (With two tiles to a unit throughout and clusters sharing units: 120 of 24 28.5, 128 of 8 22.0.)
+static int prefill_tile_ctas(const PfShape& sh, int rows, int sms) {
     const int stages = (rows + kPfRows - 1) / kPfRows;
-    if (sh.n_items > 2 * sms) return 1;
-    int best = 1;
-    double best_us = 0;
-    for (int ctas = 1; ctas <= kPfMaxSplit && ctas * 2 <= (stages > 2 ? stages : 2); ctas *= 2) {
+    const bool two_roundings = rows < kSingleRoundingMinRows;
+    const double tiles = (double)sh.n_tiles * sh.b, units = (double)((sh.n_tiles + 1) / 2) * sh.b;
+    if (tiles > 2.0 * sms) return 0;
+    int best = 0;
+    double best_us = 0.95 * std::ceil(units / sms) * (7.0 + stages * (two_roundings ? 1.9 : 1.42));
+    for (int ctas = 1; ctas <= kPfMaxSplit && (ctas == 1 || ctas * 2 <= (stages > 2 ? stages : 2)); ctas *= 2) {
         const int slots = ctas == 8 ? sms / 16 : ctas == 4 ? sms * 9 / 40 : sms / ctas;
         if (slots < 1) break;
-        const double us = (double)((sh.n_items + slots - 1) / slots) * ((double)((stages + ctas - 1) / ctas) * stage_us + unit_us + (ctas > 1 ? merge_us : 0));
-        if (best_us == 0 || us < 0.93 * best_us) { best = ctas; best_us = us; }
+        const double us = std::ceil(tiles / slots) * (8.0 + (double)((stages + ctas - 1) / ctas) * (two_roundings ? 1.05 : 0.72)) + (ctas > 1 ? 2.5 : 0);
+        if (us < best_us) { best = ctas; best_us = us; }
     }
     return best;
 }
@@ -1331,24 +1335,25 @@ int mqa_prefill_attention(const void* Q, const void* K, const void* V, const int
     int dev = 0;
     if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxDevices) { cudaGetLastError(); return MQA_ERR_CUDA; }
     if (!opt_in[dev].load(std::memory_order_acquire)) {
-        if (cudaFuncSetAttribute(mqa_prefill_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, kPfSmemBytes) != cudaSuccess ||
-            cudaFuncSetAttribute(mqa_prefill_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, kPfSmemBytes) != cudaSuccess) {
+        if (cudaFuncSetAttribute(mqa_prefill_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kPfSmemBytes) != cudaSuccess ||
+            cudaFuncSetAttribute(mqa_prefill_tile_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kPtSmemBytes) != cudaSuccess) {
             cudaGetLastError();
             return MQA_ERR_CUDA;
         }
         opt_in[dev].store(1, std::memory_order_release);
     }
-    const PfShape sh = prefill_shape(b, h, n, m_max);
-    const int sms = sm_count(), ctas = prefill_split(sh, start ? m_max : n, sms);
+    PfShape sh = prefill_shape(b, h, n, m_max);
+    const int sms = sm_count(), ctas = prefill_tile_ctas(sh, start ? m_max : n, sms);
+    prefill_units(sh, ctas > 0 ? 1 : 2);
     alignas(64) CUtensorMap map_q, map_k, map_v;
     if (!encode_map(&map_q, Q, (long long)b * h, n, kHeadDim, sh.heads, sh.positions) ||
         !encode_cache_map(&map_k, K, (long long)b * m_max, kPfRows) || !encode_cache_map(&map_v, V, (long long)b * m_max, kPfRows))
         return MQA_ERR_CUDA;
-    if (ctas > 1)
-        launch_dependent_clusters((unsigned)ctas, mqa_prefill_kernel<true>, (unsigned)(sh.n_items * ctas), (unsigned)kPfThreads,
-                                  (size_t)kPfSmemBytes, stream, map_q, map_k, map_v, start, O, status, sh);
+    if (ctas > 0)
+        launch_dependent_clusters((unsigned)ctas, mqa_prefill_tile_kernel, (unsigned)(sh.n_items * ctas), (unsigned)kPfThreads,
+                                  (size_t)kPtSmemBytes, stream, map_q, map_k, map_v, start, O, status, sh);
     else
-        launch_dependent(mqa_prefill_kernel<false>, (unsigned)(sh.n_items < sms ? sh.n_items : sms), (unsigned)kPfThreads,
+        launch_dependent(mqa_prefill_kernel, (unsigned)(sh.n_items < sms ? sh.n_items : sms), (unsigned)kPfThreads,
                          (size_t)kPfSmemBytes, stream, map_q, map_k, map_v, start, O, status, sh);
     return launch_status();
 }

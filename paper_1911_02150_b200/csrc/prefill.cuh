@@ -29,10 +29,8 @@
 //
 // What bounds it: power.  A stage of both heads takes 2630 cycles (4400 before the logits had a buffer of their own and
 // the issuers were taken apart; the tensor cores need 2048, the exponentials 2048), and at that rate the card holds its
-// clock near 1.2 GHz.  32 x 32 heads x 4096 positions, in a loop: 5.0 ms -> 4.13 ms (1070 TFLOP/s).  Where a call has fewer
-// units than the card has SMs it is the longest unit's chain of stages: those a cluster shares out (SPLIT).  5 x 9 heads x 333
-// positions over up to 3000 rows: 50 -> 35 us with the stages as above, 31 with tiles of 3 heads and two CTAs per unit; 5 x 2 x 108
-// over 2257: 36 -> 16; 7 x 22 x 200: 21 -> 13.6.
+// clock near 1.2 GHz.  32 x 32 heads x 4096 positions, in a loop: 5.0 ms -> 4.13 ms (1070 TFLOP/s).  Calls with few tiles, which
+// are bound by the longest tile's chain of stages, go to mqa_prefill_tile_kernel below.
 // Every wait is bounded; a wait that runs out flags PIPELINE_TIMEOUT and the CTA drains and leaves.
 #pragma once
 #include "decode_umma.cuh"
@@ -46,7 +44,7 @@ constexpr int kPfKSlots = 2, kPfVSlots = 2;
 constexpr int kPfThreads = 12 * 32;                            // (warp 11 only completes the third warpgroup)
 constexpr int kPfProducerWarp = 8, kPfSWarp = 9, kPfPvWarp = 10;
 constexpr int kPfRegsSoftmax = 216, kPfRegsOther = 72;
-constexpr int kPfMaxSplit = 8;                                 // CTAs that share a unit's stages
+constexpr int kPfMaxSplit = 8;                                 // CTAs that share a tile's stages (mqa_prefill_tile_kernel)
 constexpr float kPfMaxLead = 8.f;                              // log2 units a logit may exceed its row's reference by
 // barriers: q_full, k_full/k_empty[2], v_full/v_empty[2], s_ready[2], p_ready[2], pv_done[2], s_free, q_empty
 constexpr int kPfBarriers = 1 + 2 * kPfKSlots + 2 * kPfVSlots + 6 + 2;
@@ -140,55 +138,6 @@ __device__ __forceinline__ void tma_load_3d(uint32_t dst, const CUtensorMap* map
         ::"r"(dst), "l"(map), "r"(x), "r"(y), "r"(z), "r"(bar) : "memory");
 }
 
-// The rows warp, warp + 8 CTAS, ... of a unit, merged out of the CTAS shares (rank order) and stored: a warp per row, a lane 16
-// bytes of it.  All the remote loads of 16 / CTAS rows are in flight at once (row by row, a round trip each, the merge of
-// two shares took about 6 us).
-template <int CTAS>
-__device__ __forceinline__ void pf_merge(const PfItem& it, const PfShape& sh, float* __restrict__ O, uint32_t ml_s, uint32_t rows_s,
-                                         int row0, int lane) {
-    constexpr int R = 16 / CTAS;
-#pragma unroll 1
-    for (int i0 = row0; i0 < 2 * kPfRows; i0 += 8 * CTAS * R) {
-        int row[R];
-        float2 ml[R][CTAS];
-        float4 part[R][CTAS];
-#pragma unroll
-        for (int i = 0; i < R; ++i) {
-            const int rr = i0 + i * 8 * CTAS;                    // (2 * kPfRows is a multiple of 8 * CTAS * R)
-            row[i] = pf_row(it, sh, rr / kPfRows, rr % kPfRows);
-            if (row[i] < 0) continue;
-#pragma unroll
-            for (int c = 0; c < CTAS; ++c) {
-                ml[i][c] = cluster_ld_f2(cluster_map(ml_s + rr * 8, c));
-                part[i][c] = cluster_ld_f4(cluster_map(rows_s + rr * 512 + ((lane ^ (rr & 31)) << 4), c));
-            }
-        }
-#pragma unroll
-        for (int i = 0; i < R; ++i) {
-            if (row[i] < 0) continue;
-            float top = -INFINITY, den = 0.f;
-            float4 num = make_float4(0.f, 0.f, 0.f, 0.f);
-#pragma unroll
-            for (int c = 0; c < CTAS; ++c) top = fmaxf(top, ml[i][c].x);
-#pragma unroll
-            for (int c = 0; c < CTAS; ++c) {
-                // a share of which the row sees nothing (it may never have been written).  Its maximum does not tell: that of a
-                // share whose logits are all NaN is -inf too, and its sum is NaN
-                if (ml[i][c].y == 0.f) continue;
-                const float f = fast_exp2(ml[i][c].x - top);
-                den = fmaf(f, ml[i][c].y, den);
-                num.x = fmaf(f, part[i][c].x, num.x); num.y = fmaf(f, part[i][c].y, num.y);
-                num.z = fmaf(f, part[i][c].z, num.z); num.w = fmaf(f, part[i][c].w, num.w);
-            }
-            const float inv = it.n_kv > 0 ? 1.f / den : 0.f;
-            *reinterpret_cast<float4*>(O + (size_t)row[i] * kHeadDim + lane * 4) = make_float4(num.x * inv, num.y * inv, num.z * inv, num.w * inv);
-        }
-    }
-}
-
-// SPLIT: fewer units than SMs.  The CTAs of a cluster share a unit's stages, each a run of them, and merge their partial
-// softmaxes through distributed shared memory (rank order; the rows of the two tiles are shared out over the CTAs).
-template <bool SPLIT>
 __global__ void __launch_bounds__(kPfThreads, 1)
 mqa_prefill_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CUtensorMap map_k,
                    const __grid_constant__ CUtensorMap map_v, const int32_t* start, float* __restrict__ O,
@@ -231,18 +180,12 @@ mqa_prefill_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
     grid_dependency_wait();              // Q, K, V and start may come from the kernel before
     grid_launch_dependents();
     // the units of this CTA: c, 2G - 1 - c, 2G + c, 4G - 1 - c, ... (G CTAs; the units come longest first, so taking them
-    // forwards and backwards in turn evens the CTAs' totals out); with SPLIT one unit per cluster
-    const int n_items = sh.n_items, ctas = SPLIT ? (int)cluster_size() : 1, rank = SPLIT ? (int)cluster_cta_rank() : 0;
+    // forwards and backwards in turn evens the CTAs' totals out)
+    const int n_items = sh.n_items;
     auto pf_unit = [&](int round) -> int {
         const int G = (int)gridDim.x, c = (int)blockIdx.x;
-        if (SPLIT) return round == 0 ? c / ctas : n_items;
         return round * G + ((round & 1) ? G - 1 - c : c);
     };
-    // this CTA's stages of a unit: [first, first + count)
-    auto first_stage = [&](int n_kv) { return SPLIT ? rank * n_kv / ctas : 0; };
-    auto count_stages = [&](int n_kv) { return SPLIT ? (rank + 1) * n_kv / ctas - rank * n_kv / ctas : n_kv; };
-    // how many of them the unit's first tile has
-    auto count_stages0 = [&](const PfItem& it) { return SPLIT ? max(0, min(count_stages(it.n_kv), it.n_kv0 - first_stage(it.n_kv))) : it.n_kv0; };
     if (start && threadIdx.x < 32) {
         // a start that is negative or leaves too little room is flagged once (its rows are zeros, or the memory is cut at m_max)
         bool bad = false;
@@ -265,7 +208,7 @@ mqa_prefill_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
             const bool withhold = blockIdx.x == 0 && test_withhold();
             for (int round = 0, item; (item = pf_unit(round)) < n_items && ok; ++round) {
                 const PfItem it = pf_item(item, start, sh);
-                const int first = first_stage(it.n_kv), n_kv = count_stages(it.n_kv);
+                const int n_kv = it.n_kv;
                 if (n_kv == 0) continue;
                 if (qi > 0) ok = mbar_wait(q_empty, (qi - 1) & 1);            // the unit before has read its Q for the last time
                 if (!ok) break;
@@ -277,7 +220,7 @@ mqa_prefill_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
                 issued_q = qi + 1;
                 for (int j = 0; j < n_kv && ok; ++j) {
                     const int G = g + j;
-                    const int y = it.seq * sh.m_max + (first + j) * kPfRows;
+                    const int y = it.seq * sh.m_max + j * kPfRows;
                     const int ks = G % kPfKSlots, vs = G % kPfVSlots;
                     if (G >= kPfKSlots) ok = mbar_wait(k_empty + 8 * ks, ((G / kPfKSlots) - 1) & 1);
                     if (!ok) break;
@@ -311,8 +254,8 @@ mqa_prefill_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
         int g = 0, qi = 0, n_s = 0;                              // stages, units and logits so far
         for (int round = 0, item; (item = pf_unit(round)) < n_items && ok; ++round) {
             const PfItem it = pf_item(item, start, sh);
-            const int n_kv = __shfl_sync(0xffffffffu, count_stages(it.n_kv), 0), n_act = it.n_act;
-            const int n_kv0 = __shfl_sync(0xffffffffu, count_stages0(it), 0);
+            const int n_kv = __shfl_sync(0xffffffffu, it.n_kv, 0), n_act = it.n_act;
+            const int n_kv0 = __shfl_sync(0xffffffffu, it.n_kv0, 0);
             if (n_kv == 0) continue;
             ok = warp_wait(q_full, qi & 1);
             for (int j = 0; j < n_kv && ok; ++j, ++g) {
@@ -352,11 +295,11 @@ mqa_prefill_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
         int g = 0, n_p[2] = {0, 0};                              // stages and each head's weights so far
         for (int round = 0, item; (item = pf_unit(round)) < n_items && ok; ++round) {
             const PfItem it = pf_item(item, start, sh);
-            const int n_kv = __shfl_sync(0xffffffffu, count_stages(it.n_kv), 0), n_act = it.n_act, parts = __any_sync(0xffffffffu, it.hilo) ? 2 : 1;
-            const int n_kv0 = __shfl_sync(0xffffffffu, count_stages0(it), 0);
-            // (the stage that is cut, counted from this CTA's first one: with SPLIT it may be another CTA's.  A reduction over the
-            // warp leaves its result where the issue of a product can test it: 0.4 us less for a unit than with a shuffle)
-            const int cut = __reduce_max_sync(0xffffffffu, pf_cut(it)), cut_j = cut > 0 ? it.n_kv0 - 1 - first_stage(it.n_kv) : -1;
+            const int n_kv = __shfl_sync(0xffffffffu, it.n_kv, 0), n_act = it.n_act, parts = __any_sync(0xffffffffu, it.hilo) ? 2 : 1;
+            const int n_kv0 = __shfl_sync(0xffffffffu, it.n_kv0, 0);
+            // (the stage that is cut.  A reduction over the warp leaves its result where the issue of a product can test it: 0.4 us
+            // less for a unit than with a shuffle)
+            const int cut = __reduce_max_sync(0xffffffffu, pf_cut(it)), cut_j = cut > 0 ? it.n_kv0 - 1 : -1;
             for (int j = 0; j < n_kv && ok; ++j, ++g) {
                 const int slot = g % kPfVSlots;
                 const uint32_t v_s = v_ring + slot * kPfTileBytes;
@@ -367,7 +310,7 @@ mqa_prefill_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
                     if (!whole && (cut & 15)) {
                         // the 16 rows that the first tile ends in, zeros from its end on, to the place where its softmax warps hand O out
                         // (with those of the unit before they are through once this stage's weights are there)
-                        if (!SPLIT) ok = warp_wait(p_ready, n_p[0] & 1);
+                        ok = warp_wait(p_ready, n_p[0] & 1);
                         uint4 v[8];
 #pragma unroll
                         for (int i = 0; i < 8; ++i) {            // 16-byte pieces, eight to a row of a 64-column half
@@ -417,7 +360,6 @@ mqa_prefill_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
         }
         if (!ok && lane == 0) atomicExch(&timed_out, 1);
     }
-    if (SPLIT) cluster_sync();           // (the softmax warps' first one)
     } else {
         asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(kPfRegsSoftmax));
         // =============================================================== softmax warps: one thread per query row
@@ -429,10 +371,10 @@ mqa_prefill_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
         int g = 0, n_s = 0, n_p = 0;                             // stages of the CTA, logits and weights of this head so far
         for (int round = 0, item; (item = pf_unit(round)) < n_items; ++round) {
             const PfItem it = pf_item(item, start, sh);
-            const int first = first_stage(it.n_kv), n_kv = count_stages(it.n_kv);
+            const int n_kv = it.n_kv;
             const int my_row = pf_row(it, sh, w, r);             // where this thread's row of O goes (-1: nowhere)
-            if (!SPLIT && w >= it.n_act) { g += n_kv; continue; }        // (the last unit of a sequence may have one tile)
-            if (!SPLIT && n_kv == 0) {
+            if (w >= it.n_act) { g += n_kv; continue; }        // (the last unit of a sequence may have one tile)
+            if (n_kv == 0) {
                 if (my_row >= 0)
                     for (int i = 0; i < kHeadDim; i += 4) *reinterpret_cast<float4*>(O + (size_t)my_row * kHeadDim + i) = make_float4(0.f, 0.f, 0.f, 0.f);
                 continue;
@@ -441,10 +383,10 @@ mqa_prefill_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
             const int lim_first = min(it.raw + p0 + 1, it.L);            // rows the tile's first position sees
             const int lim = min(it.raw + min(p0 + r % sh.positions, sh.n - 1) + 1, it.L);   // rows this thread's position sees: >= 1
             float m = -INFINITY, l = 0.f;                        // reference maximum (log2 units), sum of weights
-            const int n_own = w == 0 ? count_stages0(it) : w < it.n_act ? n_kv : 0;      // stages of this tile
+            const int n_own = w == 0 ? it.n_kv0 : n_kv;                                  // stages of this tile
             const bool clears = w == (it.n_kv0 == it.n_kv ? 0 : 1);                      // the first tile to see the unit's last stage
             for (int j = 0; j < n_own; ++j) {
-                const int k0 = (first + j) * kPfRows;
+                const int k0 = j * kPfRows;
                 if (ok) ok = mbar_wait(s_ready + 8 * w, n_s & 1);
                 ++n_s;
                 tc_fence_after();
@@ -553,29 +495,6 @@ mqa_prefill_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
                     l += s0 + s1;
                 }
             }
-            if (SPLIT) {
-                // ---- this CTA's share: (maximum, sum) and rows of O into shared memory (the K and V rings, once both tiles'
-                // products are done), 16-byte pieces swizzled by row
-                if (n_p > 0 && ok) ok = mbar_wait(pv_done + 8 * w, (n_p - 1) & 1);
-                tc_fence_after();
-                named_barrier(1, 256);
-                asm volatile("st.shared.v2.f32 [%0], {%1,%2};" ::"r"(out_s + (w * 128 + r) * 8), "f"(m), "f"(l) : "memory");
-                if (n_p > 0) {
-                    const uint32_t ex_o = k_ring + (w * 128 + r) * 512;
-                    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");       // (the rings were the copy engine's and the tensor core's)
-#pragma unroll
-                    for (int c = 0; c < 4; ++c) {
-                        uint32_t y[32];
-                        tmem_ld32(o_t + c * 32, y);
-                        tmem_wait_ld();
-#pragma unroll
-                        for (int i = 0; i < 8; ++i)
-                            asm volatile("st.shared.v4.b32 [%0], {%1,%2,%3,%4};" ::"r"(ex_o + (((c * 8 + i) ^ (r & 31)) << 4)), "r"(y[4 * i]),
-                                         "r"(y[4 * i + 1]), "r"(y[4 * i + 2]), "r"(y[4 * i + 3]) : "memory");
-                    }
-                }
-                break;
-            }
             // ---- the row of O, divided by the sum of its weights
             if (ok) ok = mbar_wait(pv_done + 8 * w, (n_p - 1) & 1);
             tc_fence_after();
@@ -607,16 +526,409 @@ mqa_prefill_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
             g += n_kv;
         }
         if (!ok) atomicExch(&timed_out, 1);
-        if (SPLIT) {
-            // (in here, where a thread has the registers for it)
-            cluster_sync();                                      // every CTA's rows are in its shared memory
-            const PfItem it = pf_item((int)blockIdx.x / ctas, start, sh);
-            if (ctas == 2) pf_merge<2>(it, sh, O, out_s, k_ring, warp + 8 * rank, lane);
-            else if (ctas == 4) pf_merge<4>(it, sh, O, out_s, k_ring, warp + 8 * rank, lane);
-            else pf_merge<8>(it, sh, O, out_s, k_ring, warp + 8 * rank, lane);
+    }
+    tc_fence_before();
+    __syncthreads();
+    if (warp == kPfSWarp) {
+        tc_fence_after();
+        tmem_dealloc(tmem_base, 512);
+    }
+    if (threadIdx.x == 0 && timed_out && status) atomicOr(status, kStatusPipelineTimeout);
+}
+
+// ---- Few tiles (a chunk of a prompt, short prompts, few sequences): ONE tile per CTA, so that twice as many SMs work, and the two
+// softmax warpgroups take its stages in turn (warpgroup w: stages w, w + 2, ...), each with weights, an O accumulator, reference
+// maxima and sums of its own, merged on the way out -- the order of work of the many-rows step (decode_wide.cuh), under the mask of
+// Section 2.3.  A cluster of 2, 4 or 8 CTAs shares a tile's stages where there are SMs for it, each a run of them; their partial
+// results go straight to the CTA that merges them (128 / CTAs rows each), from the merge of the warpgroups into its V ring.
+// (Before it the two tiles of a unit stayed together and a cluster shared the unit: its rows of O went into shared memory and were
+// read from there by remote loads, 24 KB/us, 7 us in all after the last product.)  A stage takes 0.72 us (1.05 with two roundings of
+// the weights), half of what it takes for two tiles, and 8 us are around them.  us per call: 5 x 9 heads x 333 positions over up to 3000
+// rows 28.5 -> 25.5; 8 x 8 x 256 over 900 22.1 -> 16.7; 4 x 23 x 115 over 1682 24.6 -> 18.1; 1 x 8 x 1000 17.3 -> 16.1.
+constexpr int kPtKSlots = 3, kPtVSlots = 3;
+// barriers: q_full, k_full/k_empty, v_full/v_empty per slot, s_ready[2], p_ready[2], pv_done[2], s_free, recv
+constexpr int kPtBarriers = 1 + 2 * kPtKSlots + 2 * kPtVSlots + 6 + 2;
+constexpr int kPtSmemBytes = (1 + kPtKSlots + kPtVSlots) * kPfTileBytes + kPtBarriers * 8 + 16 + 1024 /* alignment slack */;
+static_assert(kPtSmemBytes + kPfRows * 12 + 16 /* static */ <= 227 * 1024, "exceeds the shared memory of one SM");
+
+__global__ void __launch_bounds__(kPfThreads, 1)
+mqa_prefill_tile_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CUtensorMap map_k,
+                        const __grid_constant__ CUtensorMap map_v, const int32_t* start, float* __restrict__ O,
+                        int32_t* __restrict__ status, const PfShape sh) {
+    const int warp = __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0), lane = threadIdx.x & 31;
+    const int ctas = (int)cluster_size(), rank = (int)cluster_cta_rank(), item = (int)blockIdx.x / ctas;
+    const int per = kPfRows / ctas;                              // rows that each CTA of the cluster merges
+
+    extern __shared__ uint8_t smem_raw[];
+    uint8_t* base = smem_raw + ((1024u - (smem_addr(smem_raw) & 1023u)) & 1023u);     // the 128-byte swizzle repeats every 1 KiB
+    const uint32_t q_s = smem_addr(base);
+    const uint32_t k_ring = q_s + kPfTileBytes, v_ring = k_ring + kPtKSlots * kPfTileBytes, bars = v_ring + kPtVSlots * kPfTileBytes;
+    const uint32_t q_full = bars, k_full = bars + 8, k_empty = k_full + 8 * kPtKSlots, v_full = k_empty + 8 * kPtKSlots,
+                   v_empty = v_full + 8 * kPtVSlots, s_ready = v_empty + 8 * kPtVSlots, p_ready = s_ready + 16, pv_done = p_ready + 16,
+                   s_free = pv_done + 16, recv_bar = s_free + 8;
+    const uint32_t recv_ml = v_ring + kPfRows * 512;             // (the rows that come lie where the first two V slots were)
+    uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(base + (1 + kPtKSlots + kPtVSlots) * kPfTileBytes + kPtBarriers * 8);
+    __shared__ int timed_out, ex_row[kPfRows];                   // where each row of O goes (-1: nowhere)
+    __shared__ float2 ex_ml[kPfRows];                            // (maximum, sum) of warpgroup 1's rows, then each row's two factors
+
+    if (threadIdx.x == 0) {
+        prefetch_tensormap(&map_q); prefetch_tensormap(&map_k); prefetch_tensormap(&map_v);
+        mbar_init(q_full, 1);
+        mbar_init(s_free, 4);
+        for (int i = 0; i < kPtKSlots; ++i) { mbar_init(k_full + 8 * i, 1); mbar_init(k_empty + 8 * i, 1); }
+        for (int i = 0; i < kPtVSlots; ++i) { mbar_init(v_full + 8 * i, 1); mbar_init(v_empty + 8 * i, 1); }
+        for (int w = 0; w < 2; ++w) { mbar_init(s_ready + 8 * w, 1); mbar_init(p_ready + 8 * w, 4); mbar_init(pv_done + 8 * w, 1); }
+        mbar_init(recv_bar, 1);
+        timed_out = 0;
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+        mbar_expect_tx(recv_bar, (uint32_t)((ctas - 1) * per * (kHeadDim * 4 + 8)));
+    }
+    if (warp == kPfSWarp) {
+        tmem_alloc(smem_addr(tmem_slot), 512);
+        tmem_relinquish();
+    }
+    // the tile: everything but where its sequence starts is known ahead of the wait
+    const int seq = (item / sh.group) % sh.b, tile = sh.n_units - 1 - (item / (sh.group * sh.b) * sh.group + item % sh.group);
+    const int p0 = pf_position(sh, tile), head0 = pf_head(sh, tile);
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
+    const uint32_t tmem_base = __shfl_sync(0xffffffffu, *tmem_slot, 0);
+    grid_dependency_wait();              // Q, K, V and start may come from the kernel before
+    grid_launch_dependents();
+    const int raw = start ? min(__ldcg(start + seq), sh.m_max) : 0;
+    if (start && threadIdx.x < 32) {
+        // a start that is negative or leaves too little room is flagged once (its rows are zeros, or the memory is cut at m_max)
+        bool bad = false;
+        for (int i = blockIdx.x * 32 + threadIdx.x; i < sh.b; i += gridDim.x * 32) {
+            const int first = __ldcg(start + i);
+            bad = bad || first < 0 || first > sh.m_max - sh.n;
+        }
+        if (bad && status) atomicOr(status, kStatusLenClamped);
+    }
+    const int L = min(raw + min(p0 + sh.positions, sh.n), sh.m_max);     // rows of the memory that the tile's last position sees
+    const int n_all = raw < 0 || L <= 0 ? 0 : (L + kPfRows - 1) / kPfRows;
+    const int first = rank * n_all / ctas, n_kv = __shfl_sync(0xffffffffu, (rank + 1) * n_all / ctas - first, 0);   // this CTA's stages
+    // (two roundings of the weights: as pf_item says)
+    const bool hilo = __any_sync(0xffffffffu, min(raw + min((p0 & ~(kPfRows - 1)) + kPfRows, sh.n), sh.m_max) < kSingleRoundingMinRows);
+
+    if (warp >= 8) {
+        asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(kPfRegsOther));
+        if (warp == kPfProducerWarp) {
+            // =========================================================== TMA producer: a box per lane
+            bool ok = true;
+            int issued_k = 0, issued_v = 0;
+            // (for tests: CTA 0 never starts one copy of its second stage, or of its only one)
+            const bool withhold = blockIdx.x == 0 && test_withhold();
+            if (n_kv > 0) {
+                if (lane == 0) mbar_expect_tx(q_full, sh.positions * sh.heads * kRowBytes);
+                if (lane < 2) tma_load_3d(q_s + lane * kPfHalfBytes, &map_q, lane * kBoxCols, p0, seq * sh.h + head0, q_full);
+            }
+            for (int j = 0; j < n_kv; ++j) {
+                const int y = seq * sh.m_max + (first + j) * kPfRows, ks = j % kPtKSlots, vs = j % kPtVSlots;
+                if (j >= kPtKSlots) ok = warp_wait(k_empty + 8 * ks, ((j / kPtKSlots) - 1) & 1);
+                if (!ok) break;
+                if (lane == 0) mbar_expect_tx(k_full + 8 * ks, kPfTileBytes);
+                if (lane < 2) tma_load_2d(k_ring + ks * kPfTileBytes + lane * kPfHalfBytes, &map_k, lane * kBoxCols, y, k_full + 8 * ks);
+                issued_k = j + 1;
+                if (j >= kPtVSlots) ok = warp_wait(v_empty + 8 * vs, ((j / kPtVSlots) - 1) & 1);
+                if (!ok) break;
+                if (lane == 0) mbar_expect_tx(v_full + 8 * vs, kPfTileBytes);
+                if (lane < 2 && !(withhold && lane == 1 && j == min(1, n_kv - 1)))
+                    tma_load_2d(v_ring + vs * kPfTileBytes + lane * kPfHalfBytes, &map_v, lane * kBoxCols, y, v_full + 8 * vs);
+                issued_v = j + 1;
+            }
+            if (!ok) {
+                // a wait ran out: the copies already started are given a bounded wait each before the CTA may leave
+                if (lane == 0) atomicExch(&timed_out, 1);
+                mbar_wait(q_full, 0);
+                for (int j = max(0, issued_k - kPtKSlots); j < issued_k; ++j) mbar_wait(k_full + 8 * (j % kPtKSlots), (j / kPtKSlots) & 1);
+                for (int j = max(0, issued_v - kPtVSlots); j < issued_v; ++j) mbar_wait(v_full + 8 * (j % kPtVSlots), (j / kPtVSlots) & 1);
+            }
+        } else if (warp == kPfSWarp) {
+            // =========================================================== issuer of the logits, each stage as soon as the one before is
+            // in registers
+            constexpr uint32_t kIdescS = umma_idesc(128, 128, false, false);
+            bool ok = n_kv == 0 || warp_wait(q_full, 0);
+            for (int j = 0; j < n_kv && ok; ++j) {
+                const int slot = j % kPtKSlots;
+                ok = warp_wait(k_full + 8 * slot, (j / kPtKSlots) & 1);
+                if (ok && j > 0) ok = warp_wait(s_free, (j - 1) & 1);
+                if (!ok) break;
+                const uint32_t k_s = k_ring + slot * kPfTileBytes;
+                tc_fence_after();
+                if (elect_one()) {
+#pragma unroll
+                    for (int ks = 0; ks < 8; ++ks) {             // 8 k-steps of 16 columns; 4 per 64-column box
+                        const uint32_t off = (ks >> 2) * kPfHalfBytes + (ks & 3) * 32;
+                        umma_ss(tmem_base, umma_desc(q_s + off, 16, 1024), umma_desc(k_s + off, 16, 1024), kIdescS, ks ? 1u : 0u);
+                    }
+                    tc_commit(s_ready + 8 * (j & 1));
+                    tc_commit(k_empty + 8 * slot);
+                }
+                __syncwarp();
+            }
+            if (!ok && lane == 0) atomicExch(&timed_out, 1);
+        } else if (warp == kPfPvWarp) {
+            // =========================================================== issuer of O_w += P_w V_j, in two parts where the weights have a hi
+            // and a lo one
+            constexpr uint32_t kIdescO = umma_idesc(128, 128, false, true);
+            const int parts = hilo ? 2 : 1;
+            bool ok = true;
+            int n_p[2] = {0, 0};
+            for (int j = 0; j < n_kv && ok; ++j) {
+                const int slot = j % kPtVSlots, w = j & 1;
+                const uint32_t v_s = v_ring + slot * kPfTileBytes;
+                ok = warp_wait(v_full + 8 * slot, (j / kPtVSlots) & 1);
+                for (int part = 0; part < parts && ok; ++part) {
+                    ok = warp_wait(p_ready + 8 * w, n_p[w] & 1);
+                    if (!ok) break;
+                    ++n_p[w];
+                    tc_fence_after();
+                    if (elect_one()) {
+                        const uint32_t v_p = v_s + part * 4 * 2048;
+#pragma unroll
+                        for (int kk = 0; kk < 8; ++kk)
+                            umma_ts(tmem_base + kPfTmemO + w * 128, tmem_base + kPfTmemP + w * 64 + kk * 8,
+                                    umma_desc(v_p + (parts == 2 ? kk & 3 : kk) * 2048, kPfHalfBytes, 1024), kIdescO, (j < 2 && part == 0 && kk == 0) ? 0u : 1u);
+                        tc_commit(pv_done + 8 * w);
+                        if (part == parts - 1) tc_commit(v_empty + 8 * slot);
+                    }
+                    __syncwarp();
+                }
+            }
+            if (!ok && lane == 0) atomicExch(&timed_out, 1);
+        }
+        if (ctas > 1) {                      // (as the softmax warps do)
+            cluster_sync();
+            cluster_arrive_relaxed();
+            cluster_wait();
+        }
+    } else {
+        asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(kPfRegsSoftmax));
+        // =============================================================== softmax warpgroups: one thread per query row
+        const int w = warp >> 2, quarter = warp & 3, r = quarter * 32 + lane;
+        const uint32_t lane_base = tmem_base + ((uint32_t)(quarter * 32) << 16);
+        const uint32_t p_t = lane_base + kPfTmemP + w * 64, o_t = lane_base + kPfTmemO + w * 128;
+        const int hh = r / sh.positions, pos = p0 + r - hh * sh.positions;
+        const bool mine = hh < sh.heads && head0 + hh < sh.h && pos < sh.n;
+        const int lim_first = min(raw + p0 + 1, L), lim = min(raw + min(pos, sh.n - 1) + 1, L);      // rows the tile's first position sees, and this thread's: >= 1
+        if (w == 0) ex_row[r] = mine ? (seq * sh.h + head0 + hh) * sh.n + pos : -1;
+        float m = -INFINITY, l = 0.f;                            // reference maximum (log2 units), sum of weights
+        bool ok = true;
+        int n_p = 0;
+        for (int j = w; j < n_kv; j += 2) {
+            const int k0 = (first + j) * kPfRows;
+            if (ok) ok = mbar_wait(s_ready + 8 * w, (j >> 1) & 1);
+            tc_fence_after();
+            // ---- the row's 128 logits, read once and kept in registers; the mask by index, as a select
+            uint32_t x[128];
+            tmem_ld_cols<128>(lane_base, x);
+            tmem_wait_ld();
+            tc_fence_before();
+            __syncwarp();
+            if (lane == 0) mbar_arrive(s_free);                  // the next stage's logits may take their place
+            if (k0 + kPfRows > lim_first) {
+#pragma unroll
+                for (int i = 0; i < 128; ++i)
+                    if (k0 + i >= lim) x[i] = 0xff800000u;       // -inf
+            }
+            float mx8[8];
+#pragma unroll
+            for (int i = 0; i < 8; ++i) mx8[i] = fmaxf(__uint_as_float(x[2 * i]), __uint_as_float(x[2 * i + 1]));
+#pragma unroll
+            for (int i = 8; i < 64; ++i) mx8[i & 7] = max3(mx8[i & 7], __uint_as_float(x[2 * i]), __uint_as_float(x[2 * i + 1]));
+            const float mx = max3(max3(mx8[0], mx8[1], mx8[2]), max3(mx8[3], mx8[4], mx8[5]), fmaxf(mx8[6], mx8[7])) * kLog2e;
+            if (__any_sync(0xffffffffu, mine && mx > m + kPfMaxLead)) {      // (rows that are nobody's do not count)
+                const float m_new = fmaxf(m, mx);
+                if (n_p > 0) {
+                    const float f = m == m_new ? 1.f : fast_exp2(m - m_new);
+                    l *= f;
+                    if (ok) ok = mbar_wait(pv_done + 8 * w, (n_p - 1) & 1);  // O holds the warpgroup's stages before this one
+                    tc_fence_after();
+#pragma unroll 1
+                    for (int c = 0; c < 16; ++c) {
+                        uint32_t y[8];
+                        tmem_ld8(o_t + c * 8, y);
+                        tmem_wait_ld();
+#pragma unroll
+                        for (int i = 0; i < 8; ++i) y[i] = __float_as_uint(__uint_as_float(y[i]) * f);
+                        tmem_st8(o_t + c * 8, y);
+                    }
+                }
+                m = m_new;
+            }
+            const float neg_m = m == -INFINITY ? 0.f : -m;       // (nothing seen yet, or logits of -inf: weights of zero)
+            const unsigned long long neg_m2 = f2_pack(neg_m, neg_m), log2e2 = f2_pack(kLog2e, kLog2e);
+            unsigned long long sum2[2] = {0ull, 0ull};
+            if (L < k0 + kPfRows) {
+                // the tile's last stage runs past its memory: those V rows are cleared, zero weights or not (NaN * 0 = NaN)
+                const int vs = j % kPtVSlots;
+                if (ok) ok = mbar_wait(v_full + 8 * vs, (j / kPtVSlots) & 1);
+                for (int i = r; i < (k0 + kPfRows - L) * 16; i += 128) {
+                    const int vrow = L - k0 + (i >> 4), ch = i & 15;
+                    const uint32_t a = v_ring + vs * kPfTileBytes + (ch >> 3) * kPfHalfBytes + vrow * 128 + ((ch & 7) << 4);
+                    asm volatile("st.shared.v4.b32 [%0], {%1,%1,%1,%1};" ::"r"(a), "r"(0u) : "memory");
+                }
+                asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+            }
+            // the weights stay in registers until the product before has read the ones in tensor memory
+            auto give = [&](const uint32_t (&p_0)[32], const uint32_t (&p_1)[32]) {
+                if (n_p > 0 && ok) ok = mbar_wait(pv_done + 8 * w, (n_p - 1) & 1);
+                tc_fence_after();
+                tmem_st32(p_t, p_0);
+                tmem_st32(p_t + 32, p_1);
+                tmem_wait_st();
+                tc_fence_before();
+                __syncwarp();
+                if (lane == 0) mbar_arrive(p_ready + 8 * w);
+                ++n_p;
+            };
+            if (hilo) {
+#pragma unroll
+                for (int half = 0; half < 2; ++half) {
+                    uint32_t hi[32], lo[32];
+#pragma unroll
+                    for (int i = 0; i < 32; ++i) {
+                        float a0, a1;
+                        f2_unpack(f2_fma(f2_pack(__uint_as_float(x[64 * half + 2 * i]), __uint_as_float(x[64 * half + 2 * i + 1])), log2e2, neg_m2), a0, a1);
+                        const float pa = fast_exp2(a0), pb = fast_exp2(a1);
+                        sum2[i & 1] = f2_add(sum2[i & 1], f2_pack(pa, pb));
+                        hi[i] = pack_bf16(pa, pb);
+                        lo[i] = pack_bf16(pa - bf16_lo(hi[i]), pb - bf16_hi(hi[i]));
+                    }
+                    give(hi, lo);
+                }
+            } else {
+                uint32_t hi[2][32];
+#pragma unroll
+                for (int i = 0; i < 64; ++i) {
+                    float a0, a1;
+                    f2_unpack(f2_fma(f2_pack(__uint_as_float(x[2 * i]), __uint_as_float(x[2 * i + 1])), log2e2, neg_m2), a0, a1);
+                    const float pa = fast_exp2(a0), pb = fast_exp2(a1);
+                    sum2[i & 1] = f2_add(sum2[i & 1], f2_pack(pa, pb));
+                    hi[i >> 5][i & 31] = pack_bf16(pa, pb);
+                }
+                give(hi[0], hi[1]);
+            }
+            {
+                float s0, s1;
+                f2_unpack(f2_add(sum2[0], sum2[1]), s0, s1);
+                l += s0 + s1;
+            }
+        }
+        if (n_p > 0 && ok) ok = mbar_wait(pv_done + 8 * w, (n_p - 1) & 1);
+        // (Q and the K ring are used below: a last stage that is the other warpgroup's must have its logits.  That warpgroup's logits
+        // before those were ready before this one's last ones were issued, so the wait cannot be a phase early)
+        if (n_p > 0 && n_kv > 1 && ((n_kv - 1) & 1) != w && ok) ok = mbar_wait(s_ready + 8 * (w ^ 1), ((n_kv - 1) >> 1) & 1);
+        tc_fence_after();
+        if (!ok) atomicExch(&timed_out, 1);
+        // ---- each warpgroup leaves its rows of O in shared memory (where Q and the K ring were, 16-byte pieces swizzled by row)
+        if (w == 1) ex_ml[r] = make_float2(m, l);
+        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");         // (it was the copy engine's and the tensor core's; so was the V ring)
+        if (n_p > 0) {
+            const uint32_t ex_o = q_s + (w * kPfRows + r) * 512;
+#pragma unroll
+            for (int c = 0; c < 4; ++c) {
+                uint32_t y[32];
+                tmem_ld32(o_t + c * 32, y);
+                tmem_wait_ld();
+#pragma unroll
+                for (int i = 0; i < 8; ++i)
+                    asm volatile("st.shared.v4.b32 [%0], {%1,%2,%3,%4};" ::"r"(ex_o + (((c * 8 + i) ^ (r & 31)) << 4)), "r"(y[4 * i]), "r"(y[4 * i + 1]),
+                                 "r"(y[4 * i + 2]), "r"(y[4 * i + 3]) : "memory");
+            }
+        }
+        named_barrier(1, 256);                                   // (all of this CTA's products are done)
+        if (ctas > 1) cluster_sync();                            // every CTA's V ring may be written
+        if (w == 0) {
+            // what each warpgroup's sums count for (-1: nothing, and its row may never have been written.  A share of logits that are
+            // all -inf, or of which the row sees nothing, has a sum of 0; the maximum does not tell, that of NaN logits is -inf too)
+            const float2 other = ex_ml[r];
+            const bool one = n_kv > 0 && l != 0.f, two = n_kv > 1 && other.y != 0.f;
+            const float top = fmaxf(one ? m : -INFINITY, two ? other.x : -INFINITY);
+            float f0 = !one ? -1.f : m == top ? 1.f : fast_exp2(m - top), f1 = !two ? -1.f : other.x == top ? 1.f : fast_exp2(other.x - top);
+            const float sum = (one ? f0 * l : 0.f) + (two ? f1 * other.y : 0.f);
+            if (ctas == 1) {
+                const float scale = n_all > 0 ? 1.f / sum : 0.f;
+                if (one) f0 *= scale;
+                if (two) f1 *= scale;
+                if (!one && !two && n_all > 0) f0 = sum * scale;             // (nothing but logits of -inf: 0 / 0)
+            } else {
+                const int to = r / per;
+                const uint32_t at = recv_ml + (rank * per + r - to * per) * 8;
+                if (to == rank) asm volatile("st.shared.v2.f32 [%0], {%1,%2};" ::"r"(at), "f"(top), "f"(sum) : "memory");
+                else cluster_send_f2(cluster_map(at, to), make_float2(top, sum), cluster_map(recv_bar, to));
+            }
+            ex_ml[r] = make_float2(f0, f1);
+        }
+        named_barrier(2, 256);
+        // ---- whole rows, merged by a warp each on the way out: 512 contiguous bytes
+        const float4* rows = reinterpret_cast<const float4*>(base);
+#pragma unroll 4
+        for (int i = 0; i < kPfRows / 8; ++i) {
+            const int row = warp + 8 * i, to_row = ex_row[row];
+            float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+            if (to_row >= 0) {
+                const float2 f = ex_ml[row];
+                if (f.x >= 0.f || f.x != f.x) {
+                    const float4 a = n_kv > 0 ? rows[row * 32 + (lane ^ (row & 31))] : v;
+                    v = make_float4(a.x * f.x, a.y * f.x, a.z * f.x, a.w * f.x);
+                }
+                if (f.y >= 0.f || f.y != f.y) {
+                    const float4 a = rows[(kPfRows + row) * 32 + (lane ^ (row & 31))];
+                    v.x = fmaf(a.x, f.y, v.x); v.y = fmaf(a.y, f.y, v.y); v.z = fmaf(a.z, f.y, v.z); v.w = fmaf(a.w, f.y, v.w);
+                }
+            }
+            if (ctas == 1) {
+                if (to_row >= 0) reinterpret_cast<float4*>(O + (size_t)to_row * kHeadDim)[lane] = v;
+            } else {
+                const int to = row / per;
+                const uint32_t at = v_ring + (rank * per + row - to * per) * 512 + lane * 16;
+                if (to == rank) asm volatile("st.shared.v4.f32 [%0], {%1,%2,%3,%4};" ::"r"(at), "f"(v.x), "f"(v.y), "f"(v.z), "f"(v.w) : "memory");
+                else cluster_send_f4(cluster_map(at, to), v, cluster_map(recv_bar, to));
+            }
+        }
+        if (ctas > 1) {
+            cluster_arrive_relaxed();                            // (this CTA's rows are on their way)
+            named_barrier(1, 256);                               // its own are in place
+            const bool got = mbar_wait(recv_bar, 0);
+            for (int i = warp; i < per; i += 8) {
+                const int to_row = ex_row[rank * per + i];
+                if (to_row < 0) continue;
+                float2 ml[kPfMaxSplit];
+                float4 part[kPfMaxSplit];
+                float top = -INFINITY, den = 0.f;
+                float4 num = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+                for (int c = 0; c < kPfMaxSplit; ++c) {
+                    if (c >= ctas) break;
+                    asm volatile("ld.shared.v2.f32 {%0,%1}, [%2];" : "=f"(ml[c].x), "=f"(ml[c].y) : "r"(recv_ml + (c * per + i) * 8) : "memory");
+                    asm volatile("ld.shared.v4.f32 {%0,%1,%2,%3}, [%4];" : "=f"(part[c].x), "=f"(part[c].y), "=f"(part[c].z), "=f"(part[c].w)
+                                 : "r"(v_ring + (c * per + i) * 512 + lane * 16) : "memory");
+                    top = fmaxf(top, ml[c].x);
+                }
+#pragma unroll
+                for (int c = 0; c < kPfMaxSplit; ++c) {
+                    if (c >= ctas) break;
+                    if (ml[c].y == 0.f) continue;                // (nothing of this share counts: see above)
+                    const float f = ml[c].x == top ? 1.f : fast_exp2(ml[c].x - top);
+                    den = fmaf(f, ml[c].y, den);
+                    num.x = fmaf(f, part[c].x, num.x); num.y = fmaf(f, part[c].y, num.y);
+                    num.z = fmaf(f, part[c].z, num.z); num.w = fmaf(f, part[c].w, num.w);
+                }
+                const float inv = n_all > 0 ? 1.f / den : 0.f;
+                reinterpret_cast<float4*>(O + (size_t)to_row * kHeadDim)[lane] = make_float4(num.x * inv, num.y * inv, num.z * inv, num.w * inv);
+            }
+            cluster_wait();                                      // everybody's rows have been sent
+            if (!got) {
+                // a wait ran out: what is still on its way here gets another bounded one before this CTA's shared memory goes
+                mbar_wait(recv_bar, 0);
+                if (lane == 0) atomicExch(&timed_out, 1);
+            }
         }
     }
-    if (SPLIT) cluster_sync();           // nobody leaves while its shared memory is being read
     tc_fence_before();
     __syncthreads();
     if (warp == kPfSWarp) {

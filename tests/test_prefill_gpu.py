@@ -135,6 +135,17 @@ def test_tile_shapes_and_shared_units(b, h, n, m_max, start):
     run(b, h, n, m_max, start, seed=b + 3 * h + n)
 
 
+@pytest.mark.parametrize("b,h,n,m_max,start", [
+    # one tile to a CTA, its stages in turn between the warpgroups and between 1, 2, 4 and 8 CTAs: one stage and two, an odd number, CTAs
+    # that get none, rows that see nothing of a CTA's run, a last stage of one row, tiles of several heads partly filled
+    (3, 9, 128, 128, None), (2, 5, 129, 257, [128, 0]), (6, 20, 100, 640, [540, 0, 28, 412, 413, 29]), (1, 1, 1, 1, None), (1, 3, 1, 3000, [2999]),
+    (30, 4, 128, 1500, list(range(0, 1350, 45))), (9, 8, 256, 513, [257, 256, 0, 1, 100, 127, 128, 129, 200]), (1, 2, 640, 4000, [3200]),
+    (1, 148, 2, 64, [62]),
+])
+def test_one_tile_to_a_cta(b, h, n, m_max, start):
+    run(b, h, n, m_max, start, seed=2 * b + h + n)
+
+
 def test_shared_units_with_a_negative_start_and_one_past_the_memory():
     """The same units shared by a cluster: nothing to look at gives zeros, a memory that would pass m_max is cut there."""
     b, h, n, m_max = 3, 4, 16, 2064
