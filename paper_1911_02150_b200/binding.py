@@ -8,6 +8,7 @@ no fallback: if the library is missing or was not built, importing a symbol rais
 from __future__ import annotations
 
 import ctypes
+import importlib.util
 import os
 from typing import Optional
 
@@ -96,6 +97,25 @@ def lib() -> ctypes.CDLL:
         L.mqa_status_string.restype = ctypes.c_char_p
         _lib = L
     return _lib
+
+
+_native = None
+
+
+def _checked():
+    """The wrappers' native half (csrc/checked_call.cpp): its functions check a call's tensors and make the call, or return None, with
+    nothing enqueued, where a tensor is not plainly what the call takes; the wrapper's own checks then say what is wrong."""
+    global _native
+    if _native is None:
+        lib()
+        path = os.path.join(_PKG, "checked_call.so")
+        if not os.path.exists(path):
+            raise ImportError(f"{path} is missing: build it with `python -m paper_1911_02150_b200.build`")
+        spec = importlib.util.spec_from_file_location("checked_call", path)
+        module = importlib.util.module_from_spec(spec)
+        spec.loader.exec_module(module)
+        _native = module
+    return _native
 
 
 def status_string(code: int) -> str:
@@ -201,6 +221,9 @@ def kv_cache_append(K, V, k_new, v_new, lens, advance: bool = True, status=None,
     ``K``/``V``: ``[b,m_max,128]`` (multi-query) or ``[b,kv_heads,m_max,128]`` (multi-head) bf16;
     ``k_new``/``v_new``: ``[b,128]`` or ``[b,kv_heads,128]``; ``lens``: int32 ``[b]``, advanced by one
     on the device when ``advance``."""
+    rc = (_native or _checked()).kv_cache_append(K, V, k_new, v_new, lens, advance, status, None if stream is None else stream.cuda_stream)
+    if rc is not None:
+        return _check(rc, "kv_cache_append")
     if K.dim() == 3:
         b, m_max, k = K.shape
         kvh = 1
@@ -222,6 +245,11 @@ def kv_cache_append(K, V, k_new, v_new, lens, advance: bool = True, status=None,
 
 
 def _step(name: str, multi_query: bool, q, K, V, lens, o, workspace, status, stream, phase: str):
+    if phase == "step":
+        rc = getattr(_native or _checked(), name)(q, K, V, lens, o, workspace, status, None if stream is None else stream.cuda_stream)
+        if rc is not None:
+            _check(rc, name)
+            return o
     b, h, k = q.shape
     m_max, v = K.shape[-2], V.shape[-1]
     cache = (b, m_max) if multi_query else (b, h, m_max)
@@ -419,6 +447,10 @@ def mqa_prefill_attention(Q, K, V, O, workspace, start=None, status=None, stream
     """The attention lines of the batched multi-query function under the autoregressive mask: ``Q[b,h,n,k]`` bf16 over
     the shared ``K[b,m_max,k]``, ``V[b,m_max,v]``; query t of sequence b is memory position ``start[b] + t`` (``start``
     None: zeros) and attends over the rows up to its own; ``O[b,h,n,v]`` fp32 is written."""
+    rc = (_native or _checked()).mqa_prefill_attention(Q, K, V, start, O, workspace, status, None if stream is None else stream.cuda_stream)
+    if rc is not None:
+        _check(rc, "mqa_prefill_attention")
+        return O
     b, h, n, k = Q.shape
     m_max, v = K.shape[-2], V.shape[-1]
     _need(Q, torch.bfloat16, (b, h, n, k), "Q")

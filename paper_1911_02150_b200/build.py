@@ -16,6 +16,7 @@ import sys
 PKG = os.path.dirname(os.path.abspath(__file__))
 CSRC = os.path.join(PKG, "csrc")
 LIB = os.path.join(PKG, "libmqa_decode.so")
+CHECKED_CALL = os.path.join(PKG, "checked_call.so")      # the binding's native half (csrc/checked_call.cpp), linked to the library
 INCLUDE = os.path.join(os.path.dirname(PKG), "include")
 
 NVCC_FLAGS = [
@@ -33,26 +34,41 @@ def _nvcc() -> str:
     return exe
 
 
+def _build_checked_call() -> None:
+    import sysconfig
+    import torch
+    root = os.path.dirname(torch.__file__)
+    tmp = CHECKED_CALL + f".tmp{os.getpid()}"
+    subprocess.check_call(
+        ["g++", "-O2", "-shared", "-fPIC", "-std=c++17", f"-D_GLIBCXX_USE_CXX11_ABI={int(torch._C._GLIBCXX_USE_CXX11_ABI)}",
+         "-isystem", os.path.join(root, "include"), "-isystem", os.path.join(root, "include", "torch", "csrc", "api", "include"),
+         "-isystem", os.path.join(os.path.dirname(os.path.dirname(_nvcc())), "include"), "-I", sysconfig.get_paths()["include"],
+         os.path.join(CSRC, "checked_call.cpp"), "-o", tmp, "-L", PKG, "-l:" + os.path.basename(LIB), "-Wl,-rpath,$ORIGIN",
+         "-L", os.path.join(root, "lib"), "-ltorch_python", "-ltorch_cpu", "-lc10", "-lc10_cuda"])
+    os.replace(tmp, CHECKED_CALL)
+
+
 def sources():
     return sorted(glob.glob(os.path.join(CSRC, "*.cu")))
 
 
 def _stale() -> bool:
-    if not os.path.exists(LIB):
+    if not os.path.exists(LIB) or not os.path.exists(CHECKED_CALL):
         return True
-    t = os.path.getmtime(LIB)
+    t = min(os.path.getmtime(LIB), os.path.getmtime(CHECKED_CALL))
     deps = glob.glob(os.path.join(CSRC, "*")) + glob.glob(os.path.join(INCLUDE, "*.h")) + [__file__]
     return any(os.path.getmtime(d) > t for d in deps)
 
 
 def build_library(force: bool = False, verbose: bool = False) -> str:
-    """Compile every ``csrc/*.cu`` into one shared library for sm_100a; returns its path."""
+    """Compile every ``csrc/*.cu`` into one shared library for sm_100a, and the binding's native half; returns the library's path."""
     if not force and not _stale():
         return LIB
     tmp = LIB + f".tmp{os.getpid()}"
     cmd = [_nvcc()] + NVCC_FLAGS + (["-Xptxas", "-v"] if verbose else []) + ["-I", INCLUDE, "-o", tmp] + sources()
     subprocess.check_call(cmd)
     os.replace(tmp, LIB)
+    _build_checked_call()
     return LIB
 
 
