@@ -281,7 +281,8 @@ Plan make_plan(bool multi_query, int b, int h, int m_max) {
     double best_cost = us_full * us_ragged * gain * gain * launches(old);
     auto consider = [&](const Plan& p) {
         const size_t need = plan_workspace_bytes(p);
-        if (need > MQA_NOALLOC_SCRATCH_BYTES && need > plan_workspace_bytes(old)) return;      // (what the built-in scratch held it still holds)
+        // (what the built-in scratch held it still holds, and what took no workspace takes none)
+        if (need > plan_workspace_bytes(old) && (need > MQA_NOALLOC_SCRATCH_BYTES || plan_workspace_bytes(old) == 0)) return;
         const double full = plan_us(p, m_max, 1.0, sms), ragged = plan_us(p, m_max, 0.5, sms);
         if (full > us_full || ragged > us_ragged || full * ragged * launches(p) >= best_cost) return;
         best = p;

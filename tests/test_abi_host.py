@@ -81,6 +81,14 @@ def test_plan_and_workspace_are_consistent(L):
     assert binding.plan_splits(True, 1, 8, 0) == (0, 0)
 
 
+def test_sizes_that_take_no_workspace(L):
+    """Short caches, and many sequences of a few hundred rows, are whole splits and take no scratch, on either variant."""
+    for (b, h, m) in [(1, 8, 200), (30, 32, 255), (100, 17, 129), (384, 8, 256), (600, 4, 300)]:
+        assert binding.plan_splits(True, b, h, m)[0] == 1
+    for (b, h, m) in [(1, 1, 511), (3, 8, 300), (20, 4, 500)]:
+        assert binding.plan_splits(False, b, h, m)[0] == 1
+
+
 def test_bad_arguments_are_rejected_before_any_launch(L):
     vp = ctypes.c_void_p
     a = vp(0x1000)          # plausible, 16-byte aligned, never dereferenced on the host
