@@ -83,6 +83,11 @@ __device__ __forceinline__ void send_rows(uint32_t dst, uint32_t src, uint32_t b
     asm volatile("cp.async.bulk.shared::cluster.shared::cta.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
                  ::"r"(dst), "r"(src), "r"(bytes), "r"(bar) : "memory");
 }
+// Chunk (or head) c's stage of S, and how often that stage has been used before it.  (As many stages as chunks is the common case: no
+// division by a number that the compiler does not know, 0.2 us of a layer step.)
+__device__ __forceinline__ int stage_of(int c, int S) { return c < S ? c : c % S; }
+__device__ __forceinline__ int turn_of(int c, int S) { return c < S ? 0 : c / S; }
+
 struct SumShares {
     int rank, ctas, rows, per;            // rows: of the tile; per: of a CTA (the last ones may have fewer)
     __device__ __forceinline__ int count(int r) const { return max(0, min(per, rows - r * per)); }
@@ -135,13 +140,13 @@ project_in_kernel(const __grid_constant__ CUtensorMap map_pq, const __grid_const
     const CUtensorMap* wmap = slab < h ? &map_pq : (slab == h ? &map_pk : &map_pv);
     const int wrow0 = slab < h ? slab * d : 0;
     auto issue_weights = [&](int c) {
-        const uint32_t bar = full_s + (c % S) * 8, w_s = stages_s + (c % S) * Cfg::kStageBytes;
+        const uint32_t bar = full_s + stage_of(c, S) * 8, w_s = stages_s + stage_of(c, S) * Cfg::kStageBytes;
         mbar_expect_tx(bar, kProjChunkBytes);
         tma_load_2d(w_s, wmap, 0, wrow0 + (chunk0 + c) * 128, bar);
         tma_load_2d(w_s + kProjChunkBytes / 2, wmap, kBoxCols, wrow0 + (chunk0 + c) * 128, bar);
     };
     auto issue_x = [&](int c) {
-        const uint32_t bar = full_s + (c % S) * 8, x_s = stages_s + (c % S) * Cfg::kStageBytes + kProjChunkBytes;
+        const uint32_t bar = full_s + stage_of(c, S) * 8, x_s = stages_s + stage_of(c, S) * Cfg::kStageBytes + kProjChunkBytes;
         mbar_expect_tx(bar, Cfg::kActBytes);
         tma_load_2d(x_s, &map_x, (chunk0 + c) * 128, row0, bar);              // rows past b read as zero
         tma_load_2d(x_s + Cfg::kActBytes / 2, &map_x, (chunk0 + c) * 128 + kBoxCols, row0, bar);
@@ -175,7 +180,7 @@ project_in_kernel(const __grid_constant__ CUtensorMap map_pq, const __grid_const
             bool ok = true;
             for (int c = 0; c < n_chunks && ok; ++c) {
                 if (c >= S) {
-                    ok = mbar_wait(empty_s + (c % S) * 8, ((c / S) - 1) & 1);
+                    ok = mbar_wait(empty_s + stage_of(c, S) * 8, (turn_of(c, S) - 1) & 1);
                     if (!ok) break;
                     issue_weights(c);
                 }
@@ -188,8 +193,8 @@ project_in_kernel(const __grid_constant__ CUtensorMap map_pq, const __grid_const
             constexpr uint32_t kIdesc = umma_idesc(128, NB, true, false);
             bool ok = true;
             for (int c = 0; c < n_chunks; ++c) {
-                const int st = c % S;
-                if (ok) ok = mbar_wait(full_s + st * 8, (c / S) & 1);
+                const int st = stage_of(c, S);
+                if (ok) ok = mbar_wait(full_s + st * 8, turn_of(c, S) & 1);
                 tc_fence_after();
                 if (ok) {
                     const uint32_t w_s = stages_s + st * Cfg::kStageBytes, x_s = w_s + kProjChunkBytes;
@@ -272,7 +277,7 @@ project_out_kernel(const __grid_constant__ CUtensorMap map_po, const float* __re
     }
     if (warp == kProjMmaWarp) { tmem_alloc(smem_addr(&tmem_slot), Cfg::kTmemCols); tmem_relinquish(); }
     auto issue_weights = [&](int i) {
-        const int st = i % S;
+        const int st = stage_of(i, S);
         const uint32_t bar = w_full + st * 8, w_s = stages_s + st * Cfg::kStageBytes;
         mbar_expect_tx(bar, kProjChunkBytes);
         const int yrow = (head0 + i) * d + tile * 128;
@@ -296,7 +301,7 @@ project_out_kernel(const __grid_constant__ CUtensorMap map_po, const float* __re
         if (lane == 0) {
             bool ok = true;
             for (int i = S; i < n_heads && ok; ++i) {
-                ok = mbar_wait(empty_s + (i % S) * 8, ((i / S) - 1) & 1);
+                ok = mbar_wait(empty_s + stage_of(i, S) * 8, (turn_of(i, S) - 1) & 1);
                 if (ok) issue_weights(i);
             }
             if (!ok) atomicExch(&timed_out, 1);
@@ -306,9 +311,9 @@ project_out_kernel(const __grid_constant__ CUtensorMap map_po, const float* __re
             constexpr uint32_t kIdesc = umma_idesc(128, NB, false, false);
             bool ok = true;
             for (int i = 0; i < n_heads; ++i) {
-                const int st = i % S;
-                if (ok) ok = mbar_wait(w_full + st * 8, (i / S) & 1);
-                if (ok) ok = mbar_wait(o_full + st * 8, (i / S) & 1);
+                const int st = stage_of(i, S);
+                if (ok) ok = mbar_wait(w_full + st * 8, turn_of(i, S) & 1);
+                if (ok) ok = mbar_wait(o_full + st * 8, turn_of(i, S) & 1);
                 tc_fence_after();
                 if (ok) {
                     const uint32_t w_s = stages_s + st * Cfg::kStageBytes, o_s = w_s + kProjChunkBytes;
@@ -330,7 +335,7 @@ project_out_kernel(const __grid_constant__ CUtensorMap map_po, const float* __re
         // contiguous bytes per load); all of a head's loads are in flight before the first is converted.
         bool ok = true;
         for (int i = 0; i < n_heads; ++i) {
-            const int st = i % S;
+            const int st = stage_of(i, S);
             float4 v[NB / kProjWorkWarps];
 #pragma unroll
             for (int k = 0; k < NB / kProjWorkWarps; ++k) {
@@ -338,7 +343,7 @@ project_out_kernel(const __grid_constant__ CUtensorMap map_po, const float* __re
                 v[k] = make_float4(0.f, 0.f, 0.f, 0.f);
                 if (row0 + n < b) v[k] = __ldcg(reinterpret_cast<const float4*>(o + ((size_t)(row0 + n) * h + head0 + i) * kHeadDim + lane * 4));
             }
-            if (i >= S && ok) ok = mbar_wait(empty_s + st * 8, ((i / S) - 1) & 1);   // the product that read this tile is done
+            if (i >= S && ok) ok = mbar_wait(empty_s + st * 8, (turn_of(i, S) - 1) & 1);   // the product that read this tile is done
             const uint32_t o_s = stages_s + st * Cfg::kStageBytes + kProjChunkBytes + (lane >> 4) * (Cfg::kActBytes / 2) + (lane & 1) * 8;
 #pragma unroll
             for (int k = 0; k < NB / kProjWorkWarps; ++k) {
