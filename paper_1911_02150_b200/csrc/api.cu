@@ -74,8 +74,11 @@ struct Plan {
 bool dims_ok(int b, int h, int m_max) { return b > 0 && h > 0 && m_max > 0; }
 
 // Split plan for the CUDA-core kernel (one CTA per (unit, split)): enough CTAs to fill every
-// SM several times over, but never chunks shorter than 256 rows, and a single split (no
-// combine launch) when the cache is short.
+// SM several times over, but not chunks shorter than 256 rows, and a single split (no
+// combine launch) when the cache is short.  Where that leaves SMs short of the CTAs that fit them at once, chunks down to 128
+// rows, two rounds of a CTA's warps: us per append and step, 8 sequences x 1 head x 1000 rows 9.1 -> 6.3, 20 x 4 x 1000 13.7 -> 9.2,
+// 64 x 1 x 1000 13.6 -> 8.6, 8 x 1 x 8000 14.8 -> 12.7 (beyond a wave of CTAs shorter chunks lose: 20 x 4 x 2000 18.2 in 560 CTAs,
+// 19.9 in 1280).
 Plan plan_simt(int b, int h, int m_max) {
     Plan p;
     p.units = (size_t)b * h;
@@ -90,6 +93,15 @@ Plan plan_simt(int b, int h, int m_max) {
     chunk = (chunk + 63) / 64 * 64;
     p.chunk_rows = chunk;
     p.n_splits = (m_max + chunk - 1) / chunk;
+    const long at_once = (long)sm_count() * kSimtCtasPerSm;
+    if (p.n_splits > 1 && (long)p.units * p.n_splits < at_once) {
+        long more = at_once / (long)p.units;
+        if (more > (m_max + 127) / 128) more = (m_max + 127) / 128;
+        if (more > p.n_splits) {
+            p.chunk_rows = ((int)((m_max + more - 1) / more) + 63) / 64 * 64;
+            p.n_splits = (m_max + p.chunk_rows - 1) / p.chunk_rows;
+        }
+    }
     return p;
 }
 

@@ -23,7 +23,8 @@ constexpr int kSimtThreads = kSimtWarps * 32;
 constexpr int kSimtRowsPerIter = 16;   // rows one warp consumes per loop iteration
 
 // (six CTAs per SM: with 90 registers, which it takes if it may, there are five and 64 x 16 heads x 4096 rows take 333 us, not 321)
-__global__ void __launch_bounds__(kSimtThreads, 6)
+constexpr int kSimtCtasPerSm = 6;
+__global__ void __launch_bounds__(kSimtThreads, kSimtCtasPerSm)
 decode_split_simt_kernel(const uint4* q, const uint4* __restrict__ K,
                          const uint4* __restrict__ V, const int32_t* lens,
                          float* __restrict__ o, float2* __restrict__ part_ml,
