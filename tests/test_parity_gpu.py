@@ -467,3 +467,37 @@ def test_runs_on_a_side_stream():
         mqa.mqa_decode_step(inp["q"], inp["K"], inp["V"], lens_t, o, ws)
     s.synchronize()
     assert torch.equal(o.view(torch.int32), ref.view(torch.int32))
+
+
+def test_wrappers_by_their_native_half_and_by_their_own_checks():
+    """A tensor that is not plainly one (a subclass) goes through the wrapper's own checks, with the same result; what they refuse
+    stays refused, with nothing written."""
+    class Odd(torch.Tensor):
+        pass
+
+    b, h, m = 3, 5, 600
+    inp = wl.make_inputs(b, h, m, "mha", seed=3, device=DEV)
+    lens = torch.tensor([0, 599, 64], dtype=torch.int32, device=DEV)
+    ws, status = mqa.alloc_workspace(b, h, m, DEV), torch.zeros(1, dtype=torch.int32, device=DEV)
+    side = torch.cuda.Stream()
+    side.wait_stream(torch.cuda.current_stream())
+    outs = []
+    for odd, stream in ((False, None), (True, None), (False, side)):
+        n, o = lens.clone(), torch.full((b, h, 128), float("nan"), dtype=torch.float32, device=DEV)
+        torch.cuda.synchronize()
+        q = inp["q"].as_subclass(Odd) if odd else inp["q"]
+        mqa.kv_cache_append(inp["K"], inp["V"].as_subclass(Odd) if odd else inp["V"], inp["k_new"], inp["v_new"], n, status=status, stream=stream)
+        assert mqa.mha_decode_step(q, inp["K"], inp["V"], n, o, ws, status, stream) is o
+        torch.cuda.synchronize()
+        assert n.tolist() == [1, 600, 65]
+        outs.append(o.view(torch.int32))
+    assert torch.equal(outs[0], outs[1]) and torch.equal(outs[0], outs[2]) and int(status.item()) == 0
+    o = torch.zeros(b, h, 128, dtype=torch.float32, device=DEV)
+    for bad, error in ((inp["q"].float(), TypeError), (inp["q"].cpu(), TypeError), (inp["q"].transpose(0, 1).contiguous().transpose(0, 1), ValueError),
+                       (inp["q"][:2], ValueError)):
+        with pytest.raises(error):
+            mqa.mha_decode_step(bad, inp["K"], inp["V"], lens, o, ws, status)
+    with pytest.raises(mqa.MqaError):
+        mqa.mha_decode_step(inp["q"], inp["K"], inp["V"], lens, o, torch.empty(16, dtype=torch.uint8, device=DEV), status)
+    torch.cuda.synchronize()
+    assert float(o.abs().max()) == 0.0
