@@ -5,6 +5,7 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <algorithm>
 #include <atomic>
 #include <cmath>
 #include <cstdlib>
@@ -274,6 +275,7 @@ double plan_us(const Plan& p, int m_max, double full, int sms) {
 // where it takes a second launch and the other does not.
 // Measured against the plans by size over the sizes above: -13 % on average; us per step 16 x 16 heads x 1024 rows 11.3 -> 5.5,
 // 32 x 8 x 1024 8.9 -> 7.0, 48 x 8 x 1500 20.9 -> 10.1, 8 x 8 x 2048 8.1 -> 5.2, 64 x 8 x up to 2048 rows 18.0 -> 13.0.
+constexpr long long kMaxChunkRows = 0x7fffff00;          // (a chunk, and a stage more, in an int)
 constexpr double kPlanGain = 0.87, kPlanGainLong = 0.82, kPlanSecondLaunch = 0.85;
 
 Plan make_plan(bool multi_query, int b, int h, int m_max) {
@@ -307,33 +309,31 @@ Plan make_plan(bool multi_query, int b, int h, int m_max) {
     p.units = (size_t)b * h;
     p.b = b; p.h = h;
     // fixed splits of 128 rows and multiples of them, one round of the four row-warps per 128, that fit the SMs in one wave (2 x 21 x
-    // 9909 rows: 10.2 us by size, 12.9 in 156 splits for 148 SMs)
+    // 9909 rows: 10.2 us by size, 12.9 in 156 splits for 148 SMs).  (By the number of splits: a walk over the multiples of 128 rows takes
+    // as many rounds as a cache of any length has of them, and a chunk and a rounding up do not fit an int together for the longest.)
     p.kernel = h <= 16 ? Kernel::kMma1 : Kernel::kMma2;
     const int occ = h <= 16 ? MmaCfg<1>::kMinBlocks : MmaCfg<2>::kMinBlocks;
     const bool two = keeps_second_pass(m_max) && b <= 48;          // (then nothing that is one launch)
-    for (int rows = 4 * kTileRows, before = 0; search; rows += 4 * kTileRows) {
-        const int S = (m_max + rows - 1) / rows;
-        if (S != before && S <= 128 && (S == 1 || (long long)S * b <= (long long)occ * sms) && !(two && S == 1)) {
-            p.n_splits = S;
-            p.chunk_rows = ((m_max + S - 1) / S + kTileRows - 1) / kTileRows * kTileRows;
-            p.cluster = S > 1 && m_max <= kMmaMaxCluster * 256 && clusters_fit(b, S, occ) && !keeps_second_pass(m_max);
-            if ((m_max + p.chunk_rows - 1) / p.chunk_rows == S) consider(p);
-        }
-        before = S;
-        if (S == 1) break;
+    auto splits_of = [&](long long rows) { return (m_max + rows - 1) / rows; };
+    auto chunk_of = [&](int S, int step) { return ((m_max + (long long)S - 1) / S + step - 1) / step * step; };       // of S splits, whole steps
+    auto most_splits = [&](int step, long long most) { return (int)std::max(1LL, std::min(most, splits_of(step))); };
+    for (int S = most_splits(4 * kTileRows, std::min(128LL, (long long)occ * sms / b)); search && S >= 1; --S) {
+        const long long chunk = chunk_of(S, kTileRows);
+        if (splits_of(chunk_of(S, 4 * kTileRows)) != S || splits_of(chunk) != S || chunk > kMaxChunkRows || (two && S == 1)) continue;
+        p.n_splits = S;
+        p.chunk_rows = (int)chunk;
+        p.cluster = S > 1 && m_max <= kMmaMaxCluster * 256 && clusters_fit(b, S, occ) && !keeps_second_pass(m_max);
+        consider(p);
     }
     // and of whole stages on the kernel with the query rows as tile rows, one wave of CTAs
     p.kernel = Kernel::kWide;
     p.cluster = false;
-    for (int rows = kWideRows, before = 0; search; rows += kWideRows) {
-        const int S = (m_max + rows - 1) / rows;
-        if (S != before && (long long)S * b <= sms && !(two && S == 1)) {
-            p.n_splits = S;
-            p.chunk_rows = ((m_max + S - 1) / S + kWideRows - 1) / kWideRows * kWideRows;
-            if ((m_max + p.chunk_rows - 1) / p.chunk_rows == S) consider(p);
-        }
-        before = S;
-        if (S == 1) break;
+    for (int S = most_splits(kWideRows, sms / b); search && (long long)S * b <= sms && S >= 1; --S) {
+        const long long chunk = chunk_of(S, kWideRows);
+        if (splits_of(chunk) != S || chunk > kMaxChunkRows || (two && S == 1)) continue;
+        p.n_splits = S;
+        p.chunk_rows = (int)chunk;
+        consider(p);
     }
     e = Entry{sms, b, h, m_max, best};
     return best;
