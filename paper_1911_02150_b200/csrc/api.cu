@@ -159,7 +159,7 @@ Plan plan_stream(int b, int h, int m_max) {
         if (b % g == 0 || (g % b == 0 && g / b <= kMaxClusterCtas)) { p.grid = g; found = true; }
     for (int g = sms; g >= (3 * sms + 3) / 4 && !found; --g)
         if (g % b == 0) { p.grid = g; found = true; }
-    const long long tiles = (long long)b * ((m_max + kTileRows - 1) / kTileRows);
+    const long long tiles = (long long)b * (((long long)m_max + kTileRows - 1) / kTileRows);
     p.chunk_rows = (int)((tiles + p.grid - 1) / p.grid) * kTileRows;
     int parts = (p.grid + b - 1) / b + 1;
     p.n_splits = parts < p.grid ? parts : p.grid;
@@ -185,10 +185,9 @@ Plan plan_wide(int b, int h, int m_max) {
     if (want > cap) want = cap;
     if (want > 160) want = 160;                    // (the second pass merges up to 160 pieces in one go)
     if (want < 1) want = 1;
-    int chunk = (m_max + want - 1) / want;
-    chunk = (chunk + kWideRows - 1) / kWideRows * kWideRows;
-    p.chunk_rows = chunk;
-    p.n_splits = (m_max + chunk - 1) / chunk;
+    const long long chunk = (((long long)m_max + want - 1) / want + kWideRows - 1) / kWideRows * kWideRows;
+    p.chunk_rows = (int)chunk;
+    p.n_splits = (int)((m_max + chunk - 1) / chunk);
     return p;
 }
 
@@ -203,7 +202,7 @@ Plan plan_by_size(bool multi_query, int b, int h, int m_max) {
     // 103.2 -- that tile and the groups are gone.)
     if (h > 32 && (h + kWideRows - 1) / kWideRows <= 65535 && (long long)b * h < 0x7fffffffLL) return plan_wide(b, h, m_max);
     // enough tiles to give every SM a real share: the persistent kernels; otherwise fixed splits
-    const long long tiles = (long long)b * ((m_max + kTileRows - 1) / kTileRows);
+    const long long tiles = (long long)b * (((long long)m_max + kTileRows - 1) / kTileRows);
     const int sms = sm_count();
     if (b <= kStreamMaxSeqs && tiles >= 2LL * sms && m_max >= 1024 && sms <= 256) {
         const Plan p = plan_stream(b, h, m_max);

@@ -91,13 +91,13 @@ def test_sizes_that_take_no_workspace(L):
         assert binding.plan_splits(False, b, h, m)[0] == 1
 
 
-@pytest.mark.parametrize("m_max", [1 << 28, 1_073_741_825, 1_500_000_000, 2_000_000_000, 2_147_483_646])
-def test_plans_of_the_longest_caches(L, m_max):
+def test_plans_of_the_longest_caches(L):
     """Host-only questions about caches of hundreds of millions of rows are answered, and at once (in a process of its own: one that
     overflows takes it down)."""
     code = ("import time; from paper_1911_02150_b200 import binding as m; m.lib(); t = time.perf_counter()\n"
-            f"for h in (1, 16, 32): assert m.plan_splits(True, 1, h, {m_max})[0] >= 1 and m.workspace_bytes(1, h, {m_max}) >= 0\n"
-            "assert time.perf_counter() - t < 5e-3")
+            "for rows in (1 << 28, 1_073_741_825, 1_500_000_000, 2_000_000_000, 2_147_483_646):\n"
+            "    for h in (1, 16, 32, 64): assert m.plan_splits(True, 1, h, rows)[0] > 1 and m.workspace_bytes(1, h, rows) > 0\n"
+            "assert time.perf_counter() - t < 1e-2")
     subprocess.run([sys.executable, "-c", code], check=True, cwd=ROOT)
 
 
