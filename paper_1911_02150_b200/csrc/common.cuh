@@ -8,6 +8,10 @@ namespace mqa {
 constexpr int kHeadDim = 128;                 // k == v == 128 (Section 4.1: d_k = d_v = 128)
 constexpr int kRowBytes = kHeadDim * 2;       // one bf16 cache row
 constexpr float kLog2e = 1.4426950408889634f;
+// Where a running maximum of logits stands once it has seen rows, however low: (-inf) - (-inf) is NaN, and rows whose logits are -inf
+// have to weigh nothing.  A piece that holds only such rows has this maximum and a sum of 0 (one that holds no rows has -inf and 0), so
+// that nothing but such rows gives 0 / 0 and an empty prefix zeros.
+constexpr float kLowestMax = -3.402823466e38f;
 
 // status bits (mirrors include/mqa_decode.h)
 constexpr int kStatusAppendFull = 1;

@@ -300,7 +300,7 @@ __device__ __forceinline__ void tile_logits(float (&sc)[4][4], float (&top)[2], 
             mma_bf16(sc[np * 2 + 1], qa[ks], b2, b3);
         }
     }
-    top[0] = top[1] = -INFINITY;
+    top[0] = top[1] = kLowestMax;
 #pragma unroll
     for (int nt = 0; nt < 4; ++nt) {
 #pragma unroll
@@ -373,7 +373,7 @@ __device__ __forceinline__ void consume_tile(WarpState& st, const uint32_t (&qa)
         float rescale[2];
 #pragma unroll
         for (int r = 0; r < 2; ++r) {
-            const float m_new = fmaxf(st.m[r], top[r]);     // the tile's first row is valid: finite
+            const float m_new = fmaxf(st.m[r], top[r]);     // finite
             rescale[r] = fast_exp2(st.m[r] - m_new);        // 0 on the first tile, 1 if unchanged
             st.m[r] = m_new;
             st.l[r] *= rescale[r];

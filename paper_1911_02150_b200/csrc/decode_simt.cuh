@@ -92,13 +92,13 @@ decode_split_simt_kernel(const uint4* q, const uint4* __restrict__ K,
 #pragma unroll
             for (int i = 0; i < 8; ++i) s[i] += __shfl_xor_sync(0xffffffffu, s[i], off);
         }
-        float top = -INFINITY;
+        float top = kLowestMax;
 #pragma unroll
         for (int i = 0; i < 8; ++i) {
             s[i] = (base + 2 * i + half < r1) ? s[i] * kLog2e : -INFINITY;   // select, never multiply
             top = fmaxf(top, s[i]);
         }
-        top = fmaxf(top, __shfl_xor_sync(0xffffffffu, top, 16));  // row `base` is valid: finite
+        top = fmaxf(top, __shfl_xor_sync(0xffffffffu, top, 16));
         const float m_new = fmaxf(m_run, top);
         const float rescale = fast_exp2(m_run - m_new);            // 0 on the first iteration
         m_run = m_new;

@@ -885,8 +885,8 @@ mqa_decode_stream_umma_kernel(const __grid_constant__ CUtensorMap map_k, const _
                             lead = fmaxf(lead, x[i + e] - mv[e]);           // (-inf) - (-inf) = NaN is ignored by fmaxf
                         }
                     }
-                    if (named_barrier_or(1, kUmmaSoftmaxThreads, lead > kMaxLead)) {
-                        // ---- some logit leads by too much (always on a segment's first stage): every head's
+                    if (named_barrier_or(1, kUmmaSoftmaxThreads, first || lead > kMaxLead)) {
+                        // ---- some logit leads by too much, or it is a segment's first stage: every head's
                         // reference moves to the largest logit seen so far; sums and O^T are rescaled
 #pragma unroll
                         for (int c = 0; c < NCH; ++c) {
@@ -899,9 +899,9 @@ mqa_decode_stream_umma_kernel(const __grid_constant__ CUtensorMap map_k, const _
                         named_barrier(2, kUmmaSoftmaxThreads);
                         if (tid < HP) {
                             const float m_old = first ? -INFINITY : m_sm[tid];
-                            float m_new = m_old;
+                            float m_new = first ? kLowestMax : m_old;
 #pragma unroll
-                            for (int w = 0; w < 4; ++w) m_new = fmaxf(m_new, red_m[w * HP + tid]);   // finite: the stage has a valid row
+                            for (int w = 0; w < 4; ++w) m_new = fmaxf(m_new, red_m[w * HP + tid]);   // finite
                             f_sm[tid] = fast_exp2(m_old - m_new);            // 0 on the first stage, 1 if unchanged
                             m_sm[tid] = m_new;
                         }

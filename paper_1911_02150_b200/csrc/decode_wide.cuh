@@ -421,7 +421,7 @@ mqa_decode_wide_kernel(const uint4* __restrict__ q, const __grid_constant__ CUte
                 const float top = two ? fmaxf(m, other.x) : m;
                 // (a share of logits that are all -inf has that maximum and a sum of 0)
                 const float f0 = m == top ? 1.f : fast_exp2(m - top), f1 = !two ? 0.f : other.x == top ? 1.f : fast_exp2(other.x - top);
-                ml = make_float2(top, f0 * l + (two ? f1 * other.y : 0.f));
+                ml = make_float2(fmaxf(top, kLowestMax), f0 * l + (two ? f1 * other.y : 0.f));
                 const float scale = n_splits == 1 ? 1.f / ml.y : 1.f;
                 ex_ml[r] = make_float2(f0 * scale, f1 * scale);
             }

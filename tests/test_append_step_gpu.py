@@ -330,3 +330,41 @@ def test_a_prefix_whose_rows_are_partly_nan_gives_nan(variant, b, h, m_max):
             torch.cuda.synchronize()
             assert bool(torch.isnan(o).all()), f"append step, rows {rows}: {int((~torch.isnan(o)).sum())} elements are not NaN"
     assert int(status.item()) == 0
+
+
+@pytest.mark.parametrize("variant,b,h,m_max", [
+    ("mqa", 3, 8, 100), ("mqa", 12, 16, 1000), ("mqa", 20, 32, 1500), ("mqa", 8, 16, 4096), ("mqa", 4, 9, 7909),      # fixed splits: one, clusters, a second pass
+    ("mqa", 64, 16, 4096), ("mqa", 40, 32, 2100), ("mqa", 20, 24, 9000),                                             # the streaming kernel
+    ("mqa", 5, 40, 1500), ("mqa", 96, 16, 1586),                                                                     # query rows as tile rows
+    ("mha", 3, 4, 700), ("mha", 2, 16, 100),
+])
+def test_logits_of_minus_infinity_weigh_nothing(variant, b, h, m_max):
+    """Key rows whose logit is -inf for every head: single tiles and stages of them, the first ones, later ones, the last;
+    and where there are no others, 0 / 0."""
+    inp = wl.make_inputs(b, h, m_max, variant, seed=m_max, device=DEV)
+    inp["q"][..., 0] = inp["q"][..., 0].abs() + 0.125
+    lens = torch.full((b,), m_max - 1, dtype=torch.int32, device=DEV)
+    lens[b // 2] = m_max // 2
+    ws, status = mqa.alloc_workspace(b, h, m_max, DEV), torch.zeros(1, dtype=torch.int32, device=DEV)
+    valid = torch.arange(m_max, device=DEV) <= lens[:, None]
+    for rows in (slice(0, 32), slice(0, 128), slice(32, 96), slice(0, m_max // 4), slice(m_max // 3, m_max), slice(0, m_max)):
+        K, V, o = inp["K"].clone(), inp["V"].clone(), torch.empty(b, h, 128, dtype=torch.float32, device=DEV)
+        K[..., rows, 0] = -float("inf")
+        k_new = inp["k_new"].clone()
+        if rows == slice(0, m_max):
+            k_new[..., 0] = -float("inf")
+        if variant == "mqa":
+            mqa.mqa_decode_append_step(inp["q"], K, V, k_new, inp["v_new"], lens, o, ws, status, advance=False)
+        else:
+            mqa.kv_cache_append(K, V, k_new, inp["v_new"], lens, advance=False, status=status)
+            mqa.mha_decode_step(inp["q"], K, V, lens + 1, o, ws, status)
+        torch.cuda.synchronize()
+        assert int(status.item()) == 0
+        if rows == slice(0, m_max):
+            assert bool(torch.isnan(o).all())
+            continue
+        q = inp["q"].double() if variant == "mqa" else inp["q"].double().unsqueeze(2)
+        s = q @ K.double().transpose(-1, -2)                         # (the new row is in K and V by now)
+        seen = valid[:, None] if variant == "mqa" else valid[:, None, None]
+        ref = torch.softmax(s.masked_fill(~seen, -float("inf")), -1) @ V.double()
+        check_close(o.cpu().numpy(), ref.reshape(b, h, 128).cpu().numpy(), f"rows {rows}")
