@@ -120,8 +120,8 @@ __device__ __forceinline__ PfItem pf_item(int item, const int32_t* start, const 
     it.n_kv = empty ? 0 : (it.L + kPfRows - 1) / kPfRows;        // stages
     it.L0 = min(it.raw + min(pf_position(sh, it.tile0) + sh.positions, sh.n), sh.m_max);
     it.n_kv0 = empty ? 0 : (it.L0 + kPfRows - 1) / kPfRows;
-    // one rounding of the weights from the block of 128 positions on whose last one sees kSingleRoundingMinRows rows,
-    // whatever the tiles' shape
+    // one rounding of the weights where the last position of the block of 128 that the unit's FIRST tile begins in sees
+    // kSingleRoundingMinRows rows (its second tile goes with it)
     it.hilo = min(it.raw + min((pf_position(sh, it.tile0) & ~(kPfRows - 1)) + kPfRows, sh.n), sh.m_max) < kSingleRoundingMinRows;
     return it;
 }
@@ -610,8 +610,9 @@ mqa_prefill_tile_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_
     const int L = min(raw + min(p0 + sh.positions, sh.n), sh.m_max);     // rows of the memory that the tile's last position sees
     const int n_all = raw < 0 || L <= 0 ? 0 : (L + kPfRows - 1) / kPfRows;
     const int first = rank * n_all / ctas, n_kv = __shfl_sync(0xffffffffu, (rank + 1) * n_all / ctas - first, 0);   // this CTA's stages
-    // (two roundings of the weights: as pf_item says)
-    const bool hilo = __any_sync(0xffffffffu, min(raw + min((p0 & ~(kPfRows - 1)) + kPfRows, sh.n), sh.m_max) < kSingleRoundingMinRows);
+    // two roundings of the weights: by the first of the two tiles that the other kernel takes together, as pf_item does, so that a
+    // position's precision does not depend on which kernel the batch sends it to
+    const bool hilo = __any_sync(0xffffffffu, min(raw + min((pf_position(sh, tile & ~1) & ~(kPfRows - 1)) + kPfRows, sh.n), sh.m_max) < kSingleRoundingMinRows);
 
     if (warp >= 8) {
         asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(kPfRegsOther));

@@ -331,3 +331,30 @@ def test_logits_of_minus_infinity_weigh_nothing(b, h, n, m_max, start):
     K2 = K.clone()
     K2[..., 0] = -float("inf")                             # nothing else: 0 / 0
     assert bool(torch.isnan(attend(Q, K2, V, [start] * b)).all())
+
+
+@pytest.mark.parametrize("b,h,n,m_max,start", [
+    (1, 1, 1024, 1024, 0), (2, 1, 384, 1100, 640), (3, 1, 300, 1400, 800), (5, 9, 333, 1400, 600), (40, 1, 1024, 1024, 0), (70, 3, 250, 1100, 700),
+])
+def test_two_roundings_of_the_weights_up_to_the_same_position_on_either_kernel(b, h, n, m_max, start):
+    """Positions whose tile's pair begins in a block of 128 that sees fewer than 1024 rows have weights in two bf16 parts: 2^-17 of each,
+    1e-6 to 1e-5 of a row of O; one part (2^-9 of each) leaves 5e-4 and more."""
+    gen = torch.Generator(device=DEV).manual_seed(n)
+    Q = wl.bf16_normal((b, h, n, 128), 128 ** -0.5, gen, DEV)
+    K, V = wl.bf16_normal((b, m_max, 128), 1.0, gen, DEV), wl.bf16_normal((b, m_max, 128), 1.0, gen, DEV)
+    O = attend(Q, K, V, [start] * b).double()
+    hidden = torch.arange(m_max, device=DEV)[None] > start + torch.arange(n, device=DEV)[:, None]
+    two = torch.zeros(h, n, dtype=torch.bool)
+    # the tiles: of all heads x positions with up to 128 rows the fewest tiles, among equals the most positions; heads' blocks within positions'
+    heads = min(range(1, min(h, 128) + 1), key=lambda g: (-(-n // min(128 // g, n)) * -(-h // g), g))
+    positions, blocks = min(128 // heads, n), -(-h // heads)
+    for tile in range(-(-n // positions) * blocks):
+        first = (tile & ~1) // blocks * positions // 128 * 128
+        p, g = tile // blocks * positions, tile % blocks * heads
+        two[g:g + heads, p:p + positions] = start + min(first + 128, n) < 1024
+    assert bool(two.any())
+    for i in {0, b - 1}:
+        ref = torch.softmax((Q[i].double() @ K[i].double().T).masked_fill(hidden, -float("inf")), -1) @ V[i].double()
+        rel = ((O[i] - ref).norm(dim=-1) / ref.norm(dim=-1)).cpu()
+        assert float(rel[two].max()) < 1e-4
+        assert bool(two.all()) or float(rel[~two].mean()) > 3e-4      # (the border is where it is meant to be)
