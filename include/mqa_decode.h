@@ -201,9 +201,16 @@ int mha_decode_step_combine(const int32_t* lens, float* o, const void* workspace
 /*
  * mqa_workspace_bytes -- bytes of scratch that mqa_decode_step and mha_decode_step need for
  * these sizes on the current device (an upper bound valid for both; 0 if the arguments are
- * not valid).  Host-only; touches no device memory.
+ * not valid).  Host-only; touches no device memory.  Ask for the sizes of each call: the need does not grow evenly with b (a smaller
+ * batch may be cut into more pieces, and need megabytes where a larger one needs nothing).
  */
 size_t mqa_workspace_bytes(int b, int h, int m_max, int k, int v);
+
+/*
+ * mqa_workspace_bytes_up_to -- the most that mqa_workspace_bytes gives for any batch of 1 to b sequences: what one
+ * workspace needs that serves a batch which shrinks as its sequences end.  Host-only.
+ */
+size_t mqa_workspace_bytes_up_to(int b, int h, int m_max, int k, int v);
 
 /*
  * mqa_plan_splits -- the launch plan for these sizes on the current device (`multi_query`

@@ -26,7 +26,7 @@ EXPORTS = (
     "kv_cache_append", "mqa_decode_step", "mha_decode_step",
     "mqa_decode_step_split", "mqa_decode_step_combine",
     "mha_decode_step_split", "mha_decode_step_combine",
-    "mqa_workspace_bytes", "mqa_plan_splits", "mqa_plan_kernel_name", "mqa_set_wait_limit_cycles", "mqa_set_test_withhold_copy", "mqa_prefill_attention", "mqa_prefill_workspace_bytes", "mqa_status_string", "mqa_decode_step_noalloc",
+    "mqa_workspace_bytes", "mqa_workspace_bytes_up_to", "mqa_plan_splits", "mqa_plan_kernel_name", "mqa_set_wait_limit_cycles", "mqa_set_test_withhold_copy", "mqa_prefill_attention", "mqa_prefill_workspace_bytes", "mqa_status_string", "mqa_decode_step_noalloc",
     "mqa_decode_append_step", "mqa_append_step_launches",
     "mqa_layer_decode_step", "mqa_layer_workspace_bytes", "mqa_layer_cut", "mqa_decode_local_step",
     "mqa_decode_append_step_host", "mqa_host_staging_bytes",
@@ -81,6 +81,8 @@ def lib() -> ctypes.CDLL:
         L.mqa_layer_cut.restype = I
         L.mqa_workspace_bytes.argtypes = [I, I, I, I, I]
         L.mqa_workspace_bytes.restype = sz
+        L.mqa_workspace_bytes_up_to.argtypes = [I, I, I, I, I]
+        L.mqa_workspace_bytes_up_to.restype = sz
         L.mqa_plan_splits.argtypes = [I, I, I, I, I, I, ctypes.POINTER(I)]
         L.mqa_plan_splits.restype = I
         L.mqa_plan_kernel_name.argtypes = [I, I, I, I, I, I, I]
@@ -144,9 +146,9 @@ def plan_kernel_name(multi_query: bool, whole_step: bool, b: int, h: int, m_max:
 
 
 def alloc_workspace(b: int, h: int, m_max: int, device, k: int = 128, v: int = 128) -> torch.Tensor:
-    """A byte tensor large enough for both step variants at these sizes (at least 16 bytes)."""
+    """A byte tensor large enough for both step variants at these sizes, and for any smaller batch (at least 16 bytes)."""
     with torch.cuda.device(device):
-        n = workspace_bytes(b, h, m_max, k, v)
+        n = int(lib().mqa_workspace_bytes_up_to(b, h, m_max, k, v))
     return torch.empty(max(n, 16), dtype=torch.uint8, device=device)
 
 
@@ -394,7 +396,11 @@ def layer_cut(b: int, h: int, d: int):
 
 
 def alloc_layer_workspace(b: int, h: int, d: int, m_max: int, device) -> torch.Tensor:
-    return torch.empty(max(16, layer_workspace_bytes(b, h, d, m_max)), dtype=torch.uint8, device=device)
+    """A byte tensor large enough for the layer step at these sizes, and for any smaller batch."""
+    with torch.cuda.device(device):
+        n = layer_workspace_bytes(b, h, d, m_max)
+        n += n and int(lib().mqa_workspace_bytes_up_to(b, h, m_max, 128, 128))      # (all but the attention step's own part grows with b)
+    return torch.empty(max(16, n), dtype=torch.uint8, device=device)
 
 
 def mqa_layer_decode_step(x, P_q, P_k, P_v, P_o, K, V, lens, y, workspace, status=None, advance: bool = True, stream=None):

@@ -1257,6 +1257,13 @@ size_t mqa_workspace_bytes(int b, int h, int m_max, int k, int v) {
     return a > c ? a : c;
 }
 
+size_t mqa_workspace_bytes_up_to(int b, int h, int m_max, int k, int v) {
+    size_t most = 0;
+    // (a microsecond per batch size; caches of under 256 rows are never cut)
+    for (int i = m_max < 256 ? b : 1; i <= b && i > 0; ++i) most = std::max(most, mqa_workspace_bytes(i, h, m_max, k, v));
+    return most;
+}
+
 int mqa_append_step_launches(int b, int h, int m_max, int k, int v) {
     if (!dims_ok(b, h, m_max) || k != kHeadDim || v != kHeadDim) return 0;
     const Plan p = make_plan(true, b, h, m_max);

@@ -91,6 +91,17 @@ def test_sizes_that_take_no_workspace(L):
         assert binding.plan_splits(False, b, h, m)[0] == 1
 
 
+@pytest.mark.parametrize("h,m_max,b", [(32, 1024, 128), (4, 300, 64), (16, 2048, 300), (8, 200, 5000), (40, 900, 160), (24, 33000, 50)])
+def test_a_workspace_for_every_batch_up_to_the_largest(L, h, m_max, b):
+    """The need does not grow evenly with the batch (32 heads x 1024 rows: 49 sequences need some, 128 none)."""
+    each = [binding.workspace_bytes(i, h, m_max) for i in range(1, b + 1)]
+    assert L.mqa_workspace_bytes_up_to(b, h, m_max, 128, 128) == max(each)
+    assert L.mqa_workspace_bytes_up_to(0, h, m_max, 128, 128) == L.mqa_workspace_bytes_up_to(b, h, m_max, 64, 128) == 0
+    for d in (128, 1024):        # the layer step's: all but the attention step's part grows with the batch
+        largest = binding.layer_workspace_bytes(b, h, d, m_max) + max(each)
+        assert all(binding.layer_workspace_bytes(i, h, d, m_max) <= largest for i in range(1, b + 1))
+
+
 def test_plans_of_the_longest_caches(L):
     """Host-only questions about caches of hundreds of millions of rows are answered, and at once (in a process of its own: one that
     overflows takes it down)."""

@@ -433,3 +433,20 @@ def test_splits_of_a_sequence_merged_in_a_cluster(h, m_max, chained):
         assert np.array_equal(lens_t.cpu().numpy(), lens_h)
     assert int(status.item()) == 0
     assert np.array_equal(wl.bits(inp["K"]), Kh) and np.array_equal(wl.bits(inp["V"]), Vh)
+
+
+def test_one_workspace_for_a_batch_that_shrinks():
+    """A decoder allocates for its largest batch and goes on with it as sequences end (32 heads x 1024 rows: 128 sequences need no scratch,
+    fewer do)."""
+    b, h, m_max = 128, 32, 1024
+    inp = wl.make_inputs(b, h, m_max, "mqa", seed=9, device=DEV)
+    ws, status = mqa.alloc_workspace(b, h, m_max, DEV), torch.zeros(1, dtype=torch.int32, device=DEV)
+    assert mqa.workspace_bytes(49, h, m_max) > mqa.workspace_bytes(b, h, m_max)
+    for n in (128, 90, 49, 17, 3, 1):
+        lens = torch.full((n,), m_max, dtype=torch.int32, device=DEV)
+        o = torch.empty(n, h, 128, dtype=torch.float32, device=DEV)
+        mqa.mqa_decode_step(inp["q"][:n], inp["K"][:n], inp["V"][:n], lens, o, ws, status)
+        torch.cuda.synchronize()
+        ref = oracle.mqa_decode_step(wl.bits(inp["q"][:n]), wl.bits(inp["K"][:n]), wl.bits(inp["V"][:n]), lens.cpu().numpy())
+        check_close(o.cpu().numpy(), ref, f"{n} sequences left")
+    assert int(status.item()) == 0
