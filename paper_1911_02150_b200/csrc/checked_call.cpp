@@ -62,7 +62,7 @@ bool stream_for(PyObject* tensor, PyObject* given, mqa_stream_t* stream) {
         return true;
     }
     *stream = PyLong_AsVoidPtr(given);
-    return !PyErr_Occurred();
+    return !PyErr_Occurred();        // (no handle: guarded() passes the error on)
 }
 template <typename Call>
 PyObject* without_gil(Call call) {
@@ -138,7 +138,9 @@ using Fast = PyObject* (*)(PyObject*, PyObject* const*, Py_ssize_t);
 template <Fast F>
 PyObject* guarded(PyObject* self, PyObject* const* a, Py_ssize_t n) {
     try {
-        return F(self, a, n);
+        PyObject* r = F(self, a, n);
+        if (r == Py_None && PyErr_Occurred()) { Py_DECREF(r); r = nullptr; }
+        return r;
     } catch (...) {
         PyErr_Clear();
         Py_RETURN_NONE;

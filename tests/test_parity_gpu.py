@@ -501,3 +501,19 @@ def test_wrappers_by_their_native_half_and_by_their_own_checks():
         mqa.mha_decode_step(inp["q"], inp["K"], inp["V"], lens, o, torch.empty(16, dtype=torch.uint8, device=DEV), status)
     torch.cuda.synchronize()
     assert float(o.abs().max()) == 0.0
+
+
+def test_a_stream_whose_handle_is_no_integer_is_refused():
+    class Odd:
+        cuda_stream = 1.5
+
+    b, h, m = 2, 3, 64
+    inp = wl.make_inputs(b, h, m, "mqa", seed=1, device=DEV)
+    lens, o, status = torch.full((b,), 5, dtype=torch.int32, device=DEV), torch.zeros(b, h, 128, device=DEV), torch.zeros(1, dtype=torch.int32, device=DEV)
+    before = inp["K"].clone()
+    with pytest.raises(TypeError):
+        mqa.kv_cache_append(inp["K"], inp["V"], inp["k_new"], inp["v_new"], lens, status=status, stream=Odd())
+    with pytest.raises(TypeError):
+        mqa.mqa_decode_step(inp["q"], inp["K"], inp["V"], lens, o, None, status, Odd())
+    torch.cuda.synchronize()
+    assert torch.equal(inp["K"], before) and float(o.abs().max()) == 0.0 and lens.tolist() == [5, 5]
