@@ -10,6 +10,8 @@ from __future__ import annotations
 import ctypes
 import importlib.util
 import os
+import sys
+import warnings
 from typing import Optional
 
 import torch
@@ -101,22 +103,40 @@ def lib() -> ctypes.CDLL:
     return _lib
 
 
+def checked_call_path() -> str:
+    """The binding's native half (csrc/checked_call.cpp), linked to the library, for the torch and the Python at hand: it uses torch's
+    C++ interface, which another build of torch need not have, so their versions are in its name."""
+    return os.path.join(_PKG, f"checked_call-{sys.implementation.cache_tag}-torch{torch.__version__}.so")
+
+
 _native = None
+
+
+class _OwnChecks:
+    """In the native half's place where it was not built for the torch at hand: every call goes through the wrapper's own checks."""
+    @staticmethod
+    def _none(*_):
+        return None
+
+    kv_cache_append = mqa_decode_step = mha_decode_step = mqa_prefill_attention = _none
 
 
 def _checked():
     """The wrappers' native half (csrc/checked_call.cpp): its functions check a call's tensors and make the call, or return None, with
-    nothing enqueued, where a tensor is not plainly what the call takes; the wrapper's own checks then say what is wrong."""
+    nothing enqueued, where a tensor is not plainly what the call takes; the wrapper's own checks then say what is wrong.  It only
+    spares Python time, so a library that was built under another torch works without it."""
     global _native
     if _native is None:
         lib()
-        path = os.path.join(_PKG, "checked_call.so")
+        path = checked_call_path()
         if not os.path.exists(path):
-            raise ImportError(f"{path} is missing: build it with `python -m paper_1911_02150_b200.build`")
-        spec = importlib.util.spec_from_file_location("checked_call", path)
-        module = importlib.util.module_from_spec(spec)
-        spec.loader.exec_module(module)
-        _native = module
+            warnings.warn(f"{os.path.basename(path)} is missing, calls take some microseconds more: build it with `python -m {__package__}.build`")
+            _native = _OwnChecks
+        else:
+            spec = importlib.util.spec_from_file_location("checked_call", path)
+            module = importlib.util.module_from_spec(spec)
+            spec.loader.exec_module(module)
+            _native = module
     return _native
 
 

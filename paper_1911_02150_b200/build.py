@@ -13,10 +13,11 @@ import shutil
 import subprocess
 import sys
 
+from .binding import checked_call_path
+
 PKG = os.path.dirname(os.path.abspath(__file__))
 CSRC = os.path.join(PKG, "csrc")
 LIB = os.path.join(PKG, "libmqa_decode.so")
-CHECKED_CALL = os.path.join(PKG, "checked_call.so")      # the binding's native half (csrc/checked_call.cpp), linked to the library
 INCLUDE = os.path.join(os.path.dirname(PKG), "include")
 
 NVCC_FLAGS = [
@@ -38,14 +39,15 @@ def _build_checked_call() -> None:
     import sysconfig
     import torch
     root = os.path.dirname(torch.__file__)
-    tmp = CHECKED_CALL + f".tmp{os.getpid()}"
+    path = checked_call_path()
+    tmp = path + f".tmp{os.getpid()}"
     subprocess.check_call(
         ["g++", "-O2", "-shared", "-fPIC", "-std=c++17", f"-D_GLIBCXX_USE_CXX11_ABI={int(torch._C._GLIBCXX_USE_CXX11_ABI)}",
          "-isystem", os.path.join(root, "include"), "-isystem", os.path.join(root, "include", "torch", "csrc", "api", "include"),
          "-isystem", os.path.join(os.path.dirname(os.path.dirname(_nvcc())), "include"), "-I", sysconfig.get_paths()["include"],
          os.path.join(CSRC, "checked_call.cpp"), "-o", tmp, "-L", PKG, "-l:" + os.path.basename(LIB), "-Wl,-rpath,$ORIGIN",
          "-L", os.path.join(root, "lib"), "-ltorch_python", "-ltorch_cpu", "-lc10", "-lc10_cuda"])
-    os.replace(tmp, CHECKED_CALL)
+    os.replace(tmp, path)
 
 
 def sources():
@@ -53,9 +55,10 @@ def sources():
 
 
 def _stale() -> bool:
-    if not os.path.exists(LIB) or not os.path.exists(CHECKED_CALL):
+    checked = checked_call_path()
+    if not os.path.exists(LIB) or not os.path.exists(checked):
         return True
-    t = min(os.path.getmtime(LIB), os.path.getmtime(CHECKED_CALL))
+    t = min(os.path.getmtime(LIB), os.path.getmtime(checked))
     deps = glob.glob(os.path.join(CSRC, "*")) + glob.glob(os.path.join(INCLUDE, "*.h")) + [__file__]
     return any(os.path.getmtime(d) > t for d in deps)
 

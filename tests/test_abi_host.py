@@ -148,6 +148,21 @@ def test_binding_type_checks():
         binding.mqa_decode_step(q, q, q, torch.zeros(1, dtype=torch.int32), torch.zeros(1, 8, 128))
 
 
+def test_the_native_half_belongs_to_one_torch(L, monkeypatch):
+    """Under a torch that it was not built for it is not loaded, the wrappers go by their own checks, and the build is out of date."""
+    import torch
+    from paper_1911_02150_b200 import build
+    assert os.path.exists(binding.checked_call_path()) and not build._stale()
+    monkeypatch.setattr(torch, "__version__", "0.0+other")
+    monkeypatch.setattr(binding, "_native", None)
+    assert build._stale()
+    q = torch.zeros(1, 8, 128, dtype=torch.bfloat16)
+    with pytest.warns(UserWarning), pytest.raises(TypeError):
+        binding.mqa_decode_step(q, q, q, torch.zeros(1, dtype=torch.int32), torch.zeros(1, 8, 128))
+    for name in ("kv_cache_append", "mqa_decode_step", "mha_decode_step", "mqa_prefill_attention"):
+        assert getattr(binding._native, name)(q, q, None) is None
+
+
 def test_plans_of_many_query_rows_and_of_the_batched_form(L):
     """More than 32 query rows per sequence are planned on the kernel with the query rows as tile rows, and the batched
     form's workspace and refusals are answered on the host (the plan assumes the 148 SMs of a B200 without a GPU)."""
