@@ -397,6 +397,13 @@ int mqa_set_wait_limit_cycles(long long cycles);
  */
 int mqa_set_test_withhold_copy(int on);
 
+/*
+ * mqa_set_test_cluster_room -- for tests of what a device with little room does: while most >= 0, plans take it that no more than
+ * `most` thread-block clusters of the fixed-split kernel run at once (0: none, as where a part of a card cannot place one).  The
+ * plans follow it, and with them mqa_workspace_bytes and mqa_append_step_launches.  Negative: what the device says (the default).
+ */
+int mqa_set_test_cluster_room(int most);
+
 /* mqa_status_string -- a static, human-readable name for a return code. */
 const char* mqa_status_string(int code);
 

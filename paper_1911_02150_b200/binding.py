@@ -28,7 +28,7 @@ EXPORTS = (
     "kv_cache_append", "mqa_decode_step", "mha_decode_step",
     "mqa_decode_step_split", "mqa_decode_step_combine",
     "mha_decode_step_split", "mha_decode_step_combine",
-    "mqa_workspace_bytes", "mqa_workspace_bytes_up_to", "mqa_plan_splits", "mqa_plan_kernel_name", "mqa_set_wait_limit_cycles", "mqa_set_test_withhold_copy", "mqa_prefill_attention", "mqa_prefill_workspace_bytes", "mqa_status_string", "mqa_decode_step_noalloc",
+    "mqa_workspace_bytes", "mqa_workspace_bytes_up_to", "mqa_plan_splits", "mqa_plan_kernel_name", "mqa_set_wait_limit_cycles", "mqa_set_test_withhold_copy", "mqa_set_test_cluster_room", "mqa_prefill_attention", "mqa_prefill_workspace_bytes", "mqa_status_string", "mqa_decode_step_noalloc",
     "mqa_decode_append_step", "mqa_append_step_launches",
     "mqa_layer_decode_step", "mqa_layer_workspace_bytes", "mqa_layer_cut", "mqa_decode_local_step",
     "mqa_decode_append_step_host", "mqa_host_staging_bytes",
@@ -224,6 +224,11 @@ def _step_flags(advance, chained, withhold_copy=False) -> int:
 def set_test_withhold_copy(on: bool) -> None:
     """For tests: the batched form's kernel leaves one copy of its first CTA unstarted while this is on."""
     _check(lib().mqa_set_test_withhold_copy(1 if on else 0), "mqa_set_test_withhold_copy")
+
+
+def set_test_cluster_room(most: int) -> None:
+    """For tests: plans take it that at most this many clusters of the fixed-split kernel run at once (negative: what the device says)."""
+    _check(lib().mqa_set_test_cluster_room(int(most)), "mqa_set_test_cluster_room")
 
 
 def set_wait_limit_cycles(cycles: int) -> None:

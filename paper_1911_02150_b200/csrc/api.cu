@@ -45,14 +45,20 @@ int sm_count() {
 }
 
 enum class Kernel { kSimt, kMma1, kMma2, kUmma, kWide };
+std::atomic<int> g_test_cluster_room{-1};      // mqa_set_test_cluster_room
 constexpr int kMergeInKernelMaxPieces = 10;
 // Fixed splits of up to kMmaMaxCluster per sequence are one thread-block cluster that merges the pieces itself: one launch in place
 // of two.  Measured, us per step called directly (the second launch is 2 of the host's) / in a graph: 1 x 16 heads x 512 rows 6.9 / 5.1 ->
 // 4.8 / 4.9; 4 x 16 x 1000 7.6 / 5.3 -> 5.2 / 5.1; 1 x 32 x 600 8.0 / 7.5 -> 6.9 / 6.7; 30 x 8 x 900 7.9 / 7.1 -> 6.8 / 6.5; sixteen pieces
 // (clusters beyond the portable eight): 1 x 16 x 2048 8.0 / 5.3 -> 5.9 / 5.0.
 // A cluster of S CTAs has to fit one GPC, and a launch whose clusters do not all fit at once takes a second round: at one CTA per SM (17
-// to 32 heads) 10 clusters of 8 took 6.4 us where 16 took 12.2, at two per SM 24 took 5.7 and 48 12.7.
-bool clusters_fit(int sequences, int S, int ctas_per_sm) { return S <= kMmaMaxCluster && sequences <= 17 * ctas_per_sm / S * (S <= 4 ? 8 : 7); }
+// to 32 heads) 10 clusters of 8 took 6.4 us where 16 took 12.2, at two per SM 24 took 5.7 and 48 12.7.  So many as eight (of more than four
+// CTAs: seven) GPCs of 17 SMs hold, and no more than the device at hand says it can run at once, which on a part of a card may be
+// none of that size: those sizes keep the second pass.
+int mma_clusters_at_once(int S, int ctas_per_sm);
+bool clusters_fit(int sequences, int S, int ctas_per_sm) {
+    return S <= kMmaMaxCluster && sequences <= 17 * ctas_per_sm / S * (S <= 4 ? 8 : 7) && sequences <= mma_clusters_at_once(S, ctas_per_sm);
+}
 // 257 to 319 rows keep the second pass: callers count on two launches there.
 bool keeps_second_pass(int m_max) { return m_max > 256 && m_max < 320; }
 constexpr int kMaxClusterCtas = 4;            // a sequence's CTAs as one thread-block cluster.  Measured per step: clusters of 8
@@ -282,10 +288,11 @@ Plan make_plan(bool multi_query, int b, int h, int m_max) {
     if (!multi_query || h > 32 || old.kernel == Kernel::kSimt || b > kStreamMaxSeqs) return old;
     const int sms = sm_count();
     // (a decoding loop asks for the same few plans at every step)
-    struct Entry { int sms, b, h, m_max; Plan plan; };
+    struct Entry { int sms, room, b, h, m_max; Plan plan; };
     thread_local Entry kept[32] = {};
     Entry& e = kept[((unsigned)b * 7u + (unsigned)h * 31u + (unsigned)m_max) % 32u];
-    if (e.sms == sms && e.b == b && e.h == h && e.m_max == m_max) return e.plan;
+    const int room = g_test_cluster_room.load(std::memory_order_relaxed);
+    if (e.sms == sms && e.room == room && e.b == b && e.h == h && e.m_max == m_max) return e.plan;
     const double us_full = plan_us(old, m_max, 1.0, sms), us_ragged = plan_us(old, m_max, 0.5, sms);
     auto one_launch = [](const Plan& p) { return p.stream() ? p.merge_in_kernel : p.n_splits == 1 || p.cluster; };
     auto launches = [&](const Plan& p) { return one_launch(p) ? 1.0 : 1.0 / (kPlanSecondLaunch * kPlanSecondLaunch); };
@@ -334,7 +341,7 @@ Plan make_plan(bool multi_query, int b, int h, int m_max) {
         p.chunk_rows = (int)chunk;
         consider(p);
     }
-    e = Entry{sms, b, h, m_max, best};
+    e = Entry{sms, room, b, h, m_max, best};
     return best;
 }
 
@@ -511,6 +518,53 @@ bool encode_cache_map(CUtensorMap* map, const void* base, long long rows, int bo
 
 std::atomic<int> g_smem_opt_in[kMaxDevices][12];
 
+// The shared memory of an instance of the fixed-split kernel, and clusters beyond the portable size, asked for once per device.
+template <int M_TILES, int EARLY, bool CLUSTER>
+bool mma_opt_in(int dev) {
+    auto kernel = mqa_decode_split_mma_kernel<M_TILES, EARLY, CLUSTER>;
+    constexpr int kSlot = ((M_TILES - 1) * 3 + EARLY) * 2 + (CLUSTER ? 1 : 0);
+    if (g_smem_opt_in[dev][kSlot].load(std::memory_order_acquire)) return true;
+    if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, MmaCfg<M_TILES>::smem_bytes(CLUSTER)) != cudaSuccess ||
+        (CLUSTER && cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess)) {
+        cudaGetLastError();
+        return false;
+    }
+    g_smem_opt_in[dev][kSlot].store(1, std::memory_order_release);
+    return true;
+}
+
+// How many clusters of S CTAs of the fixed-split kernel the current device runs at once (asked once per device and size; any
+// number on a machine without one, where the plan assumes a whole B200).
+template <int M_TILES>
+int clusters_of(int S) {
+    static std::atomic<int> known[kMaxDevices][kMmaMaxCluster + 1];      // the answer + 1
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess) { cudaGetLastError(); return 0x7fffffff; }
+    if (dev < 0 || dev >= kMaxDevices) return 0;
+    int n = known[dev][S].load(std::memory_order_relaxed);
+    if (n > 0) return n - 1;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)S);
+    cfg.blockDim = dim3(MmaCfg<M_TILES>::kThreads);
+    cfg.dynamicSmemBytes = MmaCfg<M_TILES>::smem_bytes(true);
+    cudaLaunchAttribute attr = {};
+    attr.id = cudaLaunchAttributeClusterDimension;
+    attr.val.clusterDim.x = (unsigned)S; attr.val.clusterDim.y = 1; attr.val.clusterDim.z = 1;
+    cfg.attrs = &attr;
+    cfg.numAttrs = 1;
+    if (!mma_opt_in<M_TILES, 0, true>(dev) || cudaOccupancyMaxActiveClusters(&n, mqa_decode_split_mma_kernel<M_TILES, 0, true>, &cfg) != cudaSuccess) {
+        cudaGetLastError();
+        n = 0;
+    }
+    known[dev][S].store(n + 1, std::memory_order_relaxed);
+    return n;
+}
+int mma_clusters_at_once(int S, int ctas_per_sm) {
+    const int room = g_test_cluster_room.load(std::memory_order_relaxed);
+    if (room >= 0) return room;
+    return ctas_per_sm == MmaCfg<1>::kMinBlocks ? clusters_of<1>(S) : clusters_of<2>(S);
+}
+
 template <int M_TILES, int EARLY = 0, bool CLUSTER = false>
 int launch_mma(const Plan& p, const void* q, const void* K, const void* V, const int32_t* lens, float* o,
                float2* part_ml, float* part_acc, int32_t* status, int b, int h, int m_max, cudaStream_t stream, int len_bias,
@@ -518,18 +572,10 @@ int launch_mma(const Plan& p, const void* q, const void* K, const void* V, const
                int mode = 0) {
     using Cfg = MmaCfg<M_TILES>;
     auto kernel = mqa_decode_split_mma_kernel<M_TILES, EARLY, CLUSTER>;
-    constexpr int kSlot = ((M_TILES - 1) * 3 + EARLY) * 2 + (CLUSTER ? 1 : 0);
-    constexpr int kSmem = CLUSTER ? Cfg::kSmemBytesCluster : Cfg::kSmemBytes;
+    constexpr int kSmem = Cfg::smem_bytes(CLUSTER);
     int dev = 0;
     if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxDevices) { cudaGetLastError(); return MQA_ERR_CUDA; }
-    if (!g_smem_opt_in[dev][kSlot].load(std::memory_order_acquire)) {
-        if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmem) != cudaSuccess ||
-            (CLUSTER && cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess)) {
-            cudaGetLastError();
-            return MQA_ERR_CUDA;
-        }
-        g_smem_opt_in[dev][kSlot].store(1, std::memory_order_release);
-    }
+    if (!mma_opt_in<M_TILES, EARLY, CLUSTER>(dev)) return MQA_ERR_CUDA;
     alignas(64) CUtensorMap map_k, map_v, map_k_big, map_v_big;
     if (!encode_cache_map(&map_k, K, (long long)b * m_max) || !encode_cache_map(&map_v, V, (long long)b * m_max) ||
         !encode_cache_map(&map_k_big, K, (long long)b * m_max, 4 * kTileRows) ||
@@ -1375,6 +1421,11 @@ int mqa_prefill_attention(const void* Q, const void* K, const void* V, const int
         launch_dependent(mqa_prefill_kernel, (unsigned)(sh.n_items < sms ? sh.n_items : sms), (unsigned)kPfThreads,
                          (size_t)kPfSmemBytes, stream, map_q, map_k, map_v, start, O, status, sh);
     return launch_status();
+}
+
+int mqa_set_test_cluster_room(int most) {
+    mqa::g_test_cluster_room.store(most < 0 ? -1 : most, std::memory_order_relaxed);
+    return MQA_OK;
 }
 
 int mqa_set_test_withhold_copy(int on) {

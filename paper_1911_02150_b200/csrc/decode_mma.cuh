@@ -73,6 +73,7 @@ struct MmaCfg {                                        // fixed-split kernel
     static constexpr int kRecvRows = M_TILES * 16 + kMmaMaxCluster;
     static constexpr int kSmemBytesCluster = kSmemBytes + kRecvRows * (kHeadDim * 4 + 8);
     static_assert(2 * kStages * 8 + 8 <= 256 && kSmemBytesCluster + 64 /* static */ <= 227 * 1024, "exceeds the shared memory of one SM");
+    static constexpr int smem_bytes(bool cluster) { return cluster ? kSmemBytesCluster : kSmemBytes; }
     static constexpr int kMinBlocks = (M_TILES == 1) ? 2 : 1;
 };
 

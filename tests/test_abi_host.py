@@ -102,10 +102,27 @@ def test_a_workspace_for_every_batch_up_to_the_largest(L, h, m_max, b):
         assert all(binding.layer_workspace_bytes(i, h, d, m_max) <= largest for i in range(1, b + 1))
 
 
+def test_sizes_whose_clusters_do_not_fit_keep_the_second_pass(L):
+    """Where the device has no room for a cluster (a part of a card), the splits of a sequence are merged by a second launch."""
+    sizes = [(1, 16, 512), (4, 16, 1000), (1, 32, 600), (8, 16, 4096), (30, 8, 900)]
+    try:
+        assert [binding.append_step_launches(*s) for s in sizes] == [1] * 5
+        binding.set_test_cluster_room(0)
+        assert [binding.append_step_launches(*s) for s in sizes] == [2] * 5
+        binding.set_test_cluster_room(4)
+        assert [binding.append_step_launches(*s) for s in sizes[:3]] == [1] * 3 and binding.append_step_launches(30, 8, 900) == 2
+    finally:
+        binding.set_test_cluster_room(-1)
+    assert [binding.append_step_launches(*s) for s in sizes] == [1] * 5
+
+
 def test_plans_of_the_longest_caches(L):
     """Host-only questions about caches of hundreds of millions of rows are answered, and at once (in a process of its own: one that
     overflows takes it down)."""
-    code = ("import time; from paper_1911_02150_b200 import binding as m; m.lib(); t = time.perf_counter()\n"
+    # (a plan first: it asks the device, where there is one, for a millisecond or so.  Walking such a cache takes 11 to 80 ms a plan)
+    code = ("import time; from paper_1911_02150_b200 import binding as m\n"
+            "for h in (16, 32): m.workspace_bytes(1, h, 4096)\n"
+            "t = time.perf_counter()\n"
             "for rows in (1 << 28, 1_073_741_825, 1_500_000_000, 2_000_000_000, 2_147_483_646):\n"
             "    for h in (1, 16, 32, 64): assert m.plan_splits(True, 1, h, rows)[0] > 1 and m.workspace_bytes(1, h, rows) > 0\n"
             "assert time.perf_counter() - t < 1e-2")

@@ -450,3 +450,27 @@ def test_one_workspace_for_a_batch_that_shrinks():
         ref = oracle.mqa_decode_step(wl.bits(inp["q"][:n]), wl.bits(inp["K"][:n]), wl.bits(inp["V"][:n]), lens.cpu().numpy())
         check_close(o.cpu().numpy(), ref, f"{n} sequences left")
     assert int(status.item()) == 0
+
+
+@pytest.mark.parametrize("b,h,m_max", [(1, 16, 512), (4, 16, 1000), (3, 32, 600), (8, 16, 4096)])
+def test_without_room_for_clusters_the_second_pass_gives_the_same(b, h, m_max):
+    """The same splits by either way of merging them are the same bits; a plan made for no clusters is right as well."""
+    inp = wl.make_inputs(b, h, m_max, "mqa", seed=b + m_max, device=DEV)
+    lens0 = np.array([m_max - 1, 0, 31, m_max // 2] * b, np.int32)[:b]
+    out = []
+    for room in (-1, 0):
+        try:
+            mqa.set_test_cluster_room(room)
+            assert mqa.append_step_launches(b, h, m_max) == (1 if room else 2)
+            lens, status = torch.from_numpy(lens0).to(DEV), torch.zeros(1, dtype=torch.int32, device=DEV)
+            o, ws = torch.empty(b, h, 128, dtype=torch.float32, device=DEV), mqa.alloc_workspace(b, h, m_max, DEV)
+            mqa.mqa_decode_append_step(inp["q"], inp["K"], inp["V"], inp["k_new"], inp["v_new"], lens, o, ws, status)
+            torch.cuda.synchronize()
+            assert int(status.item()) == 0 and np.array_equal(lens.cpu().numpy(), lens0 + 1)
+            out.append((mqa.plan_splits(True, b, h, m_max), o))
+        finally:
+            mqa.set_test_cluster_room(-1)
+    ref = oracle.mqa_decode_step(wl.bits(inp["q"]), wl.bits(inp["K"]), wl.bits(inp["V"]), lens0 + 1)
+    for _, o in out:
+        check_close(o.cpu().numpy(), ref, "step")
+    assert out[0][0] != out[1][0] or torch.equal(out[0][1].view(torch.int32), out[1][1].view(torch.int32))
