@@ -59,8 +59,6 @@ int mma_clusters_at_once(int S, int ctas_per_sm);
 bool clusters_fit(int sequences, int S, int ctas_per_sm) {
     return S <= kMmaMaxCluster && sequences <= 17 * ctas_per_sm / S * (S <= 4 ? 8 : 7) && sequences <= mma_clusters_at_once(S, ctas_per_sm);
 }
-// 257 to 319 rows keep the second pass: callers count on two launches there.
-bool keeps_second_pass(int m_max) { return m_max > 256 && m_max < 320; }
 constexpr int kMaxClusterCtas = 4;            // a sequence's CTAs as one thread-block cluster.  Measured per step: clusters of 8
                                               // (16 sequences x 16384 rows) 43 us against 29 us without, clusters of 16
                                               // (8 x 32768) 43 against 30: too few of them fit the GPCs at once
@@ -143,7 +141,7 @@ Plan plan_mma(int b, int h, int m_max) {
             p.chunk_rows = chunk;
         }
     }
-    p.cluster = p.n_splits > 1 && clusters_fit(b, p.n_splits, ctas_per_sm) && !keeps_second_pass(m_max);
+    p.cluster = p.n_splits > 1 && clusters_fit(b, p.n_splits, ctas_per_sm);
     return p;
 }
 
@@ -319,16 +317,15 @@ Plan make_plan(bool multi_query, int b, int h, int m_max) {
     // as many rounds as a cache of any length has of them, and a chunk and a rounding up do not fit an int together for the longest.)
     p.kernel = h <= 16 ? Kernel::kMma1 : Kernel::kMma2;
     const int occ = h <= 16 ? MmaCfg<1>::kMinBlocks : MmaCfg<2>::kMinBlocks;
-    const bool two = keeps_second_pass(m_max) && b <= 48;          // (then nothing that is one launch)
     auto splits_of = [&](long long rows) { return (m_max + rows - 1) / rows; };
     auto chunk_of = [&](int S, int step) { return ((m_max + (long long)S - 1) / S + step - 1) / step * step; };       // of S splits, whole steps
     auto most_splits = [&](int step, long long most) { return (int)std::max(1LL, std::min(most, splits_of(step))); };
     for (int S = most_splits(4 * kTileRows, std::min(128LL, (long long)occ * sms / b)); search && S >= 1; --S) {
         const long long chunk = chunk_of(S, kTileRows);
-        if (splits_of(chunk_of(S, 4 * kTileRows)) != S || splits_of(chunk) != S || chunk > kMaxChunkRows || (two && S == 1)) continue;
+        if (splits_of(chunk_of(S, 4 * kTileRows)) != S || splits_of(chunk) != S || chunk > kMaxChunkRows) continue;
         p.n_splits = S;
         p.chunk_rows = (int)chunk;
-        p.cluster = S > 1 && m_max <= kMmaMaxCluster * 256 && clusters_fit(b, S, occ) && !keeps_second_pass(m_max);
+        p.cluster = S > 1 && m_max <= kMmaMaxCluster * 256 && clusters_fit(b, S, occ);
         consider(p);
     }
     // and of whole stages on the kernel with the query rows as tile rows, one wave of CTAs
@@ -336,10 +333,18 @@ Plan make_plan(bool multi_query, int b, int h, int m_max) {
     p.cluster = false;
     for (int S = most_splits(kWideRows, sms / b); search && (long long)S * b <= sms && S >= 1; --S) {
         const long long chunk = chunk_of(S, kWideRows);
-        if (splits_of(chunk) != S || chunk > kMaxChunkRows || (two && S == 1)) continue;
+        if (splits_of(chunk) != S || chunk > kMaxChunkRows) continue;
         p.n_splits = S;
         p.chunk_rows = (int)chunk;
         consider(p);
+    }
+    // Up to three rounds in one split are quicker than in two whose clusters crowd the SMs, which the model does not tell apart: us, full
+    // caches, two splits / one: 76 x 8 x 257 6.4 / 5.9, 90 x 8 x 384 7.3 / 7.0, 136 x 8 x 300 7.4 / 6.2, 50 x 24 x 300 7.6 / 7.0, 64 x 24 x
+    // 384 8.0 / 7.4; 74 x 8 x 300 6.0 / 6.2, 37 x 24 x 384 6.8 / 7.4, 110 x 8 x 512 8.4 / 8.2, 64 x 24 x 512 8.7 / 8.9.
+    if (best.cluster && best.n_splits == 2 && m_max <= 3 * 4 * kTileRows && 2 * b > (h <= 16 ? sms : sms / 2)) {
+        best.n_splits = 1;
+        best.chunk_rows = (m_max + kTileRows - 1) / kTileRows * kTileRows;
+        best.cluster = false;
     }
     e = Entry{sms, room, b, h, m_max, best};
     return best;

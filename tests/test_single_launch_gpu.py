@@ -34,7 +34,9 @@ def test_launch_counts():
     assert mqa.append_step_launches(32, 32, 8192) == 1        # cut into a few pieces per sequence: merged in the kernel
     assert mqa.append_step_launches(256, 16, 2048) == 1
     assert mqa.append_step_launches(1, 16, 32768) == 2        # one sequence over every SM: second-pass kernel
-    assert mqa.append_step_launches(4, 8, 300) == 2           # small, fixed splits: pass with the append inside, second pass
+    assert mqa.append_step_launches(4, 9, 7909) == 2          # many fixed splits: pass with the append inside, second pass
+    # a few of them: merged in a cluster, at every length (257 to 319 rows took two launches for a while, 256 and 320 one)
+    assert all(mqa.append_step_launches(b, 8, m) == 1 for b in (4, 48, 64) for m in (256, 257, 300, 319, 320))
 
 
 def test_workspace_contents_do_not_matter():
