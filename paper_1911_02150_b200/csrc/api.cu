@@ -47,6 +47,7 @@ int sm_count() {
 enum class Kernel { kSimt, kMma1, kMma2, kUmma, kWide };
 std::atomic<int> g_test_cluster_room{-1};      // mqa_set_test_cluster_room
 constexpr int kMergeInKernelMaxPieces = 10;
+constexpr int kFewHeads = 8;                  // FEW of the fixed-split kernel: the rows of one half of a fragment
 // Fixed splits of up to kMmaMaxCluster per sequence are one thread-block cluster that merges the pieces itself: one launch in place
 // of two.  Measured, us per step called directly (the second launch is 2 of the host's) / in a graph: 1 x 16 heads x 512 rows 6.9 / 5.1 ->
 // 4.8 / 4.9; 4 x 16 x 1000 7.6 / 5.3 -> 5.2 / 5.1; 1 x 32 x 600 8.0 / 7.5 -> 6.9 / 6.7; 30 x 8 x 900 7.9 / 7.1 -> 6.8 / 6.5; sixteen pieces
@@ -521,13 +522,13 @@ bool encode_cache_map(CUtensorMap* map, const void* base, long long rows, int bo
     return encode_matrix_map(map, base, rows, kHeadDim, box_rows);
 }
 
-std::atomic<int> g_smem_opt_in[kMaxDevices][12];
+std::atomic<int> g_smem_opt_in[kMaxDevices][24];
 
 // The shared memory of an instance of the fixed-split kernel, and clusters beyond the portable size, asked for once per device.
-template <int M_TILES, int EARLY, bool CLUSTER>
+template <int M_TILES, int EARLY, bool CLUSTER, bool FEW = false>
 bool mma_opt_in(int dev) {
-    auto kernel = mqa_decode_split_mma_kernel<M_TILES, EARLY, CLUSTER>;
-    constexpr int kSlot = ((M_TILES - 1) * 3 + EARLY) * 2 + (CLUSTER ? 1 : 0);
+    auto kernel = mqa_decode_split_mma_kernel<M_TILES, EARLY, CLUSTER, FEW>;
+    constexpr int kSlot = (((M_TILES - 1) * 3 + EARLY) * 2 + (CLUSTER ? 1 : 0)) * 2 + (FEW ? 1 : 0);
     if (g_smem_opt_in[dev][kSlot].load(std::memory_order_acquire)) return true;
     if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, MmaCfg<M_TILES>::smem_bytes(CLUSTER)) != cudaSuccess ||
         (CLUSTER && cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess)) {
@@ -570,17 +571,17 @@ int mma_clusters_at_once(int S, int ctas_per_sm) {
     return ctas_per_sm == MmaCfg<1>::kMinBlocks ? clusters_of<1>(S) : clusters_of<2>(S);
 }
 
-template <int M_TILES, int EARLY = 0, bool CLUSTER = false>
-int launch_mma(const Plan& p, const void* q, const void* K, const void* V, const int32_t* lens, float* o,
+template <int M_TILES, int EARLY, bool CLUSTER, bool FEW>
+int launch_mma_instance(const Plan& p, const void* q, const void* K, const void* V, const int32_t* lens, float* o,
                float2* part_ml, float* part_acc, int32_t* status, int b, int h, int m_max, cudaStream_t stream, int len_bias,
-               const void* k_new = nullptr, const void* v_new = nullptr, int32_t* lens_advance = nullptr,
-               int mode = 0) {
+               const void* k_new, const void* v_new, int32_t* lens_advance,
+               int mode) {
     using Cfg = MmaCfg<M_TILES>;
-    auto kernel = mqa_decode_split_mma_kernel<M_TILES, EARLY, CLUSTER>;
+    auto kernel = mqa_decode_split_mma_kernel<M_TILES, EARLY, CLUSTER, FEW>;
     constexpr int kSmem = Cfg::smem_bytes(CLUSTER);
     int dev = 0;
     if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxDevices) { cudaGetLastError(); return MQA_ERR_CUDA; }
-    if (!mma_opt_in<M_TILES, EARLY, CLUSTER>(dev)) return MQA_ERR_CUDA;
+    if (!mma_opt_in<M_TILES, EARLY, CLUSTER, FEW>(dev)) return MQA_ERR_CUDA;
     alignas(64) CUtensorMap map_k, map_v, map_k_big, map_v_big;
     if (!encode_cache_map(&map_k, K, (long long)b * m_max) || !encode_cache_map(&map_v, V, (long long)b * m_max) ||
         !encode_cache_map(&map_k_big, K, (long long)b * m_max, 4 * kTileRows) ||
@@ -597,6 +598,18 @@ int launch_mma(const Plan& p, const void* q, const void* K, const void* V, const
                      map_k_big, map_v_big, static_cast<const uint32_t*>(q), lens, o, part_ml, part_acc, status, h, m_max, p.chunk_rows,
                      p.n_splits, len_bias, fa, lens_advance, mode);
     return cudaGetLastError() == cudaSuccess ? MQA_OK : MQA_ERR_CUDA;
+}
+
+template <int M_TILES, int EARLY = 0, bool CLUSTER = false>
+int launch_mma(const Plan& p, const void* q, const void* K, const void* V, const int32_t* lens, float* o,
+               float2* part_ml, float* part_acc, int32_t* status, int b, int h, int m_max, cudaStream_t stream, int len_bias,
+               const void* k_new = nullptr, const void* v_new = nullptr, int32_t* lens_advance = nullptr,
+               int mode = 0) {
+    auto launch = launch_mma_instance<M_TILES, EARLY, CLUSTER, false>;
+    if constexpr (M_TILES == 1) {
+        if (h <= kFewHeads) launch = launch_mma_instance<M_TILES, EARLY, CLUSTER, true>;
+    }
+    return launch(p, q, K, V, lens, o, part_ml, part_acc, status, b, h, m_max, stream, len_bias, k_new, v_new, lens_advance, mode);
 }
 
 // Sequences per SM up to which a window of several tiles gives each sequence a CTA of the fixed-split kernel (us per step, a warp per

@@ -246,32 +246,46 @@ struct QueryRows {
         }
     }
 };
-// The same fragments without shared memory, for a warp that has its query rows to itself: 16 bytes per lane and load, then the
-// four lanes that share a row swap words (4 x 4 at a time).
+// The same fragments without shared memory: 16 bytes per lane and load, then the four lanes that share a row swap words (4 x 4 at
+// a time).  HALVES: 1 where there are up to eight rows (the fragments of the upper eight are zeros), else 2.
+template <int HALVES>
+struct QueryPieces {
+    uint4 v[HALVES][4];
+    __device__ __forceinline__ void load(const uint4* q, size_t row0, int rows, int lane) {
+        const int g = lane >> 2, t4 = lane & 3;
+#pragma unroll
+        for (int r = 0; r < HALVES; ++r)
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+                v[r][j] = make_uint4(0u, 0u, 0u, 0u);
+                if (g + 8 * r < rows) v[r][j] = q[(row0 + g + 8 * r) * (kRowBytes / 16) + 4 * j + t4];
+            }
+    }
+    __device__ __forceinline__ void fragments(uint32_t (&qa)[8][4], int lane) const {
+        const bool odd = (lane & 1) != 0, upper = (lane & 2) != 0;
+#pragma unroll
+        for (int r = 0; r < 2; ++r)
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+                if (r >= HALVES) {
+                    qa[2 * j][r] = qa[2 * j][2 + r] = qa[2 * j + 1][r] = qa[2 * j + 1][2 + r] = 0u;
+                    continue;
+                }
+                const uint4 a = v[r < HALVES ? r : 0][j];           // piece 4 j + t4 of the row
+                const uint32_t s0 = __shfl_xor_sync(0xffffffffu, odd ? a.x : a.y, 1), s1 = __shfl_xor_sync(0xffffffffu, odd ? a.z : a.w, 1);
+                const uint32_t b0 = odd ? s0 : a.x, b1 = odd ? a.y : s0, b2 = odd ? s1 : a.z, b3 = odd ? a.w : s1;
+                const uint32_t s2 = __shfl_xor_sync(0xffffffffu, upper ? b0 : b2, 2), s3 = __shfl_xor_sync(0xffffffffu, upper ? b1 : b3, 2);
+                qa[2 * j][r] = upper ? s2 : b0;                     // word t4 of pieces 4 j, 4 j + 1, 4 j + 2, 4 j + 3
+                qa[2 * j][2 + r] = upper ? s3 : b1;
+                qa[2 * j + 1][r] = upper ? b2 : s2;
+                qa[2 * j + 1][2 + r] = upper ? b3 : s3;
+            }
+    }
+};
 __device__ __forceinline__ void load_q_fragments(uint32_t (&qa)[8][4], const uint4* q, size_t row0, int rows, int lane) {
-    const int g = lane >> 2, t4 = lane & 3;
-    uint4 v[2][4];
-#pragma unroll
-    for (int r = 0; r < 2; ++r)
-#pragma unroll
-        for (int j = 0; j < 4; ++j) {
-            v[r][j] = make_uint4(0u, 0u, 0u, 0u);
-            if (g + 8 * r < rows) v[r][j] = q[(row0 + g + 8 * r) * (kRowBytes / 16) + 4 * j + t4];
-        }
-    const bool odd = (t4 & 1) != 0, upper = (t4 & 2) != 0;
-#pragma unroll
-    for (int r = 0; r < 2; ++r)
-#pragma unroll
-        for (int j = 0; j < 4; ++j) {
-            const uint4 a = v[r][j];                            // piece 4 j + t4 of the row
-            const uint32_t s0 = __shfl_xor_sync(0xffffffffu, odd ? a.x : a.y, 1), s1 = __shfl_xor_sync(0xffffffffu, odd ? a.z : a.w, 1);
-            const uint32_t b0 = odd ? s0 : a.x, b1 = odd ? a.y : s0, b2 = odd ? s1 : a.z, b3 = odd ? a.w : s1;
-            const uint32_t s2 = __shfl_xor_sync(0xffffffffu, upper ? b0 : b2, 2), s3 = __shfl_xor_sync(0xffffffffu, upper ? b1 : b3, 2);
-            qa[2 * j][r] = upper ? s2 : b0;                     // word t4 of pieces 4 j, 4 j + 1, 4 j + 2, 4 j + 3
-            qa[2 * j][2 + r] = upper ? s3 : b1;
-            qa[2 * j + 1][r] = upper ? b2 : s2;
-            qa[2 * j + 1][2 + r] = upper ? b3 : s3;
-        }
+    QueryPieces<2> pieces;
+    pieces.load(q, row0, rows, lane);
+    pieces.fragments(qa, lane);
 }
 // The fragments of 16 query rows at `rows_s` (a multiple of 8 rows into a box; boxes half_stride apart).
 __device__ __forceinline__ void load_q_fragments(uint32_t (&qa)[8][4], uint32_t rows_s, uint32_t half_stride, const LaneOffsets& off) {
@@ -417,8 +431,13 @@ __device__ __forceinline__ void consume_tile(WarpState& st, const uint32_t (&qa)
 //        row-warps leaves them in into the receiver's shared memory, counted on its mbarrier.  Nothing through global memory, no
 //        second launch, the same bits as the second pass.  (Instances of their own: as a run-time flag the code cost the paper's
 //        step, which does not run it, 0.1 us.)
+// FEW    up to eight query rows: each warp has them from global memory in its registers (four loads of 16 bytes per lane), without the way
+//        through shared memory and its barrier, which costs so few rows more than it saves (two fragments of four are zeros).  us, by way of
+//        shared memory / so: a loop of 5 x 1 head to 56 rows 164 / 158, 39 x 3 to 172 567 / 540, 128 x 8 to 128 481 / 468; a step of 1 x 8 x
+//        512 4.3 / 4.1, 8 x 8 x 4096 8.2 / 7.9.  (In 32 loads of 4 bytes 154, 535, 479: quicker for one head, slower from five on.  As a
+//        run-time choice in one kernel it cost every call 1 to 10 %.)
 // =============================================================================================
-template <int M_TILES, int EARLY = 0, bool CLUSTER = false>
+template <int M_TILES, int EARLY = 0, bool CLUSTER = false, bool FEW = false>
 __global__ void __launch_bounds__(MmaCfg<M_TILES>::kThreads, MmaCfg<M_TILES>::kMinBlocks)
 mqa_decode_split_mma_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_constant__ CUtensorMap map_v,
                             const __grid_constant__ CUtensorMap map_k_big, const __grid_constant__ CUtensorMap map_v_big,
@@ -538,9 +557,14 @@ mqa_decode_split_mma_kernel(const __grid_constant__ CUtensorMap map_k, const __g
     const int mt = warp % M_TILES;                         // which 16-head tile this warp serves
     const int rw = warp / M_TILES;                         // which tiles (round-robin over kRowWarps)
     QueryRows<M_TILES * 16, Cfg::kConsumerWarps * 32> rows_q;
+    QueryPieces<1> few_q;
     if (warp < Cfg::kConsumerWarps) {
-        rows_q.load(q, (size_t)seq * h, h, threadIdx.x);
-        rows_q.store(q_s, threadIdx.x);
+        if (FEW) {
+            few_q.load(reinterpret_cast<const uint4*>(q), (size_t)seq * h, h, lane);
+        } else {
+            rows_q.load(q, (size_t)seq * h, h, threadIdx.x);
+            rows_q.store(q_s, threadIdx.x);
+        }
     }
     const bool appended = fa.k_new != nullptr && raw >= 0 && (ring || raw < m_max);
     const int new_row = ring ? raw % m_max : raw;
@@ -590,8 +614,12 @@ mqa_decode_split_mma_kernel(const __grid_constant__ CUtensorMap map_k, const __g
         LaneOffsets off;
         off.init(lane);
         uint32_t qa[8][4];
-        named_barrier(1, Cfg::kConsumerWarps * 32);        // the query rows are in place
-        load_q_fragments(qa, q_s + mt * 16 * 128, M_TILES * 16 * 128, off);
+        if (FEW) {
+            few_q.fragments(qa, lane);
+        } else {
+            named_barrier(1, Cfg::kConsumerWarps * 32);    // the query rows are in place
+            load_q_fragments(qa, q_s + mt * 16 * 128, M_TILES * 16 * 128, off);
+        }
         bool ok = true;
         for (int i = rw; i < n_tiles; i += kRowWarps) {
             const int s = i % kStages;
