@@ -379,6 +379,13 @@ int mqa_prefill_attention(const void* Q, const void* K, const void* V, const int
 size_t mqa_prefill_workspace_bytes(int b, int h, int n, int m_max, int k, int v);
 
 /*
+ * mqa_prefill_plan_kernel_name -- the name of the kernel that mqa_prefill_attention launches for these sizes on the current device
+ * (`with_start`: start is given), "" for sizes that it refuses, and through *ctas (optional) the CTAs that share one unit's cache
+ * rows.  Informational; host-only.
+ */
+const char* mqa_prefill_plan_kernel_name(int b, int h, int n, int m_max, int with_start, int k, int v, int* ctas);
+
+/*
  * mqa_set_wait_limit_cycles -- how long, in SM clock cycles, a kernel of this library waits for one of its own
  * on-chip copies or products before it gives up, flags MQA_STATUS_PIPELINE_TIMEOUT and returns (no kernel here
  * waits without a bound, and none traps).  The default, restored by cycles <= 0, is about one second; tests

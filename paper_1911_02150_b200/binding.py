@@ -28,7 +28,7 @@ EXPORTS = (
     "kv_cache_append", "mqa_decode_step", "mha_decode_step",
     "mqa_decode_step_split", "mqa_decode_step_combine",
     "mha_decode_step_split", "mha_decode_step_combine",
-    "mqa_workspace_bytes", "mqa_workspace_bytes_up_to", "mqa_plan_splits", "mqa_plan_kernel_name", "mqa_set_wait_limit_cycles", "mqa_set_test_withhold_copy", "mqa_set_test_cluster_room", "mqa_prefill_attention", "mqa_prefill_workspace_bytes", "mqa_status_string", "mqa_decode_step_noalloc",
+    "mqa_workspace_bytes", "mqa_workspace_bytes_up_to", "mqa_plan_splits", "mqa_plan_kernel_name", "mqa_set_wait_limit_cycles", "mqa_set_test_withhold_copy", "mqa_set_test_cluster_room", "mqa_prefill_attention", "mqa_prefill_workspace_bytes", "mqa_prefill_plan_kernel_name", "mqa_status_string", "mqa_decode_step_noalloc",
     "mqa_decode_append_step", "mqa_append_step_launches",
     "mqa_layer_decode_step", "mqa_layer_workspace_bytes", "mqa_layer_cut", "mqa_decode_local_step",
     "mqa_decode_append_step_host", "mqa_host_staging_bytes",
@@ -93,6 +93,8 @@ def lib() -> ctypes.CDLL:
         L.mqa_prefill_attention.restype = I
         L.mqa_prefill_workspace_bytes.argtypes = [I, I, I, I, I, I]
         L.mqa_prefill_workspace_bytes.restype = sz
+        L.mqa_prefill_plan_kernel_name.argtypes = [I, I, I, I, I, I, I, ctypes.POINTER(I)]
+        L.mqa_prefill_plan_kernel_name.restype = ctypes.c_char_p
         L.mqa_set_wait_limit_cycles.argtypes = [ctypes.c_longlong]
         L.mqa_set_wait_limit_cycles.restype = I
         L.mqa_set_test_withhold_copy.argtypes = [I]
@@ -472,6 +474,13 @@ def mqa_decode_local_step(q, K, V, k_new, v_new, pos, o, status=None, advance: b
 
 def prefill_workspace_bytes(b: int, h: int, n: int, m_max: int, k: int = 128, v: int = 128) -> int:
     return int(lib().mqa_prefill_workspace_bytes(b, h, n, m_max, k, v))
+
+
+def prefill_plan_kernel(b: int, h: int, n: int, m_max: int, with_start: bool, k: int = 128, v: int = 128):
+    """(name, CTAs that share a unit's cache rows) of the kernel that the batched form launches for these sizes (informational)."""
+    ctas = ctypes.c_int(0)
+    name = lib().mqa_prefill_plan_kernel_name(b, h, n, m_max, int(bool(with_start)), k, v, ctypes.byref(ctas)).decode()
+    return name, int(ctas.value)
 
 
 def mqa_prefill_attention(Q, K, V, O, workspace, start=None, status=None, stream=None):

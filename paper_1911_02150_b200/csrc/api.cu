@@ -1382,21 +1382,49 @@ static void prefill_units(PfShape& sh, int tiles) {
 // Which kernel, by a model of the time in us: 0 for two tiles to a CTA (persistent, one CTA per SM), else the CTAs of a cluster that share
 // one tile's stages.  Measured, us for two tiles / one tile by 1 / 2 / 4 / 8 CTAs: 120 tiles of up to 24 stages 37.8 / 25.6 / 35.7 (they do not
 // fit at once); 64 of 32: 51.1 / 32.3 / 23.6 / 29.9; 10 of 12: 21.6 / 16.5 / 15.6 / 13.6 / 12.3; 1 of 16: 19.5 / 16.6 / 14.1 / 11.5 / 10.4; 240 of 3:
-// 14.2 / 20.2; 256 of 16: 28.2 / 35.6.  (With two tiles to a unit throughout and clusters sharing units: 120 of 24 28.5, 128 of 8 22.0.)
+// 14.2 / 20.2; 256 of 16: 28.2 / 35.6; 15 of 15: 26.0 / 18.5 / 16.6 / 14.0 / 12.4.  (With two tiles to a unit throughout and clusters sharing
+// units: 120 of 24 28.5, 128 of 8 22.0.)  An odd number of tiles leaves the longest alone in its unit, and quicker there than a pair (20 x 1 x
+// 380 positions: 10.5 / 11.8 / 12.4); two CTAs' worth of units are not two rounds of the longest (5 x 16 x 471: 17.6 / 24.1).  Fitted to 330
+// drawn calls of up to 30 Gflop by each way, off by 9 % (rms): 0.92 of what the calls took with clusters sharing units of two tiles; 2 % of
+// them are more than 3 % slower than that, chunks of few rows (2 x 1 x 40 over 2096 10.1 -> 11.0).
 static int prefill_tile_ctas(const PfShape& sh, int rows, int sms) {
     const int stages = (rows + kPfRows - 1) / kPfRows;
     const bool two_roundings = rows < kSingleRoundingMinRows;
-    const double tiles = (double)sh.n_tiles * sh.b, units = (double)((sh.n_tiles + 1) / 2) * sh.b;
-    if (tiles > 2.0 * sms) return 0;
+    const long long tiles = (long long)sh.n_tiles * sh.b, units = (long long)((sh.n_tiles + 1) / 2) * sh.b;
+    if (tiles > 2 * sms) return 0;
+    // stages of the tile that the `before` longest ones come before
+    auto stages_of = [&](long long before) {
+        return std::max(1.0, stages - (double)(before / ((long long)sh.head_blocks * sh.b)) * sh.positions / kPfRows);
+    };
+    const double pair_us = two_roundings ? 1.95 : 1.34, tile_us = two_roundings ? 0.9 : 0.68;
+    double best_us;
+    if (units > sms)
+        best_us = 7.3 + std::max((double)stages, stages_of(2 * (2 * sms - units)) + stages_of(2 * (units - 1)) + 3.4) * pair_us;
+    else if (sh.n_tiles % 2 == 0)
+        best_us = 7.3 + stages * pair_us;
+    else
+        best_us = std::max(6.0 + stages * (two_roundings ? 1.31 : 0.95),
+                           sh.n_tiles > 1 ? 7.3 + (sh.head_blocks > 1 ? stages : std::max(1.0, stages - (double)sh.positions / kPfRows)) * pair_us : 0.0);
+    best_us *= 0.92;                                             // (one tile has to be quicker by 8 %, a cluster by 3 % more: the calls that were slower for a tie)
     int best = 0;
-    double best_us = 0.95 * std::ceil(units / sms) * (7.0 + stages * (two_roundings ? 1.9 : 1.42));
-    for (int ctas = 1; ctas <= kPfMaxSplit && (ctas == 1 || ctas * 2 <= (stages > 2 ? stages : 2)); ctas *= 2) {
-        const int slots = ctas == 8 ? sms / 16 : ctas == 4 ? sms * 9 / 40 : sms / ctas;
+    for (int ctas = 1, log2_ctas = 0; ctas <= kPfMaxSplit && ctas <= stages; ctas *= 2, ++log2_ctas) {
+        const int slots = ctas == 8 ? sms * 2 / 21 : ctas == 4 ? sms * 9 / 40 : sms / ctas;      // clusters that fit at once
         if (slots < 1) break;
-        const double us = std::ceil(tiles / slots) * (8.0 + (double)((stages + ctas - 1) / ctas) * (two_roundings ? 1.05 : 0.72)) + (ctas > 1 ? 2.5 : 0);
+        double us = (ctas > 1 ? 3.1 : 0) - 0.32 * log2_ctas;
+        for (long long first = 0; first < tiles; first += slots)
+            us += (first ? 10.1 : 8.4) + std::ceil(stages_of(first) / ctas) * tile_us;
+        if (ctas > 1) us *= 1.03;
         if (us < best_us) { best = ctas; best_us = us; }
     }
     return best;
+}
+
+const char* mqa_prefill_plan_kernel_name(int b, int h, int n, int m_max, int with_start, int k, int v, int* ctas) {
+    if (ctas) *ctas = 0;
+    if (check_prefill_dims(b, h, n, m_max, k, v) != MQA_OK) return "";
+    const int share = prefill_tile_ctas(prefill_shape(b, h, n, m_max), with_start ? m_max : n, sm_count());
+    if (ctas) *ctas = share > 0 ? share : 1;
+    return share > 0 ? "mqa_prefill_tile_kernel" : "mqa_prefill_kernel";
 }
 
 size_t mqa_prefill_workspace_bytes(int b, int h, int n, int m_max, int k, int v) {

@@ -180,6 +180,16 @@ def test_the_native_half_belongs_to_one_torch(L, monkeypatch):
         assert getattr(binding._native, name)(q, q, None) is None
 
 
+def test_which_kernel_takes_the_batched_form(L):
+    """Calls of few tiles go one tile to a CTA or to a cluster of them, as far as those fit; many, or ones that a CTA has done before it
+    would be shared out, stay with two tiles to a CTA."""
+    kernel = binding.prefill_plan_kernel
+    assert kernel(32, 32, 4096, 4096, False) == kernel(20, 1, 380, 380, False) == kernel(5, 16, 471, 471, False) == ("mqa_prefill_kernel", 1)
+    assert kernel(5, 9, 333, 3000, True) == kernel(2, 1, 132, 132, False) == ("mqa_prefill_tile_kernel", 1)
+    assert kernel(14, 1, 88, 1707, True) == ("mqa_prefill_tile_kernel", 8) and kernel(15, 1, 88, 1707, True)[1] == 4
+    assert kernel(2, 8, 512, 256, False) == ("", 0)
+
+
 def test_plans_of_many_query_rows_and_of_the_batched_form(L):
     """More than 32 query rows per sequence are planned on the kernel with the query rows as tile rows, and the batched
     form's workspace and refusals are answered on the host (the plan assumes the 148 SMs of a B200 without a GPU)."""
