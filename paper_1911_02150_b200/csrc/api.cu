@@ -583,10 +583,16 @@ int launch_mma_instance(const Plan& p, const void* q, const void* K, const void*
     if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxDevices) { cudaGetLastError(); return MQA_ERR_CUDA; }
     if (!mma_opt_in<M_TILES, EARLY, CLUSTER, FEW>(dev)) return MQA_ERR_CUDA;
     alignas(64) CUtensorMap map_k, map_v, map_k_big, map_v_big;
-    if (!encode_cache_map(&map_k, K, (long long)b * m_max) || !encode_cache_map(&map_v, V, (long long)b * m_max) ||
-        !encode_cache_map(&map_k_big, K, (long long)b * m_max, 4 * kTileRows) ||
-        !encode_cache_map(&map_v_big, V, (long long)b * m_max, 4 * kTileRows))
+    if (!encode_cache_map(&map_k, K, (long long)b * m_max) || !encode_cache_map(&map_v, V, (long long)b * m_max)) return MQA_ERR_CUDA;
+    // four tiles per copy: never with EARLY = 1 or from chunks of under three tiles (in_groups), which then do without these two maps (a
+    // microsecond each on new buffers)
+    if (EARLY == 1 || p.chunk_rows <= 2 * kTileRows) {
+        map_k_big = map_k;
+        map_v_big = map_v;
+    } else if (!encode_cache_map(&map_k_big, K, (long long)b * m_max, 4 * kTileRows) ||
+               !encode_cache_map(&map_v_big, V, (long long)b * m_max, 4 * kTileRows)) {
         return MQA_ERR_CUDA;
+    }
     FusedArgs fa = {};
     if (k_new) {                                       // the append-and-attend step
         fa.k_new = static_cast<const uint4*>(k_new);
