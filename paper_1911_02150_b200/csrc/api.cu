@@ -307,9 +307,11 @@ Plan make_plan(bool multi_query, int b, int h, int m_max) {
         best = p;
         best_cost = full * ragged * launches(p);
     };
-    // whole clusters of more than 16 heads stay with the streaming kernel from 2048 rows on (32 x 32 x 2048: 12.7 us, 12.8 in four splits)
+    // more than 16 heads stay with the streaming kernel in whole clusters from 2048 rows on (32 x 32 x 2048: 12.7 us, 12.8 in four splits; 16 x
+    // 32 x 4096 13.9, 12.1 so) and otherwise from 3584 on, where the model has it too slow (24 x 22 x 4080: 14.8 us, 16.5 in four splits; 22
+    // x 30 x 3876 15.1 and 16.4; 20 x 32 x 3820 14.8 and 14.2)
     const bool whole = old.stream() && old.grid % b == 0 && old.grid / b <= kMaxClusterCtas;
-    const bool search = !(whole && h > 16 && m_max >= 2048);
+    const bool search = !(old.stream() && h > 16 && m_max >= (whole ? 2048 : 3584));
     Plan p;
     p.units = (size_t)b * h;
     p.b = b; p.h = h;
