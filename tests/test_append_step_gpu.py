@@ -274,7 +274,8 @@ def test_logits_of_minus_infinity_weigh_nothing_with_many_query_rows(b, h, m_max
 @pytest.mark.parametrize("b,h,m_max", [
     (70, 8, 128), (40, 16, 1000), (8, 32, 600),        # fixed splits: one, and several
     (64, 40, 300), (9, 100, 2000),                     # many rows: one split, several
-    (40, 16, 1500), (300, 8, 1024),                    # the streaming kernel
+    (40, 16, 1500),                                    # fixed splits in clusters
+    (40, 32, 2048), (90, 16, 1800), (300, 8, 1024),   # the streaming kernel, most sequences cut and few
 ])
 def test_a_loop_of_steps_back_to_back_equals_steps_one_at_a_time(b, h, m_max):
     """60 tokens, each step behind the one before with nothing waited for, its inputs put into the same buffers; 32
@@ -307,7 +308,8 @@ def test_a_loop_of_steps_back_to_back_equals_steps_one_at_a_time(b, h, m_max):
 @pytest.mark.parametrize("variant,b,h,m_max", [
     ("mqa", 70, 8, 128), ("mqa", 40, 16, 1000), ("mqa", 8, 32, 600),            # fixed splits: one, and several
     ("mqa", 64, 40, 300), ("mqa", 9, 100, 2000), ("mqa", 2, 130, 1500), ("mqa", 1, 16, 20000),   # many rows: one split, several, dozens
-    ("mqa", 40, 16, 1500), ("mqa", 32, 32, 2048), ("mqa", 300, 8, 1024),        # streaming: merged in the kernel, by clusters, mostly whole
+    ("mqa", 40, 16, 1500), ("mqa", 4, 9, 7909),                                 # fixed splits: a cluster, a second pass
+    ("mqa", 40, 32, 2048), ("mqa", 100, 16, 3000), ("mqa", 32, 32, 2048), ("mqa", 64, 16, 4096), ("mqa", 300, 8, 1024),    # streaming: merged in the kernel, by clusters, mostly whole
     ("mha", 3, 4, 700), ("mha", 1, 2, 40000),
 ])
 def test_a_prefix_whose_rows_are_partly_nan_gives_nan(variant, b, h, m_max):

@@ -127,12 +127,14 @@ def _mixed_lens(b, m_max, seed):
 # and batches just outside it (short caches, too many sequences), which take the fixed-split kernels.
 STREAM = [
     (200, 8, 1100, 21),     # ~50 tiles per SM over 1.4 sequences: every SM crosses a sequence
-    (40, 16, 1500, 22),
+    (90, 16, 1800, 22),
+    (40, 16, 1500, 22),     # (four fixed splits in a cluster)
     (150, 17, 1030, 23),    # 17..32 heads: two 16-head groups, the second nearly empty
     (1024, 4, 1024, 24),    # the most sequences the persistent kernel indexes
     (1100, 8, 64, 25),      # more than that: fixed-split kernel
     (37, 32, 4000, 26),
-    (60, 24, 1300, 27),
+    (70, 32, 3000, 27),
+    (60, 24, 1300, 27),     # (a CTA per sequence of the kernel with the query rows as tile rows)
     (40, 48, 1500, 28),     # 33..64 heads
     (33, 64, 2100, 29),
     (300, 17, 200, 30),     # short caches: fixed-split kernel
@@ -373,7 +375,7 @@ def test_empty_and_out_of_range_lengths(variant):
     assert float(o2.abs().max()) == 0.0
 
 
-@pytest.mark.parametrize("b,h,m_max", [(40, 16, 1500), (24, 96, 2048), (6, 8, 300), (3, 200, 2100)])
+@pytest.mark.parametrize("b,h,m_max", [(40, 32, 2048), (90, 16, 1800), (40, 16, 1500), (24, 96, 2048), (6, 8, 300), (4, 9, 7909), (3, 200, 2100)])
 def test_split_and_combine_phases_equal_the_step_on_every_plan(b, h, m_max):
     """The pass and the second pass on their own give the step's bits on the streaming kernel (whose step merges inside
     the kernel), on the kernel with the query rows as tile rows (one and two row tiles) and on the fixed-split kernel."""

@@ -138,12 +138,47 @@ def test_tile_shapes_and_shared_units(b, h, n, m_max, start):
 @pytest.mark.parametrize("b,h,n,m_max,start", [
     # one tile to a CTA, its stages in turn between the warpgroups and between 1, 2, 4 and 8 CTAs: one stage and two, an odd number, CTAs
     # that get none, rows that see nothing of a CTA's run, a last stage of one row, tiles of several heads partly filled
-    (3, 9, 128, 128, None), (2, 5, 129, 257, [128, 0]), (6, 20, 100, 640, [540, 0, 28, 412, 413, 29]), (1, 1, 1, 1, None), (1, 3, 1, 3000, [2999]),
+    (2, 5, 129, 257, [128, 0]), (6, 20, 100, 640, [540, 0, 28, 412, 413, 29]), (1, 3, 1, 3000, [2999]),
     (30, 4, 128, 1500, list(range(0, 1350, 45))), (9, 8, 256, 513, [257, 256, 0, 1, 100, 127, 128, 129, 200]), (1, 2, 640, 4000, [3200]),
-    (1, 148, 2, 64, [62]),
+    (20, 2, 64, 1500, list(range(0, 1400, 70))), (60, 1, 128, 2000, list(range(0, 1800, 30))),
 ])
 def test_one_tile_to_a_cta(b, h, n, m_max, start):
+    assert mqa.prefill_plan_kernel(b, h, n, m_max, start is not None)[0] == "mqa_prefill_tile_kernel"
     run(b, h, n, m_max, start, seed=2 * b + h + n)
+
+
+@pytest.mark.parametrize("b,h,n,m_max,start", [
+    # two tiles to a CTA: one stage, one tile alone in its unit; several units to a CTA, memories of one to eight stages in any order
+    (3, 9, 128, 128, None), (1, 1, 1, 1, None), (1, 148, 2, 64, [62]), (20, 16, 128, 1100, [(251 * i) % 973 for i in range(20)]),
+    (30, 12, 200, 900, [(301 * i) % 701 for i in range(30)]), (80, 5, 130, 420, [(97 * i) % 291 for i in range(80)]),
+])
+def test_two_tiles_to_a_cta(b, h, n, m_max, start):
+    assert mqa.prefill_plan_kernel(b, h, n, m_max, start is not None)[0] == "mqa_prefill_kernel"
+    run(b, h, n, m_max, start, seed=2 * b + h + n)
+
+
+def test_starts_of_all_kinds_with_two_tiles_to_a_cta():
+    """Many tiles: a negative start in the middle of the batch gives zeros, memories that would pass m_max are cut there, and the
+    sequences beside them, on the same CTAs, are not affected."""
+    b, h, n, m_max = 20, 16, 128, 600
+    assert mqa.prefill_plan_kernel(b, h, n, m_max, True)[0] == "mqa_prefill_kernel"
+    gen = torch.Generator(device=DEV).manual_seed(43)
+    Q = wl.bf16_normal((b, h, n, 128), 128 ** -0.5, gen, DEV)
+    K, V = wl.bf16_normal((b, m_max, 128), 1.0, gen, DEV), wl.bf16_normal((b, m_max, 128), 1.0, gen, DEV)
+    st = np.array([(83 * i) % 473 for i in range(b)], np.int32)
+    st[[3, 10]] = -1, -700
+    st[[5, 11, 19]] = m_max - 1, m_max - n + 3, m_max + 40
+    O = torch.full((b, h, n, 128), float("nan"), dtype=torch.float32, device=DEV)
+    status = torch.zeros(1, dtype=torch.int32, device=DEV)
+    mqa.mqa_prefill_attention(Q, K, V, O, torch.empty(16, dtype=torch.uint8, device=DEV), torch.from_numpy(st).to(DEV), status)
+    torch.cuda.synchronize()
+    assert int(status.item()) == binding.STATUS_LEN_CLAMPED
+    assert bool((O[[3, 10]] == 0).all())
+    keep = [i for i in range(b) if i not in (3, 10)]
+    for t in (0, 1, 63, 64, 100, 126, 127):
+        lens = np.clip(st + t + 1, 0, m_max).astype(np.int32)
+        ref = oracle.mqa_decode_step(wl.bits(Q[:, :, t].contiguous()), wl.bits(K), wl.bits(V), lens)
+        check_close(O[keep, :, t].cpu().numpy(), ref[keep], f"position {t}")
 
 
 def test_shared_units_with_a_negative_start_and_one_past_the_memory():

@@ -40,7 +40,9 @@ def test_launch_counts():
 
 
 def test_workspace_contents_do_not_matter():
-    shapes = [(40, 32, 2048, 1), (64, 16, 1500, 2), (33, 64, 2100, 3), (40, 32, 2048, 4)]
+    shapes = [(40, 32, 2048, 1), (90, 16, 1800, 5), (64, 16, 1500, 2), (33, 64, 2100, 3), (40, 32, 2048, 4)]
+    assert [mqa.plan_kernel_name(True, False, b, h, m).split("<")[0] for b, h, m, _ in shapes[:4]] == [
+        "mqa_decode_stream_umma_kernel", "mqa_decode_stream_umma_kernel", "mqa_decode_split_mma_kernel", "mqa_decode_wide_kernel"]
     nbytes = max(mqa.workspace_bytes(b, h, m) for b, h, m, _ in shapes)
     gen = torch.Generator(device=DEV).manual_seed(0)
     ws = torch.randint(0, 256, (nbytes,), dtype=torch.uint8, device=DEV, generator=gen)   # garbage to begin with
@@ -86,12 +88,16 @@ def test_two_shapes_whose_counters_overlap_share_one_epoch(noalloc):
         check_close(o.cpu().numpy(), ref, f"call {rnd}: b={b}")
 
 
-@pytest.mark.parametrize("b,h,m_max,rows", [(32, 16, 1024, 300), (64, 8, 1024, 100), (32, 32, 2048, 2048), (16, 32, 4096, 4000)])
+@pytest.mark.parametrize("b,h,m_max,rows", [
+    (32, 16, 4096, 300), (64, 16, 4096, 100), (64, 8, 2048, 2048), (32, 32, 2048, 2048), (16, 32, 4096, 4000), (32, 32, 2048, 300),    # streaming
+    (32, 16, 1024, 300), (64, 8, 1024, 100),                  # fixed splits: clusters of another kind
+])
 def test_equal_sequences_in_clusters(b, h, m_max, rows):
     """A batch that divides the grid is launched as clusters, and with sequences of equal length a cluster holds one
     sequence: its CTAs take the stages in turn and merge through the cluster's shared memory.  Short sequences leave
     CTAs of a cluster without a stage (300 rows are three stages for four CTAs): their empty pieces must be skipped."""
     assert mqa.append_step_launches(b, h, m_max) == 1
+    assert ("stream_umma" if m_max >= 2048 else "split_mma") in mqa.plan_kernel_name(True, True, b, h, m_max)
     inp = wl.make_inputs(b, h, m_max, "mqa", seed=b + rows, device=DEV)
     lens0 = np.full(b, rows - 1, np.int32)
     wl.poison_tail(inp["K"], lens0); wl.poison_tail(inp["V"], lens0)
@@ -183,7 +189,7 @@ def test_reference_maximum_moves_late_in_a_long_cache():
 
 
 @pytest.mark.parametrize("chained", [True, "wrong-guess"])
-@pytest.mark.parametrize("b,h,m_max", [(40, 16, 2048), (32, 32, 4096), (33, 64, 2100), (256, 8, 1100)])
+@pytest.mark.parametrize("b,h,m_max", [(40, 16, 2048), (40, 32, 2048), (90, 16, 1800), (32, 32, 4096), (33, 64, 2100), (256, 8, 1100)])
 def test_chained_steps_in_a_loop_match_unchained_ones_and_the_oracle(b, h, m_max, chained):
     """A decoding loop whose steps carry the promise that lets the kernel fetch the cache before the step ahead of it
     has finished.  lens moves under every early guess (each step advances it), prefixes cross tile and stage

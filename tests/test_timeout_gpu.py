@@ -24,16 +24,23 @@ def check_close(got, ref, what):
     assert np.all(err.max(-1) <= REL_TOL * np.abs(ref).max(-1)), f"{what}: row-relative error"
 
 
-@pytest.mark.parametrize("b,h,m_max,chained", [
-    (40, 16, 2048, False),      # persistent kernel, pieces merged through global memory
-    (32, 32, 2048, True),       # persistent kernel launched as clusters, copies started on a guess
-    (6, 8, 300, False),         # fixed-split kernel, one CTA per sequence
-    (20, 96, 2048, False),      # many query rows: the kernel with the query rows as tile rows, pieces and a second pass
-    (160, 40, 700, False),      # the same kernel, one split per sequence
-    (20, 96, 2048, True), (160, 40, 700, True),                 # ... with a stage fetched ahead of the wait
-    (6, 8, 300, True), (8, 24, 1000, True), (8, 24, 1000, False),   # fixed splits, one and several, with tiles ahead of it and without
+@pytest.mark.parametrize("b,h,m_max,chained,kernel,launches", [
+    (40, 32, 2048, False, "stream_umma_kernel<32", 1),      # persistent kernel, pieces merged through global memory
+    (100, 16, 3000, False, "stream_umma_kernel<16", 1), (100, 16, 3000, True, "stream_umma_kernel<16", 1),
+    (32, 32, 2048, True, "stream_umma_kernel<32", 1),       # persistent kernel launched as clusters, copies started on a guess
+    (64, 16, 4096, True, "stream_umma_kernel<16", 1),
+    (40, 16, 2048, False, "split_mma_kernel<1>", 1),        # fixed splits, a cluster to a sequence
+    (6, 8, 300, False, "split_mma_kernel<1>", 1),
+    (200, 8, 200, False, "split_mma_kernel<1>", 1),         # ... and one CTA to a sequence
+    (20, 96, 2048, False, "wide_kernel", 2),                # many query rows: the kernel with the query rows as tile rows, pieces and a second pass
+    (160, 40, 700, False, "wide_kernel", 1),                # the same kernel, one split per sequence
+    (20, 96, 2048, True, "wide_kernel", 2), (160, 40, 700, True, "wide_kernel", 1),                     # ... with a stage fetched ahead of the wait
+    # fixed splits, one and several, with tiles ahead of the wait and without
+    (6, 8, 300, True, "split_mma_kernel<1>", 1), (8, 24, 1000, True, "split_mma_kernel<2>", 1), (8, 24, 1000, False, "split_mma_kernel<2>", 1),
+    (200, 8, 200, True, "split_mma_kernel<1>", 1), (4, 9, 7909, True, "split_mma_kernel<1>", 2),
 ])
-def test_a_wait_that_runs_out_is_reported_and_leaves_nothing_behind(b, h, m_max, chained):
+def test_a_wait_that_runs_out_is_reported_and_leaves_nothing_behind(b, h, m_max, chained, kernel, launches):
+    assert kernel in mqa.plan_kernel_name(True, chained, b, h, m_max) and mqa.append_step_launches(b, h, m_max) == launches
     inp = wl.make_inputs(b, h, m_max, "mqa", seed=77, device=DEV)
     lens0 = np.full(b, m_max - 1, np.int32)
     lens0[1::3] = np.random.default_rng(7).integers(m_max // 2, m_max - 1, size=len(lens0[1::3]))
@@ -101,12 +108,14 @@ def test_copies_ahead_of_the_wait_behind_the_host_inputs_that_run_out(b, h, m_ma
     check_close(o.numpy(), ref, "the call after the timed-out one")
 
 
-@pytest.mark.parametrize("b,h,n,m_max,starts", [
-    (3, 4, 512, 600, [88, 0, 31]),              # one CTA per unit
-    (1, 4, 16, 2064, [2048]),                   # a cluster of CTAs per unit: the others go on to the merge
-    (5, 9, 333, 3000, [2667, 0, 100, 1300, 700]),
+@pytest.mark.parametrize("b,h,n,m_max,starts,kernel,ctas", [
+    (3, 4, 512, 600, [88, 0, 31], "mqa_prefill_tile_kernel", 1),                 # one tile to a CTA
+    (1, 4, 16, 2064, [2048], "mqa_prefill_tile_kernel", 8),                      # a cluster of CTAs per tile: the others go on to the merge
+    (5, 9, 333, 3000, [2667, 0, 100, 1300, 700], "mqa_prefill_tile_kernel", 1),
+    (20, 16, 128, 700, [(37 * i + 300) % 570 for i in range(20)], "mqa_prefill_kernel", 1),       # two tiles to a CTA, several units to each (the first has several stages)
 ])
-def test_the_batched_form_reports_a_wait_that_runs_out_and_is_correct_again_afterwards(b, h, n, m_max, starts):
+def test_the_batched_form_reports_a_wait_that_runs_out_and_is_correct_again_afterwards(b, h, n, m_max, starts, kernel, ctas):
+    assert mqa.prefill_plan_kernel(b, h, n, m_max, True) == (kernel, ctas)
     gen = torch.Generator(device=DEV).manual_seed(4)
     Q = wl.bf16_normal((b, h, n, 128), 128 ** -0.5, gen, DEV)
     K = wl.bf16_normal((b, m_max, 128), 1.0, gen, DEV)
