@@ -591,6 +591,8 @@ mqa_prefill_tile_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_
     // the tile: everything but where its sequence starts is known ahead of the wait
     const int seq = (item / sh.group) % sh.b, tile = sh.n_units - 1 - (item / (sh.group * sh.b) * sh.group + item % sh.group);
     const int p0 = pf_position(sh, tile), head0 = pf_head(sh, tile);
+    // where the block of 128 that the pair's first tile begins in ends (see hilo below)
+    const int block_end = min((pf_position(sh, tile & ~1) & ~(kPfRows - 1)) + kPfRows, sh.n);
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
@@ -612,7 +614,7 @@ mqa_prefill_tile_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_
     const int first = rank * n_all / ctas, n_kv = __shfl_sync(0xffffffffu, (rank + 1) * n_all / ctas - first, 0);   // this CTA's stages
     // two roundings of the weights: by the first of the two tiles that the other kernel takes together, as pf_item does, so that a
     // position's precision does not depend on which kernel the batch sends it to
-    const bool hilo = __any_sync(0xffffffffu, min(raw + min((pf_position(sh, tile & ~1) & ~(kPfRows - 1)) + kPfRows, sh.n), sh.m_max) < kSingleRoundingMinRows);
+    const bool hilo = __any_sync(0xffffffffu, min(raw + block_end, sh.m_max) < kSingleRoundingMinRows);
 
     if (warp >= 8) {
         asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(kPfRegsOther));
