@@ -887,7 +887,11 @@ ProjectionCut projection_cut(int b, int columns, int depth, double act_kb, doubl
         const double total = (double)columns * batch_tiles * ctas, slots = sm_count() * (two ? 2 : 1) * 0.66 * (ctas < 8 ? 1 : two ? 0.65 : 0.95);
         return (total <= slots ? 1.0 : total / slots) * (3.1 + chunks * 0.38 + rows * chunks * act_kb / 24.8 + rows * 0.5 * (ctas - 1) / ctas / 23.5);
     };
-    if (each >= 4 && best.ctas * 2 <= kProjMaxCluster && second_look(best.ctas * 2) < 0.95 * second_look(best.ctas)) best.ctas *= 2;
+    // (not five chunks of a CTA into a cluster of three and two: 240 x 4 x 640 13.3 us a layer alone, 13.7 so; and not into more clusters of
+    // eight than fit: 248 x 31 x 1152 35.3 in clusters of four, 39.9 so)
+    const bool uneven = best.ctas == 1 && each == 5;
+    const bool too_many = best.ctas * 2 == 8 && columns * batch_tiles > (two_projections_fit(best.nb, (depth + 7) / 8) ? 28 : 14);
+    if (each >= 4 && !uneven && !too_many && best.ctas * 2 <= kProjMaxCluster && second_look(best.ctas * 2) < 0.95 * second_look(best.ctas)) best.ctas *= 2;
     return best;
 }
 
