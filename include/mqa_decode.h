@@ -113,7 +113,9 @@ int kv_cache_append(void* K, void* V, const void* k_new, const void* v_new,
  * safe, and a workspace may serve calls of different shapes one after the other.  A call that
  * reported PIPELINE_TIMEOUT moves the epoch on as well: the workspace needs no repair afterwards.
  * Between two calls the caller may overwrite the whole workspace or leave it alone, but must not
- * restore an older copy of it.  Other sizes use a second kernel to combine the pieces.
+ * restore an older copy of it.  Small problems cut into up to sixteen fixed pieces per sequence are one
+ * launch too, where the device can run them so: the pieces of a sequence are the CTAs of a thread-block
+ * cluster, which merge them through their shared memory.  Other sizes use a second kernel to combine the pieces.
  */
 int mqa_decode_step(const void* q, const void* K, const void* V, const int32_t* lens, float* o,
                     void* workspace, size_t workspace_bytes, int32_t* status,
@@ -136,8 +138,9 @@ int mha_decode_step(const void* q, const void* K, const void* V, const int32_t* 
  * the lens[b] + 1 rows (as mqa_decode_step does).  For batches large enough for the persistent
  * kernel (h <= 32) the whole step is one launch: the CTA that streams a sequence's last tile
  * writes the new row before it fetches that tile, the pieces of a sequence are merged by the
- * CTA that finishes the last one, and lens is advanced once every CTA has read it.  Other
- * sizes run the same step as separate launches (mqa_append_step_launches tells how many).
+ * CTA that finishes the last one, and lens is advanced once every CTA has read it.  Small problems
+ * are one launch as well: a CTA per sequence, or a thread-block cluster of up to sixteen that merges its
+ * pieces itself.  Other sizes run the same step as separate launches (mqa_append_step_launches tells how many).
  *
  *   q, k_new, v_new   [b, h, k], [b, k], [b, v] bf16
  *   K, V              [b, m_max, k], [b, m_max, v] bf16, read-write (row lens[b] is written)
@@ -361,11 +364,12 @@ int mqa_layer_cut(int b, int h, int d, int cut[4]);
  *          for that sequence (zeros) and flagged LEN_CLAMPED, like a bad lens.
  *   O      [b, h, n, v] fp32, written           status   optional; LEN_CLAMPED, PIPELINE_TIMEOUT
  *   workspace   at least mqa_prefill_workspace_bytes(b, h, n, m_max, k, v) bytes (see below).
- * One launch of a kernel made for this form (mqa_prefill_kernel).  A unit of work is two tiles of up to 128 query rows of a
- * sequence, each some positions of some heads -- the heads share K and V, so each staged 128-row K/V tile serves 256 query rows --
- * with the query rows as the rows of the tensor-core tiles (one thread owns one query row's logits, maximum and sum), the weights
- * handed to the second product through tensor memory, and cache rows beyond a tile's last position never multiplied.  A CTA per
- * SM walks the units; a call with few units gives each a thread-block cluster, whose CTAs share the cache rows out.  (Masked
+ * One launch of one of two kernels made for this form (mqa_prefill_plan_kernel_name tells which).  A tile is up to 128 query rows
+ * of a sequence, some positions of some heads, with the query rows as the rows of the tensor-core tiles (one thread owns one query
+ * row's logits, maximum and sum), the weights handed to the second product through tensor memory, and cache rows beyond a tile's last
+ * position never multiplied.  mqa_prefill_kernel takes two tiles at a time -- the heads share K and V, so each staged 128-row K/V tile
+ * serves 256 query rows -- and a CTA per SM walks them; mqa_prefill_tile_kernel, for calls of few tiles, gives each tile a CTA, or a
+ * thread-block cluster of 2, 4 or 8 whose CTAs share the cache rows out.  (Masked
  * logits are selected away by index; the weights of a tile's later positions are zeros that are multiplied, so a NaN or Inf in a V
  * row reaches the up to 127 positions before it that share its tile, and no others.)
  * Any n >= 1 (a tile may be partly filled); k = v = 128 (MQA_ERR_UNSUPPORTED otherwise, and for
